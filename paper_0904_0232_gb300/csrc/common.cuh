@@ -85,7 +85,12 @@ struct FieldStore {
   const T* tgt[6];
   const T* kin;  // the inner layer's relaxation table (null without it)
   const uint16_t* loc;
+  const double2* met;  // FP64: the field kernels' metric table (null: evaluated in the kernels)
 };
+
+// Metric table of an FP64 context's field kernels: (G, k_x) and (k_y, k_z), G = f / (1 + f), at location l of a cell,
+// kMetricPlanes planes of ncell double2 in the order (l, half).
+constexpr int kMetricPlanes = 12;
 
 // Metric constants of the field kernels in the field type, converted once on the host (this GPU
 // converts FP64 to FP32 on its reduced-rate FP64 pipe): centre, spin, 2m, dx^4 and 4 pi / c.
@@ -121,28 +126,32 @@ struct BStepArgs {
   const T* tgt[3];
   const T* kin;
   const uint16_t* loc;
+  const double2* met;
   FieldConsts<T> K;
   T coef;
   bool inplace;
 };
 
-// E step: d_out = d + dx4 (4 pi/c J - div h(b, d*)) at advanced edge locations, d copied
-// elsewhere; d* = d + (dx4/2)(4 pi/c J - div h(b, d)) with pred, else d.  Relaxed toward tgt in
-// the absorbing layers when tgt is set.
+// E step: d_out = d + coef (4 pi/c J - div h(b, x)) at advanced edge locations, d copied elsewhere.  Time-centred: a
+// launch with x = d, coef = dx4 / 2 gives the midpoint predictor d*, a second with x = d*, coef = dx4 the new d (relaxed
+// toward tgt in the absorbing layers when tgt is set); literal: one launch with x = d, coef = dx4.
 template <typename T>
 struct EStepArgs {
   const T* b[3];
+  const T* x[3];
   const T* d[3];
   T* out[3];
   const T* tgt[3];
   const T* kin;
   const double* J[3];
   const uint16_t* loc;
+  const double2* met;
   FieldConsts<T> K;
-  bool pred;
+  T coef;
 };
 
-// Patches of a grid for the field launches: ntx x nty patches of (x, y) columns, z in chunks.
+// Patches of a grid's advanced cells [2, n-3]^3 for the field launches: ntx x nty patches of (x, y) columns, z in
+// chunks.
 struct TileGrid {
   int ntx, nty, ntz, zchunk;
   __host__ __device__ long long count() const { return (long long)ntx * nty * ntz; }
@@ -167,13 +176,17 @@ void launch_location_flags(const Grid& g, uint16_t* loc, cudaStream_t st);
 // The inner absorbing layer's relaxation over the box g.kbox0 / g.kboxn (6 values per cell).
 template <typename T>
 void launch_inner_kappa_table(const Grid& g, T* kin, cudaStream_t st);
+// The metric table of an FP64 context (kMetricPlanes planes of g.ncell double2).
+void launch_metric_table(const Grid& g, const uint16_t* loc, double2* met, cudaStream_t st);
 // B half-steps (Eq. 10) and the E step (Eq. 12); sms sizes the z chunks of the launch.
 template <typename T>
 void launch_b_step(const Grid& g, const BStepArgs<T>& A, int sms, cudaStream_t st);
 template <typename T>
 void launch_e_step(const Grid& g, const EStepArgs<T>& A, int sms, cudaStream_t st);
-// Patch tables of one instance for the batched field launches.
-void batch_field_tiles(const Grid& g, bool fp32, TileGrid* btiles, TileGrid* etiles);
+// Patches of the instances of a batch for the batched field launches (word: bytes of a field value), and the number of
+// blocks that copy an instance's outer layers (they follow its patches in the table).
+void batch_field_tiles(const Grid* const* grids, int n, size_t word, int sms, TileGrid* tiles);
+int batch_shell_blocks(const Grid& g);
 template <typename T>
 void launch_uniform_field(const Grid& g, const Fields<T>& F, const double E[3], const double B[3], cudaStream_t st);
 template <typename T>
@@ -375,7 +388,7 @@ struct InstDesc {
   FieldConsts<double> K64;
   FieldStore<T> FS;  // b[0]: b at the start of a step (b^{n-1/2}), b[1]: b^n
   int* dcur;         // device: which d buffer holds the current d
-  TileGrid btiles, etiles;
+  TileGrid tiles;
   DevStatus* st;
   SpeciesDesc<T> sp[4];
 };
@@ -383,10 +396,8 @@ struct InstDesc {
 template <typename T>
 struct BatchTables {
   const InstDesc<T>* desc;
-  const BlockEntry* btile;  // B-step patches of every instance
-  int nbtile;
-  const BlockEntry* etile;  // E-step patches
-  int netile;
+  const BlockEntry* tile;  // field patches of every instance
+  int ntile;
   const BlockEntry* all;   // all cells, 256 per block
   int nall;
   const BlockEntry* part;  // particles of (instance, species), 128 per block
@@ -399,13 +410,12 @@ struct BatchTables {
   int npairs;
   int* pair_base;          // exclusive prefix at each pair's first bin (per step)
   int persist_blocks;      // grid size of the persistent launches
-  int persist_field_blocks;  // grid size of the persistent field launches (512-thread blocks)
 };
 
 template <typename T>
 void launch_batch_b_half(const BatchTables<T>& bt, int which, bool literal, cudaStream_t st);
 template <typename T>
-void launch_batch_e_step(const BatchTables<T>& bt, bool literal, cudaStream_t st);
+void launch_batch_e_step(const BatchTables<T>& bt, int which, bool literal, cudaStream_t st);
 template <typename T>
 void launch_batch_zero_j(const BatchTables<T>& bt, cudaStream_t st);
 // flip every instance's d parity (end of a batched step)

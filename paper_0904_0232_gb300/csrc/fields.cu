@@ -5,8 +5,13 @@
 // F^z4) on edges.  Each update needs the other form of the tensor at its own lattice points:
 //   B step:  e_i = F_i4 at the d^i edges,  b_out = b_base - coef curl e(b_src, d)   (forward diff.)
 //   E step:  h = F^jk at the b faces,       d_out = d + dx4 (4 pi/c J - div h)       (backward diff.)
-// The missing components at a lattice point are the mean of the 2, 4 or 8 nearest points of
-// their own lattice; the conversion uses the metric (f, k of Eqs. 4-6) evaluated at that point.
+// The missing components at a lattice point are the mean of the 2 or 4 nearest points of
+// their own lattice; the conversion uses the metric evaluated at that point.  With g_mn = eta + f k k
+// (Eqs. 4-6), |k| = 1 and G = f / (1 + f), lowering the tensor of Eq. 8 and eliminating gives
+//   e = -d + G [k x b + d - k (k.d)],      h = b - G [b + d x k - k (k.b)]
+// (from h = [b - f d x k + f k (k.b)] / (1 + f) and e = f k x h + (f - 1) d - f k (k.d): the k (k.b) and
+// k (k.(d x k)) terms vanish in k x h).  e_L needs neither b_L nor its eight-point mean, and h splits into a
+// part of b alone and G d x k, so the E step forms the b part and G k once for its two conversions.
 //
 // One launch per update.  A block owns a 32 x BY patch of (x, y) columns and marches up z through
 // a chunk of planes: it evaluates the conversion for the whole patch of the next plane into
@@ -18,7 +23,20 @@
 // location is not advanced), except the time-centred second B half-step, which overwrites the
 // b^{n-1/2} buffer it reads only at the cell it writes.  Per cell the launch moves the
 // prognostic words once: the conversions and the predictor live in registers and shared memory,
-// and the metric is evaluated where it is needed instead of being read from memory.
+// and in FP32 the metric is evaluated where it is needed instead of being read from memory (48 B per cell and step, as
+// much as the fields themselves).  In FP64 it is read from a table (launch_metric_table): its 40 operations at each
+// of three locations are two thirds of the kernel's, and the FP64 pipe takes longer for them than HBM for 96 B
+// (B step at 96^3: 420 us evaluated, 138 us read).
+//
+// What bounds them: FP32 the issue of instructions, FP64 the FP64 pipe.  Hence sums over pairs of planes are
+// carried from one plane of the march to the next instead of being formed again, a patch synchronises once
+// (B) or twice (E) a plane, and FP64 reciprocals and roots are FastOps64's.
+// Measured (GB300, microseconds a launch, no layers; before: the E step as one march with a halo of 3, IEEE FP64
+// divides and roots, the metric evaluated in FP64, patches over all cells and chunks of at least 4 planes):
+//            FP32 64^3   128^3   192^3 (layers)   FP64 64^3   96^3
+//   B half   24 -> 14  80 -> 43     222 -> 183    425 -> 80  1053 -> 138
+//   E step   35 -> 29 140 -> 105    467 -> 458   1147 -> 193 2310 -> 349  (both launches)
+// At 128^3 FP32 moves 38 and 2 x 68 B per cell: 43 us = 1.8 TB/s, 27 % of the measured copy rate.
 #include <algorithm>
 #include <cmath>
 
@@ -43,22 +61,29 @@ __host__ __device__ constexpr int nb_hi(int t, int s, int ax) {
 }
 
 // Reciprocal square root and reciprocal: the hardware approximations in FP32 (relative error
-// ~1e-7, below the FP32 rounding of the stencil sums), IEEE operations in FP64.
+// ~1e-7, below the FP32 rounding of the stencil sums), FastOps64 in FP64.
 __device__ __forceinline__ float rsqrt_t(float v) { return rsqrtf(v); }
-__device__ __forceinline__ double rsqrt_t(double v) { return 1.0 / sqrt(v); }
+__device__ __forceinline__ double rsqrt_t(double v) { return FastOps64::rsqrt(v); }
 __device__ __forceinline__ float rcp_t(float v) { return __fdividef(1.f, v); }
-__device__ __forceinline__ double rcp_t(double v) { return 1.0 / v; }
+__device__ __forceinline__ double rcp_t(double v) { return FastOps64::rcp(v); }
+// A product that stays one (in FP64, where the metric table has to hold what the kernels would evaluate, no product is
+// left for the compiler to fuse with a sum, which it does differently from place to place).
+__device__ __forceinline__ float mul_t(float a, float b) { return a * b; }
+__device__ __forceinline__ double mul_t(double a, double b) { return __dmul_rn(a, b); }
 
+constexpr int kTX = 32;  // threads (cells) of a patch along x: one warp per row
+
+// Metric at a point.  FP32: f and k of Eqs. 4-5; FP64: G = f / (1 + f) and k.
 template <typename T>
 struct Pt {
   T f, k0, k1, k2;
 };
 
-// f and k of Eqs. 4-6 at location l of the cell whose lower corner is (xr, yr, zr) relative to the
+// Location l of the cell whose lower corner is (xr, yr, zr) relative to the
 // centre.  The quartic's root r^2 by the cancellation-free branch form with
 // D = sqrt(p^2 + 4 a^2 z^2), p = R^2 - a^2; since the root satisfies r^4 + a^2 z^2 = r^2 (2 r^2 - p)
-// = r^2 D, f = 2 m r^3 / (r^4 + a^2 z^2) = 2 m r / D.  Excised locations (and r = 0) take the flat
-// metric, as the conversions there do.
+// = r^2 D, f = 2 m r^3 / (r^4 + a^2 z^2) = 2 m r / D and G = 2 m r / (D + 2 m r).  Excised locations
+// (and r = 0) take the flat metric, as the conversions there do.
 template <typename T>
 __device__ __forceinline__ Pt<T> metric_pt(const FieldConsts<T>& K, int l, T xr, T yr, T zr, bool excised) {
   Pt<T> P;
@@ -74,30 +99,79 @@ __device__ __forceinline__ Pt<T> metric_pt(const FieldConsts<T>& K, int l, T xr,
   const T p = fma(X, X, fma(Y, Y, fma(Z, Z, -K.a2)));
   const T disc = fma(p, p, T(4) * q);
   const T rD = rsqrt_t(disc);  // 1 / D
-  const T D = disc * rD;
-  const T r2 = p >= T(0) ? T(0.5) * (p + D) : T(2) * q * rcp_t(D - p);
+  const T D = mul_t(disc, rD);
+  const T r2 = p >= T(0) ? T(0.5) * (p + D) : mul_t(T(2) * q, rcp_t(D - p));
   if (!(r2 > T(0))) return P;
   const T ir = rsqrt_t(r2);
   const T r = r2 * ir;
   const T irho2 = rcp_t(r2 + K.a2);
-  P.f = K.two_m * r * rD;
-  P.k0 = (r * X - K.a * Y) * irho2;
-  P.k1 = (r * Y + K.a * X) * irho2;
+  if constexpr (sizeof(T) == sizeof(float)) {
+    P.f = K.two_m * r * rD;
+  } else {
+    const T F = mul_t(K.two_m, r);
+    P.f = F * rcp_t(D + F);
+  }
+  P.k0 = (r * X - mul_t(K.a, Y)) * irho2;
+  P.k1 = (r * Y + mul_t(K.a, X)) * irho2;
   P.k2 = Z * ir;
   return P;
 }
 
-// Contravariant spatial F^{jk} from covariant b and contravariant d at one point (g = eta + f k k,
-// Eq. 8): lowering gives b = M h M + f (d k^T - k d^T) with M = I + f k k^T, whose solution is
-// h = [b - f (d x k) + f k (k.b)] / (1 + f) (k.(d x k) = 0 and k.k = 1, k being null for eta).
+// Metric at location l of cell c: from the FP64 table when there is one, else evaluated.
 template <typename T>
-__device__ __forceinline__ T h_comp(int q, const Pt<T>& P, const T b[3], T dxk_q, T inv1f) {
-  const T kb = P.k0 * b[0] + P.k1 * b[1] + P.k2 * b[2];
-  const T kq = q == 0 ? P.k0 : (q == 1 ? P.k1 : P.k2);
-  return (b[q] - P.f * dxk_q + P.f * kq * kb) * inv1f;
+__device__ __forceinline__ Pt<T> metric_at(const FieldConsts<T>& K, const double2* __restrict__ met, long long ncell,
+                                           long long c, int l, T xr, T yr, T zr, bool excised) {
+  if constexpr (sizeof(T) == sizeof(double)) {
+    if (met) {
+      const double2 a = __ldg(met + 2 * l * ncell + c), b = __ldg(met + (2 * l + 1) * ncell + c);
+      return Pt<T>{a.x, a.y, b.x, b.y};
+    }
+  }
+  return metric_pt<T>(K, l, xr, yr, zr, excised);
 }
 
-constexpr int kTX = 32;        // threads (cells) of a patch along x: one warp per row
+// e_L = -d_L + G [(k x b)_L + d_L - k_L (k.d)] at an edge: dL is d_L there, sdM, sdN the sums of the four
+// nearest points of the other two d components (M = L + 1, N = L + 2 mod 3), sbM, sbN the sums of the two nearest
+// points of b_M and b_N.
+template <int L, typename T>
+__device__ __forceinline__ T edge_e(const Pt<T>& P, T dL, T sdM, T sdN, T sbM, T sbN) {
+  const T kL = L == 0 ? P.k0 : (L == 1 ? P.k1 : P.k2);
+  const T kM = L == 0 ? P.k1 : (L == 1 ? P.k2 : P.k0);
+  const T kN = L == 0 ? P.k2 : (L == 1 ? P.k0 : P.k1);
+  T G = P.f;
+  if constexpr (sizeof(T) == sizeof(float)) G = P.f * rcp_t(T(1) + P.f);
+  const T kd = fma(kL, dL, T(0.25) * fma(kM, sdM, kN * sdN));
+  const T t = fma(T(0.5), fma(kM, sbN, -(kN * sbM)), fma(-kL, kd, dL));
+  return fma(G, t, -dL);
+}
+
+// h_Q at a face: bQ is b_Q there, sbM, sbN the sums of the four nearest points of the other two b components (M = Q + 1,
+// N = Q + 2 mod 3), sdM, sdN the sums of the two nearest points of d_M and d_N; (d x k)_Q = d_M k_N - d_N k_M.
+// FP64: b_Q - G [b_Q - k_Q (k.b) + (d x k)_Q].
+// FP32: [b_Q - f (d x k)_Q + f k_Q (k.b)] / (1 + f) as it stands.  Where b is large beside d (a strong
+// uniform field), d is what the differences of these h leave of their rounding to FP32, so another form of equal
+// accuracy gives another d (measured 3e-5 apart on the 64 x 64 x 128 disk set-up, each 4e-5 from FP64).
+template <int Q, typename T>
+__device__ __forceinline__ T face_h(const Pt<T>& P, T bQ, T sbM, T sbN, T sdM, T sdN) {
+  const T kQ = Q == 0 ? P.k0 : (Q == 1 ? P.k1 : P.k2);
+  const T kM = Q == 0 ? P.k1 : (Q == 1 ? P.k2 : P.k0);
+  const T kN = Q == 0 ? P.k2 : (Q == 1 ? P.k0 : P.k1);
+  if constexpr (sizeof(T) == sizeof(float)) {
+    T b[3];
+    b[Q] = bQ;
+    b[(Q + 1) % 3] = sbM * 0.25f;
+    b[(Q + 2) % 3] = sbN * 0.25f;
+    const T dM = sdM * 0.5f, dN = sdN * 0.5f;
+    const T dxk = dM * kN - dN * kM;
+    const T kb = P.k0 * b[0] + P.k1 * b[1] + P.k2 * b[2];
+    return (bQ - P.f * dxk + P.f * kQ * kb) * rcp_t(1.f + P.f);
+  } else {
+    const T kb = fma(kQ, bQ, T(0.25) * fma(kM, sbM, kN * sbN));
+    const T t = fma(T(0.5), fma(kN, sdM, -(kM * sdN)), fma(-kQ, kb, bQ));
+    return fma(-P.f, t, bQ);
+  }
+}
+
 constexpr int kSX = kTX + 2;   // staged columns: the patch and a one-cell halo
 
 // Three components of one z plane of a patch with a one-cell halo, staged in shared memory.
@@ -105,83 +179,6 @@ template <typename T, int BY>
 struct Plane3 {
   T v[3][BY + 2][kSX];
 };
-
-// Mean of the points of source lattice SL (component SL % 3 of the staged planes S) nearest to the
-// point of target lattice TL in the cell at patch position (tx, ty); the planes at z offsets -1,
-// 0, +1 sit in slots sm, sc, sp.
-template <int TL, int SL, typename T, int BY, int NS>
-__device__ __forceinline__ T avg_s(const Plane3<T, BY> (&S)[NS], int sm, int sc, int sp, int tx, int ty) {
-  constexpr int lx = nb_lo(TL, SL, 0), hx = nb_hi(TL, SL, 0);
-  constexpr int ly = nb_lo(TL, SL, 1), hy = nb_hi(TL, SL, 1);
-  constexpr int lz = nb_lo(TL, SL, 2), hz = nb_hi(TL, SL, 2);
-  constexpr int cnt = (hx - lx + 1) * (hy - ly + 1) * (hz - lz + 1);
-  T s = T(0);
-#pragma unroll
-  for (int dz = lz; dz <= hz; ++dz) {
-    const T(&P)[BY + 2][kSX] = S[dz < 0 ? sm : (dz == 0 ? sc : sp)].v[SL % 3];
-#pragma unroll
-    for (int dy = ly; dy <= hy; ++dy)
-#pragma unroll
-      for (int dx = lx; dx <= hx; ++dx) s += P[ty + 1 + dy][tx + 1 + dx];
-  }
-  if (cnt == 1) return s;
-  return s * (T(1) / T(cnt));
-}
-
-// Covariant e_L = F_L4 at the d^L edge of the cell at (tx, ty): all six components brought to the
-// edge, h as above, then e = f (k x h) + (f - 1) d - f k (k.d).
-template <int L, typename T, int BY, int NB, int ND>
-__device__ __forceinline__ T edge_e(const FieldConsts<T>& K, const Plane3<T, BY> (&Sb)[NB], int bm, int bc, int bp,
-                                    const Plane3<T, BY> (&Sd)[ND], int dm, int dc, int dp, int tx, int ty, T xr,
-                                    T yr, T zr, bool excised) {
-  T bb[3], dd[3];
-  dd[0] = avg_s<L, 0>(Sd, dm, dc, dp, tx, ty);
-  dd[1] = avg_s<L, 1>(Sd, dm, dc, dp, tx, ty);
-  dd[2] = avg_s<L, 2>(Sd, dm, dc, dp, tx, ty);
-  bb[0] = avg_s<L, 3>(Sb, bm, bc, bp, tx, ty);
-  bb[1] = avg_s<L, 4>(Sb, bm, bc, bp, tx, ty);
-  bb[2] = avg_s<L, 5>(Sb, bm, bc, bp, tx, ty);
-  const Pt<T> P = metric_pt<T>(K, L, xr, yr, zr, excised);
-  const T inv1f = rcp_t(T(1) + P.f);
-  const T dxk0 = dd[1] * P.k2 - dd[2] * P.k1;
-  const T dxk1 = dd[2] * P.k0 - dd[0] * P.k2;
-  const T dxk2 = dd[0] * P.k1 - dd[1] * P.k0;
-  const T h0 = h_comp(0, P, bb, dxk0, inv1f), h1 = h_comp(1, P, bb, dxk1, inv1f), h2 = h_comp(2, P, bb, dxk2, inv1f);
-  const T kd = P.k0 * dd[0] + P.k1 * dd[1] + P.k2 * dd[2];
-  T kxh, kL;
-  if (L == 0) {
-    kxh = P.k1 * h2 - P.k2 * h1;
-    kL = P.k0;
-  } else if (L == 1) {
-    kxh = P.k2 * h0 - P.k0 * h2;
-    kL = P.k1;
-  } else {
-    kxh = P.k0 * h1 - P.k1 * h0;
-    kL = P.k2;
-  }
-  return P.f * kxh + (P.f - T(1)) * dd[L] - P.f * kL * kd;
-}
-
-// Contravariant h_Q = F^{jk} (Q = 0: F^yz, 1: F^zx, 2: F^xy) at the b_Q face of the cell at (tx, ty):
-// the three b components (staged planes Sb, slots bm/bc/bp) and the two d components of (d x k)_Q
-// (staged planes Sd, slots dm/dc/dp) brought to the face.
-template <int Q, typename T, int BY, int NB, int ND>
-__device__ __forceinline__ T face_h(const FieldConsts<T>& K, const Plane3<T, BY> (&Sb)[NB], int bm, int bc, int bp,
-                                    const Plane3<T, BY> (&Sd)[ND], int dm, int dc, int dp, int tx, int ty, T xr,
-                                    T yr, T zr, bool excised) {
-  constexpr int L = 3 + Q;
-  T bb[3];
-  bb[0] = avg_s<L, 3>(Sb, bm, bc, bp, tx, ty);
-  bb[1] = avg_s<L, 4>(Sb, bm, bc, bp, tx, ty);
-  bb[2] = avg_s<L, 5>(Sb, bm, bc, bp, tx, ty);
-  constexpr int A = (Q + 1) % 3, B = (Q + 2) % 3;  // (d x k)_Q = d_A k_B - d_B k_A
-  const T dA = avg_s<L, A>(Sd, dm, dc, dp, tx, ty);
-  const T dB = avg_s<L, B>(Sd, dm, dc, dp, tx, ty);
-  const Pt<T> P = metric_pt<T>(K, L, xr, yr, zr, excised);
-  const T kA = A == 0 ? P.k0 : (A == 1 ? P.k1 : P.k2);
-  const T kB = B == 0 ? P.k0 : (B == 1 ? P.k1 : P.k2);
-  return h_comp(Q, P, bb, dA * kB - dB * kA, rcp_t(T(1) + P.f));
-}
 
 // 4 pi / c J^al in the field type: FP64 J rounded to FP32 with integer operations (this GPU runs
 // conversions on its reduced-rate FP64 pipe), then scaled in FP32.
@@ -245,24 +242,24 @@ __host__ __device__ __forceinline__ long long kin_index(const Grid& g, int l, in
          (i - g.kbox0[0]);
 }
 
-// v relaxed toward the target t at location l of cell (i, j, k) with flags w: t + (1 - kappa)(v - t).
+// v relaxed toward the target t at location l of cell (i, j, k) with flags w and outer relaxation k_outer:
+// t + (1 - kappa)(v - t).
 template <typename T>
-__device__ __forceinline__ T relax(const Grid& g, const T* kin, uint16_t w, T t, T v, int l, int i, int j, int k) {
-  T kap = outer_kappa<T>(g, i, j, k);
+__device__ __forceinline__ T relax(const Grid& g, const T* kin, uint16_t w, T k_outer, T t, T v, int l, int i, int j,
+                                   int k) {
+  T kap = k_outer;
   if (w & kInnerBit) kap = fmax(kap, __ldg(kin + kin_index(g, l, i, j, k)));
   return t + (T(1) - kap) * (v - t);
 }
 
-// Asynchronous 4- or 8-byte copy global -> shared (zero-filled when ok is false: no bytes are read
-// then, and src is only a valid address), and the commit / wait of the thread's copy groups.
+// Asynchronous 4- or 8-byte copy global -> shared, and the commit / wait of the thread's copy groups.
 template <typename T>
-__device__ __forceinline__ void cp_async(T* dst, const T* src, bool ok) {
+__device__ __forceinline__ void cp_async(T* dst, const T* src) {
   const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-  const int n = ok ? (int)sizeof(T) : 0;
   if constexpr (sizeof(T) == 4)
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;\n" ::"r"(d), "l"(src), "r"(n) : "memory");
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(d), "l"(src) : "memory");
   else
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"(d), "l"(src), "r"(n) : "memory");
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(d), "l"(src) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 // wait until at most N of this thread's most recent copy groups are still in flight
@@ -273,54 +270,45 @@ __device__ __forceinline__ void cp_async_wait() {
 
 // The staged halo patch of a block: (BY + 2) x kSX elements, at most two per thread (threads
 // 32 x BY); element e of the patch is column e % kSX, row e / kSX, at grid (x0 - 1 + column,
-// y0 - 1 + row) where (x0, y0) is the grid position of thread (0, 0).
+// y0 - 1 + row) where (x0, y0) is the grid position of thread (0, 0).  Positions outside the grid, on any axis,
+// take the nearest one inside: only cells of the outer index layer reach them, and those are not converted.
 template <int BY>
 struct Stager {
-  int n;
-  int sx[2], sy[2];
-  int off[2];    // x + y nx of the element, or -1 outside the grid
+  int s0, s1;       // element in a staged component; s1 < 0: this thread stages one element only
+  unsigned o0, o1;  // x + y nx of the element
   __device__ Stager(const Grid& g, int x0, int y0) {
     const int t = threadIdx.y * kTX + threadIdx.x;
-    n = 0;
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-      const int e = t + k * kTX * BY;
-      sx[k] = sy[k] = 0;
-      off[k] = -1;
-      if (e < (BY + 2) * kSX) {
-        n = k + 1;
-        sx[k] = e % kSX;
-        sy[k] = e / kSX;
-        const int x = x0 - 1 + sx[k], y = y0 - 1 + sy[k];
-        if (x >= 0 && x < g.nx && y >= 0 && y < g.ny) off[k] = x + y * g.nx;
-      }
-    }
+    auto off = [&](int e) {
+      const int x = min(max(x0 - 1 + e % kSX, 0), g.nx - 1), y = min(max(y0 - 1 + e / kSX, 0), g.ny - 1);
+      return (unsigned)(x + y * g.nx);
+    };
+    s0 = t;
+    o0 = off(t);
+    s1 = t + kTX * BY < (BY + 2) * kSX ? t + kTX * BY : -1;
+    o1 = off(max(s1, 0));
   }
-  // start copying plane p of the three arrays src into dst (zeros outside the grid)
+  // start copying plane p of the three arrays src into dst
   template <typename T>
   __device__ __forceinline__ void stage(const Grid& g, const T* const* src, int p, Plane3<T, BY>& dst) const {
-    const bool zin = p >= 0 && p < g.nz;
-    const long long pz = zin ? (long long)p * g.nx * g.ny : 0;
+    const long long pz = (long long)min(max(p, 0), g.nz - 1) * g.nx * g.ny;
 #pragma unroll
-    for (int k = 0; k < 2; ++k) {
-      if (k < n) {
-        const bool ok = zin && off[k] >= 0;
-        const long long o = ok ? pz + off[k] : 0;
-#pragma unroll
-        for (int q = 0; q < 3; ++q) cp_async(&dst.v[q][sy[k]][sx[k]], src[q] + o, ok);
-      }
+    for (int q = 0; q < 3; ++q) {
+      const T* const plane = src[q] + pz;
+      T* const to = &dst.v[q][0][0];
+      cp_async(to + s0, plane + o0);
+      if (s1 >= 0) cp_async(to + s1, plane + o1);
     }
   }
 };
 
 // ---- B half-step ------------------------------------------------------------------------------
-// Patch: threads (tx, ty) at x = x0 + tx, y = y0 + ty; b and d of planes P-1..P+1 staged (three
-// rotating slots), e at the patch of each plane P of the chunk and of the plane above it; cells
-// with tx < 31 and ty < BY - 1 are updated (the curl reaches +1).
-// b keeps five planes (P - 1 .. P + 1 for e, P - 1 for the update, P + 2 in flight), d four.
+// Patch: threads (tx, ty) at x = x0 + tx, y = y0 + ty; e at the patch of each plane P of the chunk and of
+// the plane above it; cells with tx < 31 and ty < BY - 1 are updated (the curl reaches +1).  Iteration P reads the
+// staged planes P and P + 1 (P + 2 in flight), the sums over plane P - 1 are carried in registers, and e of plane
+// P - 1 is in the other half of E: one barrier a plane.
 template <typename T, int BY>
 struct BStepSmem {
-  Plane3<T, BY> Sb[5], Sd[4];
+  Plane3<T, BY> Sb[4], Sd[4];
   T E[2][3][BY][kTX];
 };
 
@@ -328,300 +316,346 @@ template <typename T, int BY>
 __device__ __forceinline__ void b_step_tile(const Grid& g, const BStepArgs<T>& A, int tile_x, int tile_y, int zs,
                                             int ze, BStepSmem<T, BY>& sm) {
   const int tx = threadIdx.x, ty = threadIdx.y;
-  const int x0 = tile_x * (kTX - 1), y0 = tile_y * (BY - 1);
+  const int cx = tx + 1, cy = ty + 1;  // the cell in the staged planes
+  const int x0 = 2 + tile_x * (kTX - 1), y0 = 2 + tile_y * (BY - 1);
   const int x = x0 + tx, y = y0 + ty;
   const bool in_xy = x < g.nx && y < g.ny;
   const bool conv_xy = x >= 1 && x <= g.nx - 2 && y >= 1 && y <= g.ny - 2;
-  const bool out_xy = in_xy && tx < kTX - 1 && ty < BY - 1;
+  const bool out_xy = x <= g.nx - 3 && y <= g.ny - 3 && tx < kTX - 1 && ty < BY - 1;
   const T xr = (T)x - A.K.xc, yr = (T)y - A.K.yc;
   const Stager<BY> st(g, x0, y0);
-  auto sb = [](int p) { return (p + 5) % 5; };
-  auto sd = [](int p) { return (p + 4) & 3; };
-  // planes zs - 1 .. zs + 1 in one copy group; each iteration P starts plane P + 2
   for (int q = zs - 1; q <= zs + 1; ++q) {
-    st.stage(g, A.src, q, sm.Sb[sb(q)]);
-    st.stage(g, A.d, q, sm.Sd[sd(q)]);
+    st.stage(g, A.src, q, sm.Sb[q & 3]);
+    st.stage(g, A.d, q, sm.Sd[q & 3]);
   }
   cp_async_commit();
-  const long long splane = (long long)g.nx * g.ny;
-  uint16_t w_prev = 0;  // flags of plane P - 1, loaded one iteration ahead
+  cp_async_wait<0>();
+  __syncthreads();
+  // carried from plane P - 1: d_z summed over the x and the y pair, b; from plane P: d_x, d_y and their sums with
+  // the neighbour below in x and in y
+  T d2x_m, d2y_m, b_m[3], d0, d0x, d1, d1y;
+  {
+    const Plane3<T, BY>&B = sm.Sb[(zs - 1) & 3], &D = sm.Sd[(zs - 1) & 3], &C = sm.Sd[zs & 3];
+    d2x_m = D.v[2][cy][cx] + D.v[2][cy][cx + 1];
+    d2y_m = D.v[2][cy][cx] + D.v[2][cy + 1][cx];
+#pragma unroll
+    for (int q = 0; q < 3; ++q) b_m[q] = B.v[q][cy][cx];
+    d0 = C.v[0][cy][cx];
+    d0x = d0 + C.v[0][cy][cx - 1];
+    d1 = C.v[1][cy][cx];
+    d1y = d1 + C.v[1][cy - 1][cx];
+  }
+  T em[3] = {T(0), T(0), T(0)};  // e of plane P - 1 at the cell
+  const int splane = g.nx * g.ny;
+  long long cP = ((long long)zs * g.ny + y) * g.nx + x;  // the cell in plane P
+  T zr = (T)zs - A.K.zc;
+  // loaded one iteration ahead: the flags of plane P + 1 and, for the in-place update, b^{n-1/2} of plane P
+  uint16_t w_prev = 0, w = in_xy ? __ldg(A.loc + cP) : (uint16_t)0;
+  T old_next[3] = {T(0), T(0), T(0)};
   for (int P = zs; P <= ze; ++P) {
-    st.stage(g, A.src, P + 2, sm.Sb[sb(P + 2)]);
-    st.stage(g, A.d, P + 2, sm.Sd[sd(P + 2)]);
+    if (P < ze) {
+      st.stage(g, A.src, P + 2, sm.Sb[(P + 2) & 3]);
+      st.stage(g, A.d, P + 2, sm.Sd[(P + 2) & 3]);
+    }
     cp_async_commit();
-    // loads of this iteration issued ahead of the waits: the flags of plane P and, for the in-place
-    // update of plane P - 1, its b^{n-1/2}
-    const long long cP = ((long long)P * g.ny + y) * g.nx + x;
-    const uint16_t w_cur = (in_xy && P < g.nz) ? __ldg(A.loc + cP) : (uint16_t)0;
+    const uint16_t w_next = in_xy && P < ze ? __ldg(A.loc + cP + splane) : (uint16_t)0;
     const int p = P - 1;
     const bool upd = p >= zs && out_xy;
-    T base_old[3] = {T(0), T(0), T(0)};
-    if (A.inplace && upd) {
+    T old[3] = {b_m[0], b_m[1], b_m[2]};
+    if (A.inplace) {
 #pragma unroll
-      for (int q = 0; q < 3; ++q) base_old[q] = A.base[q][cP - splane];
+      for (int q = 0; q < 3; ++q) {
+        old[q] = old_next[q];
+        if (out_xy && P < ze) old_next[q] = A.base[q][cP];
+      }
     }
     cp_async_wait<1>();  // planes up to P + 1 have landed
     __syncthreads();
     // e at plane P
-    {
-      const int buf = P & 1;
-      T e0 = T(0), e1 = T(0), e2 = T(0);
-      if (conv_xy && P >= 1 && P <= g.nz - 2) {
-        const uint16_t w = w_cur;
-        const T zr = (T)P - A.K.zc;
-        const int b0 = sb(P - 1), b1 = sb(P), b2 = sb(P + 1);
-        const int d0 = sd(P - 1), d1 = sd(P), d2 = sd(P + 1);
-        e0 = edge_e<0>(A.K, sm.Sb, b0, b1, b2, sm.Sd, d0, d1, d2, tx, ty, xr, yr, zr, exc(w, 0));
-        e1 = edge_e<1>(A.K, sm.Sb, b0, b1, b2, sm.Sd, d0, d1, d2, tx, ty, xr, yr, zr, exc(w, 1));
-        e2 = edge_e<2>(A.K, sm.Sb, b0, b1, b2, sm.Sd, d0, d1, d2, tx, ty, xr, yr, zr, exc(w, 2));
-      }
-      sm.E[buf][0][ty][tx] = e0;
-      sm.E[buf][1][ty][tx] = e1;
-      sm.E[buf][2][ty][tx] = e2;
+    const Plane3<T, BY>&B = sm.Sb[P & 3], &D = sm.Sd[P & 3], &N = sm.Sd[(P + 1) & 3];
+    const T b0 = B.v[0][cy][cx], b1 = B.v[1][cy][cx], b2 = B.v[2][cy][cx];
+    const T d2 = D.v[2][cy][cx];
+    const T d2x = d2 + D.v[2][cy][cx + 1], d2y = d2 + D.v[2][cy + 1][cx];
+    const T n0 = N.v[0][cy][cx], n1 = N.v[1][cy][cx];
+    const T n0x = n0 + N.v[0][cy][cx - 1], n1y = n1 + N.v[1][cy - 1][cx];
+    T e[3] = {T(0), T(0), T(0)};
+    if (conv_xy) {  // (the planes of the march, 2 .. n - 2, are all converted)
+      auto metric = [&](int l) { return metric_at<T>(A.K, A.met, g.ncell, cP, l, xr, yr, zr, exc(w, l)); };
+      e[0] = edge_e<0>(metric(0), d0,
+                       d1y + (D.v[1][cy][cx + 1] + D.v[1][cy - 1][cx + 1]), d2x_m + d2x, b_m[1] + b1,
+                       B.v[2][cy - 1][cx] + b2);
+      e[1] = edge_e<1>(metric(1), d1, d2y_m + d2y,
+                       d0x + (D.v[0][cy + 1][cx] + D.v[0][cy + 1][cx - 1]), B.v[2][cy][cx - 1] + b2, b_m[0] + b0);
+      e[2] = edge_e<2>(metric(2), d2, d0x + n0x, d1y + n1y,
+                       B.v[0][cy - 1][cx] + b0, B.v[1][cy][cx - 1] + b1);
     }
-    __syncthreads();
-    // b update at plane P - 1 from e of planes P - 1 and P
+    T(&E)[3][BY][kTX] = sm.E[P & 1];
+#pragma unroll
+    for (int q = 0; q < 3; ++q) E[q][ty][tx] = e[q];
+    // b update at plane P - 1 from e of planes P - 1 (the neighbours' in shared memory) and P (own)
     if (upd) {
       const long long c = cP - splane;
-      const uint16_t w = w_prev;
-      const T (&E)[3][BY][kTX] = sm.E[p & 1];
-      const T (&En)[3][BY][kTX] = sm.E[P & 1];
+      const T(&Em)[3][BY][kTX] = sm.E[p & 1];
       // curl e at the three faces: b_x = F_yz: d_y e_z - d_z e_y; b_y = F_zx: d_z e_x - d_x e_z;
       // b_z = F_xy: d_x e_y - d_y e_x
-      const T cx = (E[2][ty + 1][tx] - E[2][ty][tx]) - (En[1][ty][tx] - E[1][ty][tx]);
-      const T cy = (En[0][ty][tx] - E[0][ty][tx]) - (E[2][ty][tx + 1] - E[2][ty][tx]);
-      const T cz = (E[1][ty][tx + 1] - E[1][ty][tx]) - (E[0][ty + 1][tx] - E[0][ty][tx]);
-      const T cu[3] = {cx, cy, cz};
+      const T cu[3] = {(Em[2][ty + 1][tx] - em[2]) - (e[1] - em[1]), (e[0] - em[0]) - (Em[2][ty][tx + 1] - em[2]),
+                       (Em[1][ty][tx + 1] - em[1]) - (Em[0][ty + 1][tx] - em[0])};
+      T v[3];
 #pragma unroll
-      for (int q = 0; q < 3; ++q) {
-        // b at the cell: the staged b^n when the base is the source, else the other buffer
-        const T old = A.inplace ? base_old[q] : sm.Sb[sb(p)].v[q][ty + 1][tx + 1];
-        if (adv(w, 3 + q)) {
-          T v = old - A.coef * cu[q];
-          if (A.tgt[0] && in_layer(w)) v = relax<T>(g, A.kin, w, A.tgt[q][c], v, 3 + q, x, y, p);
-          A.out[q][c] = v;
-        } else if (!A.inplace) {
-          A.out[q][c] = old;
-        }
+      for (int q = 0; q < 3; ++q) v[q] = adv(w_prev, 3 + q) ? fma(-A.coef, cu[q], old[q]) : old[q];
+      if (A.tgt[0] && in_layer(w_prev)) {
+        const T ko = outer_kappa<T>(g, x, y, p);
+#pragma unroll
+        for (int q = 0; q < 3; ++q)
+          if (adv(w_prev, 3 + q)) v[q] = relax<T>(g, A.kin, w_prev, ko, A.tgt[q][c], v[q], 3 + q, x, y, p);
       }
+#pragma unroll
+      for (int q = 0; q < 3; ++q) A.out[q][c] = v[q];
     }
-    w_prev = w_cur;
+    d2x_m = d2x;
+    d2y_m = d2y;
+    b_m[0] = b0;
+    b_m[1] = b1;
+    b_m[2] = b2;
+    d0 = n0;
+    d0x = n0x;
+    d1 = n1;
+    d1y = n1y;
+#pragma unroll
+    for (int q = 0; q < 3; ++q) em[q] = e[q];
+    w_prev = w;
+    w = w_next;
+    cP += splane;
+    zr += T(1);
   }
   cp_async_wait<0>();
 }
 
-// div_al h at a cell from the face values of its plane (C) and of the plane below (M):
-// F^{al nu} = +-h_q with q = 3 - al - nu, backward differences (Eq. 12):
-//   div_x = (h_z - h_z[-y]) - (h_y - h_y[-z]),  div_y = (h_x - h_x[-z]) - (h_z - h_z[-x]),
-//   div_z = (h_y - h_y[-x]) - (h_x - h_x[-y])
-template <typename T, int BY>
-__device__ __forceinline__ void div_h(const T (&C)[3][BY][kTX], const T (&M)[3][BY][kTX], int tx, int ty, T out[3]) {
-  out[0] = (C[2][ty][tx] - C[2][ty - 1][tx]) - (C[1][ty][tx] - M[1][ty][tx]);
-  out[1] = (C[0][ty][tx] - M[0][ty][tx]) - (C[2][ty][tx] - C[2][ty][tx - 1]);
-  out[2] = (C[1][ty][tx] - C[1][ty][tx - 1]) - (C[0][ty][tx] - C[0][ty - 1][tx]);
-}
-
 // ---- E step -----------------------------------------------------------------------------------
-// Patch: threads (tx, ty) at x = x0 + tx, y = y0 + ty with (x0, y0) two cells before the block's
-// first output column and row.  b and d are staged plane by plane (four rotating slots each).
-// Marching up z, iteration p:
-//   A  h1 = h(b, d) at plane p+1, whole patch                                   [predictor only]
-//   B  d* at plane p+1: d + (dx4/2)(4 pi/c J - div h1), or d where not advanced  (tx, ty >= 1)
-//   C  h2 = h(b, d*) at plane p (d* at offsets 0, +1)            (1 <= tx <= 30, 1 <= ty <= BY-2)
-//   D  d_out at plane p: d + dx4 (4 pi/c J - div h2)             (2 <= tx <= 30, 2 <= ty <= BY-2)
-// The literal step (no predictor) skips A and takes d* = d.  The march starts 3 planes below the
-// chunk, so that every buffer holds its plane when the first output plane is reached.
-// b and d keep five planes each (p - 1 .. p + 2 in use, p + 3 in flight).
+// d_out = d + coef (4 pi/c J - div h(b, x)) at advanced edge locations.  The time-centred step is two launches: the
+// predictor d* (x = d, coef = dx4 / 2) and the update (x = d*, coef = dx4); the literal step is one (x = d).
+// (One launch for both, with h of d and of d* in one march, overlaps patches by 3 cells instead of 1 and needs
+// two barriers a plane and 80 registers: slower at every size, see the figures above.)
+// Patch: threads (tx, ty) at x = x0 + tx, y = y0 + ty, h at the patch of each plane of the chunk and of the plane
+// below it; cells with tx >= 1 and ty >= 1 are updated (the divergence reaches -1).  Iteration q reads the staged planes
+// q and q + 1 (q + 2 in flight) for h of plane q and updates plane q - 1 from the h that the last iteration left in
+// the other half of H: one barrier a plane.
 template <typename T, int BY>
 struct EStepSmem {
-  Plane3<T, BY> Sb[5], Sd[5], DP[2];
-  T H1[2][3][BY][kTX];
-  T H2[2][3][BY][kTX];
+  Plane3<T, BY> Sb[4], Sx[4];
+  T H[2][3][BY][kTX];
 };
 
 template <typename T, int BY>
 __device__ __forceinline__ void e_step_tile(const Grid& g, const EStepArgs<T>& A, int tile_x, int tile_y, int zs,
                                             int ze, EStepSmem<T, BY>& sm) {
   const int tx = threadIdx.x, ty = threadIdx.y;
-  const int x0 = tile_x * (kTX - 3) - 2, y0 = tile_y * (BY - 3) - 2;
+  const int cx = tx + 1, cy = ty + 1;
+  const int x0 = 1 + tile_x * (kTX - 1), y0 = 1 + tile_y * (BY - 1);
   const int x = x0 + tx, y = y0 + ty;
-  const bool in_xy = x >= 0 && x < g.nx && y >= 0 && y < g.ny;
-  const bool conv_xy = x >= 1 && x <= g.nx - 2 && y >= 1 && y <= g.ny - 2;
-  const bool dp_xy = in_xy && tx >= 1 && ty >= 1;
-  const bool h2_xy = conv_xy && tx >= 1 && tx <= kTX - 2 && ty >= 1 && ty <= BY - 2;
-  const bool out_xy = in_xy && tx >= 2 && tx <= kTX - 2 && ty >= 2 && ty <= BY - 2;
+  const bool conv_xy = x <= g.nx - 2 && y <= g.ny - 2;  // (x, y >= 1)
+  const bool out_xy = x <= g.nx - 3 && y <= g.ny - 3 && tx >= 1 && ty >= 1;
+  const bool own = A.x[0] == A.d[0];
   const T xr = (T)x - A.K.xc, yr = (T)y - A.K.yc;
-  const T dx4 = A.K.dx4;
-  const T half_dx4 = dx4 * T(0.5);
   const Stager<BY> st(g, x0, y0);
-  auto s5 = [](int p) { return (p + 10) % 5; };
-  // planes zs - 3 .. zs - 1 in one copy group; iteration p starts plane p + 3
-  for (int q = zs - 3; q <= zs - 1; ++q) {
-    st.stage(g, A.b, q, sm.Sb[s5(q)]);
-    st.stage(g, A.d, q, sm.Sd[s5(q)]);
+  for (int q = zs - 2; q <= zs; ++q) {
+    st.stage(g, A.b, q, sm.Sb[q & 3]);
+    st.stage(g, A.x, q, sm.Sx[q & 3]);
   }
   cp_async_commit();
-  int cur = 0;  // buffer of plane p in H1, DP, H2 (plane p + 1 in the other)
-  // flags and source of plane p, carried from the iteration that loaded them as plane p + 1
-  uint16_t w_cur = 0;
-  T src_cur[3] = {T(0), T(0), T(0)};
-  const long long splane = (long long)g.nx * g.ny;
-  for (int p = zs - 3; p < ze; ++p) {
-    const int nxt = cur ^ 1;
-    st.stage(g, A.b, p + 3, sm.Sb[s5(p + 3)]);
-    st.stage(g, A.d, p + 3, sm.Sd[s5(p + 3)]);
+  cp_async_wait<0>();
+  __syncthreads();
+  // carried from plane q - 1: b_x summed over the x pair, b_y over the y pair; h, d and J there, and h of plane q - 2
+  T b0x_m, b1y_m;
+  {
+    const Plane3<T, BY>& B = sm.Sb[(zs - 2) & 3];
+    b0x_m = B.v[0][cy][cx] + B.v[0][cy][cx + 1];
+    b1y_m = B.v[1][cy][cx] + B.v[1][cy + 1][cx];
+  }
+  T hm[3] = {T(0), T(0), T(0)}, hmm[2] = {T(0), T(0)}, dm[3] = {T(0), T(0), T(0)};
+  double jm[3] = {0.0, 0.0, 0.0};
+  const int splane = g.nx * g.ny;
+  long long cq = ((long long)(zs - 1) * g.ny + y) * g.nx + x;  // the cell in plane q
+  T zr = (T)(zs - 1) - A.K.zc;
+  uint16_t w_prev = 0, w = conv_xy ? __ldg(A.loc + cq) : (uint16_t)0;  // flags of planes q - 1, q
+  for (int q = zs - 1; q <= ze; ++q) {
+    if (q + 2 <= ze) {
+      st.stage(g, A.b, q + 2, sm.Sb[(q + 2) & 3]);
+      st.stage(g, A.x, q + 2, sm.Sx[(q + 2) & 3]);
+    }
     cp_async_commit();
-    // flags and J of plane p + 1, issued ahead of the waits (J is converted where it is used)
-    const int pp = p + 1;
-    const bool row_in = in_xy && pp >= 0 && pp < g.nz;
-    const long long cn = ((long long)pp * g.ny + y) * g.nx + x;
-    const uint16_t w_next = row_in ? __ldg(A.loc + cn) : (uint16_t)0;
-    double j_next[3] = {0.0, 0.0, 0.0};
-    if (row_in) {
+    // loaded one iteration ahead: the flags of plane q + 1, J and (where it is not staged) d of plane q
+    const uint16_t w_next = conv_xy && q < ze ? __ldg(A.loc + cq + splane) : (uint16_t)0;
+    double jq[3] = {0.0, 0.0, 0.0};
+    T dq[3] = {T(0), T(0), T(0)};
+    if (out_xy && q < ze) {
 #pragma unroll
-      for (int al = 0; al < 3; ++al) j_next[al] = __ldg(A.J[al] + cn);
-    }
-    cp_async_wait<1>();  // planes up to p + 2 have landed
-    __syncthreads();
-    // A: h1 at plane p + 1
-    if (A.pred) {
-      T v0 = T(0), v1 = T(0), v2 = T(0);
-      const int pp = p + 1;
-      if (conv_xy && pp >= 1 && pp <= g.nz - 2) {
-        const uint16_t w = w_next;
-        const T zr = (T)pp - A.K.zc;
-        const int a = s5(p), b = s5(p + 1), d = s5(p + 2);
-        v0 = face_h<0>(A.K, sm.Sb, a, b, d, sm.Sd, a, b, d, tx, ty, xr, yr, zr, exc(w, 3));
-        v1 = face_h<1>(A.K, sm.Sb, a, b, d, sm.Sd, a, b, d, tx, ty, xr, yr, zr, exc(w, 4));
-        v2 = face_h<2>(A.K, sm.Sb, a, b, d, sm.Sd, a, b, d, tx, ty, xr, yr, zr, exc(w, 5));
-      }
-      sm.H1[nxt][0][ty][tx] = v0;
-      sm.H1[nxt][1][ty][tx] = v1;
-      sm.H1[nxt][2][ty][tx] = v2;
-    }
-    __syncthreads();
-    // B: d* at plane p + 1
-    T src_next[3];
+      for (int al = 0; al < 3; ++al) jq[al] = __ldg(A.J[al] + cq);
+      if (!own) {
 #pragma unroll
-    for (int al = 0; al < 3; ++al) src_next[al] = source<T>(A.K, j_next[al]);
-    {
-      if (dp_xy && pp >= 0 && pp < g.nz && p >= zs - 2) {
-        const Plane3<T, BY>& Dn = sm.Sd[s5(pp)];
-        T dv[3] = {Dn.v[0][ty + 1][tx + 1], Dn.v[1][ty + 1][tx + 1], Dn.v[2][ty + 1][tx + 1]};
-        if (A.pred) {
-          T dv_h[3];
-          div_h<T, BY>(sm.H1[nxt], sm.H1[cur], tx, ty, dv_h);
-#pragma unroll
-          for (int al = 0; al < 3; ++al)
-            if (adv(w_next, al)) dv[al] += (src_next[al] - dv_h[al]) * half_dx4;
-        }
-        sm.DP[nxt].v[0][ty + 1][tx + 1] = dv[0];
-        sm.DP[nxt].v[1][ty + 1][tx + 1] = dv[1];
-        sm.DP[nxt].v[2][ty + 1][tx + 1] = dv[2];
+        for (int al = 0; al < 3; ++al) dq[al] = __ldg(A.d[al] + cq);
       }
     }
+    cp_async_wait<1>();  // planes up to q + 1 have landed
     __syncthreads();
-    // C: h2 = h(b, d*) at plane p (d* of planes p and p + 1 in DP[cur], DP[nxt])
-    if (p >= zs - 1) {
-      T v0 = T(0), v1 = T(0), v2 = T(0);
-      if (h2_xy && p >= 1 && p <= g.nz - 2) {
-        const uint16_t w = w_cur;
-        const T zr = (T)p - A.K.zc;
-        const int a = s5(p - 1), b = s5(p), d = s5(p + 1);
-        v0 = face_h<0>(A.K, sm.Sb, a, b, d, sm.DP, nxt, cur, nxt, tx, ty, xr, yr, zr, exc(w, 3));
-        v1 = face_h<1>(A.K, sm.Sb, a, b, d, sm.DP, nxt, cur, nxt, tx, ty, xr, yr, zr, exc(w, 4));
-        v2 = face_h<2>(A.K, sm.Sb, a, b, d, sm.DP, nxt, cur, nxt, tx, ty, xr, yr, zr, exc(w, 5));
+    T h[3] = {T(0), T(0), T(0)};
+    if (q < ze && conv_xy) {
+      const Plane3<T, BY>&B = sm.Sb[q & 3], &Bn = sm.Sb[(q + 1) & 3], &X = sm.Sx[q & 3], &Xn = sm.Sx[(q + 1) & 3];
+      auto metric = [&](int l) { return metric_at<T>(A.K, A.met, g.ncell, cq, l, xr, yr, zr, exc(w, l)); };
+      // (sums over points in the order z, y, x)
+      const T b0 = B.v[0][cy][cx], b0r = B.v[0][cy][cx + 1], b1 = B.v[1][cy][cx], b1u = B.v[1][cy + 1][cx];
+      const T b2 = B.v[2][cy][cx], b2n = Bn.v[2][cy][cx];
+      const T x0v = X.v[0][cy][cx], x1v = X.v[1][cy][cx], x2v = X.v[2][cy][cx];
+      h[0] = face_h<0>(metric(3), b0, B.v[1][cy][cx - 1] + b1 + B.v[1][cy + 1][cx - 1] + b1u,
+                       B.v[2][cy][cx - 1] + b2 + Bn.v[2][cy][cx - 1] + b2n, x1v + Xn.v[1][cy][cx],
+                       x2v + X.v[2][cy + 1][cx]);
+      h[1] = face_h<1>(metric(4), b1, B.v[2][cy - 1][cx] + b2 + Bn.v[2][cy - 1][cx] + b2n,
+                       B.v[0][cy - 1][cx] + B.v[0][cy - 1][cx + 1] + b0 + b0r, x2v + X.v[2][cy][cx + 1],
+                       x0v + Xn.v[0][cy][cx]);
+      h[2] = face_h<2>(metric(5), b2, b0x_m + b0 + b0r, b1y_m + b1 + b1u, x0v + X.v[0][cy + 1][cx],
+                       x1v + X.v[1][cy][cx + 1]);
+      b0x_m = b0 + b0r;
+      b1y_m = b1 + b1u;
+      if (own) {
+        dq[0] = x0v;
+        dq[1] = x1v;
+        dq[2] = x2v;
       }
-      sm.H2[cur][0][ty][tx] = v0;
-      sm.H2[cur][1][ty][tx] = v1;
-      sm.H2[cur][2][ty][tx] = v2;
     }
-    __syncthreads();
-    // D: d_out at plane p (h2 of plane p in H2[cur], of plane p - 1 in H2[nxt])
+#pragma unroll
+    for (int al = 0; al < 3; ++al) sm.H[q & 1][al][ty][tx] = h[al];
+    // d_out at plane q - 1: div_al h, F^{al nu} = +-h_q with q = 3 - al - nu, backward differences (Eq. 12)
+    const int p = q - 1;
     if (p >= zs && out_xy) {
-      const long long c = cn - splane;
-      const Plane3<T, BY>& Dc = sm.Sd[s5(p)];
-      T dv_h[3];
-      div_h<T, BY>(sm.H2[cur], sm.H2[nxt], tx, ty, dv_h);
-#pragma unroll
+      const long long c = cq - splane;
+      const T(&M)[3][BY][kTX] = sm.H[p & 1];
+      const T dv[3] = {(hm[2] - M[2][ty - 1][tx]) - (hm[1] - hmm[1]), (hm[0] - hmm[0]) - (hm[2] - M[2][ty][tx - 1]),
+                       (hm[1] - M[1][ty][tx - 1]) - (hm[0] - M[0][ty - 1][tx])};
       T v[3];
 #pragma unroll
-      for (int al = 0; al < 3; ++al) {
-        const T dold = Dc.v[al][ty + 1][tx + 1];
-        v[al] = adv(w_cur, al) ? dold + (src_cur[al] - dv_h[al]) * dx4 : dold;
-      }
-      if (A.tgt[0] && in_layer(w_cur)) {
+      for (int al = 0; al < 3; ++al)
+        v[al] = adv(w_prev, al) ? dm[al] + (source<T>(A.K, jm[al]) - dv[al]) * A.coef : dm[al];
+      if (A.tgt[0] && in_layer(w_prev)) {
+        const T ko = outer_kappa<T>(g, x, y, p);
+#pragma unroll
         for (int al = 0; al < 3; ++al)
-          if (adv(w_cur, al)) v[al] = relax<T>(g, A.kin, w_cur, A.tgt[al][c], v[al], al, x, y, p);
+          if (adv(w_prev, al)) v[al] = relax<T>(g, A.kin, w_prev, ko, A.tgt[al][c], v[al], al, x, y, p);
       }
 #pragma unroll
       for (int al = 0; al < 3; ++al) A.out[al][c] = v[al];
     }
-    cur = nxt;
-    w_cur = w_next;
+    hmm[0] = hm[0];
+    hmm[1] = hm[1];
 #pragma unroll
-    for (int al = 0; al < 3; ++al) src_cur[al] = src_next[al];
+    for (int al = 0; al < 3; ++al) {
+      hm[al] = h[al];
+      dm[al] = dq[al];
+      jm[al] = jq[al];
+    }
+    w_prev = w;
+    w = w_next;
+    cq += splane;
+    zr += T(1);
   }
   cp_async_wait<0>();
 }
 
-// Rows of a patch: FP32 16, FP64 8.
-template <typename T>
-constexpr int patch_rows() {
-  return sizeof(T) == sizeof(float) ? 16 : 8;
-}
+// Resident blocks per SM: 64 registers a thread for the FP32 patches, 128 for the FP64 ones.
+constexpr int patch_blocks(size_t word, int rows) { return (word == 4 ? 32 : 16) / rows; }
 
-// Patches of a grid for the B step (out = 31 x (BY - 1) cells) or the E step (29 x (BY - 3)), and the
-// z chunk (4 to 64 planes) that minimises the estimated time: a chunk marches `halo` planes beyond
-// its own and the busiest of the `sms` multiprocessors runs ceil(patches / sms) of them.
-TileGrid tile_grid(const Grid& g, bool e_step, int rows, int sms) {
+// Patches over the advanced cells [2, n-3] per axis (31 x (rows - 1) cells each), and the split of z that minimises the
+// estimated time: a chunk marches `halo` planes beyond its own and the busiest of the `slots` runs
+// ceil(patches / slots) of them.
+TileGrid tile_grid(const Grid& g, int rows, int slots, double* cost_out = nullptr) {
   TileGrid t;
-  const int ox = e_step ? kTX - 3 : kTX - 1, oy = e_step ? rows - 3 : rows - 1;
-  const int halo = e_step ? 4 : 2;  // planes marched (and staged) below and above the chunk
-  t.ntx = (g.nx + ox - 1) / ox;
-  t.nty = (g.ny + oy - 1) / oy;
+  const int ox = kTX - 1, oy = rows - 1;
+  const int halo = 2;
+  const int nzi = g.nz - 4;
+  t.ntx = (g.nx - 4 + ox - 1) / ox;
+  t.nty = (g.ny - 4 + oy - 1) / oy;
   double best = 1e300;
-  for (int zc = 64; zc >= 4; zc /= 2) {
-    const long long nt = (long long)t.ntx * t.nty * ((g.nz + zc - 1) / zc);
-    const double per_sm = std::ceil((double)nt / sms);
-    const double cost = per_sm * (zc + halo);  // time ~ blocks of the busiest SM x planes marched
+  for (int nc = (nzi + 63) / 64; nc <= nzi; ++nc) {
+    const int zc = (nzi + nc - 1) / nc;
+    const long long nt = (long long)t.ntx * t.nty * ((nzi + zc - 1) / zc);
+    const double per_slot = std::ceil((double)nt / slots);
+    const double cost = per_slot * (zc + halo);  // time ~ blocks of the busiest slot x planes marched
     if (cost < best * 0.999) {
       best = cost;
       t.zchunk = zc;
     }
   }
-  t.ntz = (g.nz + t.zchunk - 1) / t.zchunk;
+  t.ntz = (nzi + t.zchunk - 1) / t.zchunk;
+  if (cost_out) *cost_out = best;
   return t;
+}
+
+// The outer two index layers are never advanced: a step into another buffer copies them with blocks of its own
+// beside the patches (blocks of kTX * rows threads, one cell a thread).  Cells by index: the z layers, then the
+// y layers of the planes between them, then the x layers of the rows between those.
+__host__ __device__ inline long long shell_cells(const Grid& g) {
+  return g.ncell - (long long)(g.nx - 4) * (g.ny - 4) * (g.nz - 4);
+}
+inline int shell_blocks(const Grid& g, int rows) {
+  return (int)((shell_cells(g) + kTX * rows - 1) / (kTX * rows));
+}
+__device__ __forceinline__ int outer_layer(int q, int n) { return q < 2 ? q : n - 4 + q; }  // q = 0..3
+template <typename T>
+__device__ __forceinline__ void copy_shell(const Grid& g, const T* const* src, T* const* dst, long long block) {
+  long long s = block * (blockDim.x * blockDim.y) + threadIdx.y * kTX + threadIdx.x;
+  int x, y, z;
+  const long long nz4 = 4ll * g.nx * g.ny, ny4 = 4ll * g.nx * (g.nz - 4);
+  if (s < nz4) {
+    x = (int)(s % g.nx);
+    y = (int)(s / g.nx % g.ny);
+    z = outer_layer((int)(s / ((long long)g.nx * g.ny)), g.nz);
+  } else if (s < nz4 + ny4) {
+    s -= nz4;
+    x = (int)(s % g.nx);
+    y = outer_layer((int)(s / g.nx % 4), g.ny);
+    z = 2 + (int)(s / (4ll * g.nx));
+  } else if (s < shell_cells(g)) {
+    s -= nz4 + ny4;
+    x = outer_layer((int)(s % 4), g.nx);
+    y = 2 + (int)(s / 4 % (g.ny - 4));
+    z = 2 + (int)(s / (4ll * (g.ny - 4)));
+  } else {
+    return;
+  }
+  const long long c = ((long long)z * g.ny + y) * g.nx + x;
+#pragma unroll
+  for (int q = 0; q < 3; ++q) dst[q][c] = src[q][c];
 }
 
 __device__ __forceinline__ void decode_tile(const TileGrid& t, long long q, int& tx, int& ty, int& zs) {
   tx = (int)(q % t.ntx);
   const long long r = q / t.ntx;
   ty = (int)(r % t.nty);
-  zs = (int)(r / t.nty) * t.zchunk;
+  zs = 2 + (int)(r / t.nty) * t.zchunk;
 }
 
 template <typename T, int BY>
-__global__ void __launch_bounds__(kTX * BY, 2) k_b_step(const Grid g, const BStepArgs<T> A, const TileGrid t) {
+__global__ void __launch_bounds__(kTX * BY, patch_blocks(sizeof(T), BY)) k_b_step(const Grid g, const BStepArgs<T> A, const TileGrid t) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   auto& sm = *reinterpret_cast<BStepSmem<T, BY>*>(smem_raw);
   int tx, ty, zs;
+  if (blockIdx.x >= t.count()) return copy_shell<T>(g, A.base, A.out, blockIdx.x - t.count());
   decode_tile(t, blockIdx.x, tx, ty, zs);
-  b_step_tile<T, BY>(g, A, tx, ty, zs, min(zs + t.zchunk, g.nz), sm);
+  b_step_tile<T, BY>(g, A, tx, ty, zs, min(zs + t.zchunk, g.nz - 2), sm);
 }
 
 template <typename T, int BY>
-__global__ void __launch_bounds__(kTX * BY, 2) k_e_step(const Grid g, const EStepArgs<T> A, const TileGrid t) {
+__global__ void __launch_bounds__(kTX * BY, patch_blocks(sizeof(T), BY)) k_e_step(const Grid g, const EStepArgs<T> A, const TileGrid t) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   auto& sm = *reinterpret_cast<EStepSmem<T, BY>*>(smem_raw);
   int tx, ty, zs;
+  if (blockIdx.x >= t.count()) return copy_shell<T>(g, A.d, A.out, blockIdx.x - t.count());
   decode_tile(t, blockIdx.x, tx, ty, zs);
-  e_step_tile<T, BY>(g, A, tx, ty, zs, min(zs + t.zchunk, g.nz), sm);
+  e_step_tile<T, BY>(g, A, tx, ty, zs, min(zs + t.zchunk, g.nz - 2), sm);
 }
 
-// ---- batched: persistent grid-stride over a table of (instance, patch) work items --------------
-// which: 0 first B half (b[0] -> b[1]), 1 second B half, 2 E step.  The instance's d buffer
-// parity is read from the device (flipped by launch_batch_flip_d at the end of a step).
+// ---- batched: one block per entry of a table of (instance, patch) work items ---------------------
+// which (B): 0 first half (b[0] -> b[1]), 1 second half; (E): 0 predictor (into b[1], free by then), 1 update.
+// The instance's d buffer parity is read from the device (flipped by launch_batch_flip_d at the end of a step).
 template <typename T>
 __device__ __forceinline__ const FieldConsts<T>& inst_consts(const InstDesc<T>& D) {
   if constexpr (sizeof(T) == sizeof(float))
@@ -651,58 +685,76 @@ __device__ __forceinline__ BStepArgs<T> batch_b_args(const InstDesc<T>& D, int w
   for (int q = 0; q < 3; ++q) A.tgt[q] = which == 1 ? D.FS.tgt[3 + q] : nullptr;
   A.kin = D.FS.kin;
   A.loc = D.FS.loc;
+  A.met = D.FS.met;
   A.coef = (which == 1 && !literal) ? dx4 : dx4 * T(0.5);
   A.inplace = which == 1 && !literal;
   return A;
 }
 
 template <typename T>
-__device__ __forceinline__ EStepArgs<T> batch_e_args(const InstDesc<T>& D, bool literal) {
+__device__ __forceinline__ EStepArgs<T> batch_e_args(const InstDesc<T>& D, int which, bool literal) {
   EStepArgs<T> A;
   const int dc = *D.dcur;
   A.K = inst_consts(D);
+  const bool pred = which == 0;
   for (int q = 0; q < 3; ++q) {
     A.b[q] = D.FS.b[0][q];
     A.d[q] = D.FS.d[dc][q];
-    A.out[q] = D.FS.d[dc ^ 1][q];
+    A.x[q] = pred || literal ? D.FS.d[dc][q] : D.FS.b[1][q];
+    A.out[q] = pred ? D.FS.b[1][q] : D.FS.d[dc ^ 1][q];
     A.J[q] = D.FS.J[q];
-    A.tgt[q] = D.FS.tgt[q];
+    A.tgt[q] = pred ? nullptr : D.FS.tgt[q];
   }
+  A.coef = pred ? A.K.dx4 * T(0.5) : A.K.dx4;
   A.kin = D.FS.kin;
   A.loc = D.FS.loc;
-  A.pred = !literal;
+  A.met = D.FS.met;
   return A;
 }
 
 template <typename T, int BY>
-__global__ void __launch_bounds__(kTX * BY) k_batch_b_step(const InstDesc<T>* __restrict__ desc,
-                                                           const BlockEntry* __restrict__ blk, int nblk, int which,
-                                                           bool literal) {
+__global__ void __launch_bounds__(kTX * BY, patch_blocks(sizeof(T), BY))
+    k_batch_b_step(const InstDesc<T>* __restrict__ desc, const BlockEntry* __restrict__ blk, int which, bool literal) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ BStepArgs<T> A;  // (in registers, as a kernel parameter is not, it would spill)
+  __shared__ Grid g;
   auto& sm = *reinterpret_cast<BStepSmem<T, BY>*>(smem_raw);
-  for (int bi = blockIdx.x; bi < nblk; bi += gridDim.x) {
-    const BlockEntry e = blk[bi];
-    const InstDesc<T>& D = desc[e.inst];
-    int tx, ty, zs;
-    decode_tile(D.btiles, e.block, tx, ty, zs);
-    b_step_tile<T, BY>(D.g, batch_b_args(D, which, literal), tx, ty, zs, min(zs + D.btiles.zchunk, D.g.nz), sm);
-    __syncthreads();  // the next item restages the planes
+  const BlockEntry e = blk[blockIdx.x];
+  const InstDesc<T>& D = desc[e.inst];
+  if (threadIdx.x == 0 && threadIdx.y == 0) {
+    A = batch_b_args(D, which, literal);
+    g = D.g;
   }
+  const TileGrid t = D.tiles;
+  __syncthreads();
+  if (e.block >= t.count()) {
+    if (!A.inplace) copy_shell<T>(g, A.base, A.out, e.block - t.count());
+    return;
+  }
+  int tx, ty, zs;
+  decode_tile(t, e.block, tx, ty, zs);
+  b_step_tile<T, BY>(g, A, tx, ty, zs, min(zs + t.zchunk, g.nz - 2), sm);
 }
 
 template <typename T, int BY>
-__global__ void __launch_bounds__(kTX * BY) k_batch_e_step(const InstDesc<T>* __restrict__ desc,
-                                                           const BlockEntry* __restrict__ blk, int nblk, bool literal) {
+__global__ void __launch_bounds__(kTX * BY, patch_blocks(sizeof(T), BY))
+    k_batch_e_step(const InstDesc<T>* __restrict__ desc, const BlockEntry* __restrict__ blk, int which, bool literal) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ EStepArgs<T> A;
+  __shared__ Grid g;
   auto& sm = *reinterpret_cast<EStepSmem<T, BY>*>(smem_raw);
-  for (int bi = blockIdx.x; bi < nblk; bi += gridDim.x) {
-    const BlockEntry e = blk[bi];
-    const InstDesc<T>& D = desc[e.inst];
-    int tx, ty, zs;
-    decode_tile(D.etiles, e.block, tx, ty, zs);
-    e_step_tile<T, BY>(D.g, batch_e_args(D, literal), tx, ty, zs, min(zs + D.etiles.zchunk, D.g.nz), sm);
-    __syncthreads();
+  const BlockEntry e = blk[blockIdx.x];
+  const InstDesc<T>& D = desc[e.inst];
+  if (threadIdx.x == 0 && threadIdx.y == 0) {
+    A = batch_e_args(D, which, literal);
+    g = D.g;
   }
+  const TileGrid t = D.tiles;
+  __syncthreads();
+  if (e.block >= t.count()) return copy_shell<T>(g, A.d, A.out, e.block - t.count());
+  int tx, ty, zs;
+  decode_tile(t, e.block, tx, ty, zs);
+  e_step_tile<T, BY>(g, A, tx, ty, zs, min(zs + t.zchunk, g.nz - 2), sm);
 }
 
 template <typename T>
@@ -787,14 +839,13 @@ __global__ void k_uniform_field(const Grid g, const Fields<T> F, double E0, doub
 }
 
 // ---- read-out of the contravariant face components --------------------------------------------
-// Mean of the points of source lattice SL nearest to the point of target lattice TL in cell
-// (i, j, k), from global memory, in the order of avg_s.
+// Sum of the points of source lattice SL nearest to the point of target lattice TL in cell
+// (i, j, k), from global memory.
 template <int TL, int SL, typename T>
-__device__ __forceinline__ T avg_g(const T* __restrict__ F, const Grid& g, int i, int j, int k) {
+__device__ __forceinline__ T sum_g(const T* __restrict__ F, const Grid& g, int i, int j, int k) {
   constexpr int lx = nb_lo(TL, SL, 0), hx = nb_hi(TL, SL, 0);
   constexpr int ly = nb_lo(TL, SL, 1), hy = nb_hi(TL, SL, 1);
   constexpr int lz = nb_lo(TL, SL, 2), hz = nb_hi(TL, SL, 2);
-  constexpr int cnt = (hx - lx + 1) * (hy - ly + 1) * (hz - lz + 1);
   T s = T(0);
 #pragma unroll
   for (int dz = lz; dz <= hz; ++dz)
@@ -802,25 +853,17 @@ __device__ __forceinline__ T avg_g(const T* __restrict__ F, const Grid& g, int i
     for (int dy = ly; dy <= hy; ++dy)
 #pragma unroll
       for (int dx = lx; dx <= hx; ++dx) s += F[((long long)(k + dz) * g.ny + (j + dy)) * g.nx + (i + dx)];
-  if (cnt == 1) return s;
-  return s * (T(1) / T(cnt));
+  return s;
 }
 
 template <int Q, typename T>
 __device__ __forceinline__ double face_h_g(const Grid& g, const FieldConsts<T>& K, const Fields<T>& F, int i, int j,
                                            int k, bool excised) {
-  constexpr int L = 3 + Q;
-  T bb[3];
-  bb[0] = avg_g<L, 3>(F.b[0], g, i, j, k);
-  bb[1] = avg_g<L, 4>(F.b[1], g, i, j, k);
-  bb[2] = avg_g<L, 5>(F.b[2], g, i, j, k);
-  constexpr int A = (Q + 1) % 3, B = (Q + 2) % 3;  // (d x k)_Q = d_A k_B - d_B k_A
-  const T dA = avg_g<L, A>(F.d[A], g, i, j, k);
-  const T dB = avg_g<L, B>(F.d[B], g, i, j, k);
+  constexpr int L = 3 + Q, M = (Q + 1) % 3, N = (Q + 2) % 3;
   const Pt<T> P = metric_pt<T>(K, L, (T)i - K.xc, (T)j - K.yc, (T)k - K.zc, excised);
-  const T kA = A == 0 ? P.k0 : (A == 1 ? P.k1 : P.k2);
-  const T kB = B == 0 ? P.k0 : (B == 1 ? P.k1 : P.k2);
-  return (double)h_comp(Q, P, bb, dA * kB - dB * kA, rcp_t(T(1) + P.f));
+  return (double)face_h<Q>(P, F.b[Q][((long long)k * g.ny + j) * g.nx + i], sum_g<L, 3 + M>(F.b[M], g, i, j, k),
+                           sum_g<L, 3 + N>(F.b[N], g, i, j, k), sum_g<L, M>(F.d[M], g, i, j, k),
+                           sum_g<L, N>(F.d[N], g, i, j, k));
 }
 
 // h (F^yz, F^zx, F^xy) at every b face of the cells 1 .. n-2 per axis, as the E step converts the
@@ -891,64 +934,130 @@ void launch_inner_kappa_table(const Grid& g, T* kin, cudaStream_t st) {
 template void launch_inner_kappa_table<float>(const Grid&, float*, cudaStream_t);
 template void launch_inner_kappa_table<double>(const Grid&, double*, cudaStream_t);
 
+__global__ void k_metric_table(const Grid g, const FieldConsts<double> K, const uint16_t* __restrict__ loc,
+                               double2* __restrict__ met) {
+  const long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (c >= g.ncell) return;
+  const int i = (int)(c % g.nx);
+  const int j = (int)((c / g.nx) % g.ny);
+  const int k = (int)(c / ((long long)g.nx * g.ny));
+  const uint16_t w = loc[c];
+#pragma unroll 1
+  for (int l = 0; l < 6; ++l) {
+    const Pt<double> P = metric_pt<double>(K, l, i - K.xc, j - K.yc, k - K.zc, exc(w, l));
+    met[2 * l * g.ncell + c] = make_double2(P.f, P.k0);
+    met[(2 * l + 1) * g.ncell + c] = make_double2(P.k1, P.k2);
+  }
+}
+
+void launch_metric_table(const Grid& g, const uint16_t* loc, double2* met, cudaStream_t st) {
+  k_metric_table<<<blocks_for(g.ncell, 256), 256, 0, st>>>(g, field_consts<double>(g), loc, met);
+}
+
 // Dynamic shared memory of the field kernels (above the 48 KB default): set once per kernel.
 template <typename K>
 void allow_smem(K kernel, size_t bytes) {
   cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
-template <typename T>
-void launch_b_step(const Grid& g, const BStepArgs<T>& A, int sms, cudaStream_t st) {
-  constexpr int BY = patch_rows<T>();
+template <typename T, int BY>
+void launch_b_rows(const Grid& g, const BStepArgs<T>& A, const TileGrid& t, cudaStream_t st) {
   constexpr size_t smem = sizeof(BStepSmem<T, BY>);
   static bool once = (allow_smem(k_b_step<T, BY>, smem), true);
   (void)once;
-  const TileGrid t = tile_grid(g, false, BY, sms);
-  k_b_step<T, BY><<<(unsigned)t.count(), dim3(kTX, BY), smem, st>>>(g, A, t);
+  const long long nb = t.count() + (A.inplace ? 0 : shell_blocks(g, BY));
+  k_b_step<T, BY><<<(unsigned)nb, dim3(kTX, BY), smem, st>>>(g, A, t);
+}
+
+template <typename T, int BY>
+void launch_e_rows(const Grid& g, const EStepArgs<T>& A, const TileGrid& t, cudaStream_t st) {
+  constexpr size_t smem = sizeof(EStepSmem<T, BY>);
+  static bool once = (allow_smem(k_e_step<T, BY>, smem), true);
+  (void)once;
+  k_e_step<T, BY><<<(unsigned)(t.count() + shell_blocks(g, BY)), dim3(kTX, BY), smem, st>>>(g, A, t);
+}
+
+// FP32 patches (and the batched FP64 ones) have 16 rows.  Other FP64 patches, bound by the FP64 pipe whatever their
+// shape, take the rows (8 or 16) with the lower estimated time: 16 waste less on the overlap, 8 divide a small grid
+// more evenly.
+// B step at 32^3 FP64: 8 rows 78 us, 16 rows 144 us (metric evaluated); E step at 64^3: 16 rows 393 us, 8 rows 607 us.
+template <typename T>
+TileGrid choose_rows(const Grid& g, int sms, int* rows) {
+  double c16 = 0.0, c8 = 0.0;
+  const TileGrid t16 = tile_grid(g, 16, sms * patch_blocks(sizeof(T), 16), &c16);
+  *rows = 16;
+  if (sizeof(T) == sizeof(float)) return t16;
+  const TileGrid t8 = tile_grid(g, 8, sms, &c8);  // (two blocks share an SM's FP64 pipe)
+  if (0.5 * c8 >= c16) return t16;
+  *rows = 8;
+  return t8;
+}
+
+template <typename T>
+void launch_b_step(const Grid& g, const BStepArgs<T>& A, int sms, cudaStream_t st) {
+  int rows;
+  const TileGrid t = choose_rows<T>(g, sms, &rows);
+  if constexpr (sizeof(T) == sizeof(double)) {
+    if (rows == 8) return launch_b_rows<T, 8>(g, A, t, st);
+  }
+  launch_b_rows<T, 16>(g, A, t, st);
 }
 
 template <typename T>
 void launch_e_step(const Grid& g, const EStepArgs<T>& A, int sms, cudaStream_t st) {
-  constexpr int BY = patch_rows<T>();
-  constexpr size_t smem = sizeof(EStepSmem<T, BY>);
-  static bool once = (allow_smem(k_e_step<T, BY>, smem), true);
-  (void)once;
-  const TileGrid t = tile_grid(g, true, BY, sms);
-  k_e_step<T, BY><<<(unsigned)t.count(), dim3(kTX, BY), smem, st>>>(g, A, t);
+  int rows;
+  const TileGrid t = choose_rows<T>(g, sms, &rows);
+  if constexpr (sizeof(T) == sizeof(double)) {
+    if (rows == 8) return launch_e_rows<T, 8>(g, A, t, st);
+  }
+  launch_e_rows<T, 16>(g, A, t, st);
 }
 
-// Patch tables of an instance for the batched field launches: z chunks of 16 planes, the
-// instances themselves supplying the parallelism.
-void batch_field_tiles(const Grid& g, bool fp32, TileGrid* btiles, TileGrid* etiles) {
-  const int rows = fp32 ? patch_rows<float>() : patch_rows<double>();
-  for (int e = 0; e < 2; ++e) {
-    TileGrid t = tile_grid(g, e == 1, rows, 1);
-    t.zchunk = 16;
-    t.ntz = (g.nz + 15) / 16;
-    *(e ? etiles : btiles) = t;
+// Patches of the instances of a batch (16 rows), the z chunks the ones (of one length for all) that minimise the
+// estimated time as in tile_grid; blocks of the copied outer layers follow an instance's patches.
+constexpr int kBatchRows = 16;
+int batch_shell_blocks(const Grid& g) { return shell_blocks(g, kBatchRows); }
+void batch_field_tiles(const Grid* const* grids, int n, size_t word, int sms, TileGrid* tiles) {
+  const int slots = sms * patch_blocks(word, kBatchRows);
+  double best = 1e300;
+  int zbest = 64;
+  for (int zc = 64; zc >= 1; zc -= zc > 16 ? 4 : 1) {
+    long long nt = 0;
+    for (int i = 0; i < n; ++i) {
+      TileGrid t = tile_grid(*grids[i], kBatchRows, 1);
+      nt += (long long)t.ntx * t.nty * ((grids[i]->nz - 4 + zc - 1) / zc);
+    }
+    const double cost = std::ceil((double)nt / slots) * (zc + 2);
+    if (cost < best * 0.999) {
+      best = cost;
+      zbest = zc;
+    }
+  }
+  for (int i = 0; i < n; ++i) {
+    tiles[i] = tile_grid(*grids[i], kBatchRows, 1);
+    tiles[i].zchunk = zbest;
+    tiles[i].ntz = (grids[i]->nz - 4 + zbest - 1) / zbest;
   }
 }
 
 template <typename T>
 void launch_batch_b_half(const BatchTables<T>& bt, int which, bool literal, cudaStream_t st) {
-  constexpr int BY = patch_rows<T>();
+  constexpr int BY = kBatchRows;
   constexpr size_t smem = sizeof(BStepSmem<T, BY>);
   static bool once = (allow_smem(k_batch_b_step<T, BY>, smem), true);
   (void)once;
-  if (bt.nbtile == 0) return;
-  k_batch_b_step<T, BY><<<std::min(bt.nbtile, bt.persist_field_blocks), dim3(kTX, BY), smem, st>>>(
-      bt.desc, bt.btile, bt.nbtile, which, literal);
+  if (bt.ntile == 0) return;
+  k_batch_b_step<T, BY><<<bt.ntile, dim3(kTX, BY), smem, st>>>(bt.desc, bt.tile, which, literal);
 }
 
 template <typename T>
-void launch_batch_e_step(const BatchTables<T>& bt, bool literal, cudaStream_t st) {
-  constexpr int BY = patch_rows<T>();
+void launch_batch_e_step(const BatchTables<T>& bt, int which, bool literal, cudaStream_t st) {
+  constexpr int BY = kBatchRows;
   constexpr size_t smem = sizeof(EStepSmem<T, BY>);
   static bool once = (allow_smem(k_batch_e_step<T, BY>, smem), true);
   (void)once;
-  if (bt.netile == 0) return;
-  k_batch_e_step<T, BY><<<std::min(bt.netile, bt.persist_field_blocks), dim3(kTX, BY), smem, st>>>(
-      bt.desc, bt.etile, bt.netile, literal);
+  if (bt.ntile == 0) return;
+  k_batch_e_step<T, BY><<<bt.ntile, dim3(kTX, BY), smem, st>>>(bt.desc, bt.tile, which, literal);
 }
 
 template <typename T>
@@ -992,7 +1101,7 @@ void launch_convert_out(double* dst, const T* src, long long n, cudaStream_t st)
   template void launch_convert_in<T>(T*, const double*, long long, cudaStream_t);                       \
   template void launch_convert_out<T>(double*, const T*, long long, cudaStream_t);                      \
   template void launch_batch_b_half<T>(const BatchTables<T>&, int, bool, cudaStream_t);                 \
-  template void launch_batch_e_step<T>(const BatchTables<T>&, bool, cudaStream_t);                      \
+  template void launch_batch_e_step<T>(const BatchTables<T>&, int, bool, cudaStream_t);                      \
   template void launch_batch_zero_j<T>(const BatchTables<T>&, cudaStream_t);                            \
   template void launch_batch_flip_d<T>(const BatchTables<T>&, int, cudaStream_t);
 

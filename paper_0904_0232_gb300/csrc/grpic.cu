@@ -7,8 +7,8 @@
 #include <string>
 #include <vector>
 
-#include "../../include/grpic.h"
 #include "common.cuh"
+#include "internal.h"
 
 using namespace grpic;
 
@@ -53,11 +53,15 @@ struct grpic_ctx {
   void* tgt = nullptr;     // absorbing layers: 6 planes of T, the target d and b (null without layers)
   void* kin = nullptr;     // inner absorbing layer: relaxation table over g.kbox0 / g.kboxn (T)
   double* J = nullptr;     // 3 planes
+  double2* met = nullptr;  // FP64: metric table of the field kernels (may be given up for memory, see dev_alloc)
+  bool met_held = false;   // a batch's tables refer to it
   float4* atab = nullptr;  // per-cell area fits of the far-field deposit (built when tune.area_table is set)
   uint16_t* loc = nullptr;  // per-cell location flags
   // field ping-pong state: buffer of the current d and b; bprev: buffer holding b^{n-1/2} after the
   // first B half-step (time-centred second half-step)
   int dcur = 0, bcur = 0, bprev = 0;
+  bool bprev_held = false;  // between a first B half-step and its second: the idle b buffer is b^{n-1/2}
+  void* dstar = nullptr;    // 3 planes of T for the E step's predictor in that state (hand-driven stages only)
   DevStatus* st = nullptr;
   DevStatus* st_host = nullptr;  // pinned
   SortScratch sort{};
@@ -86,8 +90,7 @@ struct grpic_ctx {
 
 namespace {
 
-void* dev_alloc(grpic_ctx* c, size_t bytes) {
-  if (bytes == 0) bytes = 256;
+void* raw_alloc(grpic_ctx* c, size_t bytes) {
   if (c->cfg.alloc) return c->cfg.alloc(bytes, c->cfg.alloc_user);
   void* p = nullptr;
   if (cudaMalloc(&p, bytes) != cudaSuccess) {
@@ -104,6 +107,18 @@ void dev_free(grpic_ctx* c, void* p) {
     return;
   }
   cudaFree(p);
+}
+
+// Device memory of the context.  The metric table only saves time, so it makes room for anything else: where an
+// allocation fails it is freed (unless a batch refers to it) and the allocation tried again.
+void* dev_alloc(grpic_ctx* c, size_t bytes) {
+  if (bytes == 0) bytes = 256;
+  void* p = raw_alloc(c, bytes);
+  if (p || !c->met || c->met_held) return p;
+  cudaStreamSynchronize(c->stream);
+  dev_free(c, c->met);
+  c->met = nullptr;
+  return raw_alloc(c, bytes);
 }
 
 grpic_status fail(grpic_ctx* c, grpic_status s, const std::string& msg) {
@@ -292,6 +307,7 @@ void enqueue_stage(grpic_ctx* c, int stage) {
       }
       A.kin = static_cast<const T*>(c->kin);
       A.loc = c->loc;
+      A.met = c->met;
       A.K = field_consts<T>(c->g);
       const T dx4 = grid_dx4<T>(c->g);
       A.coef = centred ? dx4 : dx4 * T(0.5);
@@ -299,6 +315,7 @@ void enqueue_stage(grpic_ctx* c, int stage) {
       launch_b_step<T>(c->g, A, c->sms, c->stream);
       c->launches += 1;
       if (!second) c->bprev = c->bcur;
+      c->bprev_held = !second;
       c->bcur = out;
       break;
     }
@@ -324,18 +341,35 @@ void enqueue_stage(grpic_ctx* c, int stage) {
       c->pushes += 1;
       break;
     case GRPIC_STAGE_E: {
+      // the predictor goes to the idle b buffer (b^n: the next first half-step writes all of it), or to planes of its own
+      // where that buffer is still to be read (grpic_stage)
+      const bool literal = literal_fields(c);
       EStepArgs<T> A;
       for (int q = 0; q < 3; ++q) {
         A.b[q] = F.b[q];
+        A.x[q] = F.d[q];
         A.d[q] = F.d[q];
-        A.out[q] = field_plane<T>(c, false, 1 - c->dcur, q);
+        A.out[q] = c->bprev_held ? static_cast<T*>(c->dstar) + (size_t)q * c->g.ncell
+                                 : field_plane<T>(c, true, 1 - c->bcur, q);
         A.J[q] = F.J[q];
-        A.tgt[q] = target_plane<T>(c, q);
+        A.tgt[q] = nullptr;
       }
       A.kin = static_cast<const T*>(c->kin);
       A.loc = c->loc;
+      A.met = c->met;
       A.K = field_consts<T>(c->g);
-      A.pred = !literal_fields(c);
+      const T dx4 = grid_dx4<T>(c->g);
+      A.coef = dx4 * T(0.5);
+      if (!literal) {
+        launch_e_step<T>(c->g, A, c->sms, c->stream);
+        c->launches += 1;
+      }
+      for (int q = 0; q < 3; ++q) {
+        if (!literal) A.x[q] = A.out[q];
+        A.out[q] = field_plane<T>(c, false, 1 - c->dcur, q);
+        A.tgt[q] = target_plane<T>(c, q);
+      }
+      A.coef = dx4;
       launch_e_step<T>(c->g, A, c->sms, c->stream);
       c->launches += 1;
       c->dcur = 1 - c->dcur;
@@ -487,6 +521,12 @@ const char* grpic_status_string(grpic_status s) {
 const char* grpic_last_error(const grpic_ctx* c) { return c ? c->err.c_str() : "null context"; }
 
 grpic_status grpic_create(const grpic_config* cfg, void* stream, grpic_ctx** out) {
+  return grpic::create_context(cfg, stream, /*metric_table=*/true, out);
+}
+
+}  // extern "C"
+
+grpic_status grpic::create_context(const grpic_config* cfg, void* stream, bool metric_table, grpic_ctx** out) {
   if (!cfg || !out) return GRPIC_ERR_INVALID;
   *out = nullptr;
   if (cfg->nx < 8 || cfg->ny < 8 || cfg->nz < 8) return GRPIC_ERR_INVALID;
@@ -610,6 +650,10 @@ grpic_status grpic_create(const grpic_config* cfg, void* stream, grpic_ctx** out
     else
       launch_inner_kappa_table<double>(g, static_cast<double*>(c->kin), c->stream);
   }
+  if (!c->mixed && metric_table && g.m > 0.0) {
+    c->met = static_cast<double2*>(raw_alloc(c, sizeof(double2) * kMetricPlanes * (size_t)ncell));
+    if (c->met) launch_metric_table(g, c->loc, c->met, c->stream);
+  }
   grpic_status s = cuda_check(c, cudaGetLastError(), "create");
   if (s == GRPIC_OK) s = cuda_check(c, cudaStreamSynchronize(c->stream), "create sync");
   if (s != GRPIC_OK) {
@@ -620,6 +664,8 @@ grpic_status grpic_create(const grpic_config* cfg, void* stream, grpic_ctx** out
   return GRPIC_OK;
 }
 
+extern "C" {
+
 grpic_status grpic_destroy(grpic_ctx* c) {
   if (!c) return GRPIC_ERR_INVALID;
   cudaStreamSynchronize(c->stream);
@@ -627,6 +673,8 @@ grpic_status grpic_destroy(grpic_ctx* c) {
   dev_free(c, c->tgt);
   dev_free(c, c->kin);
   dev_free(c, c->atab);
+  dev_free(c, c->met);
+  dev_free(c, c->dstar);
   dev_free(c, c->J);
   dev_free(c, c->loc);
   dev_free(c, c->st);
@@ -812,6 +860,10 @@ grpic_status grpic_step(grpic_ctx* c, int nsteps) {
 
 grpic_status grpic_stage(grpic_ctx* c, int stage) {
   if (!c || stage < GRPIC_STAGE_B_HALF || stage > GRPIC_STAGE_B_HALF2) return GRPIC_ERR_INVALID;
+  if (stage == GRPIC_STAGE_E && c->bprev_held && !c->dstar && !literal_fields(c)) {
+    c->dstar = dev_alloc(c, 3 * (size_t)c->g.ncell * c->tsize);
+    if (!c->dstar) return fail(c, GRPIC_ERR_OOM, "predictor planes");
+  }
   enqueue_stage_any(c, stage);
   grpic_status s = cuda_check(c, cudaGetLastError(), "stage launch");
   if (s != GRPIC_OK) return s;
@@ -1224,15 +1276,14 @@ struct grpic_batch {
   int quad = 2;
   std::vector<void*> allocs;
   void* desc = nullptr;
-  BlockEntry *btile = nullptr, *etile = nullptr, *all = nullptr, *part = nullptr;
-  int nbtile = 0, netile = 0, nall = 0, npart = 0;
+  BlockEntry *tile = nullptr, *all = nullptr, *part = nullptr;
+  int ntile = 0, nall = 0, npart = 0;
   int* dcur = nullptr;  // device d-buffer parity per instance
   int *counts = nullptr, *offsets = nullptr, *tiles = nullptr, *pairs = nullptr, *pair_base = nullptr;
   int* cur = nullptr;  // device ping-pong index per (instance, species)
   long long nbins = 0;
   int npairs = 0;
   int persist_blocks = 0;
-  int persist_field_blocks = 0;
   int sms = 1;
   std::vector<long long> pair_n;  // work upper bound of each pair when the batch was built
   // One captured step per step parity k: every step flips each particle store (the sort) and each d
@@ -1275,10 +1326,8 @@ template <typename T>
 BatchTables<T> batch_tables(grpic_batch* b) {
   BatchTables<T> t;
   t.desc = static_cast<const InstDesc<T>*>(b->desc);
-  t.btile = b->btile;
-  t.nbtile = b->nbtile;
-  t.etile = b->etile;
-  t.netile = b->netile;
+  t.tile = b->tile;
+  t.ntile = b->ntile;
   t.all = b->all;
   t.nall = b->nall;
   t.part = b->part;
@@ -1291,7 +1340,6 @@ BatchTables<T> batch_tables(grpic_batch* b) {
   t.npairs = b->npairs;
   t.pair_base = b->pair_base;
   t.persist_blocks = b->persist_blocks;
-  t.persist_field_blocks = b->persist_field_blocks;
   return t;
 }
 
@@ -1304,7 +1352,7 @@ template <typename T>
 grpic_status batch_build(grpic_batch* b) {
   const int n = (int)b->ctxs.size();
   std::vector<InstDesc<T>> desc(n);
-  std::vector<BlockEntry> btile, etile, all, part;
+  std::vector<BlockEntry> tile, all, part;
   std::vector<int> pairs, cur_init, dcur_init(n, 0);
   std::vector<long long> bin_base;
   long long nbins = 0;
@@ -1314,6 +1362,10 @@ grpic_status batch_build(grpic_batch* b) {
   b->dcur = static_cast<int*>(batch_alloc(b, sizeof(int) * n));
   if (!b->dcur) return GRPIC_ERR_OOM;
   cur_init.assign(4 * n, 0);
+  std::vector<const Grid*> grids(n);
+  std::vector<TileGrid> tiles(n);
+  for (int i = 0; i < n; ++i) grids[i] = &b->ctxs[i]->g;
+  batch_field_tiles(grids.data(), n, sizeof(T), b->sms, tiles.data());
   for (int i = 0; i < n; ++i) {
     grpic_ctx* c = b->ctxs[i];
     InstDesc<T>& D = desc[i];
@@ -1331,13 +1383,15 @@ grpic_status batch_build(grpic_batch* b) {
     for (int q = 0; q < 6; ++q) D.FS.tgt[q] = target_plane<T>(c, q);
     D.FS.kin = static_cast<const T*>(c->kin);
     D.FS.loc = c->loc;
+    D.FS.met = c->met;
+    c->met_held = true;
     D.dcur = b->dcur + i;
     dcur_init[i] = c->dcur;
     D.st = c->st;
     const Grid& g = c->g;
-    batch_field_tiles(g, sizeof(T) == sizeof(float), &D.btiles, &D.etiles);
-    for (long long q = 0; q < D.btiles.count(); ++q) btile.push_back(BlockEntry{i, (int)q});
-    for (long long q = 0; q < D.etiles.count(); ++q) etile.push_back(BlockEntry{i, (int)q});
+    D.tiles = tiles[i];
+    const long long ntile = D.tiles.count() + batch_shell_blocks(g);
+    for (long long q = 0; q < ntile; ++q) tile.push_back(BlockEntry{i, (int)q});
     append_blocks(all, i, g.ncell, 256);
     for (int s = 0; s < kMaxSpecies; ++s) {
       SpeciesStore& S = c->sp[s];
@@ -1363,13 +1417,11 @@ grpic_status batch_build(grpic_batch* b) {
   }
   b->npairs = (int)pairs.size();
   b->nbins = std::max<long long>(nbins, 1);
-  b->nbtile = (int)btile.size();
-  b->netile = (int)etile.size();
+  b->ntile = (int)tile.size();
   b->nall = (int)all.size();
   b->npart = (int)part.size();
   b->desc = batch_alloc(b, sizeof(InstDesc<T>) * n);
-  b->btile = static_cast<BlockEntry*>(batch_alloc(b, sizeof(BlockEntry) * std::max<size_t>(1, btile.size())));
-  b->etile = static_cast<BlockEntry*>(batch_alloc(b, sizeof(BlockEntry) * std::max<size_t>(1, etile.size())));
+  b->tile = static_cast<BlockEntry*>(batch_alloc(b, sizeof(BlockEntry) * std::max<size_t>(1, tile.size())));
   b->all = static_cast<BlockEntry*>(batch_alloc(b, sizeof(BlockEntry) * std::max<size_t>(1, all.size())));
   b->part = static_cast<BlockEntry*>(batch_alloc(b, sizeof(BlockEntry) * std::max<size_t>(1, part.size())));
   b->counts = static_cast<int*>(batch_alloc(b, sizeof(int) * b->nbins));
@@ -1378,15 +1430,14 @@ grpic_status batch_build(grpic_batch* b) {
   b->pairs = static_cast<int*>(batch_alloc(b, sizeof(int) * std::max(1, b->npairs)));
   // pair_base: npairs per-step bases, then pair_of_inst for every instance * 4 + species
   b->pair_base = static_cast<int*>(batch_alloc(b, sizeof(int) * (b->npairs + 4 * n)));
-  if (!b->desc || !b->btile || !b->etile || !b->all || !b->part || !b->counts || !b->offsets || !b->tiles ||
+  if (!b->desc || !b->tile || !b->all || !b->part || !b->counts || !b->offsets || !b->tiles ||
       !b->pairs || !b->pair_base)
     return GRPIC_ERR_OOM;
   std::vector<int> pair_of_inst(4 * n, 0);
   for (int p = 0; p < b->npairs; ++p) pair_of_inst[pairs[p]] = p;
   cudaStream_t st = b->stream;
   cudaMemcpyAsync(b->desc, desc.data(), sizeof(InstDesc<T>) * n, cudaMemcpyHostToDevice, st);
-  cudaMemcpyAsync(b->btile, btile.data(), sizeof(BlockEntry) * btile.size(), cudaMemcpyHostToDevice, st);
-  cudaMemcpyAsync(b->etile, etile.data(), sizeof(BlockEntry) * etile.size(), cudaMemcpyHostToDevice, st);
+  cudaMemcpyAsync(b->tile, tile.data(), sizeof(BlockEntry) * tile.size(), cudaMemcpyHostToDevice, st);
   cudaMemcpyAsync(b->dcur, dcur_init.data(), sizeof(int) * n, cudaMemcpyHostToDevice, st);
   cudaMemcpyAsync(b->all, all.data(), sizeof(BlockEntry) * all.size(), cudaMemcpyHostToDevice, st);
   if (!part.empty())
@@ -1452,7 +1503,8 @@ void batch_enqueue_step(grpic_batch* b, int k) {
   else
     launch_batch_push<T>(t, b->quad, b->stream);
   launch_batch_b_half<T>(t, 1, b->literal, b->stream);
-  launch_batch_e_step<T>(t, b->literal, b->stream);
+  if (!b->literal) launch_batch_e_step<T>(t, 0, b->literal, b->stream);
+  launch_batch_e_step<T>(t, 1, b->literal, b->stream);
   launch_batch_flip_d<T>(t, (int)b->ctxs.size(), b->stream);
   launch_batch_sort<T>(t, b->stream);
 }
@@ -1482,7 +1534,6 @@ grpic_status grpic_batch_create(grpic_ctx* const* ctxs, int n, void* stream, grp
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   b->sms = std::max(1, sms);
   b->persist_blocks = b->sms * 8;
-  b->persist_field_blocks = b->sms * 2;
   bool ok = cudaStreamCreateWithFlags(&b->stream, cudaStreamNonBlocking) == cudaSuccess &&
             cudaEventCreateWithFlags(&b->ev, cudaEventDisableTiming) == cudaSuccess &&
             cudaEventCreateWithFlags(&b->ev_fork, cudaEventDisableTiming) == cudaSuccess;
@@ -1499,10 +1550,10 @@ grpic_status grpic_batch_create(grpic_ctx* const* ctxs, int n, void* stream, grp
     grpic_batch_destroy(b);
     return s;
   }
-  // kernels per step: B halves 2, zero J 1, push (FP32-mixed: one per pair; FP64: 1), E 1, d parity 1,
+  // kernels per step: B halves 2, zero J 1, push (FP32-mixed: one per pair; FP64: 1), E 2 (literal 1), d parity 1,
   // sort 5 (+2 with particles; and 1 memset)
   const int push_launches = b->npart > 0 ? (b->mixed ? b->npairs : 1) : 0;
-  b->kernels_per_step = 2 + 1 + push_launches + 1 + 1 + (b->npairs ? 5 + 2 * (b->npart > 0 ? 1 : 0) : 0);
+  b->kernels_per_step = 2 + 1 + push_launches + (b->literal ? 1 : 2) + 1 + (b->npairs ? 5 + 2 * (b->npart > 0 ? 1 : 0) : 0);
   *out = b;
   return GRPIC_OK;
 }
@@ -1608,7 +1659,7 @@ grpic_status grpic_batch_set_blocks_per_sm(grpic_batch* b, int blocks_per_sm) {
 grpic_status grpic_batch_info(grpic_batch* b, int64_t* kernels_per_step, int64_t* work_blocks) {
   if (!b) return GRPIC_ERR_INVALID;
   if (kernels_per_step) *kernels_per_step = b->kernels_per_step;
-  if (work_blocks) *work_blocks = (int64_t)b->nbtile + b->netile + b->nall + b->npart;
+  if (work_blocks) *work_blocks = (int64_t)b->ntile + b->nall + b->npart;
   return GRPIC_OK;
 }
 

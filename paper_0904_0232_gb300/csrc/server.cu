@@ -13,7 +13,7 @@
 #include <map>
 #include <vector>
 
-#include "../../include/grpic.h"
+#include "internal.h"
 
 namespace {
 
@@ -169,7 +169,7 @@ grpic_status start_run(grpic_server* s, Run* r) {
   cfg.free_fn = s->free_fn;
   cfg.alloc_user = s->user;
   cfg.sort_interval = 1;
-  grpic_status st = grpic_create(&cfg, s->stream, &r->ctx);
+  grpic_status st = grpic::create_context(&cfg, s->stream, /*metric_table=*/false, &r->ctx);
   if (st != GRPIC_OK) return st;
   st = grpic_set_uniform_field(r->ctx, r->req.E_contra, r->req.B_contra);
   if (st != GRPIC_OK) return st;
