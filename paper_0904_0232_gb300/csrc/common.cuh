@@ -188,7 +188,8 @@ void launch_e_step(const Grid& g, const EStepArgs<T>& A, int sms, cudaStream_t s
 void batch_field_tiles(const Grid* const* grids, int n, size_t word, int sms, TileGrid* tiles);
 int batch_shell_blocks(const Grid& g);
 template <typename T>
-void launch_uniform_field(const Grid& g, const Fields<T>& F, const double E[3], const double B[3], cudaStream_t st);
+void launch_uniform_field(const Grid& g, const Fields<T>& F, const uint16_t* loc, const double E[3], const double B[3],
+                          cudaStream_t st);
 template <typename T>
 void launch_convert_in(T* dst, const double* src, long long n, cudaStream_t st);
 template <typename T>

@@ -71,6 +71,17 @@ __device__ __forceinline__ double rcp_t(double v) { return FastOps64::rcp(v); }
 __device__ __forceinline__ float mul_t(float a, float b) { return a * b; }
 __device__ __forceinline__ double mul_t(double a, double b) { return __dmul_rn(a, b); }
 
+// Conversions between FP64 and the field type with integer operations (the hardware's run on the FP64 pipe).
+template <typename T>
+__device__ __forceinline__ T narrow_t(double v) {
+  if constexpr (sizeof(T) == sizeof(float))
+    return narrow(v);
+  else
+    return v;
+}
+__device__ __forceinline__ double widen_t(float v) { return widen(v); }
+__device__ __forceinline__ double widen_t(double v) { return v; }
+
 constexpr int kTX = 32;  // threads (cells) of a patch along x: one warp per row
 
 // Metric at a point.  FP32: f and k of Eqs. 4-5; FP64: G = f / (1 + f) and k.
@@ -811,31 +822,38 @@ __global__ void k_location_flags(const Grid g, uint16_t* __restrict__ loc) {
 }
 
 // ---- initial conditions / conversions ----------------------------------------------------
+// b_Q = h_Q + f (v x k)_Q at its face with v = k x h + d, the contravariant (h, d) uniform (g = eta + f k k
+// lowers the tensor of Eq. 8).  FP64-pipe bound: FastOps64, and the excised locations from the flags.
+//@UNIFORM@
+template <int Q, typename T>
+__device__ __forceinline__ T uniform_b(const Grid& g, int i, int j, int k, bool excised, const double h[3],
+                                       const double d[3]) {
+  if (excised || !(g.m > 0.0)) return (T)h[Q];
+  constexpr int L = 3 + Q, M = (Q + 1) % 3, N = (Q + 2) % 3;
+  const Kerr<double> K = kerr_eval_fast(i + 0.5 * half(L, 0) - g.xc, j + 0.5 * half(L, 1) - g.yc,
+                                        k + 0.5 * half(L, 2) - g.zc, g.m, g.a);
+  const double kv[3] = {K.k0, K.k1, K.k2};
+  const double vM = fma(kv[N], h[Q], fma(-kv[Q], h[N], d[M])), vN = fma(kv[Q], h[M], fma(-kv[M], h[Q], d[N]));
+  return narrow_t<T>(fma(K.f, fma(vM, kv[N], -(kv[M] * vN)), h[Q]));
+}
+
 template <typename T>
-__global__ void k_uniform_field(const Grid g, const Fields<T> F, double E0, double E1, double E2, double B0,
-                                double B1, double B2) {
+__global__ void k_uniform_field(const Grid g, const Fields<T> F, const uint16_t* __restrict__ loc, double E0, double E1,
+                                double E2, double B0, double B1, double B2) {
   const long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (c >= g.ncell) return;
   const int i = (int)(c % g.nx);
   const int j = (int)((c / g.nx) % g.ny);
   const int k = (int)(c / ((long long)g.nx * g.ny));
+  const uint16_t w = loc[c];
   const double h[3] = {B0, B1, B2};
   const double d[3] = {-E0, -E1, -E2};
   F.d[0][c] = (T)d[0];
   F.d[1][c] = (T)d[1];
   F.d[2][c] = (T)d[2];
-#pragma unroll
-  for (int q = 0; q < 3; ++q) {
-    const int l = 3 + q;
-    const double X = i + 0.5 * half(l, 0) - g.xc;
-    const double Y = j + 0.5 * half(l, 1) - g.yc;
-    const double Z = k + 0.5 * half(l, 2) - g.zc;
-    const Kerr<double> K = kerr_eval<double>(X, Y, Z, g.m, g.a);
-    const bool excised = K.flat || K.r < g.r_exc;
-    double bl[3];
-    lower_spatial<double>(excised ? 0.0 : K.f, K.k0, K.k1, K.k2, h, d, bl);
-    F.b[q][c] = (T)bl[q];
-  }
+  F.b[0][c] = uniform_b<0, T>(g, i, j, k, exc(w, 3), h, d);
+  F.b[1][c] = uniform_b<1, T>(g, i, j, k, exc(w, 4), h, d);
+  F.b[2][c] = uniform_b<2, T>(g, i, j, k, exc(w, 5), h, d);
 }
 
 // ---- read-out of the contravariant face components --------------------------------------------
@@ -889,12 +907,12 @@ __global__ void k_contra_h(const Grid g, const FieldConsts<T> K, const Fields<T>
 template <typename T>
 __global__ void k_convert_in(T* __restrict__ dst, const double* __restrict__ src, long long n) {
   const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (i < n) dst[i] = (T)src[i];
+  if (i < n) dst[i] = narrow_t<T>(src[i]);
 }
 template <typename T>
 __global__ void k_convert_out(double* __restrict__ dst, const T* __restrict__ src, long long n) {
   const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (i < n) dst[i] = (double)src[i];
+  if (i < n) dst[i] = widen_t(src[i]);
 }
 
 inline unsigned blocks_for(long long n, int bs) { return (unsigned)((n + bs - 1) / bs); }
@@ -1071,8 +1089,9 @@ void launch_batch_flip_d(const BatchTables<T>& bt, int ninst, cudaStream_t st) {
 }
 
 template <typename T>
-void launch_uniform_field(const Grid& g, const Fields<T>& F, const double E[3], const double B[3], cudaStream_t st) {
-  k_uniform_field<T><<<blocks_for(g.ncell, 256), 256, 0, st>>>(g, F, E[0], E[1], E[2], B[0], B[1], B[2]);
+void launch_uniform_field(const Grid& g, const Fields<T>& F, const uint16_t* loc, const double E[3], const double B[3],
+                          cudaStream_t st) {
+  k_uniform_field<T><<<blocks_for(g.ncell, 256), 256, 0, st>>>(g, F, loc, E[0], E[1], E[2], B[0], B[1], B[2]);
 }
 
 __global__ void k_add_f64(double* __restrict__ dst, const double* __restrict__ src, long long n) {
@@ -1096,8 +1115,8 @@ void launch_convert_out(double* dst, const T* src, long long n, cudaStream_t st)
 #define GRPIC_INST_FIELDS(T)                                                                             \
   template void launch_b_step<T>(const Grid&, const BStepArgs<T>&, int, cudaStream_t);                  \
   template void launch_e_step<T>(const Grid&, const EStepArgs<T>&, int, cudaStream_t);                  \
-  template void launch_uniform_field<T>(const Grid&, const Fields<T>&, const double*, const double*,     \
-                                        cudaStream_t);                                                   \
+  template void launch_uniform_field<T>(const Grid&, const Fields<T>&, const uint16_t*, const double*,   \
+                                        const double*, cudaStream_t);                                    \
   template void launch_convert_in<T>(T*, const double*, long long, cudaStream_t);                       \
   template void launch_convert_out<T>(double*, const T*, long long, cudaStream_t);                      \
   template void launch_batch_b_half<T>(const BatchTables<T>&, int, bool, cudaStream_t);                 \

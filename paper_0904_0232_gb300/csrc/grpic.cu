@@ -758,9 +758,9 @@ grpic_status grpic_set_fields(grpic_ctx* c, const double* d3, const double* b3, 
 grpic_status grpic_set_uniform_field(grpic_ctx* c, const double E[3], const double B[3]) {
   if (!c || !E || !B) return GRPIC_ERR_INVALID;
   if (c->mixed)
-    launch_uniform_field<float>(c->g, fields_view<float>(c), E, B, c->stream);
+    launch_uniform_field<float>(c->g, fields_view<float>(c), c->loc, E, B, c->stream);
   else
-    launch_uniform_field<double>(c->g, fields_view<double>(c), E, B, c->stream);
+    launch_uniform_field<double>(c->g, fields_view<double>(c), c->loc, E, B, c->stream);
   snapshot_target(c);
   grpic_status s = cuda_check(c, cudaGetLastError(), "set_uniform_field");
   if (s == GRPIC_OK) s = cuda_check(c, cudaStreamSynchronize(c->stream), "set_uniform_field sync");

@@ -80,28 +80,88 @@ struct SeededOps64 {
   }
 };
 
-// FP64 reciprocal and reciprocal square root to FP64 accuracy without the compiler's divide and root
-// sequences: the hardware's approximate values (relative error e below 2^-18) refined once by the
-// third-order step of the series (1 - e)^-1 = 1 + e + e^2 + O(e^3) and
-// (1 - e)^-1/2 = 1 + e/2 + 3 e^2/8 + O(e^3), e = 1 - x y or 1 - x y^2 formed with a fused multiply-add;
-// the truncation (e^3, below 2^-54) stays under the rounding of the last operation.  3 and 5 FP64 operations;
-// this GPU issues one FP64 warp instruction per 16 cycles and SM, and its FP64 kernels are bound by their count
-// (IEEE 1/x, sqrt x and 1/sqrt x take about 9, 10 and 20).  0, subnormals and infinities give NaN or the
-// hardware's limit, which every caller screens as it screens the IEEE results.
+// FP64 reciprocal, square root and reciprocal square root to FP64 accuracy with 1, 2 and 2 FP64 operations.  This GPU issues
+// one FP64 warp instruction per 16 cycles and SM, 64 times slower than FP32 and integer ones, and its FP64 kernels are
+// bound by their count (IEEE 1/x, sqrt x and 1/sqrt x take about 9, 10 and 20), so everything else is done beside the FP64
+// pipe:
+//   1. the argument's mantissa as two floats xh + xl (46 bits), y0 ~ xh^-1/2 (or xh^-1) from the FP32 approximation,
+//      r = 1 - x y0^2 (1 - x y0) in FP32 with fused multiply-adds, whose rounding (2^-24 of r ~ 2^-21) leaves
+//      y = y0 (1 + r/2 + 3 r^2/8) (y0 (1 + r + r^2)) within about 2^-44; the sum is an integer addition to y0's bits;
+//   2. in FP64 the residual e = 1 - x y^2 (with s = x y for the root) or 1 - x y;
+//   3. the first-order step y (1 + e/2), s (1 + e/2) or y (1 + e), whose correction is below 2^12 units in the last place:
+//      formed in FP32, rounded to an integer and added to the bits (where that crosses a power of two, which changes the
+//      unit, in FP64).  The truncation is of order e^2.
+// The result is within one unit in the last place (measured: 0.75).  Arguments are positive normal numbers (rcp:
+// of either sign); root gives 0 for 0 and subnormals.  Others give no useful value, and callers screen them.
 struct FastOps64 {
+ private:
+  // mantissa of x in [1, 2), or [1, 4) where odd, as xh + xl
+  __device__ static __forceinline__ void split(int hi, int lo, int odd, float* xh, float* xl) {
+    const unsigned m = ((unsigned)(hi & 0xfffff) << 3) | ((unsigned)lo >> 29);
+    *xh = __uint_as_float(((127u + odd) << 23) | m);
+    const float low = __uint_as_float(0x4B000000u | (((unsigned)lo & 0x1fffffffu) >> 6)) - 8388608.f;
+    *xl = low * (odd ? 0x1p-45f : 0x1p-46f);
+  }
+  // y0 + c (y0 in [0.5, 1]) times 2^-shift, as a double
+  __device__ static __forceinline__ double assemble(float y0, float c, int shift) {
+    const long long bits = ((long long)__float_as_uint(y0) << 29) + ((long long)(896 - shift) << 52);
+    return __longlong_as_double(bits + __float2int_rn(c * 0x1p53f));
+  }
+  // y (1 + e scale), |e| < 2^-40
+  __device__ static __forceinline__ double correct(double y, double e, float scale) {
+    const int eh = __double2hiint(e);
+    const unsigned ee = ((unsigned)eh >> 20) & 0x7ffu;
+    const float ef = ee < 923u ? 0.f
+                               : __uint_as_float(((unsigned)eh & 0x80000000u) | ((ee - 896u) << 23) |
+                                                 (((unsigned)eh & 0xfffffu) << 3) | ((unsigned)__double2loint(e) >> 29));
+    const float m = __uint_as_float(0x3f800000u | (((unsigned)__double2hiint(y) & 0xfffffu) << 3) |
+                                    ((unsigned)__double2loint(y) >> 29));
+    const long long b0 = __double_as_longlong(y), b1 = b0 + __float2int_rn(ef * (m * scale));
+    if (((b0 ^ b1) >> 52) != 0) return crossing(y, e, scale);
+    return __longlong_as_double(b1);
+  }
+  __device__ static __noinline__ double crossing(double y, double e, float scale) {
+    return fma(y * e, scale == 0x1p52f ? 1.0 : 0.5, y);
+  }
+  __device__ static __forceinline__ double rsqrt_start(double x) {
+    const int hi = __double2hiint(x), lo = __double2loint(x);
+    const int E = (hi >> 20) - 1023, odd = E & 1;
+    float xh, xl;
+    split(hi, lo, odd, &xh, &xl);
+    const float y0 = fminf(fmaxf(rsqrtf(xh), 0.5f), 1.f);
+    const float t = __fmul_rn(xh, y0);
+    float r = __fmaf_rn(-t, y0, 1.f);
+    r = __fmaf_rn(-__fmaf_rn(xh, y0, -t), y0, r);
+    r = __fmaf_rn(-__fmul_rn(xl, y0), y0, r);
+    return assemble(y0, y0 * (r * __fmaf_rn(0.375f, r, 0.5f)), (E - odd) >> 1);
+  }
+
+ public:
   __device__ static __forceinline__ double rcp(double x) {
-    double y;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    const double e = fma(-x, y, 1.0);
-    return fma(y, fma(e, e, e), y);
+    const int hi = __double2hiint(x), lo = __double2loint(x);
+    float xh, xl, y0;
+    split(hi, lo, 0, &xh, &xl);
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y0) : "f"(xh));
+    y0 = fminf(fmaxf(y0, 0.5f), 1.f);
+    float r = __fmaf_rn(-xh, y0, 1.f);
+    r = __fmaf_rn(-xl, y0, r);
+    const double y = assemble(y0, y0 * __fmaf_rn(r, r, r), ((hi & 0x7fffffff) >> 20) - 1023);
+    const double ys = __hiloint2double(__double2hiint(y) | (hi & 0x80000000), __double2loint(y));
+    return correct(ys, fma(-x, ys, 1.0), 0x1p52f);
   }
   __device__ static __forceinline__ double rsqrt(double x) {
-    double y;
-    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    const double e = fma(-x * y, y, 1.0);
-    return fma(y * e, fma(0.375, e, 0.5), y);
+    const double y = rsqrt_start(x);
+    return correct(y, fma(-x * y, y, 1.0), 0x1p51f);
+  }
+  __device__ static __forceinline__ double root(double x) {
+    const double y = rsqrt_start(x), s = x * y;
+    const double v = correct(s, fma(-s, y, 1.0), 0x1p51f);
+    return (__double2hiint(x) & 0x7fffffff) < 0x00100000 ? 0.0 : v;
   }
 };
+
+// x / 2 for a positive normal x, without an FP64 operation.
+__device__ __forceinline__ double halve(double x) { return __hiloint2double(__double2hiint(x) - 0x00100000, __double2loint(x)); }
 
 template <typename S>
 struct Kerr {
@@ -152,30 +212,86 @@ __device__ __forceinline__ Kerr<S> kerr_from_r2(S x, S y, S z, S m, S a, S r2, S
   return K;
 }
 
-// Integrand of Eq. 18 for the plane normal to axis K: g_II g_JJ - g_IJ^2 = 1 + f (k_I^2 + k_J^2)
-// and, k being null for eta (Eq. 6), k_I^2 + k_J^2 = 1 - k_K^2.  Given r^2 from Eq. 6.
-template <typename S>
-__device__ __forceinline__ S area_density(S x, S y, S z, S m, S a, S r2, int K) {
-  if (!(r2 > S(0))) return S(1);
-  const S r = sqrt(r2);
-  const S a2 = a * a;
-  const S sig = r2 * r2 + a2 * z * z;
-  if (K == 2) {
-    // f (1 - z^2/r^2) = 2 m r (r^2 - z^2) / Sigma
-    return sqrt(S(1) + S(2) * m * r * (r2 - z * z) / sig);
-  }
-  // f (1 - k_K^2) with k_x = (r x - a y)/(r^2+a^2), k_y = (r y + a x)/(r^2+a^2)
-  const S num = (K == 0) ? (r * x - a * y) : (r * y + a * x);
-  const S rho2 = r2 + a2;
-  const S kk = num * num / (rho2 * rho2);
-  return sqrt(S(1) + S(2) * m * r * r2 * (S(1) - kk) / sig);
-}
-
 template <typename S, typename Ops = IeeeOps>
 __device__ __forceinline__ Kerr<S> kerr_eval(S x, S y, S z, S m, S a) {
   S D;
   const S r2 = kerr_r2<S, Ops>(x, y, z, a, &D);
   return kerr_from_r2<S, Ops>(x, y, z, m, a, r2, D);
+}
+
+// kerr_eval in FP64 with FastOps64; since the root satisfies Sigma = r^4 + a^2 z^2 = r^2 D, 1 / Sigma and f = 2 m r / D
+// need no division.  The root for p = R^2 - a^2 < 0 is out of line (its operations would be issued for every point).
+static __device__ __noinline__ double kerr_root_inside(double p, double q4, double D) {
+  return halve(q4 * FastOps64::rcp(D - p));
+}
+__device__ __forceinline__ Kerr<double> kerr_eval_fast(double x, double y, double z, double m, double a) {
+  Kerr<double> K;
+  const double a2 = a * a;
+  const double q4 = 4.0 * a2 * (z * z);
+  const double p = fma(x, x, fma(y, y, fma(z, z, -a2)));
+  const double D2 = fma(p, p, q4);
+  K.inv_D = FastOps64::rsqrt(D2);
+  K.D = D2 * K.inv_D;
+  double r2 = halve(p + K.D);
+  if (__double2hiint(p) < 0) r2 = kerr_root_inside(p, q4, K.D);
+  if (__double2hiint(D2) < 0x00100000 || __double2hiint(r2) < 0x00100000) {  // r = 0
+    K.flat = true;
+    K.r = K.f = K.k0 = K.k1 = 0.0;
+    K.k2 = 1.0;
+    return K;
+  }
+  K.flat = false;
+  K.inv_r = FastOps64::rsqrt(r2);
+  K.r = r2 * K.inv_r;
+  K.inv_rho2 = FastOps64::rcp(r2 + a2);
+  K.inv_sig = K.inv_D * (K.inv_r * K.inv_r);
+  K.f = 2.0 * m * K.r * K.inv_D;
+  K.k0 = fma(K.r, x, -(a * y)) * K.inv_rho2;
+  K.k1 = fma(K.r, y, a * x) * K.inv_rho2;
+  K.k2 = z * K.inv_r;
+  return K;
+}
+
+// christoffel_uu (below) in FP64 without forming d_i k_j.  With u.r = u^i d_i r, k_x = (r x - a y) / rho^2 and so on,
+//   D_x = [x u.r + r u^x - a u^y - 2 r (u.r) k_x] / rho^2,  D_y alike,  D_z = (u^z - k_z u.r) / r,
+//   E_j = A d_j r + ((r u^x + a u^y) / rho^2, (r u^y - a u^x) / rho^2, u^z / r)_j,
+//   A = [u^x x + u^y y - 2 r (u^x k_x + u^y k_y)] / rho^2 - u^z k_z / r,
+// and d_r f = f (3 / r - 4 r / D).
+__device__ __forceinline__ void christoffel_uu_fast(const Kerr<double>& K, double x, double y, double z, double a,
+                                                    const double u[4], double out[4]) {
+  if (K.flat) {
+    out[0] = out[1] = out[2] = out[3] = 0.0;
+    return;
+  }
+  const double r = K.r, f = K.f, k0 = K.k0, k1 = K.k1, k2 = K.k2, ir = K.inv_r, ip = K.inv_rho2;
+  const double rD = r * K.inv_D, two_r = r + r, a2 = a * a;
+  const double rx = x * rD, ry = y * rD, rz = z * (fma(r, r, a2) * (K.inv_D * ir));
+  const double fr = f * fma(3.0, ir, -4.0 * rD);
+  const double fx = fr * rx, fy = fr * ry, fz = fma(fr, rz, -2.0 * a2 * z * (f * K.inv_sig));
+  const double ur = fma(u[0], rx, fma(u[1], ry, u[2] * rz));
+  const double t = two_r * ur;
+  const double p0 = r * u[0], p1 = r * u[1];
+  const double D0 = fma(-t, k0, fma(x, ur, fma(-a, u[1], p0))) * ip;
+  const double D1 = fma(-t, k1, fma(y, ur, fma(a, u[0], p1))) * ip;
+  const double D2 = fma(-k2, ur, u[2]) * ir;
+  const double uk = fma(u[0], k0, u[1] * k1), u2i = u[2] * ir;
+  const double A = fma(fma(-two_r, uk, fma(u[0], x, u[1] * y)), ip, -(k2 * u2i));
+  const double E0 = fma(A, rx, fma(a, u[1], p0) * ip);
+  const double E1 = fma(A, ry, fma(-a, u[0], p1) * ip);
+  const double E2 = fma(A, rz, u2i);
+  const double s = fma(k2, u[2], uk) + u[3];
+  const double uf = fma(u[0], fx, fma(u[1], fy, u[2] * fz));
+  const double uD = fma(u[0], D0, fma(u[1], D1, u[2] * D2));
+  const double c1 = fma(uf, s, f * uD), fs = f * s, hs2 = -0.5 * s * s;
+  const double w0 = fma(c1, k0, fma(fs, D0 - E0, hs2 * fx));
+  const double w1 = fma(c1, k1, fma(fs, D1 - E1, hs2 * fy));
+  const double w2 = fma(c1, k2, fma(fs, D2 - E2, hs2 * fz));
+  const double kw = fma(k0, w0, fma(k1, w1, fma(k2, w2, -c1)));
+  const double fk = f * kw;
+  out[0] = fma(-fk, k0, w0);
+  out[1] = fma(-fk, k1, w1);
+  out[2] = fma(-fk, k2, w2);
+  out[3] = fk - c1;
 }
 
 // Gamma^a_mn u^m u^n = g^ab (u^m d_m g_bn u^n - 1/2 d_b g_mn u^m u^n) for g = eta + f k k.
@@ -256,13 +372,14 @@ __device__ __forceinline__ void contra_spatial(S f, S k0, S k1, S k2, const S b[
   h[2] = (al2 + ka * k2) * inv;
 }
 
-template <typename S>
-__device__ __forceinline__ void cov_electric(S f, S k0, S k1, S k2, const S h[3], const S d[3], S e[3]) {
-  const S kd = k0 * d[0] + k1 * d[1] + k2 * d[2];
-  const S fm1 = f - S(1);
-  e[0] = f * (k1 * h[2] - k2 * h[1]) + fm1 * d[0] - f * k0 * kd;
-  e[1] = f * (k2 * h[0] - k0 * h[2]) + fm1 * d[1] - f * k1 * kd;
-  e[2] = f * (k0 * h[1] - k1 * h[0]) + fm1 * d[2] - f * k2 * kd;
+// contra_spatial in FP64: with G = f / (1 + f) the same tensor is h = b - G [b + d x k - k (k.b)].
+__device__ __forceinline__ void contra_spatial_fast(double f, double k0, double k1, double k2, const double b[3],
+                                                    const double d[3], double h[3]) {
+  const double G = f * FastOps64::rcp(1.0 + f);
+  const double kb = fma(k0, b[0], fma(k1, b[1], k2 * b[2]));
+  h[0] = fma(-G, fma(-k0, kb, b[0]) + fma(d[1], k2, -(d[2] * k1)), b[0]);
+  h[1] = fma(-G, fma(-k1, kb, b[1]) + fma(d[2], k0, -(d[0] * k2)), b[1]);
+  h[2] = fma(-G, fma(-k2, kb, b[2]) + fma(d[0], k1, -(d[1] * k0)), b[2]);
 }
 
 // Lorentz part of Eq. 15, (q/m) F^a_b u^b = (q/m) F^ac u_c, with u_c = g_cb u^b:
@@ -280,27 +397,14 @@ __device__ __forceinline__ void lorentz(S qm, S f, S k0, S k1, S k2, const S h[3
   out[3] = -qm * (d[0] * c0 + d[1] * c1 + d[2] * c2);
 }
 
-// Covariant spatial block of a contravariant tensor given as (h, d): with v_i = F^{i b} k_b,
-// (g F g)_ij = F^ij + f (v_i k_j - k_i v_j).  Returns (F_yz, F_zx, F_xy).
-template <typename S>
-__device__ __forceinline__ void lower_spatial(S f, S k0, S k1, S k2, const S h[3], const S d[3], S b[3]) {
-  // F^{ij} k_j = (k x h) components with sign: F^{il} k_l = eps_ilm k_l h_m = (k x h)_i
-  const S v0 = (k1 * h[2] - k2 * h[1]) + d[0];
-  const S v1 = (k2 * h[0] - k0 * h[2]) + d[1];
-  const S v2 = (k0 * h[1] - k1 * h[0]) + d[2];
-  b[0] = h[0] + f * (v1 * k2 - k1 * v2);
-  b[1] = h[1] + f * (v2 * k0 - k2 * v0);
-  b[2] = h[2] + f * (v0 * k1 - k0 * v1);
-}
-
 // Eq. 16: gamma = [u^4/c + sqrt((u^4/c)^2 + 4 a^4 dt / (2c))] / 2; a negative argument or a
 // non-positive result falls back to u^4/c (the caller counts it).
-template <typename S>
+template <typename S, typename Ops = IeeeOps>
 __device__ __forceinline__ S gamma_step(S u4, S a4, S inv_c, S dt, bool* fallback) {
   const S w = u4 * inv_c;
   const S arg = w * w + S(2) * a4 * dt * inv_c;
   S g = S(-1);
-  if (arg >= S(0)) g = S(0.5) * (w + sqrt(arg));
+  if (arg >= S(0)) g = S(0.5) * (w + Ops::root(arg));
   if (!(g > S(0))) {
     *fallback = true;
     return w;

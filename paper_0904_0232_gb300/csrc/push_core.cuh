@@ -28,6 +28,7 @@
 #include <cuda_fp16.h>
 
 #include <cmath>
+#include <type_traits>
 
 #include "common.cuh"
 #include "metric.cuh"
@@ -156,6 +157,30 @@ __device__ __forceinline__ void christoffel_uu_x2(const Kerr<float>& K, float x,
   out[3] = -c1 + f * kw;
 }
 
+// floor of x as an integer and in T.  FP64: from the bits (the FP64 pipe, which would also do the conversions, stays
+// free); negative, huge and non-finite x take the conversions.
+__device__ __forceinline__ void floor_split(float x, int& i, float& fl) {
+  i = (int)floorf(x);
+  fl = (float)i;
+}
+__device__ __forceinline__ void floor_split(double x, int& i, double& fl) {
+  const int hi = __double2hiint(x), e = (hi >> 20) - 1023;
+  if ((unsigned)hi < 0x41400000u) {  // 0 <= x < 2^21
+    const int drop = 20 - max(e, 0);
+    const int mask = e < 0 ? 0 : (int)(0xffffffffu << drop);
+    i = e < 0 ? 0 : ((hi & 0xfffff) | 0x100000) >> drop;
+    fl = __hiloint2double(hi & mask, 0);
+  } else {
+    i = (int)floor(x);
+    fl = (double)i;
+  }
+}
+__device__ __forceinline__ bool finite_t(float v) { return isfinite(v); }
+__device__ __forceinline__ bool finite_t(double v) { return (__double2hiint(v) & 0x7ff00000) != 0x7ff00000; }
+// |v| < 1 (false for NaN)
+__device__ __forceinline__ bool below_one(float v) { return fabsf(v) < 1.f; }
+__device__ __forceinline__ bool below_one(double v) { return (__double2hiint(v) & 0x7fffffff) < 0x3ff00000; }
+
 template <typename T>
 __device__ __forceinline__ T lerp(T a, T b, T w) {
   return fma(w, b - a, a);
@@ -242,6 +267,20 @@ __device__ __forceinline__ void accel(const Grid& g, const Fields<T>& F, const C
 #pragma unroll
   for (int ax = 0; ax < 3; ++ax) {
     const T s0 = x[ax];
+    if constexpr (sizeof(T) == sizeof(double)) {
+      int a0;
+      double fl;
+      floor_split(s0, a0, fl);
+      const double w = s0 - fl;  // exact, and so is the half lattice's w -+ 1/2
+      const bool upper = __double2hiint(w) >= 0x3fe00000;  // w >= 1/2
+      if (a0 >= 1 && a0 <= nn[ax] - 2) {
+        ii[ax] = a0;
+        ih[ax] = upper ? a0 : a0 - 1;
+        wi[ax] = w;
+        wh[ax] = upper ? w - 0.5 : w + 0.5;
+        continue;
+      }
+    }
     const T s1 = x[ax] - T(0.5);
     if (!(s1 >= T(0)) || !(s0 <= T(nn[ax] - 1))) flags |= ST_RANGE;
     int a0 = (int)floor(s0), a1 = (int)floor(s1);
@@ -294,7 +333,7 @@ __device__ __forceinline__ void accel(const Grid& g, const Fields<T>& F, const C
     // far-field warps: every stage has R > |a| (the quartic's p > 0 branch)
     Kt = mixed ? kerr_eval<T>(X, Y, Z, C.m, C.a) : kerr_far(X, Y, Z, C.m, C.a);
   } else {
-    Kt = kerr_eval<T>(X, Y, Z, C.m, C.a);
+    Kt = kerr_eval_fast(X, Y, Z, C.m, C.a);
   }
   bool promoted = false;
   if constexpr (sizeof(T) == sizeof(float)) {
@@ -317,105 +356,164 @@ __device__ __forceinline__ void accel(const Grid& g, const Fields<T>& F, const C
     if constexpr (sizeof(T) == sizeof(float))
       christoffel_uu_x2(Kt, X, Y, Z, C.a, u, gam);
     else
-      christoffel_uu<T>(Kt, X, Y, Z, C.a, u, gam);
+      christoffel_uu_fast(Kt, X, Y, Z, C.a, u, gam);
     f = Kt.f;
     k0 = Kt.k0;
     k1 = Kt.k1;
     k2 = Kt.k2;
   }
   T h[3], lor[4];
-  contra_spatial(f, k0, k1, k2, b, d, h);
+  if constexpr (sizeof(T) == sizeof(double))
+    contra_spatial_fast(f, k0, k1, k2, b, d, h);
+  else
+    contra_spatial(f, k0, k1, k2, b, d, h);
   lorentz(C.qm, f, k0, k1, k2, h, d, u, lor);
 #pragma unroll
   for (int q = 0; q < 4; ++q) out[q] = lor[q] - gam[q];
 }
 
-// Integrand of Eq. 18, sqrt(g_II g_JJ - g_IJ^2) = sqrt(1 + f (k_I^2 + k_J^2)), at a grid
-// position (the FP64 path; the FP32 paths use deposit_lattice).
-template <typename T>
-__device__ __forceinline__ T area_integrand(const Consts<T>& C, T px, T py, T pz, int K) {
-  const T X = px - C.xc, Y = py - C.yc, Z = pz - C.zc;
-  T D;
-  const T r2 = kerr_r2<T>(X, Y, Z, C.a, &D);
-  return area_density<T>(X, Y, Z, C.m, C.a, r2, K);
-}
-
-// AREA of Eq. 18 over [Is, If] x [Js, Jf] in the plane x^K = xK.
-template <typename T, int Q>
-__device__ __forceinline__ T area(const Consts<T>& C, int K, T xK, T Is, T If, T Js, T Jf) {
-  T s = T(0);
-  const T ci = T(0.5) * (Is + If), hi = T(0.5) * (If - Is);
-  const T cj = T(0.5) * (Js + Jf), hj = T(0.5) * (Jf - Js);
+// The four sub-rectangle AREAs of Eq. 18 of a face in FP64, plane x^K = XK (relative to the centre), the cell's lower
+// corner at (oI, oJ) relative to the centre along (I, J) = (K+1, K+2) mod 3, split at the fractions (u, v).  The Q x Q
+// Gauss nodes of the four rectangles make a 2Q x 2Q lattice, on which p = R^2 - a^2, 4 q = 4 a^2 z^2 and the spin
+// term of k_K's numerator are sums of a row and a column term.  With D = sqrt(p^2 + 4 q), r^2 = (p + D) / 2 and
+// f = 2 m r / D the integrand 1 + f (1 - k_K^2) (k being null, Eq. 6) is N / M,
+//   M = D rho^4, N = M + 2 m r (rho^4 - num^2), k_K = num / rho^2    (K = 0: num = r x - a y, 1: r y + a x)
+//   M = D r,     N = M + 2 m (r^2 - z^2)                             (K = 2),
+// so that a node takes two roots and one reciprocal root, sqrt(N / M) = N / sqrt(N M).
+// FP64 operations bound the push in FP64 (one FP64 warp instruction per 16 cycles and SM): 19 a node (15 for K = 2) and 96
+// nodes a particle-step at Q = 2, where one IEEE evaluation of the integrand per node took about 78.
+//@PUSH64@
+// r = 0 takes the flat limit 1.
+// A00 = [u,1] x [v,1], A10 = [0,u] x [v,1], A01 = [u,1] x [0,v], A11 = [0,u] x [0,v].
+template <int Q, int K>
+__device__ __forceinline__ void lattice_areas(const Consts<double>& C, double XK, double oI, double oJ, double u,
+                                              double v, double& A00, double& A10, double& A01, double& A11) {
+  const double wu = 1.0 - u, wv = 1.0 - v;
+  const double zz = XK * XK;
+  const double a4 = 4.0 * C.a2, pK = zz - C.a2, qK = a4 * zz;
+  double pJ[2 * Q], qJ[2 * Q], tJ[2 * Q];
+  const double oJv = oJ + v;
 #pragma unroll
-  for (int p = 0; p < Q; ++p)
+  for (int j = 0; j < 2 * Q; ++j) {
+    const double gx = 0.5 + 0.5 * Gauss<Q>::x(j % Q);
+    const double X = j < Q ? fma(v, gx, oJ) : fma(wv, gx, oJv);
+    pJ[j] = X * X;
+    qJ[j] = K == 0 ? a4 * pJ[j] : 0.0;
+    tJ[j] = K == 1 ? C.a * X : 0.0;
+  }
+  double S[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
 #pragma unroll
-    for (int q = 0; q < Q; ++q) {
-      const T xi = ci + hi * (T)Gauss<Q>::x(p);
-      const T xj = cj + hj * (T)Gauss<Q>::x(q);
-      // (x^K, x^I, x^J) -> (x, y, z) with I = K+1, J = K+2 (mod 3)
-      const T px = sel3(K, xK, xj, xi);
-      const T py = sel3(K, xi, xK, xj);
-      const T pz = sel3(K, xj, xi, xK);
-      s += (T)Gauss<Q>::w(p) * (T)Gauss<Q>::w(q) * area_integrand<T>(C, px, py, pz, K);
+  for (int si = 0; si < 2; ++si) {
+    const double lo = si ? oI + u : oI, w = si ? wu : u;
+#pragma unroll 1
+    for (int pi = 0; pi < Q; ++pi) {
+      double gx = 0.5 + 0.5 * Gauss<Q>::x(0), gw = Gauss<Q>::w(0);
+#pragma unroll
+      for (int t = 1; t < Q; ++t)
+        if (pi == t) {
+          gx = 0.5 + 0.5 * Gauss<Q>::x(t);
+          gw = Gauss<Q>::w(t);
+        }
+      const double X = fma(w, gx, lo);
+      const double pR = fma(X, X, pK);
+      const double qR = K == 1 ? a4 * (X * X) : qK;
+      const double tR = K == 0 ? -C.a * X : 0.0;
+#pragma unroll
+      for (int j = 0; j < 2 * Q; ++j) {
+        const double p = pR + pJ[j];
+        const double q4 = K == 0 ? qJ[j] : qR;
+        const double D = FastOps64::root(fma(p, p, q4));
+        double r2 = halve(p + D);
+        if (__double2hiint(p) < 0) r2 = kerr_root_inside(p, q4, D);
+        const double r = FastOps64::root(r2);
+        double M, N;
+        if (K == 2) {
+          M = D * r;
+          N = fma(C.two_m, r2 - zz, M);
+        } else {
+          const double num = fma(r, XK, K == 0 ? tR : tJ[j]);
+          const double rho2 = r2 + C.a2;
+          const double rho4 = rho2 * rho2;
+          M = D * rho4;
+          N = fma(C.two_m * r, fma(-num, num, rho4), M);
+        }
+        double val = N * FastOps64::rsqrt(N * M);
+        if (__double2hiint(r2) < 0x00100000) val = 1.0;  // r = 0: the flat limit
+        if (Q == 2)
+          S[si][j / Q] += val;  // unit Gauss weights
+        else
+          S[si][j / Q] = fma(gw * Gauss<Q>::w(j % Q), val, S[si][j / Q]);
+      }
     }
-  return s * T(0.25) * (If - Is) * (Jf - Js);
+  }
+  A00 = S[1][1] * (wu * wv);
+  A10 = S[0][1] * (u * wv);
+  A01 = S[1][0] * (wu * v);
+  A11 = S[0][0] * (u * v);
 }
 
-// Umeda zig-zag deposit of the move x0 -> x0 + dx.  The segment displacements are carried
+// Umeda zig-zag deposit of the move x0 -> x0 + dx in FP64.  The segment displacements are carried
 // as offsets from x0 (s1 = relay - x0, s2 = dx - s1), so the flux keeps the accuracy of the RK4
 // increment instead of inheriting the rounding of the stored positions.  With |dx| < 1 the
 // relay point min(min(a,b)+1, max(max(a,b), mid)) is the midpoint when the cell does not
 // change along an axis and the shared face otherwise.
-template <typename T, int Q>
-__device__ __forceinline__ void deposit(const Grid& g, const Fields<T>& F, const Consts<T>& C, const T x0[3],
-                                        const T dx[3], T qg, T inv_dt, unsigned& flags) {
+template <int Q>
+__device__ __forceinline__ void deposit64(const Grid& g, const Fields<double>& F, const Consts<double>& C,
+                                          const double x0[3], const double dx[3], double qg, double inv_dt,
+                                          unsigned& flags) {
   const int nn[3] = {g.nx, g.ny, g.nz};
+  const double cen[3] = {C.xc, C.yc, C.zc};
   int c1[3], c2[3];
-  T s1[3], s2[3];
+  double s1[3], s2[3];
 #pragma unroll
   for (int ax = 0; ax < 3; ++ax) {
-    int a = (int)floor(x0[ax]), b = (int)floor(x0[ax] + dx[ax]);
-    if (a < 0 || b < 0 || a > nn[ax] - 2 || b > nn[ax] - 2) flags |= ST_RANGE;
-    a = min(max(a, 0), nn[ax] - 2);
-    b = min(max(b, 0), nn[ax] - 2);
+    int a, b;
+    double fa, fb;
+    floor_split(x0[ax], a, fa);
+    floor_split(x0[ax] + dx[ax], b, fb);
+    if (a < 0 || b < 0 || a > nn[ax] - 2 || b > nn[ax] - 2) {
+      flags |= ST_RANGE;
+      a = min(max(a, 0), nn[ax] - 2);
+      b = min(max(b, 0), nn[ax] - 2);
+      fa = a;
+      fb = b;
+    }
     c1[ax] = a;
     c2[ax] = b;
-    s1[ax] = (a == b) ? T(0.5) * dx[ax] : (T)max(a, b) - x0[ax];
+    s1[ax] = (a == b) ? 0.5 * dx[ax] : (a > b ? fa : fb) - x0[ax];
     s2[ax] = dx[ax] - s1[ax];
   }
   const long long sy = g.nx, sz = (long long)g.nx * g.ny;
 #pragma unroll 1
   for (int seg = 0; seg < 2; ++seg) {
     const int cx = seg ? c2[0] : c1[0], cy = seg ? c2[1] : c1[1], cz = seg ? c2[2] : c1[2];
-    T P[3], dseg[3];
+    const int cell[3] = {cx, cy, cz};
+    // the segment midpoint's fraction fr of its cell and the cell's corner relative to the centre
+    double dseg[3], fr[3], o[3];
 #pragma unroll
     for (int ax = 0; ax < 3; ++ax) {
+      const double cd = __hiloint2double(0x43300000, cell[ax]) - 4503599627370496.0;  // (double)cell
       dseg[ax] = seg ? s2[ax] : s1[ax];
-      P[ax] = seg ? x0[ax] + (s1[ax] + T(0.5) * s2[ax]) : x0[ax] + T(0.5) * s1[ax];
+      fr[ax] = (x0[ax] - cd) + (seg ? fma(0.5, s2[ax], s1[ax]) : 0.5 * s1[ax]);
+      o[ax] = cd - cen[ax];
     }
     const long long base = ((long long)cz * g.ny + cy) * g.nx + cx;
-#pragma unroll 1
-    for (int K = 0; K < 3; ++K) {
-      const T dK = sel3(K, dseg[0], dseg[1], dseg[2]);
-      if (dK == T(0)) continue;
-      const T flux = qg * dK * inv_dt;
-      const T PK = sel3(K, P[0], P[1], P[2]);
-      const T PI = sel3(K, P[1], P[2], P[0]);
-      const T PJ = sel3(K, P[2], P[0], P[1]);
-      const T i0 = (T)sel3(K, cy, cz, cx), j0 = (T)sel3(K, cz, cx, cy);
-      const T A00 = area<T, Q>(C, K, PK, PI, i0 + T(1), PJ, j0 + T(1));
-      const T A10 = area<T, Q>(C, K, PK, i0, PI, PJ, j0 + T(1));
-      const T A01 = area<T, Q>(C, K, PK, PI, i0 + T(1), j0, PJ);
-      const T A11 = area<T, Q>(C, K, PK, i0, PI, j0, PJ);
-      const T FA = A00 + A10 + A01 + A11;
-      const T W00 = A00 / FA, W10 = A10 / FA, W01 = A01 / FA, W11 = A11 / FA;
-      const long long stI = sel3(K, sy, sz, 1ll), stJ = sel3(K, sz, 1ll, sy);
-      double* JK = sel3(K, F.J[0], F.J[1], F.J[2]);
-      atomicAdd(JK + base, to_f64(flux * W00));
-      atomicAdd(JK + base + stI, to_f64(flux * W10));
-      atomicAdd(JK + base + stJ, to_f64(flux * W01));
-      atomicAdd(JK + base + stI + stJ, to_f64(flux * W11));
-    }
+    auto face = [&](auto axis) {
+      constexpr int K = decltype(axis)::value, I = (K + 1) % 3, J = (K + 2) % 3;
+      if (dseg[K] == 0.0) return;
+      double A00, A10, A01, A11;
+      lattice_areas<Q, K>(C, o[K] + fr[K], o[I], o[J], fr[I], fr[J], A00, A10, A01, A11);
+      const double fw = qg * dseg[K] * inv_dt * FastOps64::rcp((A00 + A10) + (A01 + A11));
+      const long long stI = K == 0 ? sy : (K == 1 ? sz : 1), stJ = K == 0 ? sz : (K == 1 ? 1 : sy);
+      double* JK = F.J[K] + base;
+      atomicAdd(JK, fw * A00);
+      atomicAdd(JK + stI, fw * A10);
+      atomicAdd(JK + stJ, fw * A01);
+      atomicAdd(JK + stI + stJ, fw * A11);
+    };
+    face(std::integral_constant<int, 0>());
+    face(std::integral_constant<int, 1>());
+    face(std::integral_constant<int, 2>());
   }
 }
 
@@ -566,7 +664,7 @@ __device__ __forceinline__ void table_areas(const float4* __restrict__ t, float 
   A00 = S1.y * (wu * wv);
 }
 
-// FP32 deposit (the zig-zag split, fluxes and Eq. 18 weights of deposit() below) evaluated on a
+// FP32 deposit (the zig-zag split, fluxes and Eq. 18 weights of deposit64) evaluated on a
 // per-face node lattice: the Q x Q Gauss nodes of the four sub-rectangles of a face make a
 // 2Q x 2Q lattice in (x^I, x^J), so node coordinates, their squares and the spin terms are
 // formed once per face (column terms) or row (row terms), roots are v * rsqrt(v) and each node
@@ -866,7 +964,12 @@ __device__ __forceinline__ Move<T> push_move(const Grid& g, const Fields<T>& F, 
 #pragma unroll 1
   for (int stage = 0; stage < 4; ++stage) {
     accel<T>(g, F, C, xs, us, a, flags, n64, mixed);
-    if (stage == 0) h = C.dt / gamma_step<T>(us[3], a[3], C.inv_c, C.dt, &fb);
+    if (stage == 0) {
+      if constexpr (sizeof(T) == sizeof(double))
+        h = C.dt * FastOps64::rcp(gamma_step<T, FastOps64>(us[3], a[3], C.inv_c, C.dt, &fb));
+      else
+        h = C.dt / gamma_step<T>(us[3], a[3], C.inv_c, C.dt, &fb);
+    }
     const T wgt = (stage == 0 || stage == 3) ? T(1) : T(2);
     const T frac = (stage == 2) ? h : T(0.5) * h;
 #pragma unroll
@@ -878,7 +981,7 @@ __device__ __forceinline__ Move<T> push_move(const Grid& g, const Fields<T>& F, 
     }
   }
   T x0[3], x1[4], u1[4], dx[3];
-  const T h6 = h / T(6);
+  const T h6 = sizeof(T) == sizeof(double) ? h * T(1.0 / 6.0) : h / T(6);
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     const T xq = reload(P.x[q] + i), d = h6 * sx[q];
@@ -890,14 +993,18 @@ __device__ __forceinline__ Move<T> push_move(const Grid& g, const Fields<T>& F, 
     u1[q] = reload(P.u[q] + i) + h6 * su[q];
   }
   x1[3] -= C.cdt;  // x^4 is stored relative to c t
-  const T gbar = C.gamma_in_j ? (reload(P.u[3] + i) + u1[3]) / (T(2) * C.c) : T(1);
+  T gbar = T(1);
+  if (C.gamma_in_j) {
+    const T u4s = reload(P.u[3] + i) + u1[3];
+    gbar = sizeof(T) == sizeof(double) ? u4s * (T(0.5) * C.inv_c) : u4s / (T(2) * C.c);
+  }
   bool finite = true;
 #pragma unroll
-  for (int q = 0; q < 4; ++q) finite = finite && isfinite(x1[q]) && isfinite(u1[q]);
+  for (int q = 0; q < 4; ++q) finite = finite && finite_t(x1[q]) && finite_t(u1[q]);
   if (!finite) flags |= ST_NONFINITE;
 #pragma unroll
   for (int q = 0; q < 3; ++q)
-    if (!(fabs(x1[q] - x0[q]) < T(1))) flags |= ST_CFL;
+    if (!below_one(x1[q] - x0[q])) flags |= ST_CFL;
   // streaming (evict-first) stores: the new state is read again only by the next step or the sort
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
@@ -907,16 +1014,32 @@ __device__ __forceinline__ Move<T> push_move(const Grid& g, const Fields<T>& F, 
   // removal (r <= r_+ or outside [1, n-2]) and the sort key
   bool outer = !finite;
   const int nn[3] = {g.nx, g.ny, g.nz};
+  int ci[3];
 #pragma unroll
-  for (int q = 0; q < 3; ++q)
-    if (!(x1[q] >= T(1) && x1[q] <= T(nn[q] - 2))) outer = true;
+  for (int q = 0; q < 3; ++q) {
+    if constexpr (sizeof(T) == sizeof(double)) {
+      double fl;
+      floor_split(x1[q], ci[q], fl);
+      if (ci[q] < 1 || ci[q] > nn[q] - 2 || (ci[q] == nn[q] - 2 && !(x1[q] == fl))) outer = true;
+    } else {
+      if (!(x1[q] >= T(1) && x1[q] <= T(nn[q] - 2))) outer = true;
+      ci[q] = (int)floor(x1[q]);
+    }
+  }
   bool horizon = false;
   if (finite && C.massive) {
-    // screen in T, decide in FP64 near r_+
-    const T X = x1[0] - C.xc, Y = x1[1] - C.yc, Z = x1[2] - C.zc;
-    T D;
-    const T r2 = kerr_r2<T>(X, Y, Z, C.a, &D);
-    if (r2 < C.rcheck2) {
+    // screen in FP32, decide in FP64 near r_+
+    float r2;
+    if constexpr (sizeof(T) == sizeof(double)) {
+      const float X = narrow(x1[0] - C.xc), Y = narrow(x1[1] - C.yc), Z = narrow(x1[2] - C.zc);
+      float D;
+      r2 = kerr_r2<float>(X, Y, Z, (float)C.a, &D);
+    } else {
+      const T X = x1[0] - C.xc, Y = x1[1] - C.yc, Z = x1[2] - C.zc;
+      T D;
+      r2 = kerr_r2<T>(X, Y, Z, C.a, &D);
+    }
+    if (r2 < (float)C.rcheck2) {
       double Dd;
       const double r2d =
           kerr_r2<double>(to_f64(x1[0]) - C.dxc, to_f64(x1[1]) - C.dyc, to_f64(x1[2]) - C.dzc, C.da, &Dd);
@@ -927,8 +1050,7 @@ __device__ __forceinline__ Move<T> push_move(const Grid& g, const Fields<T>& F, 
     __stcs(key_out, kDead);
     atomicAdd(horizon ? &st->removed_horizon : &st->removed_outer, 1ull);
   } else {
-    const int ci = (int)floor(x1[0]), cj = (int)floor(x1[1]), ck = (int)floor(x1[2]);
-    __stcs(key_out, (uint32_t)(((long long)ck * g.ny + cj) * g.nx + ci));
+    __stcs(key_out, (uint32_t)(((long long)ci[2] * g.ny + ci[1]) * g.nx + ci[0]));
   }
   if (fb) atomicAdd(&st->fallbacks, 1ull);
   Move<T> mv;
@@ -952,7 +1074,7 @@ __device__ __forceinline__ void deposit_move(const Grid& g, const Fields<T>& F, 
   if constexpr (sizeof(T) == sizeof(float))
     deposit_lattice<Q, TAB>(g, F, C, mv.x0, mv.dx, mv.qg, C.inv_dt, flags, n64, mixed, jt, atab);
   else
-    deposit<T, Q>(g, F, C, mv.x0, mv.dx, mv.qg, C.inv_dt, flags);
+    deposit64<Q>(g, F, C, mv.x0, mv.dx, mv.qg, C.inv_dt, flags);
 }
 
 // One particle-step of particle i: RK4 push, new state stored, removal flag and sort key
