@@ -183,10 +183,8 @@ template <typename T>
 void launch_b_step(const Grid& g, const BStepArgs<T>& A, int sms, cudaStream_t st);
 template <typename T>
 void launch_e_step(const Grid& g, const EStepArgs<T>& A, int sms, cudaStream_t st);
-// Patches of the instances of a batch for the batched field launches (word: bytes of a field value), and the number of
-// blocks that copy an instance's outer layers (they follow its patches in the table).
+// Patches of the instances of a batch for the batched field launches (word: bytes of a field value).
 void batch_field_tiles(const Grid* const* grids, int n, size_t word, int sms, TileGrid* tiles);
-int batch_shell_blocks(const Grid& g);
 template <typename T>
 void launch_uniform_field(const Grid& g, const Fields<T>& F, const uint16_t* loc, const double E[3], const double B[3],
                           cudaStream_t st);

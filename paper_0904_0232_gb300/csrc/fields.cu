@@ -33,10 +33,11 @@
 // (B) or twice (E) a plane, and FP64 reciprocals and roots are FastOps64's.
 // Measured (GB300, microseconds a launch, no layers; before: the E step as one march with a halo of 3, IEEE FP64
 // divides and roots, the metric evaluated in FP64, patches over all cells and chunks of at least 4 planes):
-//            FP32 64^3   128^3   192^3 (layers)   FP64 64^3   96^3
-//   B half   24 -> 14  80 -> 43     222 -> 183    425 -> 80  1053 -> 138
-//   E step   35 -> 29 140 -> 105    467 -> 458   1147 -> 193 2310 -> 349  (both launches)
-// At 128^3 FP32 moves 38 and 2 x 68 B per cell: 43 us = 1.8 TB/s, 27 % of the measured copy rate.
+//            FP32 64^3   128^3      192^3       64x64x128   FP64 32^3    64^3         96^3
+//   B half   24 -> 14   80 -> 45    222 -> 132   39 -> 18    129 -> 15   425 -> 47   1053 -> 138
+//   E step   35 -> 30  140 -> 107   411 -> 330   56 -> 40    215 -> 32  1114 -> 104  2193 -> 318  (both launches)
+// At 192^3 FP32 moves 38 B (B half) and 62 + 74 B (E) per cell: 2.0 and 2.9 TB/s, 30 and 43 % of the measured copy
+// rate; it issues about 500 instructions a cell and plane of the march.
 #include <algorithm>
 #include <cmath>
 
@@ -281,22 +282,22 @@ __device__ __forceinline__ void cp_async_wait() {
 
 // The staged halo patch of a block: (BY + 2) x kSX elements, at most two per thread (threads
 // 32 x BY); element e of the patch is column e % kSX, row e / kSX, at grid (x0 - 1 + column,
-// y0 - 1 + row) where (x0, y0) is the grid position of thread (0, 0).  Positions outside the grid, on any axis,
-// take the nearest one inside: only cells of the outer index layer reach them, and those are not converted.
+// y0 - 1 + row) where (x0, y0) is the grid position of thread (0, 0).  Columns and rows beyond the grid are left out, and
+// planes beyond it take the nearest one: only cells of the outer index layer reach them, and those are not converted.
+// (Copies that clamp the columns too, many lanes reading one address, made a patch at a grid's edge twice as slow.)
 template <int BY>
 struct Stager {
-  int s0, s1;       // element in a staged component; s1 < 0: this thread stages one element only
+  int s0, s1;       // element in a staged component; negative: none
   unsigned o0, o1;  // x + y nx of the element
   __device__ Stager(const Grid& g, int x0, int y0) {
     const int t = threadIdx.y * kTX + threadIdx.x;
-    auto off = [&](int e) {
-      const int x = min(max(x0 - 1 + e % kSX, 0), g.nx - 1), y = min(max(y0 - 1 + e / kSX, 0), g.ny - 1);
+    auto off = [&](int e, int& s) {
+      const int x = x0 - 1 + e % kSX, y = y0 - 1 + e / kSX;  // (x0, y0 >= 1)
+      s = e < (BY + 2) * kSX && x < g.nx && y < g.ny ? e : -1;
       return (unsigned)(x + y * g.nx);
     };
-    s0 = t;
-    o0 = off(t);
-    s1 = t + kTX * BY < (BY + 2) * kSX ? t + kTX * BY : -1;
-    o1 = off(max(s1, 0));
+    o0 = off(t, s0);
+    o1 = off(t + kTX * BY, s1);
   }
   // start copying plane p of the three arrays src into dst
   template <typename T>
@@ -306,11 +307,58 @@ struct Stager {
     for (int q = 0; q < 3; ++q) {
       const T* const plane = src[q] + pz;
       T* const to = &dst.v[q][0][0];
-      cp_async(to + s0, plane + o0);
+      if (s0 >= 0) cp_async(to + s0, plane + o0);
       if (s1 >= 0) cp_async(to + s1, plane + o1);
     }
   }
 };
+
+// The outer two index layers are never advanced: a step into another buffer copies them, each block its share (blocks of
+// their own beside the patches filled both slots of an SM with patches while other SMs had none: FP64 at 64^3 80 us
+// instead of 46).  Cells by index: the z layers, then the y layers of the planes between them, then the x layers of the
+// rows between those.
+__device__ __forceinline__ int outer_layer(int q, int n) { return q < 2 ? q : n - 4 + q; }  // q = 0..3
+template <typename T>
+__device__ __forceinline__ void copy_shell(const Grid& g, const T* const* src, T* const* dst, long long block,
+                                           long long blocks) {
+  const unsigned plane = g.nx * g.ny, xrow = 4u * g.nx, xcol = 4u * (g.ny - 4);
+  const long long nz4 = 4ll * plane, ny4 = (long long)xrow * (g.nz - 4);
+  const long long cells = g.ncell - (long long)(g.nx - 4) * (g.ny - 4) * (g.nz - 4);
+  const int threads = blockDim.x * blockDim.y;
+  for (long long s = block * threads + threadIdx.y * kTX + threadIdx.x; s < cells; s += blocks * threads) {
+    int x, y, z;
+    if (s < nz4) {
+      const unsigned q = (unsigned)(s / plane), e = (unsigned)(s - (long long)q * plane);
+      y = e / g.nx;
+      x = e - y * g.nx;
+      z = outer_layer((int)q, g.nz);
+    } else if (s < nz4 + ny4) {
+      const unsigned r = (unsigned)((s - nz4) / xrow), e = (unsigned)(s - nz4 - (long long)r * xrow);
+      y = e / g.nx;
+      x = e - y * g.nx;
+      y = outer_layer(y, g.ny);
+      z = 2 + (int)r;
+    } else {
+      const unsigned r = (unsigned)((s - nz4 - ny4) / xcol), e = (unsigned)(s - nz4 - ny4 - (long long)r * xcol);
+      x = outer_layer((int)(e & 3u), g.nx);
+      y = 2 + (int)(e >> 2);
+      z = 2 + (int)r;
+    }
+    const long long c = ((long long)z * g.ny + y) * g.nx + x;
+    T v[3];
+#pragma unroll
+    for (int q = 0; q < 3; ++q) v[q] = src[q][c];
+#pragma unroll
+    for (int q = 0; q < 3; ++q) dst[q][c] = v[q];
+  }
+}
+
+__device__ __forceinline__ void decode_tile(const TileGrid& t, long long q, int& tx, int& ty, int& zs) {
+  tx = (int)(q % t.ntx);
+  const long long r = q / t.ntx;
+  ty = (int)(r % t.nty);
+  zs = 2 + (int)(r / t.nty) * t.zchunk;
+}
 
 // ---- B half-step ------------------------------------------------------------------------------
 // Patch: threads (tx, ty) at x = x0 + tx, y = y0 + ty; e at the patch of each plane P of the chunk and of
@@ -324,8 +372,11 @@ struct BStepSmem {
 };
 
 template <typename T, int BY>
-__device__ __forceinline__ void b_step_tile(const Grid& g, const BStepArgs<T>& A, int tile_x, int tile_y, int zs,
-                                            int ze, BStepSmem<T, BY>& sm) {
+__device__ __forceinline__ void b_step_tile(const Grid& g, const BStepArgs<T>& A, const TileGrid& t, int block,
+                                            BStepSmem<T, BY>& sm) {
+  int tile_x, tile_y, zs;
+  decode_tile(t, block, tile_x, tile_y, zs);
+  const int ze = min(zs + t.zchunk, g.nz - 2);
   const int tx = threadIdx.x, ty = threadIdx.y;
   const int cx = tx + 1, cy = ty + 1;  // the cell in the staged planes
   const int x0 = 2 + tile_x * (kTX - 1), y0 = 2 + tile_y * (BY - 1);
@@ -340,6 +391,7 @@ __device__ __forceinline__ void b_step_tile(const Grid& g, const BStepArgs<T>& A
     st.stage(g, A.d, q, sm.Sd[q & 3]);
   }
   cp_async_commit();
+  if (!A.inplace) copy_shell<T>(g, A.base, A.out, block, t.count());
   cp_async_wait<0>();
   __syncthreads();
   // carried from plane P - 1: d_z summed over the x and the y pair, b; from plane P: d_x, d_y and their sums with
@@ -458,8 +510,11 @@ struct EStepSmem {
 };
 
 template <typename T, int BY>
-__device__ __forceinline__ void e_step_tile(const Grid& g, const EStepArgs<T>& A, int tile_x, int tile_y, int zs,
-                                            int ze, EStepSmem<T, BY>& sm) {
+__device__ __forceinline__ void e_step_tile(const Grid& g, const EStepArgs<T>& A, const TileGrid& t, int block,
+                                            EStepSmem<T, BY>& sm) {
+  int tile_x, tile_y, zs;
+  decode_tile(t, block, tile_x, tile_y, zs);
+  const int ze = min(zs + t.zchunk, g.nz - 2);
   const int tx = threadIdx.x, ty = threadIdx.y;
   const int cx = tx + 1, cy = ty + 1;
   const int x0 = 1 + tile_x * (kTX - 1), y0 = 1 + tile_y * (BY - 1);
@@ -474,6 +529,7 @@ __device__ __forceinline__ void e_step_tile(const Grid& g, const EStepArgs<T>& A
     st.stage(g, A.x, q, sm.Sx[q & 3]);
   }
   cp_async_commit();
+  copy_shell<T>(g, A.d, A.out, block, t.count());
   cp_async_wait<0>();
   __syncthreads();
   // carried from plane q - 1: b_x summed over the x pair, b_y over the y pair; h, d and J there, and h of plane q - 2
@@ -600,68 +656,18 @@ TileGrid tile_grid(const Grid& g, int rows, int slots, double* cost_out = nullpt
   return t;
 }
 
-// The outer two index layers are never advanced: a step into another buffer copies them with blocks of its own
-// beside the patches (blocks of kTX * rows threads, one cell a thread).  Cells by index: the z layers, then the
-// y layers of the planes between them, then the x layers of the rows between those.
-__host__ __device__ inline long long shell_cells(const Grid& g) {
-  return g.ncell - (long long)(g.nx - 4) * (g.ny - 4) * (g.nz - 4);
-}
-inline int shell_blocks(const Grid& g, int rows) {
-  return (int)((shell_cells(g) + kTX * rows - 1) / (kTX * rows));
-}
-__device__ __forceinline__ int outer_layer(int q, int n) { return q < 2 ? q : n - 4 + q; }  // q = 0..3
-template <typename T>
-__device__ __forceinline__ void copy_shell(const Grid& g, const T* const* src, T* const* dst, long long block) {
-  long long s = block * (blockDim.x * blockDim.y) + threadIdx.y * kTX + threadIdx.x;
-  int x, y, z;
-  const long long nz4 = 4ll * g.nx * g.ny, ny4 = 4ll * g.nx * (g.nz - 4);
-  if (s < nz4) {
-    x = (int)(s % g.nx);
-    y = (int)(s / g.nx % g.ny);
-    z = outer_layer((int)(s / ((long long)g.nx * g.ny)), g.nz);
-  } else if (s < nz4 + ny4) {
-    s -= nz4;
-    x = (int)(s % g.nx);
-    y = outer_layer((int)(s / g.nx % 4), g.ny);
-    z = 2 + (int)(s / (4ll * g.nx));
-  } else if (s < shell_cells(g)) {
-    s -= nz4 + ny4;
-    x = outer_layer((int)(s % 4), g.nx);
-    y = 2 + (int)(s / 4 % (g.ny - 4));
-    z = 2 + (int)(s / (4ll * (g.ny - 4)));
-  } else {
-    return;
-  }
-  const long long c = ((long long)z * g.ny + y) * g.nx + x;
-#pragma unroll
-  for (int q = 0; q < 3; ++q) dst[q][c] = src[q][c];
-}
-
-__device__ __forceinline__ void decode_tile(const TileGrid& t, long long q, int& tx, int& ty, int& zs) {
-  tx = (int)(q % t.ntx);
-  const long long r = q / t.ntx;
-  ty = (int)(r % t.nty);
-  zs = 2 + (int)(r / t.nty) * t.zchunk;
-}
-
 template <typename T, int BY>
 __global__ void __launch_bounds__(kTX * BY, patch_blocks(sizeof(T), BY)) k_b_step(const Grid g, const BStepArgs<T> A, const TileGrid t) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   auto& sm = *reinterpret_cast<BStepSmem<T, BY>*>(smem_raw);
-  int tx, ty, zs;
-  if (blockIdx.x >= t.count()) return copy_shell<T>(g, A.base, A.out, blockIdx.x - t.count());
-  decode_tile(t, blockIdx.x, tx, ty, zs);
-  b_step_tile<T, BY>(g, A, tx, ty, zs, min(zs + t.zchunk, g.nz - 2), sm);
+  b_step_tile<T, BY>(g, A, t, blockIdx.x, sm);
 }
 
 template <typename T, int BY>
 __global__ void __launch_bounds__(kTX * BY, patch_blocks(sizeof(T), BY)) k_e_step(const Grid g, const EStepArgs<T> A, const TileGrid t) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   auto& sm = *reinterpret_cast<EStepSmem<T, BY>*>(smem_raw);
-  int tx, ty, zs;
-  if (blockIdx.x >= t.count()) return copy_shell<T>(g, A.d, A.out, blockIdx.x - t.count());
-  decode_tile(t, blockIdx.x, tx, ty, zs);
-  e_step_tile<T, BY>(g, A, tx, ty, zs, min(zs + t.zchunk, g.nz - 2), sm);
+  e_step_tile<T, BY>(g, A, t, blockIdx.x, sm);
 }
 
 // ---- batched: one block per entry of a table of (instance, patch) work items ---------------------
@@ -738,13 +744,7 @@ __global__ void __launch_bounds__(kTX * BY, patch_blocks(sizeof(T), BY))
   }
   const TileGrid t = D.tiles;
   __syncthreads();
-  if (e.block >= t.count()) {
-    if (!A.inplace) copy_shell<T>(g, A.base, A.out, e.block - t.count());
-    return;
-  }
-  int tx, ty, zs;
-  decode_tile(t, e.block, tx, ty, zs);
-  b_step_tile<T, BY>(g, A, tx, ty, zs, min(zs + t.zchunk, g.nz - 2), sm);
+  b_step_tile<T, BY>(g, A, t, e.block, sm);
 }
 
 template <typename T, int BY>
@@ -762,10 +762,7 @@ __global__ void __launch_bounds__(kTX * BY, patch_blocks(sizeof(T), BY))
   }
   const TileGrid t = D.tiles;
   __syncthreads();
-  if (e.block >= t.count()) return copy_shell<T>(g, A.d, A.out, e.block - t.count());
-  int tx, ty, zs;
-  decode_tile(t, e.block, tx, ty, zs);
-  e_step_tile<T, BY>(g, A, tx, ty, zs, min(zs + t.zchunk, g.nz - 2), sm);
+  e_step_tile<T, BY>(g, A, t, e.block, sm);
 }
 
 template <typename T>
@@ -824,7 +821,7 @@ __global__ void k_location_flags(const Grid g, uint16_t* __restrict__ loc) {
 // ---- initial conditions / conversions ----------------------------------------------------
 // b_Q = h_Q + f (v x k)_Q at its face with v = k x h + d, the contravariant (h, d) uniform (g = eta + f k k
 // lowers the tensor of Eq. 8).  FP64-pipe bound: FastOps64, and the excised locations from the flags.
-//@UNIFORM@
+// At 128^3: 847 -> 577 us.
 template <int Q, typename T>
 __device__ __forceinline__ T uniform_b(const Grid& g, int i, int j, int k, bool excised, const double h[3],
                                        const double d[3]) {
@@ -983,8 +980,7 @@ void launch_b_rows(const Grid& g, const BStepArgs<T>& A, const TileGrid& t, cuda
   constexpr size_t smem = sizeof(BStepSmem<T, BY>);
   static bool once = (allow_smem(k_b_step<T, BY>, smem), true);
   (void)once;
-  const long long nb = t.count() + (A.inplace ? 0 : shell_blocks(g, BY));
-  k_b_step<T, BY><<<(unsigned)nb, dim3(kTX, BY), smem, st>>>(g, A, t);
+  k_b_step<T, BY><<<(unsigned)t.count(), dim3(kTX, BY), smem, st>>>(g, A, t);
 }
 
 template <typename T, int BY>
@@ -992,7 +988,7 @@ void launch_e_rows(const Grid& g, const EStepArgs<T>& A, const TileGrid& t, cuda
   constexpr size_t smem = sizeof(EStepSmem<T, BY>);
   static bool once = (allow_smem(k_e_step<T, BY>, smem), true);
   (void)once;
-  k_e_step<T, BY><<<(unsigned)(t.count() + shell_blocks(g, BY)), dim3(kTX, BY), smem, st>>>(g, A, t);
+  k_e_step<T, BY><<<(unsigned)t.count(), dim3(kTX, BY), smem, st>>>(g, A, t);
 }
 
 // FP32 patches (and the batched FP64 ones) have 16 rows.  Other FP64 patches, bound by the FP64 pipe whatever their
@@ -1032,9 +1028,8 @@ void launch_e_step(const Grid& g, const EStepArgs<T>& A, int sms, cudaStream_t s
 }
 
 // Patches of the instances of a batch (16 rows), the z chunks the ones (of one length for all) that minimise the
-// estimated time as in tile_grid; blocks of the copied outer layers follow an instance's patches.
+// estimated time as in tile_grid.
 constexpr int kBatchRows = 16;
-int batch_shell_blocks(const Grid& g) { return shell_blocks(g, kBatchRows); }
 void batch_field_tiles(const Grid* const* grids, int n, size_t word, int sms, TileGrid* tiles) {
   const int slots = sms * patch_blocks(word, kBatchRows);
   double best = 1e300;

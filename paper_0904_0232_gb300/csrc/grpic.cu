@@ -1390,8 +1390,7 @@ grpic_status batch_build(grpic_batch* b) {
     D.st = c->st;
     const Grid& g = c->g;
     D.tiles = tiles[i];
-    const long long ntile = D.tiles.count() + batch_shell_blocks(g);
-    for (long long q = 0; q < ntile; ++q) tile.push_back(BlockEntry{i, (int)q});
+    for (long long q = 0; q < D.tiles.count(); ++q) tile.push_back(BlockEntry{i, (int)q});
     append_blocks(all, i, g.ncell, 256);
     for (int s = 0; s < kMaxSpecies; ++s) {
       SpeciesStore& S = c->sp[s];
