@@ -214,6 +214,7 @@ struct Consts {
   T qm, qmacro;              // q/m (Lorentz term of Eq. 15), macro-particle charge (deposit)
   T rcheck2;                 // removal screen: r^2 below this -> FP64 test against r_+
   float r_fp64, r2_fp64;     // FP32-mixed: promote where the FP32 r is below r_fp64
+  float r2_hot;              // ... which no node does in a cell whose R^2 at any point is above this (nor R <= |a|)
   bool massive;              // m > 0
   bool gamma_in_j;           // J = rho gamma v (else the plain Umeda flux)
   double dxc, dyc, dzc, dm, da, da2, r_plus;
@@ -239,6 +240,9 @@ __host__ __device__ inline Consts<T> make_consts(const Grid& g, const Species& s
   C.rcheck2 = (T)(1.2 * g.r_plus * g.r_plus + 1.0);
   C.r_fp64 = (float)g.r_fp64;
   C.r2_fp64 = C.r_fp64 > 0.f ? C.r_fp64 * C.r_fp64 : -1.f;  // negative: never promote
+  // a cell's points lie within sqrt(3) < 1.8 of each other, r >= R - |a| (Eq. 6)
+  const double r_hot = (g.r_fp64 > 0.0 ? g.r_fp64 : 0.0) + (g.a < 0.0 ? -g.a : g.a) + 1.8;
+  C.r2_hot = (float)(r_hot * r_hot);
   C.massive = g.m > 0.0;
   C.gamma_in_j = (g.flags & 1u) == 0;
   C.dxc = g.xc;
@@ -317,6 +321,15 @@ inline int spread_log2(int group) {
   while ((1 << lg) < group) ++lg;
   return lg;
 }
+// A push launch of few blocks: warps near the hole take several times as long as the others (FP64 pipe), so where an SM
+// gets only a handful of warps, blocks of one warp (a register file holds as many warps of them) spread the near ones
+// over the SMs, and another species' launch runs beside it (grpic.cu).  Larger launches keep blocks of four warps, whose
+// common cells stay in L1.
+// Measured, us per push stage, 128-thread blocks one after another / small launches as here: 2 x 46 K particles at 32^3
+// 228 / 121 (FP64 695 / 603), 2 x 400 K + 2 x 85 K at 64 x 64 x 128 380 / 248; blocks of one warp for 2 x 0.9 M
+// particles at 64^3 cost 1142 instead of 941.
+constexpr long long kSmallPush = 311296;  // 4 waves of 128-thread blocks at 4 an SM
+inline bool small_push(long long n) { return n <= kSmallPush; }
 // Unsplit alternative: one launch, far-field or FP32-mixed code chosen per warp by the same
 // near_radius criterion.  atab (non-null, Q = 2, no tile): far-field warps deposit with the
 // per-cell area fits, and the criterion becomes table_radius.
@@ -372,7 +385,6 @@ struct BlockEntry {
 template <typename T>
 struct SpeciesDesc {
   Consts<T> C;          // launch constants of this (instance, species)
-  float r_near2;        // near_radius^2 of the instance (FP32-mixed far-field criterion)
   double qm, qmacro;
   Particles<T> buf[2];  // the two ping-pong buffers (n = work upper bound, n_dev = live count)
   int* cur;             // device int: index of the current buffer
@@ -420,8 +432,8 @@ void launch_batch_zero_j(const BatchTables<T>& bt, cudaStream_t st);
 // flip every instance's d parity (end of a batched step)
 template <typename T>
 void launch_batch_flip_d(const BatchTables<T>& bt, int ninst, cudaStream_t st);
-template <typename T>
-void launch_batch_push(const BatchTables<T>& bt, int quad_order, cudaStream_t st);
+// the FP64 push of a batched step (FP32-mixed batches launch the per-warp select kernel per instance and species)
+void launch_batch_push(const BatchTables<double>& bt, int quad_order, cudaStream_t st);
 template <typename T>
 void launch_batch_sort(const BatchTables<T>& bt, cudaStream_t st);
 

@@ -211,17 +211,44 @@ void enqueue_rho(grpic_ctx* c, bool with_gamma, double* rho) {
 // The area fits the per-warp select push uses, or null.
 const float4* area_table_of(const grpic_ctx* c) { return c->tune.area_table ? c->atab : nullptr; }
 
+// One push launch per species, launch(species, stream).  Small launches (small_push) do not fill the GPU: where another
+// species is loaded they go to the side stream, ahead of and beside the others (all add into J atomically), and the context
+// stream waits for them.  The buffers belong to the context stream, which is joined before anything else uses them.
+template <typename Launch>
+void enqueue_species_pushes(grpic_ctx* c, Launch launch) {
+  int order[kMaxSpecies], n = 0;
+  for (int s = 0; s < kMaxSpecies; ++s) {
+    if (!c->sp[s].loaded || c->sp[s].n == 0) continue;
+    refresh_count(c->sp[s]);
+    order[n++] = s;
+  }
+  std::stable_sort(order, order + n, [c](int a, int b) { return c->sp[a].n < c->sp[b].n; });
+  // the smaller launches, but never all of them: two small ones run beside each other
+  int side = 0;
+  while (side < n - 1 && small_push(c->sp[order[side]].n)) ++side;
+  if (side == n - 1 && n > 2 && small_push(c->sp[order[n - 1]].n)) side = n / 2;
+  if (side > 0) {
+    cudaEventRecord(c->ev_fork, c->stream);
+    cudaStreamWaitEvent(c->side, c->ev_fork, 0);
+  }
+  for (int q = 0; q < n; ++q) {
+    launch(order[q], q < side ? c->side : c->stream);
+    c->launches += 1;
+  }
+  if (side > 0) {
+    cudaEventRecord(c->ev_join, c->side);
+    cudaStreamWaitEvent(c->stream, c->ev_join, 0);
+  }
+}
+
 // Unsplit FP32-mixed push: one launch per species, far-field or mixed code chosen per warp.
 void enqueue_select_push(grpic_ctx* c) {
   Fields<float> F = fields_view<float>(c);
-  for (int s = 0; s < kMaxSpecies; ++s) {
+  enqueue_species_pushes(c, [&](int s, cudaStream_t st) {
     SpeciesStore& S = c->sp[s];
-    if (!S.loaded || S.n == 0) continue;
-    refresh_count(S);
     launch_push_select(c->g, F, particles_view<float>(c, s, S.cur), Species{S.qm, S.qmacro}, c->st,
-                       c->tune.far_min_blocks, c->tune.j_tile != 0, c->tune.spread, area_table_of(c), c->stream);
-    c->launches += 1;
-  }
+                       c->tune.far_min_blocks, c->tune.j_tile != 0, c->tune.spread, area_table_of(c), st);
+  });
 }
 
 void enqueue_far(grpic_ctx* c, const Fields<float>& F) {
@@ -329,14 +356,11 @@ void enqueue_stage(grpic_ctx* c, int stage) {
         else
           enqueue_select_push(c);
       } else {
-        for (int s = 0; s < kMaxSpecies; ++s) {
+        enqueue_species_pushes(c, [&](int s, cudaStream_t st) {
           SpeciesStore& S = c->sp[s];
-          if (!S.loaded || S.n == 0) continue;
-          refresh_count(S);
-          Species spc{S.qm, S.qmacro};
-          launch_push_deposit<T>(c->g, F, particles_view<T>(c, s, S.cur), spc, c->st, c->mixed, 0.0, c->stream);
-          c->launches += 1;
-        }
+          launch_push_deposit<T>(c->g, F, particles_view<T>(c, s, S.cur), Species{S.qm, S.qmacro}, c->st, c->mixed, 0.0,
+                                 st);
+        });
       }
       c->pushes += 1;
       break;
@@ -1399,8 +1423,6 @@ grpic_status batch_build(grpic_batch* b) {
       SD.qm = S.qm;
       SD.qmacro = S.qmacro;
       SD.C = make_consts<T>(g, Species{S.qm, S.qmacro});
-      const double rn = near_radius(g);
-      SD.r_near2 = (float)(rn * rn);
       SD.cur = b->cur + 4 * i + s;
       SD.bin_base = 0;
       if (!S.loaded) continue;
@@ -1500,7 +1522,7 @@ void batch_enqueue_step(grpic_batch* b, int k) {
   if constexpr (sizeof(T) == sizeof(float))
     batch_enqueue_push_items(b, k);
   else
-    launch_batch_push<T>(t, b->quad, b->stream);
+    launch_batch_push(t, b->quad, b->stream);
   launch_batch_b_half<T>(t, 1, b->literal, b->stream);
   if (!b->literal) launch_batch_e_step<T>(t, 0, b->literal, b->stream);
   launch_batch_e_step<T>(t, 1, b->literal, b->stream);

@@ -10,14 +10,14 @@ namespace grpic {
 
 namespace {
 
-template <typename T, int Q, bool MIXED>
-__global__ void __launch_bounds__(128, 4) k_push_deposit(const Grid g, const Fields<T> F, const Particles<T> P,
+template <typename T, int Q, bool MIXED, int THREADS>
+__global__ void __launch_bounds__(THREADS, 4 * (128 / THREADS)) k_push_deposit(const Grid g, const Fields<T> F, const Particles<T> P,
                                                            const Consts<T> C, DevStatus* st) {
   const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   unsigned flags = 0, n64 = 0;
   bool active = i < P.n && i < (long long)(*P.n_dev);
   if (active) active = P.key[i] != kDead;
-  if (active) push_particle<T, Q>(g, F, P, C, i, st, flags, n64, P.key + i, MIXED);
+  if (active) push_particle<T, Q, MIXED>(g, F, P, C, i, st, flags, n64, P.key + i);
   warp_status(st, flags, n64, active);
 }
 
@@ -51,7 +51,7 @@ __global__ void __launch_bounds__(128, 4) k_push_near(const Grid g, const Fields
     const int j = base + threadIdx.x;
     const bool active = j < n;
     unsigned flags = 0, n64 = 0;
-    if (active) push_particle<float, Q>(g, F, P, C, (long long)list[j], st, flags, n64, keys + j, true);
+    if (active) push_particle<float, Q, true>(g, F, P, C, (long long)list[j], st, flags, n64, keys + j);
     warp_status(st, flags, n64, active);
   }
 }
@@ -63,28 +63,26 @@ __global__ void k_near_keys(uint32_t* __restrict__ key, const uint32_t* __restri
   for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) key[list[j]] = keys[j];
 }
 
-// Batched: one CTA per (instance * 4 + species, block) work item; each block belongs to one
+// Batched FP64 push: one CTA per (instance * 4 + species, block) work item; each block belongs to one
 // instance and species, so the warp-level status stays per instance.  The block stages its
 // instance descriptor (with the host-built launch constants) in shared memory.  The block -> item map is the same
-// coprime permutation as k_push_select's (perm; 1 = in order), spreading FP64-heavy items.
-// FP32-mixed: each warp takes the far-field code unless one of its particles lies within the
-// instance's near_radius.
-template <typename T, int Q, bool MIXED>
-__global__ void __launch_bounds__(128, 4) k_push_deposit_batch(const InstDesc<T>* __restrict__ desc,
+// coprime permutation as k_push_select's (perm; 1 = in order).
+template <int Q>
+__global__ void __launch_bounds__(128, 4) k_push_deposit_batch(const InstDesc<double>* __restrict__ desc,
                                                                  const BlockEntry* __restrict__ blk, int nblk,
                                                                  unsigned perm) {
   __shared__ Grid sg;
-  __shared__ Fields<T> sF;
-  __shared__ SpeciesDesc<T> sS;
+  __shared__ Fields<double> sF;
+  __shared__ SpeciesDesc<double> sS;
   __shared__ DevStatus* sst;
   __shared__ int s_cur;
   const int bi = (int)spread_chunk(blockIdx.x, (unsigned)nblk, perm, kBatchSpreadLog2);
   const BlockEntry e = blk[bi];
   // stage the descriptor parts this block needs with one coalesced copy by all threads (the
   // launch constants were built on the host)
-  const InstDesc<T>& D = desc[e.inst >> 2];
+  const InstDesc<double>& D = desc[e.inst >> 2];
   copy_words(&sg, &D.g, sizeof(Grid));
-  copy_words(&sS, &D.sp[e.inst & 3], sizeof(SpeciesDesc<T>));
+  copy_words(&sS, &D.sp[e.inst & 3], sizeof(SpeciesDesc<double>));
   if (threadIdx.x == 0) {
     sst = D.st;
     s_cur = *D.sp[e.inst & 3].cur;
@@ -97,27 +95,12 @@ __global__ void __launch_bounds__(128, 4) k_push_deposit_batch(const InstDesc<T>
     }
   }
   __syncthreads();
-  const Particles<T>& sP = sS.buf[s_cur];
-  const Consts<T>& sC = sS.C;
-  const float s_rnear2 = sS.r_near2;
+  const Particles<double>& sP = sS.buf[s_cur];
   const long long i = (long long)e.block * blockDim.x + threadIdx.x;
   unsigned flags = 0, n64 = 0;
   bool active = i < sP.n && i < (long long)(*sP.n_dev);
   if (active) active = sP.key[i] != kDead;
-  bool mixed = false;
-  if constexpr (MIXED) {
-    bool near = false;
-    if (active) {
-      const float X = sP.x[0][i] - sC.xc, Y = sP.x[1][i] - sC.yc, Z = sP.x[2][i] - sC.zc;
-      near = X * X + Y * Y + Z * Z < s_rnear2;
-    }
-    mixed = __any_sync(0xffffffffu, near);
-  }
-  if (mixed) {  // two inlined copies with a constant flag (see k_push_select)
-    if (active) push_particle<T, Q>(sg, sF, sP, sC, i, sst, flags, n64, sP.key + i, true);
-  } else {
-    if (active) push_particle<T, Q>(sg, sF, sP, sC, i, sst, flags, n64, sP.key + i, false);
-  }
+  if (active) push_particle<double, Q, false>(sg, sF, sP, sS.C, i, sst, flags, n64, sP.key + i);
   warp_status(sst, flags, n64, active);
 }
 
@@ -231,29 +214,33 @@ inline unsigned blocks_for(long long n, int bs) { return (unsigned)((n + bs - 1)
 
 }  // namespace
 
-template <typename T, bool MIXED>
+template <typename T, bool MIXED, int THREADS>
 void launch_push_q(const Grid& g, const Fields<T>& F, const Particles<T>& P, const Species& sp, DevStatus* st,
                    cudaStream_t stream) {
-  const unsigned nb = blocks_for(P.n, 128);
+  const unsigned nb = blocks_for(P.n, THREADS);
   const Consts<T> C = make_consts<T>(g, sp);
   if (g.quad_order == 1)
-    k_push_deposit<T, 1, MIXED><<<nb, 128, 0, stream>>>(g, F, P, C, st);
+    k_push_deposit<T, 1, MIXED, THREADS><<<nb, THREADS, 0, stream>>>(g, F, P, C, st);
   else if (g.quad_order == 3)
-    k_push_deposit<T, 3, MIXED><<<nb, 128, 0, stream>>>(g, F, P, C, st);
+    k_push_deposit<T, 3, MIXED, THREADS><<<nb, THREADS, 0, stream>>>(g, F, P, C, st);
   else
-    k_push_deposit<T, 2, MIXED><<<nb, 128, 0, stream>>>(g, F, P, C, st);
+    k_push_deposit<T, 2, MIXED, THREADS><<<nb, THREADS, 0, stream>>>(g, F, P, C, st);
 }
 
 // FP64 runs pure double; FP32 runs the mixed policy.
 template <>
 void launch_push_deposit<double>(const Grid& g, const Fields<double>& F, const Particles<double>& P,
                                  const Species& sp, DevStatus* st, bool, double, cudaStream_t stream) {
-  if (P.n > 0) launch_push_q<double, false>(g, F, P, sp, st, stream);
+  if (P.n <= 0) return;
+  if (small_push(P.n))
+    launch_push_q<double, false, 32>(g, F, P, sp, st, stream);
+  else
+    launch_push_q<double, false, 128>(g, F, P, sp, st, stream);
 }
 template <>
 void launch_push_deposit<float>(const Grid& g, const Fields<float>& F, const Particles<float>& P,
                                 const Species& sp, DevStatus* st, bool, double, cudaStream_t stream) {
-  if (P.n > 0) launch_push_q<float, true>(g, F, P, sp, st, stream);
+  if (P.n > 0) launch_push_q<float, true, 128>(g, F, P, sp, st, stream);
 }
 
 void launch_push_near(const Grid& g, const Fields<float>& F, const Particles<float>& P, const Species& sp,
@@ -275,28 +262,18 @@ void launch_near_keys(const Particles<float>& P, const uint32_t* list, const uin
   k_near_keys<<<nblocks, 256, 0, stream>>>(P.key, list, keys, count);
 }
 
-template <typename T, bool MIXED>
-void launch_batch_push_q(const BatchTables<T>& bt, int quad_order, cudaStream_t stream) {
+void launch_batch_push(const BatchTables<double>& bt, int quad_order, cudaStream_t stream) {
   // one block per work item: each block stages its instance descriptor once, and the hardware
   // scheduler balances instances of very different cost
   const unsigned nb = (unsigned)bt.npart;
   if (bt.npart == 0) return;
   const unsigned perm = spread_multiplier(nb, kBatchSpreadLog2);
   if (quad_order == 1)
-    k_push_deposit_batch<T, 1, MIXED><<<nb, 128, 0, stream>>>(bt.desc, bt.part, bt.npart, perm);
+    k_push_deposit_batch<1><<<nb, 128, 0, stream>>>(bt.desc, bt.part, bt.npart, perm);
   else if (quad_order == 3)
-    k_push_deposit_batch<T, 3, MIXED><<<nb, 128, 0, stream>>>(bt.desc, bt.part, bt.npart, perm);
+    k_push_deposit_batch<3><<<nb, 128, 0, stream>>>(bt.desc, bt.part, bt.npart, perm);
   else
-    k_push_deposit_batch<T, 2, MIXED><<<nb, 128, 0, stream>>>(bt.desc, bt.part, bt.npart, perm);
-}
-
-template <>
-void launch_batch_push<double>(const BatchTables<double>& bt, int quad_order, cudaStream_t stream) {
-  launch_batch_push_q<double, false>(bt, quad_order, stream);
-}
-template <>
-void launch_batch_push<float>(const BatchTables<float>& bt, int quad_order, cudaStream_t stream) {
-  launch_batch_push_q<float, true>(bt, quad_order, stream);
+    k_push_deposit_batch<2><<<nb, 128, 0, stream>>>(bt.desc, bt.part, bt.npart, perm);
 }
 
 template <typename T>

@@ -240,10 +240,26 @@ __device__ __noinline__ void metric_christoffel_fp64(const Consts<float>& C, flo
   const double Xd = widen(x) - C.dxc, Yd = widen(y) - C.dyc, Zd = widen(z) - C.dzc;
   double p;
   const double s = quartic_newton(C, Xd, Yd, Zd, rf * rf, Df, &p);
-  const Kerr<double> K = kerr_from_r2<double, SeededOps64>(Xd, Yd, Zd, C.dm, C.da, s, 2.0 * s - p);
+  Kerr<double> K;
+  K.flat = !(s > 0.0);
+  if (!K.flat) {
+    K.D = 2.0 * s - p;
+    K.r = SeededOps64::root(s);
+    K.inv_r = SeededOps64::rcp(K.r);
+    K.inv_D = SeededOps64::rcp(K.D);
+    K.inv_rho2 = SeededOps64::rcp(s + C.da2);
+    K.inv_sig = K.inv_D * (K.inv_r * K.inv_r);  // Sigma = r^2 D at the root
+    K.f = 2.0 * C.dm * (K.r * K.inv_D);
+    K.k0 = fma(K.r, Xd, -C.da * Yd) * K.inv_rho2;
+    K.k1 = fma(K.r, Yd, C.da * Xd) * K.inv_rho2;
+    K.k2 = Zd * K.inv_r;
+  } else {
+    K.f = K.k0 = K.k1 = 0.0;
+    K.k2 = 1.0;
+  }
   const double ud[4] = {widen(u0), widen(u1), widen(u2), widen(u3)};
   double gd[4];
-  christoffel_uu<double, SeededOps64>(K, Xd, Yd, Zd, C.da, ud, gd);
+  christoffel_uu_fast(K, Xd, Yd, Zd, C.da, ud, gd);
   out[0] = narrow(K.f);
   out[1] = narrow(K.k0);
   out[2] = narrow(K.k1);
@@ -255,11 +271,11 @@ __device__ __noinline__ void metric_christoffel_fp64(const Consts<float>& C, flo
 }
 
 // a~ at (x, u): gather, convert, Lorentz - Christoffel.
-// mixed: the FP32-mixed policy applies (T = float): where the FP32 r is below r_fp64 the metric
+// MIXED: the FP32-mixed policy applies (T = float): where the FP32 r is below r_fp64 the metric
 // and the Christoffel contraction are taken from metric_christoffel_fp64.
-template <typename T>
+template <typename T, bool MIXED>
 __device__ __forceinline__ void accel(const Grid& g, const Fields<T>& F, const Consts<T>& C, const T x[3],
-                                      const T u[4], T out[4], unsigned& flags, unsigned& n64, bool mixed) {
+                                      const T u[4], T out[4], unsigned& flags, unsigned& n64) {
   // --- CIC gather: integer lattice (floor x) and half lattice (floor(x - 1/2)) per axis
   int ii[3], ih[3];
   T wi[3], wh[3];
@@ -331,13 +347,13 @@ __device__ __forceinline__ void accel(const Grid& g, const Fields<T>& F, const C
   Kerr<T> Kt;
   if constexpr (sizeof(T) == sizeof(float)) {
     // far-field warps: every stage has R > |a| (the quartic's p > 0 branch)
-    Kt = mixed ? kerr_eval<T>(X, Y, Z, C.m, C.a) : kerr_far(X, Y, Z, C.m, C.a);
+    Kt = MIXED ? kerr_eval<T>(X, Y, Z, C.m, C.a) : kerr_far(X, Y, Z, C.m, C.a);
   } else {
     Kt = kerr_eval_fast(X, Y, Z, C.m, C.a);
   }
   bool promoted = false;
-  if constexpr (sizeof(T) == sizeof(float)) {
-    if (mixed && Kt.r < C.r_fp64) {
+  if constexpr (sizeof(T) == sizeof(float) && MIXED) {
+    if (Kt.r < C.r_fp64) {
       float o[8];
       metric_christoffel_fp64(C, x[0], x[1], x[2], u[0], u[1], u[2], u[3], Kt.r, Kt.D, o);
       f = o[0];
@@ -518,8 +534,7 @@ __device__ __forceinline__ void deposit64(const Grid& g, const Fields<double>& F
   }
 }
 
-// The per-face quantities of deposit_lattice and the per-node terms they are built from (one
-// definition, so that the deferred near-hole nodes see exactly the values of the main loop).
+// The per-face quantities of deposit_lattice and the per-node terms they are built from.
 struct FaceLattice {
   int K;
   float PK, XK, PI, PJ, i0, j0, cI, cJ, wI0, wI1, pK, qK;
@@ -558,31 +573,24 @@ __device__ __forceinline__ float col_coord(const FaceLattice& L, int jb) {
   const float lo_j = sub ? L.PJ : L.j0, hi_j = sub ? L.j0 + 1.f : L.PJ;
   return fmaf(0.5f * (hi_j - lo_j), gx, 0.5f * (lo_j + hi_j));
 }
-__device__ __forceinline__ void col_terms(const Consts<float>& C, const FaceLattice& L, float AJ, float& pJ,
-                                          float& qJ, float& tJ) {
-  const float XJ = AJ - L.cJ;
-  pJ = XJ * XJ;
-  qJ = L.qJ * pJ;
-  tJ = L.tJ * XJ;
-}
-
-// Eq. 18 integrand at one node from its r^2 (scalar form, for the deferred nodes).
-__device__ __forceinline__ float node_value(const Consts<float>& C, const FaceLattice& L, float r2, float q,
-                                            float t) {
-  if (!(r2 > 0.f)) return 1.f;  // the flat limit r = 0
-  const float r = r2 * rsqrtf(r2);
-  const float sig = fmaf(r2, r2, q);
-  float fperp;
-  if (L.K == 2) {
-    fperp = __fdividef(C.two_m * r * (r2 - L.XK * L.XK), sig);
-  } else {
-    const float num = fmaf(r, L.XK, t);
-    const float rho2 = r2 + C.a2;
-    const float rho4 = rho2 * rho2;
-    fperp = __fdividef(C.two_m * r * r2 * fmaf(-num, num, rho4), rho4 * sig);
+// FP32-mixed: r^2 of one node of a hot cell, and 2 / D with it.  h = p / 2, q, D2 = h^2 + q, their FP32 root r2 (of the
+// p > 0 form) and 2 / D come in; the cancellation-free root where p <= 0, then one FP64 Newton step on the FP64 p64, q64
+// where the policy asks for it, and 2 / D = 2 r^2 / Sigma from the corrected root (near the ring the FP32 D has
+// lost its digits).  Straight-line but for the rare closed form, so that a row's nodes overlap.
+__device__ __forceinline__ void hot_node(const Consts<float>& C, float h, float q, double p64, double q64, float& r2,
+                                         float& rD2, unsigned& n64) {
+  const float D2 = fmaf(h, h, q);
+  const float sq = h > 0.f ? D2 * rD2 : sqrtf(D2);
+  float s0 = h > 0.f ? r2 : __fdividef(q, sq - h);
+  const bool promote = !(s0 >= C.r2_fp64);
+  if (promote) {
+    s0 = node_newton64(p64, q64, s0, 2.f * sq);
+    ++n64;
   }
-  const float v = 1.f + fperp;
-  return v * rsqrtf(v);
+  if (promote || !(h > 0.f)) {
+    r2 = s0;
+    rD2 = __fdividef(2.f * s0, fmaf(s0, s0, q));
+  }
 }
 
 // Means of t^i (i = 0..4) over [0, x] (lane x: x^i / (i+1)) and over [x, 1] (lane y:
@@ -675,18 +683,18 @@ __device__ __forceinline__ void table_areas(const float4* __restrict__ t, float 
 //   1 - k_y^2 = (rho^4 - (r y + a x)^2) / rho^4,  rho^2 = r^2 + a^2.
 // With (I, J) = (K+1, K+2) mod 3: K = 0 -> (x, y, z) = (x^K, x^I, x^J); K = 1 -> (x^J, x^K, x^I);
 // K = 2 -> (x^I, x^J, x^K).
-// Every node first takes the far-field form: for a particle outside the near radius every node
+// Every node takes the far-field form: for a particle outside the near radius every node
 // has R > |a|, so the quartic takes its p = R^2 - a^2 > 0 branch and every root argument is
-// positive.  With mixed (a warp-uniform flag) a node with p <= 0 or an FP32 r below r_fp64 is
-// left out of the sums and marked; after the lattice each marked node is evaluated again -- the
-// cancellation-free form of the root, then the FP64 policy (node_newton64 on FP64 p and q) where
-// it applies; r = 0 gives the flat limit -- and added.  The main loop has no call in it.
-template <int Q, bool TAB = false>
+// positive.  With MIXED the roots of a row in a hot cell (one near enough that a node may have p <= 0 or an
+// FP32 r below r_fp64) go through hot_node before the integrand; r = 0 gives the flat limit.  FP64 p and q are sums of
+// FP64 face, row and column terms, like their FP32 counterparts.
+// (Marked nodes evaluated one at a time after the lattice, each a serial chain of FP64 and integer operations with a
+// warp's lanes out of step: 136 us instead of 114 for 46 K particles at 32^3, a quarter of them near; 128^3 2.95 -> 2.89 ms.)
+template <int Q, bool MIXED, bool TAB = false>
 __device__ __forceinline__ void deposit_lattice(const Grid& g, const Fields<float>& F, const Consts<float>& C,
                                                 const float x0[3], const float dx[3], float qg, float inv_dt,
-                                                unsigned& flags, unsigned& n64, bool mixed, const JTile& jt,
+                                                unsigned& flags, unsigned& n64, const JTile& jt,
                                                 const float4* __restrict__ atab = nullptr) {
-  static_assert(4 * Q * Q <= 64, "node mask");
   const int nn[3] = {g.nx, g.ny, g.nz};
   int c1[3], c2[3];
   float s1[3], s2[3];
@@ -761,13 +769,30 @@ __device__ __forceinline__ void deposit_lattice(const Grid& g, const Fields<floa
           tJ2[k] = mul2(f2(L.tJ), XJ);
         }
         const float nzz = -(L.XK * L.XK);
+        // a hot cell's FP64 face and column terms (p and q of a node as sums)
+        bool hot = false;
+        double cI64 = 0.0, pK64 = 0.0, qK64 = 0.0, sqJ[2 * Q];
+        if (MIXED) {
+          const float XI = L.PI - L.cI, XJ = L.PJ - L.cJ;
+          hot = fmaf(XJ, XJ, fmaf(XI, XI, L.XK * L.XK)) < C.r2_hot;
+          if (hot) {
+            cI64 = sel3(K, C.dyc, C.dzc, C.dxc);
+            const double XK64 = widen(L.PK) - sel3(K, C.dxc, C.dyc, C.dzc), cJ64 = sel3(K, C.dzc, C.dxc, C.dyc);
+            pK64 = fma(XK64, XK64, -C.da2);
+            qK64 = K == 2 ? C.da2 * XK64 * XK64 : 0.0;
+#pragma unroll
+            for (int jb = 0; jb < 2 * Q; ++jb) {
+              const double XJ64 = widen(col_coord<Q>(L, jb)) - cJ64;
+              sqJ[jb] = XJ64 * XJ64;
+            }
+          }
+        }
         // acc[si][k]: lane-wise sums over the rows of sub-interval si, node pair k of a row
         float2 acc[2][Q];
   #pragma unroll
         for (int si = 0; si < 2; ++si)
   #pragma unroll
           for (int k = 0; k < Q; ++k) acc[si][k] = f2(0.f);
-        unsigned long long slow = 0ull;  // marked nodes, bit (si * Q + pi) * 2Q + jb
   #pragma unroll 1
         for (int pi = 0; pi < Q; ++pi) {
           float gw = (float)Gauss<Q>::w(0);
@@ -777,17 +802,43 @@ __device__ __forceinline__ void deposit_lattice(const Grid& g, const Fields<floa
   #pragma unroll
           for (int si = 0; si < 2; ++si) {
             float pRow, qRow, tRow;
-            row_terms(C, L, row_coord<Q>(L, si, pi), pRow, qRow, tRow);
+            const float AIa = row_coord<Q>(L, si, pi);
+            row_terms(C, L, AIa, pRow, qRow, tRow);
             const float2 pR = f2(0.5f * pRow), qR = f2(qRow), tR = f2(tRow);
+            // with h = p / 2 (the halves of the row and column terms, exact):
+            // r^2 = h + sqrt(h^2 + q), the root's p > 0 form
+            auto root = [&](int k, float2& rD2, float2& r2) {
+              const float2 p = add2(pR, pJ2[k]);
+              const float2 D2 = fma2(p, p, add2(qR, qJ2[k]));
+              rD2 = rsqrt2(D2);  // 2 / D
+              r2 = fma2(D2, rD2, p);
+            };
+            float2 rD2s[Q], r2s[Q];
+            if (MIXED) {
+  #pragma unroll
+              for (int k = 0; k < Q; ++k) root(k, rD2s[k], r2s[k]);
+              if (hot) {
+                const double XI64 = widen(AIa) - cI64;
+                const double pRow64 = fma(XI64, XI64, pK64);
+                const double qRow64 = K == 1 ? C.da2 * XI64 * XI64 : qK64;
+  #pragma unroll
+                for (int k = 0; k < Q; ++k) {
+                  const float2 h = add2(pR, pJ2[k]), q = add2(qR, qJ2[k]);
+                  const double sx = sqJ[2 * k], sy = sqJ[2 * k + 1];
+                  hot_node(C, h.x, q.x, pRow64 + sx, K == 0 ? C.da2 * sx : qRow64, r2s[k].x, rD2s[k].x, n64);
+                  hot_node(C, h.y, q.y, pRow64 + sy, K == 0 ? C.da2 * sy : qRow64, r2s[k].y, rD2s[k].y, n64);
+                }
+              }
+            }
   #pragma unroll
             for (int k = 0; k < Q; ++k) {
-              // with h = p / 2 (the halves of the row and column terms, exact):
-              // r^2 = h + sqrt(h^2 + q), the root's p > 0 form
-              const float2 p = add2(pR, pJ2[k]);
-              const float2 q = add2(qR, qJ2[k]);
-              const float2 D2 = fma2(p, p, q);
-              const float2 rD2 = rsqrt2(D2);  // 2 / D
-              const float2 r2 = fma2(D2, rD2, p);
+              float2 rD2, r2;
+              if (MIXED) {
+                rD2 = rD2s[k];
+                r2 = r2s[k];
+              } else {
+                root(k, rD2, r2);
+              }
               const float2 ir = rsqrt2(r2);
               // at the root r^4 + a^2 z^2 = r^2 D, so f = 2 m r^3 / Sigma = 2 m r / D = m r rsqrt(D2)
               float2 v;
@@ -802,18 +853,11 @@ __device__ __forceinline__ void deposit_lattice(const Grid& g, const Fields<floa
                 const float2 omk2 = fma2(kK, make_float2(-kK.x, -kK.y), f2(1.f));
                 v = fma2(mul2(mul2(f2(C.m), r), rD2), omk2, f2(1.f));
               }
-              float2 rv = rsqrt2(v);
-              if (mixed) {
-                const int bit = (si * Q + pi) * 2 * Q + 2 * k;
-                if (!(p.x > 0.f) || !(r2.x >= C.r2_fp64)) {
-                  v.x = rv.x = 0.f;
-                  slow |= 1ull << bit;
-                }
-                if (!(p.y > 0.f) || !(r2.y >= C.r2_fp64)) {
-                  v.y = rv.y = 0.f;
-                  slow |= 1ull << (bit + 1);
-                }
+              if (MIXED && hot) {  // r = 0: the flat limit
+                if (!(r2.x > 0.f)) v.x = 1.f;
+                if (!(r2.y > 0.f)) v.y = 1.f;
               }
+              const float2 rv = rsqrt2(v);
               if (Q == 2) {
                 acc[si][k] = fma2(v, rv, acc[si][k]);  // unit Gauss weights
               } else {
@@ -833,66 +877,6 @@ __device__ __forceinline__ void deposit_lattice(const Grid& g, const Fields<floa
             S[si][(2 * k) >= Q ? 1 : 0] += acc[si][k].x;
             S[si][(2 * k + 1) >= Q ? 1 : 0] += acc[si][k].y;
           }
-        // The marked nodes of FP32-mixed warps.  p and q in FP64 are sums of FP64 face, row and
-        // column terms, like their FP32 counterparts: face, row and column terms are formed once.
-        if (slow) {
-          const double cK = sel3(K, C.dxc, C.dyc, C.dzc), cI = sel3(K, C.dyc, C.dzc, C.dxc);
-          const double cJ = sel3(K, C.dzc, C.dxc, C.dyc);
-          const double XK64 = widen(L.PK) - cK;
-          const double pK64 = fma(XK64, XK64, -C.da2);
-          const double qK64 = K == 2 ? C.da2 * XK64 * XK64 : 0.0;
-          double sqJ[2 * Q];  // squared FP64 offsets of the columns
-  #pragma unroll
-          for (int jb = 0; jb < 2 * Q; ++jb) {
-            const double XJ64 = widen(col_coord<Q>(L, jb)) - cJ;
-            sqJ[jb] = XJ64 * XJ64;
-          }
-          int row = -1;
-          double pRow64 = 0.0, qRow64 = 0.0;
-          do {
-            const int b = __ffsll((long long)slow) - 1;
-            slow &= slow - 1ull;
-            const int ia = b / (2 * Q), jb = b - ia * 2 * Q;
-            const int si = ia / Q, pi = ia - si * Q;
-            const float AIa = row_coord<Q>(L, si, pi), AJ = col_coord<Q>(L, jb);
-            float pRow, qRow, tRow, pJ, qJ, tJ;
-            row_terms(C, L, AIa, pRow, qRow, tRow);
-            col_terms(C, L, AJ, pJ, qJ, tJ);
-            const float p = pRow + pJ, q = qRow + qJ;
-            // FP32 root by the cancellation-free form; FP64 where the policy asks for it (a node
-            // with p > 0 was marked only for that)
-            const float D = sqrtf(fmaf(p, p, 4.f * q));
-            float r2 = p >= 0.f ? 0.5f * (p + D) : __fdividef(2.f * q, D - p);
-            if (p > 0.f || !(r2 >= C.r2_fp64)) {
-              if (ia != row) {
-                row = ia;
-                const double XI64 = widen(AIa) - cI;
-                pRow64 = fma(XI64, XI64, pK64);
-                qRow64 = K == 1 ? C.da2 * XI64 * XI64 : qK64;
-              }
-              double sq = sqJ[0];
-  #pragma unroll
-              for (int t = 1; t < 2 * Q; ++t)
-                if (jb == t) sq = sqJ[t];
-              const double p64 = pRow64 + sq;
-              const double q64 = K == 0 ? C.da2 * sq : qRow64;
-              r2 = node_newton64(p64, q64, r2, D);
-              ++n64;
-            }
-            float w = (float)Gauss<Q>::w(0), wj = (float)Gauss<Q>::w(0);
-  #pragma unroll
-            for (int t = 1; t < Q; ++t) {
-              if (pi == t) w = (float)Gauss<Q>::w(t);
-              if (jb % Q == t) wj = (float)Gauss<Q>::w(t);
-            }
-            const float add = w * wj * node_value(C, L, r2, q, tRow + tJ);
-            const int sj = jb >= Q ? 1 : 0;
-            S[0][0] += (si == 0 && sj == 0) ? add : 0.f;
-            S[0][1] += (si == 0 && sj == 1) ? add : 0.f;
-            S[1][0] += (si == 1 && sj == 0) ? add : 0.f;
-            S[1][1] += (si == 1 && sj == 1) ? add : 0.f;
-          } while (slow);
-        }
         const float wI[2] = {L.wI0, L.wI1};
         A00 = S[1][1] * 0.25f * wI[1] * wJ[1];
         A10 = S[0][1] * 0.25f * wI[0] * wJ[1];
@@ -946,10 +930,10 @@ struct Move {
 };
 
 // One particle-step of particle i without its deposit (push_particle below, up to the deposit).
-template <typename T, int Q>
+template <typename T, bool MIXED>
 __device__ __forceinline__ Move<T> push_move(const Grid& g, const Fields<T>& F, const Particles<T>& P,
                                              const Consts<T>& C, long long i, DevStatus* st, unsigned& flags,
-                                             unsigned& n64, uint32_t* key_out, bool mixed) {
+                                             unsigned& n64, uint32_t* key_out) {
   // RK4 in proper time: stages at offsets 0, h/2, h/2, h; h = dt / gamma_1 (Eq. 16).  x^4 does
   // not enter a~ (the metric is stationary), so the stages carry x^1..x^3 only.
   T xs[3], us[4], a[4], sx[4], su[4];
@@ -964,7 +948,7 @@ __device__ __forceinline__ Move<T> push_move(const Grid& g, const Fields<T>& F, 
   bool fb = false;
 #pragma unroll 1
   for (int stage = 0; stage < 4; ++stage) {
-    accel<T>(g, F, C, xs, us, a, flags, n64, mixed);
+    accel<T, MIXED>(g, F, C, xs, us, a, flags, n64);
     if (stage == 0) {
       if constexpr (sizeof(T) == sizeof(double))
         h = C.dt * FastOps64::rcp(gamma_step<T, FastOps64>(us[3], a[3], C.inv_c, C.dt, &fb));
@@ -1067,13 +1051,12 @@ __device__ __forceinline__ Move<T> push_move(const Grid& g, const Fields<T>& F, 
 
 // The deposit of a move (Sec. 4).  TAB (far-field warps, T = float): face areas from the per-cell
 // fits atab.
-template <typename T, int Q, bool TAB = false>
+template <typename T, int Q, bool MIXED, bool TAB>
 __device__ __forceinline__ void deposit_move(const Grid& g, const Fields<T>& F, const Consts<T>& C, const Move<T>& mv,
-                                             unsigned& flags, unsigned& n64, bool mixed, const JTile& jt = JTile(),
-                                             const float4* atab = nullptr) {
+                                             unsigned& flags, unsigned& n64, const JTile& jt, const float4* atab) {
   if (!mv.go) return;
   if constexpr (sizeof(T) == sizeof(float))
-    deposit_lattice<Q, TAB>(g, F, C, mv.x0, mv.dx, mv.qg, C.inv_dt, flags, n64, mixed, jt, atab);
+    deposit_lattice<Q, MIXED, TAB>(g, F, C, mv.x0, mv.dx, mv.qg, C.inv_dt, flags, n64, jt, atab);
   else
     deposit64<Q>(g, F, C, mv.x0, mv.dx, mv.qg, C.inv_dt, flags);
 }
@@ -1081,16 +1064,16 @@ __device__ __forceinline__ void deposit_move(const Grid& g, const Fields<T>& F, 
 // One particle-step of particle i: RK4 push, new state stored, removal flag and sort key
 // (written to *key_out: P.key + i, or a side array where another kernel still reads P.key
 // concurrently), then the deposit of the move (which needs only x_n and the increment).
-// mixed (T = float): the FP32-mixed policy applies to this warp's particles (a warp-uniform
-// flag; false only where every particle lies outside near_radius).  T = double ignores it.
+// MIXED (T = float): the FP32-mixed policy applies to this warp's particles (false only where every particle lies
+// outside near_radius).
 // TAB (far-field warps, T = float): the deposit takes its face areas from the per-cell fits atab.
-template <typename T, int Q, bool TAB = false>
+template <typename T, int Q, bool MIXED, bool TAB = false>
 __device__ __forceinline__ void push_particle(const Grid& g, const Fields<T>& F, const Particles<T>& P,
                                               const Consts<T>& C, long long i, DevStatus* st, unsigned& flags,
-                                              unsigned& n64, uint32_t* key_out, bool mixed,
-                                              const JTile& jt = JTile(), const float4* atab = nullptr) {
-  const Move<T> mv = push_move<T, Q>(g, F, P, C, i, st, flags, n64, key_out, mixed);
-  deposit_move<T, Q, TAB>(g, F, C, mv, flags, n64, mixed, jt, atab);
+                                              unsigned& n64, uint32_t* key_out, const JTile& jt = JTile(),
+                                              const float4* atab = nullptr) {
+  const Move<T> mv = push_move<T, MIXED>(g, F, P, C, i, st, flags, n64, key_out);
+  deposit_move<T, Q, MIXED, TAB>(g, F, C, mv, flags, n64, jt, atab);
 }
 
 // Warp-aggregated status: flags, FP64 evaluations and particle-steps of the warp's lanes.

@@ -50,7 +50,7 @@ __global__ void __launch_bounds__(128, MINB) k_push_far(const Grid g, const Fiel
     const uint32_t k = P.key[i];
     active = k != kDead && k != kNear;
   }
-  if (active) push_particle<float, Q>(g, F, P, C, i, st, flags, n64, P.key + i, false);
+  if (active) push_particle<float, Q, false>(g, F, P, C, i, st, flags, n64, P.key + i);
   warp_status(st, flags, n64, active);
 }
 
@@ -70,11 +70,10 @@ constexpr int kJTileFloats = 3072;
 // perm: the block -> particle-chunk map (spread_chunk in common.cuh; 1 = in order).
 // TAB: the far-field copy deposits with the per-cell area fits atab; r_near2 is then
 // table_radius^2, so that every far particle lies where the fits hold.
-template <int Q, int MINB, bool TILE, bool TAB = false>
-__global__ void __launch_bounds__(128, MINB) k_push_select(const Grid g, const Fields<float> F,
-                                                           const Particles<float> P, const Consts<float> C,
-                                                           float r_near2, unsigned perm, int lg, DevStatus* st,
-                                                           const float4* __restrict__ atab) {
+template <int Q, int MINB, bool TILE, bool TAB, int THREADS>
+__global__ void __launch_bounds__(THREADS, MINB * (128 / THREADS))
+    k_push_select(const Grid g, const Fields<float> F, const Particles<float> P, const Consts<float> C,
+                  float r_near2, unsigned perm, int lg, DevStatus* st, const float4* __restrict__ atab) {
   const unsigned chunk = spread_chunk(blockIdx.x, gridDim.x, perm, lg);
   const long long i = chunk * (long long)blockDim.x + threadIdx.x;
   unsigned flags = 0, n64 = 0;
@@ -133,7 +132,7 @@ __global__ void __launch_bounds__(128, MINB) k_push_select(const Grid g, const F
   // two inlined copies, each with the flag a constant: the far-field copy has no out-of-line
   // calls at all (a call site in the loop would cost every warp registers and stack traffic)
   if (__any_sync(0xffffffffu, near)) {
-    if (active) push_particle<float, Q>(g, F, P, C, i, st, flags, n64, P.key + i, true, jt);
+    if (active) push_particle<float, Q, true>(g, F, P, C, i, st, flags, n64, P.key + i, jt);
   } else if constexpr (TAB) {
     if (active) {
       // the fits of x_n's cell (the deposit's first segment) into L2 now, read after the RK4 stages
@@ -144,10 +143,10 @@ __global__ void __launch_bounds__(128, MINB) k_push_select(const Grid g, const F
       const char* t = reinterpret_cast<const char*>(atab + cell_index(g, c[0], c[1], c[2]) * kAreaTableStride);
 #pragma unroll
       for (int b = 0; b < 16 * kAreaTableStride; b += 128) asm volatile("prefetch.global.L2 [%0];" ::"l"(t + b));
-      push_particle<float, Q, true>(g, F, P, C, i, st, flags, n64, P.key + i, false, jt, atab);
+      push_particle<float, Q, false, true>(g, F, P, C, i, st, flags, n64, P.key + i, jt, atab);
     }
   } else if (active) {
-    push_particle<float, Q>(g, F, P, C, i, st, flags, n64, P.key + i, false, jt);
+    push_particle<float, Q, false>(g, F, P, C, i, st, flags, n64, P.key + i, jt);
   }
   warp_status(st, flags, n64, active);
   if constexpr (TILE) {
@@ -216,32 +215,42 @@ unsigned coprime_multiplier(unsigned n) {
   return m % n;
 }
 
+template <int Q, int MINB, bool TILE, bool TAB, int THREADS>
+void launch_select(const Grid& g, const Fields<float>& F, const Particles<float>& P, const Consts<float>& C,
+                   int spread, DevStatus* st, const float4* atab, cudaStream_t stream) {
+  const double rn = TAB ? table_radius(g) : near_radius(g);
+  const unsigned nb = blocks_for(P.n, THREADS);
+  // groups of `spread` chunks of 128 particles
+  const int lg = spread > 0 ? spread_log2(spread * (128 / THREADS)) : 0;
+  const unsigned perm = spread > 0 ? spread_multiplier(nb, lg) : 1u;
+  k_push_select<Q, MINB, TILE, TAB, THREADS><<<nb, THREADS, 0, stream>>>(g, F, P, C, (float)(rn * rn), perm, lg, st,
+                                                                         atab);
+}
+
 void launch_push_select(const Grid& g, const Fields<float>& F, const Particles<float>& P, const Species& sp,
                         DevStatus* st, int minb, bool tile, int spread, const float4* atab, cudaStream_t stream) {
   if (P.n <= 0) return;
-  const unsigned nb = blocks_for(P.n, 128);
   const Consts<float> C = make_consts<float>(g, sp);
   const bool tab = atab != nullptr && g.quad_order == 2 && !tile;
-  const double rn = tab ? table_radius(g) : near_radius(g);
-  const float r_near2 = (float)(rn * rn);
-  const int lg = spread > 0 ? spread_log2(spread) : 0;
-  const unsigned perm = spread > 0 ? spread_multiplier(nb, lg) : 1u;
+  const bool small = small_push(P.n) && !tile;
   if (g.quad_order == 1)
-    k_push_select<1, 4, false><<<nb, 128, 0, stream>>>(g, F, P, C, r_near2, perm, lg, st, nullptr);
+    small ? launch_select<1, 4, false, false, 32>(g, F, P, C, spread, st, nullptr, stream)
+          : launch_select<1, 4, false, false, 128>(g, F, P, C, spread, st, nullptr, stream);
   else if (g.quad_order == 3)
-    k_push_select<3, 4, false><<<nb, 128, 0, stream>>>(g, F, P, C, r_near2, perm, lg, st, nullptr);
-  else if (tab && minb >= 5)
-    k_push_select<2, 5, false, true><<<nb, 128, 0, stream>>>(g, F, P, C, r_near2, perm, lg, st, atab);
+    small ? launch_select<3, 4, false, false, 32>(g, F, P, C, spread, st, nullptr, stream)
+          : launch_select<3, 4, false, false, 128>(g, F, P, C, spread, st, nullptr, stream);
+  else if (small)
+    tab ? launch_select<2, 4, false, true, 32>(g, F, P, C, spread, st, atab, stream)
+        : launch_select<2, 4, false, false, 32>(g, F, P, C, spread, st, nullptr, stream);
   else if (tab)
-    k_push_select<2, 4, false, true><<<nb, 128, 0, stream>>>(g, F, P, C, r_near2, perm, lg, st, atab);
-  else if (tile && minb >= 5)
-    k_push_select<2, 5, true><<<nb, 128, 0, stream>>>(g, F, P, C, r_near2, perm, lg, st, nullptr);
+    minb >= 5 ? launch_select<2, 5, false, true, 128>(g, F, P, C, spread, st, atab, stream)
+              : launch_select<2, 4, false, true, 128>(g, F, P, C, spread, st, atab, stream);
   else if (tile)
-    k_push_select<2, 4, true><<<nb, 128, 0, stream>>>(g, F, P, C, r_near2, perm, lg, st, nullptr);
-  else if (minb >= 5)
-    k_push_select<2, 5, false><<<nb, 128, 0, stream>>>(g, F, P, C, r_near2, perm, lg, st, nullptr);
+    minb >= 5 ? launch_select<2, 5, true, false, 128>(g, F, P, C, spread, st, nullptr, stream)
+              : launch_select<2, 4, true, false, 128>(g, F, P, C, spread, st, nullptr, stream);
   else
-    k_push_select<2, 4, false><<<nb, 128, 0, stream>>>(g, F, P, C, r_near2, perm, lg, st, nullptr);
+    minb >= 5 ? launch_select<2, 5, false, false, 128>(g, F, P, C, spread, st, nullptr, stream)
+              : launch_select<2, 4, false, false, 128>(g, F, P, C, spread, st, nullptr, stream);
 }
 
 }  // namespace grpic
