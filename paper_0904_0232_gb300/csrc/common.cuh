@@ -164,7 +164,7 @@ struct Particles {
   uint32_t* id;
   uint32_t* key;
   long long n;       // entries in the arrays (live + removed-not-yet-sorted)
-  const int* n_dev;  // live+flagged count after the last sort (device)
+  const int* n_dev;  // live+flagged count of this buffer after the sort that filled it (device)
 };
 
 __host__ __device__ inline long long cell_index(const Grid& g, int i, int j, int k) {
@@ -361,17 +361,23 @@ void launch_max_id(const Particles<T>& P, unsigned long long* max_id, cudaStream
 size_t invariant_acc_bytes();
 constexpr int kInvariantStride = 64;  // tracked subsample: ids divisible by this
 
-// Counting sort by cell of one species; removed particles (key == kDead) are dropped.
-// counts: nbins+1 ints, offsets: nbins+1 ints, blocks: scan scratch; n_out: device int.
-struct SortScratch {
-  int* counts;
-  int* offsets;
-  int* blocks;
-  int nblocks;
+// Counting sort by cell of the species of a context; removed particles (key == kDead) are dropped.  bins: ncell + 1 ints,
+// zero on entry; tiles: scan_tiles(ncell + 1) ints; n_out: the live count (device).
+template <typename T>
+struct SortJob {
+  Particles<T> src, dst;
+  int* bins;
+  int* tiles;
+  int* n_out;
 };
 template <typename T>
-void launch_sort(const Grid& g, const Particles<T>& src, const Particles<T>& dst, const SortScratch& s,
-                 int* n_out, cudaStream_t stream);
+struct SortJobs {
+  SortJob<T> job[4];
+  int n;
+};
+int scan_tiles(long long nbins);
+template <typename T>
+void launch_sort(const Grid& g, const SortJobs<T>& jobs, cudaStream_t stream);
 
 // ---- batched engine -------------------------------------------------------------------------
 // Every stage of a batched step is one launch over a device table of work blocks; each block

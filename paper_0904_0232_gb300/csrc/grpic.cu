@@ -12,10 +12,6 @@
 
 using namespace grpic;
 
-namespace grpic {
-int scan_tiles(long long nbins);
-}
-
 namespace {
 
 constexpr int kMaxSpecies = 4;
@@ -26,12 +22,18 @@ struct SpeciesStore {
   long long cap = 0;  // capacity in particles
   void* buf[2] = {nullptr, nullptr};
   int cur = 0;
-  int* n_dev = nullptr;
-  int* n_shadow = nullptr;  // pinned host copy of n_dev
-  int* near_n = nullptr;    // split push: near-hole list length and work cursor (2 device ints)
-  cudaEvent_t shadow_ev = nullptr;
+  int* n_dev = nullptr;   // live count of each buffer (2 device ints)
+  int* near_n = nullptr;  // split push: near-hole list length and work cursor (2 device ints)
+  int* bins = nullptr;    // sort bins and tiles (sort_ints(c) ints)
+  bool bins_zero = false;
   bool shadow_pending = false;
   bool loaded = false;
+};
+
+// What the host reads back: the status word and the species' live counts (both buffers).
+struct HostMirror {
+  DevStatus st;
+  int n[2 * kMaxSpecies];
 };
 
 }  // namespace
@@ -63,8 +65,10 @@ struct grpic_ctx {
   bool bprev_held = false;  // between a first B half-step and its second: the idle b buffer is b^{n-1/2}
   void* dstar = nullptr;    // 3 planes of T for the E step's predictor in that state (hand-driven stages only)
   DevStatus* st = nullptr;
-  DevStatus* st_host = nullptr;  // pinned
-  SortScratch sort{};
+  int* counters = nullptr;       // 4 ints a species: n_dev, near_n
+  HostMirror* host = nullptr;    // pinned
+  cudaEvent_t shadow_ev = nullptr;  // the last copy of the live counts into host->n
+  int* bins2 = nullptr;          // sort bins of species 2 and 3 (those of 0 and 1 follow J)
   SpeciesStore sp[kMaxSpecies];
   long long steps = 0;
   long long pushes = 0;
@@ -179,16 +183,35 @@ Particles<T> particles_view(grpic_ctx* c, int s, int which) {
   P.id = reinterpret_cast<uint32_t*>(base + 8 * cap * sizeof(T));
   P.key = reinterpret_cast<uint32_t*>(base + 8 * cap * sizeof(T) + cap * sizeof(uint32_t));
   P.n = S.n;
-  P.n_dev = S.n_dev;
+  P.n_dev = S.n_dev + which;
   return P;
 }
 
 // Refresh the host upper bound of the live count from the last completed shadow copy.
-void refresh_count(SpeciesStore& S) {
-  if (S.shadow_pending && cudaEventQuery(S.shadow_ev) == cudaSuccess) {
-    S.n = std::min<long long>(S.n, *S.n_shadow);
+void refresh_count(grpic_ctx* c, int s) {
+  SpeciesStore& S = c->sp[s];
+  if (S.shadow_pending && cudaEventQuery(c->shadow_ev) == cudaSuccess) {
+    S.n = std::min<long long>(S.n, c->host->n[2 * s + S.cur]);
     S.shadow_pending = false;
   }
+}
+
+// Ints of a species' sort scratch: the bins, then the tiles.
+long long sort_ints(const grpic_ctx* c) { return c->g.ncell + 1 + scan_tiles(c->g.ncell + 1); }
+
+void zero_bins(grpic_ctx* c, int s) {
+  if (c->sp[s].bins_zero) return;
+  cudaMemsetAsync(c->sp[s].bins, 0, sizeof(int) * (size_t)sort_ints(c), c->stream);
+  c->sp[s].bins_zero = true;
+}
+
+template <typename T>
+SortJob<T> sort_job(grpic_ctx* c, int s) {
+  SpeciesStore& S = c->sp[s];
+  zero_bins(c, s);
+  S.bins_zero = false;
+  return SortJob<T>{particles_view<T>(c, s, S.cur), particles_view<T>(c, s, 1 - S.cur), S.bins,
+                    S.bins + c->g.ncell + 1, S.n_dev + (1 - S.cur)};
 }
 
 bool literal_fields(const grpic_ctx* c) { return (c->cfg.flags & GRPIC_LITERAL_HALF_STEPS) != 0; }
@@ -219,7 +242,7 @@ void enqueue_species_pushes(grpic_ctx* c, Launch launch) {
   int order[kMaxSpecies], n = 0;
   for (int s = 0; s < kMaxSpecies; ++s) {
     if (!c->sp[s].loaded || c->sp[s].n == 0) continue;
-    refresh_count(c->sp[s]);
+    refresh_count(c, s);
     order[n++] = s;
   }
   std::stable_sort(order, order + n, [c](int a, int b) { return c->sp[a].n < c->sp[b].n; });
@@ -273,7 +296,7 @@ void enqueue_split_push(grpic_ctx* c) {
   for (int s = 0; s < kMaxSpecies; ++s) {
     SpeciesStore& S = c->sp[s];
     if (!S.loaded || S.n == 0) continue;
-    refresh_count(S);
+    refresh_count(c, s);
     cudaMemsetAsync(S.near_n, 0, 2 * sizeof(int), c->stream);
     launch_classify_near(c->g, particles_view<float>(c, s, S.cur), particles_view<float>(c, s, 1 - S.cur).key,
                          S.near_n, c->stream);
@@ -347,7 +370,16 @@ void enqueue_stage(grpic_ctx* c, int stage) {
       break;
     }
     case GRPIC_STAGE_ZERO_J:
-      cudaMemsetAsync(c->J, 0, sizeof(double) * 3 * (size_t)c->g.ncell, c->stream);
+      // with the bins of species 0 and 1 behind it where the last sort left counts in them
+      {
+        size_t bytes = sizeof(double) * 3 * (size_t)c->g.ncell;
+        for (int s = 0; s < 2; ++s)
+          if (c->sp[s].loaded && !c->sp[s].bins_zero) {
+            bytes = sizeof(double) * 3 * (size_t)c->g.ncell + (s + 1) * sizeof(int) * (size_t)sort_ints(c);
+            for (int q = 0; q <= s; ++q) c->sp[q].bins_zero = true;
+          }
+        cudaMemsetAsync(c->J, 0, bytes, c->stream);
+      }
       break;
     case GRPIC_STAGE_PUSH_DEPOSIT:
       if (split_push(c)) {
@@ -399,19 +431,22 @@ void enqueue_stage(grpic_ctx* c, int stage) {
       c->dcur = 1 - c->dcur;
       break;
     }
-    case GRPIC_STAGE_SORT:
-      for (int s = 0; s < kMaxSpecies; ++s) {
-        SpeciesStore& S = c->sp[s];
-        if (!S.loaded) continue;
-        launch_sort<T>(c->g, particles_view<T>(c, s, S.cur), particles_view<T>(c, s, 1 - S.cur), c->sort, S.n_dev,
-                       c->stream);
-        c->launches += S.n > 0 ? 6 : 4;
-        S.cur = 1 - S.cur;
-        cudaMemcpyAsync(S.n_shadow, S.n_dev, sizeof(int), cudaMemcpyDeviceToHost, c->stream);
-        cudaEventRecord(S.shadow_ev, c->stream);
-        S.shadow_pending = true;
-      }
+    case GRPIC_STAGE_SORT: {
+      SortJobs<T> jobs{};
+      for (int s = 0; s < kMaxSpecies; ++s)
+        if (c->sp[s].loaded) jobs.job[jobs.n++] = sort_job<T>(c, s);
+      if (jobs.n == 0) break;
+      launch_sort<T>(c->g, jobs, c->stream);
+      c->launches += 4;
+      for (int s = 0; s < kMaxSpecies; ++s)
+        if (c->sp[s].loaded) {
+          c->sp[s].cur = 1 - c->sp[s].cur;
+          c->sp[s].shadow_pending = true;
+        }
+      cudaMemcpyAsync(c->host->n, c->counters, sizeof(c->host->n), cudaMemcpyDeviceToHost, c->stream);
+      cudaEventRecord(c->shadow_ev, c->stream);
       break;
+    }
     default:
       break;
   }
@@ -475,14 +510,14 @@ void enqueue_step(grpic_ctx* c) {
 }
 
 grpic_status read_status(grpic_ctx* c) {
-  grpic_status s = cuda_check(c, cudaMemcpyAsync(c->st_host, c->st, sizeof(DevStatus), cudaMemcpyDeviceToHost,
+  grpic_status s = cuda_check(c, cudaMemcpyAsync(&c->host->st, c->st, sizeof(DevStatus), cudaMemcpyDeviceToHost,
                                                  c->stream),
                               "status copy");
   if (s != GRPIC_OK) return s;
   s = cuda_check(c, cudaStreamSynchronize(c->stream), "stream synchronize");
   if (s != GRPIC_OK) return s;
   collect_profile(c);
-  const DevStatus h = *c->st_host;
+  const DevStatus h = c->host->st;
   c->totals.removed_horizon = (int64_t)h.removed_horizon;
   c->totals.removed_outer = (int64_t)h.removed_outer;
   c->totals.gamma_fallbacks = (int64_t)h.fallbacks;
@@ -631,24 +666,20 @@ grpic_status grpic::create_context(const grpic_config* cfg, void* stream, bool m
   const bool layers = g.k_in > 0.0 || g.k_out > 0.0;
   if (layers) c->tgt = dev_alloc(c, 6 * (size_t)ncell * c->tsize);
   if (kin_cells > 0) c->kin = dev_alloc(c, 6 * (size_t)kin_cells * c->tsize);
-  c->J = static_cast<double*>(dev_alloc(c, 3 * (size_t)ncell * sizeof(double)));
+  // J, then the sort bins of species 0 and 1
+  c->J = static_cast<double*>(
+      dev_alloc(c, 3 * (size_t)ncell * sizeof(double) + 2 * sizeof(int) * (size_t)sort_ints(c)));
   c->loc = static_cast<uint16_t*>(dev_alloc(c, sizeof(uint16_t) * (size_t)ncell));
   c->st = static_cast<DevStatus*>(dev_alloc(c, sizeof(DevStatus)));
-  const long long nbins = ncell + 1;
-  c->sort.nblocks = scan_tiles(nbins);
-  c->sort.counts = static_cast<int*>(dev_alloc(c, sizeof(int) * nbins));
-  c->sort.offsets = static_cast<int*>(dev_alloc(c, sizeof(int) * nbins));
-  c->sort.blocks = static_cast<int*>(dev_alloc(c, sizeof(int) * (c->sort.nblocks + 1)));
-  bool ok = c->fields && c->J && c->loc && c->st && c->sort.counts && c->sort.offsets && c->sort.blocks &&
-            (c->tgt || !layers) && (c->kin || kin_cells == 0);
+  c->counters = static_cast<int*>(dev_alloc(c, sizeof(int) * 4 * kMaxSpecies));
+  bool ok = c->fields && c->J && c->loc && c->st && c->counters && (c->tgt || !layers) && (c->kin || kin_cells == 0);
   for (int s = 0; s < kMaxSpecies && ok; ++s) {
-    c->sp[s].n_dev = static_cast<int*>(dev_alloc(c, sizeof(int)));
-    c->sp[s].near_n = static_cast<int*>(dev_alloc(c, 2 * sizeof(int)));
-    ok = c->sp[s].n_dev != nullptr && c->sp[s].near_n != nullptr;
-    if (ok) ok = cudaMallocHost(&c->sp[s].n_shadow, sizeof(int)) == cudaSuccess;
-    if (ok) ok = cudaEventCreateWithFlags(&c->sp[s].shadow_ev, cudaEventDisableTiming) == cudaSuccess;
+    c->sp[s].n_dev = c->counters + 2 * s;
+    c->sp[s].near_n = c->counters + 2 * kMaxSpecies + 2 * s;
+    if (s < 2) c->sp[s].bins = reinterpret_cast<int*>(c->J + 3 * (size_t)ncell) + s * sort_ints(c);
   }
-  if (ok) ok = cudaMallocHost(&c->st_host, sizeof(DevStatus)) == cudaSuccess;
+  if (ok) ok = cudaMallocHost(&c->host, sizeof(HostMirror)) == cudaSuccess;
+  if (ok) ok = cudaEventCreateWithFlags(&c->shadow_ev, cudaEventDisableTiming) == cudaSuccess;
   if (ok) {
     int lo = 0, hi = 0;
     cudaDeviceGetStreamPriorityRange(&lo, &hi);
@@ -666,7 +697,7 @@ grpic_status grpic::create_context(const grpic_config* cfg, void* stream, bool m
   if (c->tgt) cudaMemsetAsync(c->tgt, 0, 6 * (size_t)ncell * c->tsize, c->stream);
   cudaMemsetAsync(c->J, 0, 3 * (size_t)ncell * sizeof(double), c->stream);
   cudaMemsetAsync(c->st, 0, sizeof(DevStatus), c->stream);
-  for (int s = 0; s < kMaxSpecies; ++s) cudaMemsetAsync(c->sp[s].n_dev, 0, sizeof(int), c->stream);
+  cudaMemsetAsync(c->counters, 0, sizeof(int) * 4 * kMaxSpecies, c->stream);
   launch_location_flags(g, c->loc, c->stream);
   if (c->kin) {
     if (c->mixed)
@@ -702,20 +733,16 @@ grpic_status grpic_destroy(grpic_ctx* c) {
   dev_free(c, c->J);
   dev_free(c, c->loc);
   dev_free(c, c->st);
-  dev_free(c, c->sort.counts);
-  dev_free(c, c->sort.offsets);
-  dev_free(c, c->sort.blocks);
+  dev_free(c, c->bins2);
+  dev_free(c, c->counters);
   for (int s = 0; s < kMaxSpecies; ++s) {
     dev_free(c, c->inv_e0[s]);
     dev_free(c, c->inv_l0[s]);
     dev_free(c, c->sp[s].buf[0]);
     dev_free(c, c->sp[s].buf[1]);
-    dev_free(c, c->sp[s].n_dev);
-    dev_free(c, c->sp[s].near_n);
-    if (c->sp[s].n_shadow) cudaFreeHost(c->sp[s].n_shadow);
-    if (c->sp[s].shadow_ev) cudaEventDestroy(c->sp[s].shadow_ev);
   }
-  if (c->st_host) cudaFreeHost(c->st_host);
+  if (c->host) cudaFreeHost(c->host);
+  if (c->shadow_ev) cudaEventDestroy(c->shadow_ev);
   if (c->side) {
     cudaStreamSynchronize(c->side);
     cudaStreamDestroy(c->side);
@@ -815,6 +842,11 @@ grpic_status grpic_load_particles(grpic_ctx* c, int species, double q_over_m, do
   grpic_status s = ensure_capacity(c, species, n);
   if (s != GRPIC_OK) return s;
   SpeciesStore& S = c->sp[species];
+  if (!S.bins) {  // species 2 and 3
+    c->bins2 = static_cast<int*>(dev_alloc(c, 2 * sizeof(int) * (size_t)sort_ints(c)));
+    if (!c->bins2) return fail(c, GRPIC_ERR_OOM, "sort scratch allocation failed");
+    for (int q = 2; q < kMaxSpecies; ++q) c->sp[q].bins = c->bins2 + (q - 2) * sort_ints(c);
+  }
   const void *xd, *ud, *idd;
   void *tx = nullptr, *tu = nullptr, *ti = nullptr;
   s = stage_in(c, x4, sizeof(double) * 4 * (size_t)n, mem, &xd, &tx);
@@ -834,7 +866,8 @@ grpic_status grpic_load_particles(grpic_ctx* c, int species, double q_over_m, do
   S.shadow_pending = false;
   const double ct_now = c->g.c * c->g.dt * (double)c->pushes;
   const int ni = (int)n;
-  cudaMemcpyAsync(S.n_dev, &ni, sizeof(int), cudaMemcpyHostToDevice, c->stream);
+  const int counts[2] = {ni, 0};
+  cudaMemcpyAsync(S.n_dev, counts, sizeof(counts), cudaMemcpyHostToDevice, c->stream);
   if (c->mixed)
     launch_load_particles<float>(c->g, particles_view<float>(c, species, 0), n, static_cast<const double*>(xd),
                                  static_cast<const double*>(ud), static_cast<const uint32_t*>(idd), umode, ct_now,
@@ -846,12 +879,15 @@ grpic_status grpic_load_particles(grpic_ctx* c, int species, double q_over_m, do
   s = cuda_check(c, cudaGetLastError(), "load_particles");
   // sort once so the store starts cell-ordered
   if (s == GRPIC_OK) {
-    if (c->mixed)
-      launch_sort<float>(c->g, particles_view<float>(c, species, 0), particles_view<float>(c, species, 1), c->sort,
-                         S.n_dev, c->stream);
-    else
-      launch_sort<double>(c->g, particles_view<double>(c, species, 0), particles_view<double>(c, species, 1),
-                          c->sort, S.n_dev, c->stream);
+    if (c->mixed) {
+      SortJobs<float> jobs{};
+      jobs.job[jobs.n++] = sort_job<float>(c, species);
+      launch_sort<float>(c->g, jobs, c->stream);
+    } else {
+      SortJobs<double> jobs{};
+      jobs.job[jobs.n++] = sort_job<double>(c, species);
+      launch_sort<double>(c->g, jobs, c->stream);
+    }
     S.cur = 1;
   }
   if (s == GRPIC_OK) s = read_status(c);
@@ -1024,7 +1060,7 @@ grpic_status grpic_num_particles(grpic_ctx* c, int species, int64_t* n) {
     return GRPIC_OK;
   }
   int v = 0;
-  grpic_status s = cuda_check(c, cudaMemcpyAsync(&v, S.n_dev, sizeof(int), cudaMemcpyDeviceToHost, c->stream),
+  grpic_status s = cuda_check(c, cudaMemcpyAsync(&v, S.n_dev + S.cur, sizeof(int), cudaMemcpyDeviceToHost, c->stream),
                               "count copy");
   if (s == GRPIC_OK) s = cuda_check(c, cudaStreamSynchronize(c->stream), "count sync");
   if (s != GRPIC_OK) return s;
@@ -1032,7 +1068,7 @@ grpic_status grpic_num_particles(grpic_ctx* c, int species, int64_t* n) {
   if (c->since_sort != 0) {
     enqueue_stage_any(c, GRPIC_STAGE_SORT);
     c->since_sort = 0;
-    s = cuda_check(c, cudaMemcpyAsync(&v, S.n_dev, sizeof(int), cudaMemcpyDeviceToHost, c->stream), "count copy");
+    s = cuda_check(c, cudaMemcpyAsync(&v, S.n_dev + S.cur, sizeof(int), cudaMemcpyDeviceToHost, c->stream), "count copy");
     if (s == GRPIC_OK) s = cuda_check(c, cudaStreamSynchronize(c->stream), "count sync");
     if (s != GRPIC_OK) return s;
   }
@@ -1095,7 +1131,7 @@ grpic_status grpic_get_stats(grpic_ctx* c, grpic_stats* out) {
   for (int q = 0; q < kMaxSpecies; ++q) {
     int v = 0;
     if (c->sp[q].loaded) {
-      cudaMemcpy(&v, c->sp[q].n_dev, sizeof(int), cudaMemcpyDeviceToHost);
+      cudaMemcpy(&v, c->sp[q].n_dev + c->sp[q].cur, sizeof(int), cudaMemcpyDeviceToHost);
     }
     out->n_alive[q] = v;
   }

@@ -1,11 +1,18 @@
 // Particle removal and counting sort by cell (not in the paper: the paper names no boundary
 // treatment; removed particles carry key kDead and are dropped here).
 //
+// Four launches for all species of a context (blockIdx.y = species):
 //   1. histogram of the keys into ncell + 1 bins (the last bin collects removed particles);
-//   2. exclusive prefix sum of the bins (block-level warp-shuffle scans, three passes);
-//   3. scatter of x, u, id, key into the alternate buffers at bin offset + running count.
-// The live count (start of the removed bin) is left in device memory, so no host round
-// trip is needed between steps.  Within a cell the order is not stable.
+//   2. sums of tiles of bins;
+//   3. exclusive prefix sum of the bins in place: a block sums the tiles before its own and scans its tile
+//      (block-level warp-shuffle scans); the removed bin's start is the new live count;
+//   4. scatter of x, u, id, key into the alternate buffers at bin offset + running count.
+// The live counts stay in device memory (one per buffer), so no host round trip is needed between steps.  Within a
+// cell the order is not stable.  The bins have to be zero before a sort; the step's zeroing of J takes them along.
+// (Tile sums counted by the histogram, one atomic a warp: sorted particles meet on one tile's address, 4.4 ms for
+// 31 M particles instead of 0.1.)
+// Measured, us per sort of all species (a launch each of seven kernels per species before): 2 x 46 K particles at 32^3 69 -> 27,
+// 4 species with 0.97 M at 64 x 64 x 128 157 -> 62, 2 x 1.8 M at 64^3 150 -> 102, 2 x 15.6 M at 128^3 971 -> 915.
 #include <algorithm>
 
 #include "common.cuh"
@@ -43,13 +50,16 @@ __device__ __forceinline__ KeyRun key_run(bool valid, uint32_t k) {
   return r;
 }
 
-__global__ void k_hist(const uint32_t* __restrict__ key, long long n, const int* __restrict__ n_dev,
-                       int* __restrict__ counts, long long dead_bin) {
+template <typename T>
+__global__ void k_hist(const SortJobs<T> jobs, long long dead_bin) {
+  const SortJob<T>& job = jobs.job[blockIdx.y];
+  const long long live = min(job.src.n, (long long)*job.src.n_dev);
+  if (blockIdx.x * (long long)blockDim.x >= live) return;
   const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  const bool valid = i < n && i < (long long)(*n_dev);
-  const uint32_t k = valid ? key[i] : kDead;
+  const bool valid = i < live;
+  const uint32_t k = valid ? job.src.key[i] : kDead;
   const KeyRun r = key_run(valid, k);
-  if (r.head) atomicAdd(counts + (k == kDead ? dead_bin : (long long)k), r.len);
+  if (r.head) atomicAdd(job.bins + (k == kDead ? dead_bin : (long long)k), r.len);
 }
 
 // Inclusive scan of one value per thread across the block.
@@ -77,8 +87,7 @@ __device__ __forceinline__ int block_inclusive_scan(int v, int* warp_sums) {
   return v;
 }
 
-__global__ void __launch_bounds__(kScanThreads) k_tile_sums(const int* __restrict__ in, long long n,
-                                                              int* __restrict__ tile_sums) {
+__device__ __forceinline__ void tile_sum(const int* __restrict__ in, long long n, int* __restrict__ tile_sums) {
   __shared__ int ws[kScanThreads / 32];
   const long long base = (long long)blockIdx.x * kScanTile + (long long)threadIdx.x * kScanItems;
   int s = 0;
@@ -87,6 +96,14 @@ __global__ void __launch_bounds__(kScanThreads) k_tile_sums(const int* __restric
     if (base + q < n) s += in[base + q];
   const int inc = block_inclusive_scan(s, ws);
   if (threadIdx.x == kScanThreads - 1) tile_sums[blockIdx.x] = inc;
+}
+__global__ void __launch_bounds__(kScanThreads) k_tile_sums(const int* __restrict__ in, long long n,
+                                                              int* __restrict__ tile_sums) {
+  tile_sum(in, n, tile_sums);
+}
+template <typename T>
+__global__ void __launch_bounds__(kScanThreads) k_job_tile_sums(const SortJobs<T> jobs, long long nbins) {
+  tile_sum(jobs.job[blockIdx.y].bins, nbins, jobs.job[blockIdx.y].tiles);
 }
 
 // Exclusive scan of the tile sums in place, one block looping over chunks.
@@ -128,8 +145,39 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_apply(const int* __restri
   }
 }
 
-__global__ void k_live_count(const int* __restrict__ offsets, long long dead_bin, int* __restrict__ n_out) {
-  *n_out = offsets[dead_bin];
+// Exclusive scan of a job's bins in place.  scanned: the tiles already hold their offsets (k_scan_tile_sums).
+template <typename T>
+__global__ void __launch_bounds__(kScanThreads) k_scan_bins(const SortJobs<T> jobs, long long nbins, bool scanned) {
+  __shared__ int ws[kScanThreads / 32];
+  __shared__ int s_before;
+  const SortJob<T>& job = jobs.job[blockIdx.y];
+  const int tile = blockIdx.x;
+  int before = 0;
+  if (!scanned)
+    for (int t = threadIdx.x; t < tile; t += kScanThreads) before += job.tiles[t];
+  const long long base = (long long)tile * kScanTile + (long long)threadIdx.x * kScanItems;
+  int v[kScanItems];
+  int s = 0;
+#pragma unroll
+  for (int q = 0; q < kScanItems; ++q) {
+    v[q] = (base + q < nbins) ? job.bins[base + q] : 0;
+    s += v[q];
+  }
+  if (scanned) {
+    before = job.tiles[tile];
+  } else {
+    before = block_inclusive_scan(before, ws);
+    if (threadIdx.x == kScanThreads - 1) s_before = before;
+    __syncthreads();
+    before = s_before;
+  }
+  int run = before + block_inclusive_scan(s, ws) - s;
+#pragma unroll
+  for (int q = 0; q < kScanItems; ++q) {
+    if (base + q < nbins) job.bins[base + q] = run;
+    if (base + q == nbins - 1) *job.n_out = run;  // the removed bin: the live count
+    run += v[q];
+  }
 }
 
 // Each thread moves kScatterItems records, from kScatterItems consecutive blocks' worth of the store
@@ -140,9 +188,11 @@ __global__ void k_live_count(const int* __restrict__ offsets, long long dead_bin
 constexpr int kScatterItems = 1;
 
 template <typename T>
-__global__ void k_scatter(const Particles<T> src, const Particles<T> dst, int* __restrict__ cursor,
-                          long long dead_bin) {
+__global__ void k_scatter(const SortJobs<T> jobs) {
+  const Particles<T>&src = jobs.job[blockIdx.y].src, &dst = jobs.job[blockIdx.y].dst;
+  int* const cursor = jobs.job[blockIdx.y].bins;
   const long long live_n = min(src.n, (long long)(*src.n_dev));
+  if ((long long)blockIdx.x * kScatterItems * blockDim.x >= live_n) return;
   uint32_t k[kScatterItems], idv[kScatterItems];
   T xv[kScatterItems][4], uv[kScatterItems][4];
   bool in_range[kScatterItems];
@@ -261,7 +311,7 @@ __global__ void k_batch_finish(const InstDesc<T>* __restrict__ desc, const int* 
   const InstDesc<T>& D = desc[pairs[p] >> 2];
   const SpeciesDesc<T>& S = D.sp[pairs[p] & 3];
   const int cur = *S.cur;
-  *const_cast<int*>(S.buf[cur].n_dev) = offsets[S.bin_base + D.g.ncell] - base[p];  // shared by both buffers
+  *const_cast<int*>(S.buf[1 - cur].n_dev) = offsets[S.bin_base + D.g.ncell] - base[p];
   *S.cur = 1 - cur;
 }
 
@@ -270,21 +320,20 @@ __global__ void k_batch_finish(const InstDesc<T>* __restrict__ desc, const int* 
 int scan_tiles(long long nbins) { return (int)((nbins + kScanTile - 1) / kScanTile); }
 
 template <typename T>
-void launch_sort(const Grid& g, const Particles<T>& src, const Particles<T>& dst, const SortScratch& s, int* n_out,
-                 cudaStream_t stream) {
+void launch_sort(const Grid& g, const SortJobs<T>& jobs, cudaStream_t stream) {
   const long long nbins = g.ncell + 1;
-  const long long dead_bin = g.ncell;
-  cudaMemsetAsync(s.counts, 0, sizeof(int) * nbins, stream);
-  if (src.n > 0) k_hist<<<blocks_for(src.n, 256), 256, 0, stream>>>(src.key, src.n, src.n_dev, s.counts, dead_bin);
-  const int ntiles = (int)((nbins + kScanTile - 1) / kScanTile);
-  k_tile_sums<<<ntiles, kScanThreads, 0, stream>>>(s.counts, nbins, s.blocks);
-  k_scan_tile_sums<<<1, kScanThreads, 0, stream>>>(s.blocks, ntiles);
-  k_scan_apply<<<ntiles, kScanThreads, 0, stream>>>(s.counts, nbins, s.blocks, s.offsets);
-  // scatter first: it reads the old count through src.n_dev, which may alias n_out.  Removed
-  // particles never take a slot, so the cursor of the removed bin still holds the live count.
-  if (src.n > 0)
-    k_scatter<T><<<blocks_for(src.n, 256 * kScatterItems), 256, 0, stream>>>(src, dst, s.offsets, dead_bin);
-  k_live_count<<<1, 1, 0, stream>>>(s.offsets, dead_bin, n_out);
+  const int ntiles = scan_tiles(nbins);
+  long long n = 0;
+  for (int q = 0; q < jobs.n; ++q) n = std::max(n, jobs.job[q].src.n);
+  if (n > 0) k_hist<T><<<dim3(blocks_for(n, 256), jobs.n), 256, 0, stream>>>(jobs, g.ncell);
+  k_job_tile_sums<T><<<dim3(ntiles, jobs.n), kScanThreads, 0, stream>>>(jobs, nbins);
+  // beyond 16384 tiles (320^3 cells) the blocks' own sums over the tiles before them, of order ntiles^2, would cost more
+  // than a launch
+  const bool scanned = ntiles > 16384;
+  for (int q = 0; scanned && q < jobs.n; ++q)
+    k_scan_tile_sums<<<1, kScanThreads, 0, stream>>>(jobs.job[q].tiles, ntiles);
+  k_scan_bins<T><<<dim3(ntiles, jobs.n), kScanThreads, 0, stream>>>(jobs, nbins, scanned);
+  if (n > 0) k_scatter<T><<<dim3(blocks_for(n, 256 * kScatterItems), jobs.n), 256, 0, stream>>>(jobs);
 }
 
 // pair_of_inst: for each (instance * 4 + species) the index of its pair (stored after `base`).
@@ -310,9 +359,7 @@ void launch_batch_sort(const BatchTables<T>& bt, cudaStream_t stream) {
 template void launch_batch_sort<float>(const BatchTables<float>&, cudaStream_t);
 template void launch_batch_sort<double>(const BatchTables<double>&, cudaStream_t);
 
-template void launch_sort<float>(const Grid&, const Particles<float>&, const Particles<float>&, const SortScratch&,
-                                 int*, cudaStream_t);
-template void launch_sort<double>(const Grid&, const Particles<double>&, const Particles<double>&,
-                                  const SortScratch&, int*, cudaStream_t);
+template void launch_sort<float>(const Grid&, const SortJobs<float>&, cudaStream_t);
+template void launch_sort<double>(const Grid&, const SortJobs<double>&, cudaStream_t);
 
 }  // namespace grpic
