@@ -56,6 +56,25 @@ __device__ __forceinline__ float narrow(double d) {
   return __uint_as_float(r);
 }
 
+// floor of x as an integer and in T.  FP64: from the bits (the FP64 pipe, which would also do the conversions, stays
+// free); negative, huge and non-finite x take the conversions.
+__device__ __forceinline__ void floor_split(float x, int& i, float& fl) {
+  i = (int)floorf(x);
+  fl = (float)i;
+}
+__device__ __forceinline__ void floor_split(double x, int& i, double& fl) {
+  const int hi = __double2hiint(x), e = (hi >> 20) - 1023;
+  if ((unsigned)hi < 0x41400000u) {  // 0 <= x < 2^21
+    const int drop = 20 - max(e, 0);
+    const int mask = e < 0 ? 0 : (int)(0xffffffffu << drop);
+    i = e < 0 ? 0 : ((hi & 0xfffff) | 0x100000) >> drop;
+    fl = __hiloint2double(hi & mask, 0);
+  } else {
+    i = (int)floor(x);
+    fl = (double)i;
+  }
+}
+
 // FP64 reciprocal, quotient and square root for evaluations whose results are rounded to FP32
 // afterwards (the FP32-mixed policy near the hole), where IEEE rounding of the last FP64 bit
 // buys nothing: an FP32 estimate (the approximate reciprocal / reciprocal square root, relative

@@ -157,24 +157,6 @@ __device__ __forceinline__ void christoffel_uu_x2(const Kerr<float>& K, float x,
   out[3] = -c1 + f * kw;
 }
 
-// floor of x as an integer and in T.  FP64: from the bits (the FP64 pipe, which would also do the conversions, stays
-// free); negative, huge and non-finite x take the conversions.
-__device__ __forceinline__ void floor_split(float x, int& i, float& fl) {
-  i = (int)floorf(x);
-  fl = (float)i;
-}
-__device__ __forceinline__ void floor_split(double x, int& i, double& fl) {
-  const int hi = __double2hiint(x), e = (hi >> 20) - 1023;
-  if ((unsigned)hi < 0x41400000u) {  // 0 <= x < 2^21
-    const int drop = 20 - max(e, 0);
-    const int mask = e < 0 ? 0 : (int)(0xffffffffu << drop);
-    i = e < 0 ? 0 : ((hi & 0xfffff) | 0x100000) >> drop;
-    fl = __hiloint2double(hi & mask, 0);
-  } else {
-    i = (int)floor(x);
-    fl = (double)i;
-  }
-}
 __device__ __forceinline__ bool finite_t(float v) { return isfinite(v); }
 __device__ __forceinline__ bool finite_t(double v) { return (__double2hiint(v) & 0x7ff00000) != 0x7ff00000; }
 // |v| < 1 (false for NaN)
