@@ -252,10 +252,16 @@ __device__ __noinline__ void metric_christoffel_fp64(const Consts<float>& C, flo
   out[7] = narrow(gd[3]);
 }
 
+// Node indices of the gathers and deposits (ncell < 2^31).  32 bits save address arithmetic: the push of 2 x 2.1 M particles at
+// 64^3 936 -> 917 us, at 75 x 50 x 91, Q = 3, 1108 -> 1085.  The kernels with area fits keep 64 (WIDE): with 32 their 96-register
+// build went from 5764 to 5966 us (2 x 16.8 M particles, 128^3).
+template <bool WIDE>
+using NodeIndex = std::conditional_t<WIDE, long long, int>;
+
 // a~ at (x, u): gather, convert, Lorentz - Christoffel.
 // MIXED: the FP32-mixed policy applies (T = float): where the FP32 r is below r_fp64 the metric
 // and the Christoffel contraction are taken from metric_christoffel_fp64.
-template <typename T, bool MIXED>
+template <typename T, bool MIXED, bool WIDE>
 __device__ __forceinline__ void accel(const Grid& g, const Fields<T>& F, const Consts<T>& C, const T x[3],
                                       const T u[4], T out[4], unsigned& flags, unsigned& n64) {
   // --- CIC gather: integer lattice (floor x) and half lattice (floor(x - 1/2)) per axis
@@ -289,7 +295,8 @@ __device__ __forceinline__ void accel(const Grid& g, const Fields<T>& F, const C
     wi[ax] = s0 - T(a0);
     wh[ax] = s1 - T(a1);
   }
-  const long long sy = g.nx, sz = (long long)g.nx * g.ny;
+  using Ix = NodeIndex<WIDE>;
+  const Ix sy = g.nx, sz = (Ix)g.nx * g.ny;
   T val[6];
 #pragma unroll
   for (int comp = 0; comp < 6; ++comp) {
@@ -300,7 +307,7 @@ __device__ __forceinline__ void accel(const Grid& g, const Fields<T>& F, const C
     const int i0 = hx ? ih[0] : ii[0], j0 = hy ? ih[1] : ii[1], k0 = hz ? ih[2] : ii[2];
     const T w0 = hx ? wh[0] : wi[0], w1 = hy ? wh[1] : wi[1], w2 = hz ? wh[2] : wi[2];
     const T* arr = comp < 3 ? F.d[comp] : F.b[comp - 3];
-    const T* q = arr + (((long long)k0 * g.ny + j0) * g.nx + i0);
+    const T* q = arr + (((Ix)k0 * g.ny + j0) * g.nx + i0);
     // trilinear as nested linear interpolations (the weight products expanded, 7 lerps)
     if constexpr (sizeof(T) == sizeof(float)) {
       // the lerps along x of the (z0, z1) pairs at y0 and at y1, then along y, as packed pairs;
@@ -672,7 +679,7 @@ __device__ __forceinline__ void table_areas(const float4* __restrict__ t, float 
 // FP64 face, row and column terms, like their FP32 counterparts.
 // (Marked nodes evaluated one at a time after the lattice, each a serial chain of FP64 and integer operations with a
 // warp's lanes out of step: 136 us instead of 114 for 46 K particles at 32^3, a quarter of them near; 128^3 2.95 -> 2.89 ms.)
-template <int Q, bool MIXED, bool TAB = false>
+template <int Q, bool MIXED, bool TAB, bool WIDE>
 __device__ __forceinline__ void deposit_lattice(const Grid& g, const Fields<float>& F, const Consts<float>& C,
                                                 const float x0[3], const float dx[3], float qg, float inv_dt,
                                                 unsigned& flags, unsigned& n64, const JTile& jt,
@@ -691,7 +698,8 @@ __device__ __forceinline__ void deposit_lattice(const Grid& g, const Fields<floa
     s1[ax] = (a == b) ? 0.5f * dx[ax] : (float)max(a, b) - x0[ax];
     s2[ax] = dx[ax] - s1[ax];
   }
-  const long long sy = g.nx, sz = (long long)g.nx * g.ny;
+  using Ix = NodeIndex<WIDE>;
+  const Ix sy = g.nx, sz = (Ix)g.nx * g.ny;
   const float cen[3] = {C.xc, C.yc, C.zc};
 #pragma unroll 1
   for (int seg = 0; seg < 2; ++seg) {
@@ -706,7 +714,7 @@ __device__ __forceinline__ void deposit_lattice(const Grid& g, const Fields<floa
       dseg[ax] = seg ? s2[ax] : s1[ax];
       fr[ax] = seg ? (x0[ax] - (float)c2[ax]) + (s1[ax] + 0.5f * s2[ax]) : (x0[ax] - (float)c1[ax]) + 0.5f * s1[ax];
     }
-    const long long base = ((long long)cz * g.ny + cy) * g.nx + cx;
+    const Ix base = ((Ix)cz * g.ny + cy) * g.nx + cx;
 #pragma unroll 1
     for (int K = 0; K < 3; ++K) {
       const float dK = sel3(K, dseg[0], dseg[1], dseg[2]);
@@ -715,7 +723,7 @@ __device__ __forceinline__ void deposit_lattice(const Grid& g, const Fields<floa
       const float frI = sel3(K, fr[1], fr[2], fr[0]), frJ = sel3(K, fr[2], fr[0], fr[1]);
       float A00, A10, A01, A11;  // sub-rectangle areas; a node's weight is the area opposite it
       if constexpr (TAB) {
-        table_areas(atab + base * kAreaTableStride + 5 * K, frI, frJ, sel3(K, fr[0], fr[1], fr[2]), A00, A10,
+        table_areas(atab + (long long)base * kAreaTableStride + 5 * K, frI, frJ, sel3(K, fr[0], fr[1], fr[2]), A00, A10,
                     A01, A11);
       } else {
         FaceLattice L;
@@ -878,7 +886,7 @@ __device__ __forceinline__ void deposit_lattice(const Grid& g, const Fields<floa
         atomicAdd(TK + tJ, flux * (A01 * rFA));
         atomicAdd(TK + tI + tJ, flux * (A11 * rFA));
       } else {
-        const long long stI = sel3(K, sy, sz, 1ll), stJ = sel3(K, sz, 1ll, sy);
+        const Ix stI = sel3(K, sy, sz, (Ix)1), stJ = sel3(K, sz, (Ix)1, sy);
         double* JK = sel3(K, F.J[0], F.J[1], F.J[2]);
         atomicAdd(JK + base, widen(flux * (A00 * rFA)));
         atomicAdd(JK + base + stI, widen(flux * (A10 * rFA)));
@@ -912,7 +920,7 @@ struct Move {
 };
 
 // One particle-step of particle i without its deposit (push_particle below, up to the deposit).
-template <typename T, bool MIXED>
+template <typename T, bool MIXED, bool WIDE>
 __device__ __forceinline__ Move<T> push_move(const Grid& g, const Fields<T>& F, const Particles<T>& P,
                                              const Consts<T>& C, long long i, DevStatus* st, unsigned& flags,
                                              unsigned& n64, uint32_t* key_out) {
@@ -930,7 +938,7 @@ __device__ __forceinline__ Move<T> push_move(const Grid& g, const Fields<T>& F, 
   bool fb = false;
 #pragma unroll 1
   for (int stage = 0; stage < 4; ++stage) {
-    accel<T, MIXED>(g, F, C, xs, us, a, flags, n64);
+    accel<T, MIXED, WIDE>(g, F, C, xs, us, a, flags, n64);
     if (stage == 0) {
       if constexpr (sizeof(T) == sizeof(double))
         h = C.dt * FastOps64::rcp(gamma_step<T, FastOps64>(us[3], a[3], C.inv_c, C.dt, &fb));
@@ -1033,12 +1041,12 @@ __device__ __forceinline__ Move<T> push_move(const Grid& g, const Fields<T>& F, 
 
 // The deposit of a move (Sec. 4).  TAB (far-field warps, T = float): face areas from the per-cell
 // fits atab.
-template <typename T, int Q, bool MIXED, bool TAB>
+template <typename T, int Q, bool MIXED, bool TAB, bool WIDE>
 __device__ __forceinline__ void deposit_move(const Grid& g, const Fields<T>& F, const Consts<T>& C, const Move<T>& mv,
                                              unsigned& flags, unsigned& n64, const JTile& jt, const float4* atab) {
   if (!mv.go) return;
   if constexpr (sizeof(T) == sizeof(float))
-    deposit_lattice<Q, MIXED, TAB>(g, F, C, mv.x0, mv.dx, mv.qg, C.inv_dt, flags, n64, jt, atab);
+    deposit_lattice<Q, MIXED, TAB, WIDE>(g, F, C, mv.x0, mv.dx, mv.qg, C.inv_dt, flags, n64, jt, atab);
   else
     deposit64<Q>(g, F, C, mv.x0, mv.dx, mv.qg, C.inv_dt, flags);
 }
@@ -1049,13 +1057,13 @@ __device__ __forceinline__ void deposit_move(const Grid& g, const Fields<T>& F, 
 // MIXED (T = float): the FP32-mixed policy applies to this warp's particles (false only where every particle lies
 // outside near_radius).
 // TAB (far-field warps, T = float): the deposit takes its face areas from the per-cell fits atab.
-template <typename T, int Q, bool MIXED, bool TAB = false>
+template <typename T, int Q, bool MIXED, bool TAB = false, bool WIDE = TAB>
 __device__ __forceinline__ void push_particle(const Grid& g, const Fields<T>& F, const Particles<T>& P,
                                               const Consts<T>& C, long long i, DevStatus* st, unsigned& flags,
                                               unsigned& n64, uint32_t* key_out, const JTile& jt = JTile(),
                                               const float4* atab = nullptr) {
-  const Move<T> mv = push_move<T, MIXED>(g, F, P, C, i, st, flags, n64, key_out);
-  deposit_move<T, Q, MIXED, TAB>(g, F, C, mv, flags, n64, jt, atab);
+  const Move<T> mv = push_move<T, MIXED, WIDE>(g, F, P, C, i, st, flags, n64, key_out);
+  deposit_move<T, Q, MIXED, TAB, WIDE>(g, F, C, mv, flags, n64, jt, atab);
 }
 
 // Warp-aggregated status: flags, FP64 evaluations and particle-steps of the warp's lanes.
