@@ -73,8 +73,8 @@ constexpr int kJTileFloats = 3072;
 template <int Q, int MINB, bool TILE, bool TAB, int THREADS>
 __global__ void __launch_bounds__(THREADS, MINB * (128 / THREADS))
     k_push_select(const Grid g, const Fields<float> F, const Particles<float> P, const Consts<float> C,
-                  float r_near2, unsigned perm, int lg, DevStatus* st, const float4* __restrict__ atab) {
-  const unsigned chunk = spread_chunk(blockIdx.x, gridDim.x, perm, lg);
+                  float r_near2, unsigned perm, int lg, unsigned tail, DevStatus* st, const float4* __restrict__ atab) {
+  const unsigned chunk = spread_chunk(blockIdx.x, gridDim.x, perm, lg, tail);
   const long long i = chunk * (long long)blockDim.x + threadIdx.x;
   unsigned flags = 0, n64 = 0;
   bool active = i < P.n && i < (long long)(*P.n_dev);
@@ -215,6 +215,14 @@ unsigned coprime_multiplier(unsigned n) {
   return m % n;
 }
 
+// A block near the hole takes several times as long as another, so one that starts late leaves the GPU idle but for its SM.
+// The last kTailWaves waves of a spread launch (152 SMs, as many blocks an SM as the kernel is compiled for), at most half of
+// it, take the chunks from both ends of the cell order, the farthest from the hole; the others go before them, permuted.
+// Push stage without / with, us: 2 x 46 K particles at 32^3 124 / 111, 2 x 2.1 M at 64^3 916 / 840, 2 x 1.6 M at 75 x 50 x 91,
+// Q = 3, 1087 / 945, 2 x 400 K + 2 x 85 K at 64 x 64 x 128 249 / 238, 2 x 16.8 M at 128^3 with fits 5765 / 5700.  4 waves give 860 and
+// 1004 for the second and third, 13 give 854 and 935.
+constexpr unsigned kTailWaves = 8;
+
 template <int Q, int MINB, bool TILE, bool TAB, int THREADS>
 void launch_select(const Grid& g, const Fields<float>& F, const Particles<float>& P, const Consts<float>& C,
                    int spread, DevStatus* st, const float4* atab, cudaStream_t stream) {
@@ -222,8 +230,9 @@ void launch_select(const Grid& g, const Fields<float>& F, const Particles<float>
   const unsigned nb = blocks_for(P.n, THREADS);
   // groups of `spread` chunks of 128 particles
   const int lg = spread > 0 ? spread_log2(spread * (128 / THREADS)) : 0;
-  const unsigned perm = spread > 0 ? spread_multiplier(nb, lg) : 1u;
-  k_push_select<Q, MINB, TILE, TAB, THREADS><<<nb, THREADS, 0, stream>>>(g, F, P, C, (float)(rn * rn), perm, lg, st,
+  const unsigned tail = spread > 0 ? std::min(kTailWaves * (152u * MINB * (128 / THREADS)) / 2 >> lg, (nb >> lg) / 4) : 0u;
+  const unsigned perm = spread > 0 ? spread_multiplier(nb, lg, tail) : 1u;
+  k_push_select<Q, MINB, TILE, TAB, THREADS><<<nb, THREADS, 0, stream>>>(g, F, P, C, (float)(rn * rn), perm, lg, tail, st,
                                                                          atab);
 }
 
