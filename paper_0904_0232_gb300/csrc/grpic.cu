@@ -234,9 +234,12 @@ void enqueue_rho(grpic_ctx* c, bool with_gamma, double* rho) {
 // The area fits the per-warp select push uses, or null.
 const float4* area_table_of(const grpic_ctx* c) { return c->tune.area_table ? c->atab : nullptr; }
 
-// One push launch per species, launch(species, stream).  Small launches (small_push) do not fill the GPU: where another
-// species is loaded they go to the side stream, ahead of and beside the others (all add into J atomically), and the context
-// stream waits for them.  The buffers belong to the context stream, which is joined before anything else uses them.
+// One push launch per species, launch(species, stream).  The smaller half of them go to the side stream, ahead of and beside
+// the others (all add into J atomically), and the context stream waits for them: small launches (small_push) do not fill the
+// GPU, and the blocks of one take the SMs that the last blocks of another leave idle.  The buffers belong to the context
+// stream, which is joined before anything else uses them.
+// Large ones beside each other, us per push stage: 2 x 2.1 M particles at 64^3 840 -> 831, 2 x 1.6 M at 75 x 50 x 91, Q = 3,
+// 927 -> 914, 2 x 16.8 M at 128^3 5715 -> 5705.
 template <typename Launch>
 void enqueue_species_pushes(grpic_ctx* c, Launch launch) {
   int order[kMaxSpecies], n = 0;
@@ -246,10 +249,7 @@ void enqueue_species_pushes(grpic_ctx* c, Launch launch) {
     order[n++] = s;
   }
   std::stable_sort(order, order + n, [c](int a, int b) { return c->sp[a].n < c->sp[b].n; });
-  // the smaller launches, but never all of them: two small ones run beside each other
-  int side = 0;
-  while (side < n - 1 && small_push(c->sp[order[side]].n)) ++side;
-  if (side == n - 1 && n > 2 && small_push(c->sp[order[n - 1]].n)) side = n / 2;
+  const int side = n / 2;
   if (side > 0) {
     cudaEventRecord(c->ev_fork, c->stream);
     cudaStreamWaitEvent(c->side, c->ev_fork, 0);
