@@ -243,10 +243,10 @@ __device__ __forceinline__ Kerr<S> kerr_eval(S x, S y, S z, S m, S a) {
 static __device__ __noinline__ double kerr_root_inside(double p, double q4, double D) {
   return halve(q4 * FastOps64::rcp(D - p));
 }
-__device__ __forceinline__ Kerr<double> kerr_eval_fast(double x, double y, double z, double m, double a) {
+__device__ __forceinline__ Kerr<double> kerr_eval_fast(double x, double y, double z, double two_m, double a, double a2,
+                                                       double a2_4) {
   Kerr<double> K;
-  const double a2 = a * a;
-  const double q4 = 4.0 * a2 * (z * z);
+  const double q4 = a2_4 * (z * z);
   const double p = fma(x, x, fma(y, y, fma(z, z, -a2)));
   const double D2 = fma(p, p, q4);
   K.inv_D = FastOps64::rsqrt(D2);
@@ -264,11 +264,15 @@ __device__ __forceinline__ Kerr<double> kerr_eval_fast(double x, double y, doubl
   K.r = r2 * K.inv_r;
   K.inv_rho2 = FastOps64::rcp(r2 + a2);
   K.inv_sig = K.inv_D * (K.inv_r * K.inv_r);
-  K.f = 2.0 * m * K.r * K.inv_D;
+  K.f = two_m * K.r * K.inv_D;
   K.k0 = fma(K.r, x, -(a * y)) * K.inv_rho2;
   K.k1 = fma(K.r, y, a * x) * K.inv_rho2;
   K.k2 = z * K.inv_r;
   return K;
+}
+__device__ __forceinline__ Kerr<double> kerr_eval_fast(double x, double y, double z, double m, double a) {
+  const double a2 = a * a;
+  return kerr_eval_fast(x, y, z, 2.0 * m, a, a2, 4.0 * a2);
 }
 
 // christoffel_uu (below) in FP64 without forming d_i k_j.  With u.r = u^i d_i r, k_x = (r x - a y) / rho^2 and so on,

@@ -117,18 +117,27 @@ __device__ __forceinline__ bool inside_horizon(const Grid& g, double X, double Y
   return K.flat || K.r <= g.r_plus;
 }
 
+// v > 0, normal and finite (from the bits)
+__device__ __forceinline__ bool normal_positive(double v) {
+  return (unsigned)__double2hiint(v) - 0x00100000u < 0x7fe00000u;
+}
+
 // Completion of u^a from its spatial part.  Covariant u_i (umode 1): g^mn u_m u_n = -c^2 with g^mn = eta^mn - f k^m k^n,
 // k^m = (k_i, -1), is (1 + f) u_4^2 - 2 f (k.u) u_4 - C = 0, C = |u|^2 - f (k.u)^2 + c^2; for its roots
 // u_4 = [f (k.u) -+ S] / (1 + f), S^2 = f^2 (k.u)^2 + (1 + f) C, u^4 = -u_4 + f (k.u - u_4) is +-S, so the
 // future-directed one has u^4 = S.  Contravariant u^i (umode 2): (1 - f) u4^2 - 2 f (k.u) u4 - C = 0 with
 // C = |u|^2 + f (k.u)^2 + c^2, u^4 = [f (k.u) + S] / (1 - f), S^2 = f^2 (k.u)^2 + (1 - f) C.
 // The load is bound by the FP64 pipe: one FP64 evaluation of the metric by FastOps64 and 20 operations a particle (two IEEE
-// evaluations and the two roots of each quadratic before: 5.1 ms for 15.6 M particles of an FP32-mixed context,
-// now 2.2 ms, 0.7 TB/s).
+// evaluations and the two roots of each quadratic before: 5.1 ms for 15.6 M particles of an FP32-mixed context; 2.2 ms with
+// the constants formed and the signs compared in FP64 as well; now 2.0 ms).
+// FP64 products of the grid's constants, formed once on the host.
+struct LoadConsts {
+  double two_m, a2, a2_4, c2;
+};
 template <typename T>
 __global__ void k_load(const Grid g, const Particles<T> P, long long n, const double* __restrict__ x4,
                        const double* __restrict__ u4, const uint32_t* __restrict__ ids, int umode, double ct_now,
-                       DevStatus* st) {
+                       const LoadConsts C, DevStatus* st) {
   const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (i >= n) return;
   const double x[3] = {x4[i], x4[n + i], x4[2 * n + i]};
@@ -140,7 +149,8 @@ __global__ void k_load(const Grid g, const Particles<T> P, long long n, const do
     double fl;
     floor_split(x[q], cell[q], fl);
     // x in [1, n - 2] (NaN fails both)
-    if (!(cell[q] >= 1 && (cell[q] < nn[q] - 2 || (cell[q] == nn[q] - 2 && x[q] == fl)))) bad |= ST_LOAD_INVALID;
+    const bool whole = __double_as_longlong(x[q]) == __double_as_longlong(fl);
+    if (!(cell[q] >= 1 && (cell[q] < nn[q] - 2 || (cell[q] == nn[q] - 2 && whole)))) bad |= ST_LOAD_INVALID;
     cell[q] = min(max(cell[q], 0), nn[q] - 2);
   }
   double u[4] = {u4[i], u4[n + i], u4[2 * n + i], umode == 0 ? u4[3 * n + i] : 0.0};
@@ -152,16 +162,16 @@ __global__ void k_load(const Grid g, const Particles<T> P, long long n, const do
     if (inside) atomicAdd(&st->removed_horizon, 1ull);
   }
   if (!bad && !inside && umode != 0) {
-    const Kerr<double> K = kerr_eval_fast(X, Y, Z, g.m, g.a);
+    const Kerr<double> K = kerr_eval_fast(X, Y, Z, C.two_m, g.a, C.a2, C.a2_4);
     const double f = K.f, kk[3] = {K.k0, K.k1, K.k2};
     const double ku = fma(kk[0], u[0], fma(kk[1], u[1], kk[2] * u[2]));
     const double fk = f * ku;
-    const double uu = fma(u[0], u[0], fma(u[1], u[1], fma(u[2], u[2], g.c * g.c)));
+    const double uu = fma(u[0], u[0], fma(u[1], u[1], fma(u[2], u[2], C.c2)));
     if (umode == 1) {
       const double A = 1.0 + f;
       const double S2 = fma(fk, fk, A * fma(-fk, ku, uu));
       const double S = FastOps64::root(S2);
-      if (!(S2 >= 0.0) || !(S > 0.0)) {
+      if (!normal_positive(S2)) {
         bad |= ST_LOAD_INVALID;
       } else {
         // raise: u^i = u_i - f k_i (k.u - u_4)
@@ -280,7 +290,8 @@ template <typename T>
 void launch_load_particles(const Grid& g, const Particles<T>& P, long long n, const double* x4, const double* u4,
                            const uint32_t* ids, int umode, double ct_now, DevStatus* st, cudaStream_t stream) {
   if (n <= 0) return;
-  k_load<T><<<blocks_for(n, 256), 256, 0, stream>>>(g, P, n, x4, u4, ids, umode, ct_now, st);
+  k_load<T><<<blocks_for(n, 256), 256, 0, stream>>>(g, P, n, x4, u4, ids, umode, ct_now,
+                                              LoadConsts{2.0 * g.m, g.a * g.a, 4.0 * (g.a * g.a), g.c * g.c}, st);
 }
 
 template <typename T>
