@@ -302,12 +302,13 @@ unsigned coprime_multiplier(unsigned n);
 // Block -> work-chunk map of the push launches: groups of 2^lg consecutive chunks are permuted,
 // group g -> g * perm mod (number of full groups), perm coprime to that number (1 keeps the order;
 // a partial last group stays in place).  With `tail` groups at either end set apart, the others are permuted among
-// themselves and go first, the lower end's and the upper end's after them.  Cell-sorted particles put the FP64-heavy chunks near the
+// themselves and go first, the lower end's and the upper end's after them.  perm = 0: from the middle outwards.  Cell-sorted particles put the FP64-heavy chunks near the
 // hole in one contiguous run; the permutation spreads them over the whole launch, so the FP64
 // pipes of all SMs share that work alongside FP32 work, while the blocks of a group, which run at
 // about the same time, keep neighbouring cells together (their field stencils and J nodes stay in
 // L2).  Larger groups favour that locality, smaller ones the spreading of FP64 work.
 __device__ __forceinline__ unsigned spread_chunk(unsigned b, unsigned n, unsigned perm, int lg, unsigned tail = 0) {
+  if (perm == 0u) return b & 1u ? (n - 1) / 2 + (b + 1) / 2 : (n - 1) / 2 - b / 2;
   const unsigned nfull = n >> lg;
   if (perm == 1u || b >= (nfull << lg)) return b;
   const unsigned mask = (1u << lg) - 1u, main = nfull - 2 * tail, i = b >> lg;
@@ -330,7 +331,7 @@ inline int spread_log2(int group) {
 // over the SMs, and another species' launch runs beside it (grpic.cu).  Larger launches keep blocks of four warps, whose
 // common cells stay in L1.
 // Measured, us per push stage, 128-thread blocks one after another / small launches as here: 2 x 46 K particles at 32^3
-// 228 / 111 (FP64 695 / 603), 2 x 400 K + 2 x 85 K at 64 x 64 x 128 380 / 238; blocks of one warp for 2 x 0.9 M
+// 228 / 105 (FP64 695 / 603), 2 x 400 K + 2 x 85 K at 64 x 64 x 128 380 / 238; blocks of one warp for 2 x 0.9 M
 // particles at 64^3 cost 1142 instead of 941.
 constexpr long long kSmallPush = 311296;  // 4 waves of 128-thread blocks at 4 an SM
 inline bool small_push(long long n) { return n <= kSmallPush; }
