@@ -254,8 +254,8 @@ void launch_push_select(const Grid& g, const Fields<float>& F, const Particles<f
   else if (small)
     tab ? launch_select<2, 4, false, true, 32>(g, F, P, C, spread, st, atab, stream)
         : launch_select<2, 4, false, false, 32>(g, F, P, C, spread, st, nullptr, stream);
-  else if (tab)  // 80 registers for 5 and 6 blocks: 5641 us against 5712 with 96 (2 x 16.8 M particles, 128^3); 128 give 6055
-    minb >= 5 ? launch_select<2, 6, false, true, 128>(g, F, P, C, spread, st, atab, stream)
+  else if (tab)
+    minb >= 5 ? launch_select<2, 5, false, true, 128>(g, F, P, C, spread, st, atab, stream)
               : launch_select<2, 4, false, true, 128>(g, F, P, C, spread, st, atab, stream);
   else if (tile)
     minb >= 5 ? launch_select<2, 5, true, false, 128>(g, F, P, C, spread, st, nullptr, stream)
