@@ -679,7 +679,13 @@ __device__ __forceinline__ void table_areas(const float4* __restrict__ t, float 
 // FP64 face, row and column terms, like their FP32 counterparts.
 // (Marked nodes evaluated one at a time after the lattice, each a serial chain of FP64 and integer operations with a
 // warp's lanes out of step: 136 us instead of 114 for 46 K particles at 32^3, a quarter of them near; 128^3 2.95 -> 2.89 ms.)
-template <int Q, bool MIXED, bool TAB, bool WIDE>
+// ROWS: rows of the lattice in flight (1 or 2).  FP32-mixed code takes 1: its rows carry the corrections, and with two of them
+// unrolled the far and the FP32-mixed copies of a kernel no longer fit the instruction cache together (no_instruction 2.1
+// cycles per issue, with one row 0.9 before the corrections moved into the rows).  Push stage 2 -> 1: 2 x 2.1 M particles at
+// 64^3 834 -> 791 us, 2 x 1.6 M at 75 x 50 x 91, Q = 3, 918 -> 870, 2 x 15.6 M at 128^3 with fits over steps 4-203 6.75 ->
+// 6.59 ms.  A far-field lattice with 1 loses its overlap (822 and 937 us), and so do the near warps of small launches (2 x 46 K
+// particles at 32^3: 104 -> 107).
+template <int Q, bool MIXED, bool TAB, bool WIDE, int ROWS>
 __device__ __forceinline__ void deposit_lattice(const Grid& g, const Fields<float>& F, const Consts<float>& C,
                                                 const float x0[3], const float dx[3], float qg, float inv_dt,
                                                 unsigned& flags, unsigned& n64, const JTile& jt,
@@ -789,7 +795,7 @@ __device__ __forceinline__ void deposit_lattice(const Grid& g, const Fields<floa
   #pragma unroll
           for (int t = 1; t < Q; ++t)
             if (pi == t) gw = (float)Gauss<Q>::w(t);
-  #pragma unroll
+  #pragma unroll ROWS
           for (int si = 0; si < 2; ++si) {
             float pRow, qRow, tRow;
             const float AIa = row_coord<Q>(L, si, pi);
@@ -848,13 +854,18 @@ __device__ __forceinline__ void deposit_lattice(const Grid& g, const Fields<floa
                 if (!(r2.y > 0.f)) v.y = 1.f;
               }
               const float2 rv = rsqrt2(v);
+              float2 sum = si ? acc[1][k] : acc[0][k];
               if (Q == 2) {
-                acc[si][k] = fma2(v, rv, acc[si][k]);  // unit Gauss weights
+                sum = fma2(v, rv, sum);  // unit Gauss weights
               } else {
                 const float2 w = make_float2(gw * (float)Gauss<Q>::w((2 * k) % Q),
                                              gw * (float)Gauss<Q>::w((2 * k + 1) % Q));
-                acc[si][k] = fma2(w, mul2(v, rv), acc[si][k]);
+                sum = fma2(w, mul2(v, rv), sum);
               }
+              if (si)
+                acc[1][k] = sum;
+              else
+                acc[0][k] = sum;
             }
           }
         }
@@ -1041,12 +1052,12 @@ __device__ __forceinline__ Move<T> push_move(const Grid& g, const Fields<T>& F, 
 
 // The deposit of a move (Sec. 4).  TAB (far-field warps, T = float): face areas from the per-cell
 // fits atab.
-template <typename T, int Q, bool MIXED, bool TAB, bool WIDE>
+template <typename T, int Q, bool MIXED, bool TAB, bool WIDE, int ROWS>
 __device__ __forceinline__ void deposit_move(const Grid& g, const Fields<T>& F, const Consts<T>& C, const Move<T>& mv,
                                              unsigned& flags, unsigned& n64, const JTile& jt, const float4* atab) {
   if (!mv.go) return;
   if constexpr (sizeof(T) == sizeof(float))
-    deposit_lattice<Q, MIXED, TAB, WIDE>(g, F, C, mv.x0, mv.dx, mv.qg, C.inv_dt, flags, n64, jt, atab);
+    deposit_lattice<Q, MIXED, TAB, WIDE, ROWS>(g, F, C, mv.x0, mv.dx, mv.qg, C.inv_dt, flags, n64, jt, atab);
   else
     deposit64<Q>(g, F, C, mv.x0, mv.dx, mv.qg, C.inv_dt, flags);
 }
@@ -1057,13 +1068,13 @@ __device__ __forceinline__ void deposit_move(const Grid& g, const Fields<T>& F, 
 // MIXED (T = float): the FP32-mixed policy applies to this warp's particles (false only where every particle lies
 // outside near_radius).
 // TAB (far-field warps, T = float): the deposit takes its face areas from the per-cell fits atab.
-template <typename T, int Q, bool MIXED, bool TAB = false, bool WIDE = TAB>
+template <typename T, int Q, bool MIXED, bool TAB = false, bool WIDE = TAB, int ROWS = MIXED ? 1 : 2>
 __device__ __forceinline__ void push_particle(const Grid& g, const Fields<T>& F, const Particles<T>& P,
                                               const Consts<T>& C, long long i, DevStatus* st, unsigned& flags,
                                               unsigned& n64, uint32_t* key_out, const JTile& jt = JTile(),
                                               const float4* atab = nullptr) {
   const Move<T> mv = push_move<T, MIXED, WIDE>(g, F, P, C, i, st, flags, n64, key_out);
-  deposit_move<T, Q, MIXED, TAB, WIDE>(g, F, C, mv, flags, n64, jt, atab);
+  deposit_move<T, Q, MIXED, TAB, WIDE, ROWS>(g, F, C, mv, flags, n64, jt, atab);
 }
 
 // Warp-aggregated status: flags, FP64 evaluations and particle-steps of the warp's lanes.

@@ -132,7 +132,8 @@ __global__ void __launch_bounds__(THREADS, MINB * (128 / THREADS))
   // two inlined copies, each with the flag a constant: the far-field copy has no out-of-line
   // calls at all (a call site in the loop would cost every warp registers and stack traffic)
   if (__any_sync(0xffffffffu, near)) {
-    if (active) push_particle<float, Q, true, false, TAB>(g, F, P, C, i, st, flags, n64, P.key + i, jt);
+    if (active)
+      push_particle<float, Q, true, false, TAB, THREADS == 32 ? 2 : 1>(g, F, P, C, i, st, flags, n64, P.key + i, jt);
   } else if constexpr (TAB) {
     if (active) {
       // the fits of x_n's cell (the deposit's first segment) into L2 now, read after the RK4 stages
