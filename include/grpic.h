@@ -303,7 +303,8 @@ grpic_status grpic_gauss_residual(grpic_ctx* ctx, double* res, int mem, double* 
  *   spread:             split = 0: G = 1, 2, 4, ... 64 maps blocks to particle chunks by a permutation of
  *                       groups of G consecutive chunks, spreading the near-hole (FP64-heavy) chunks over
  *                       the launch while each group keeps neighbouring cells together (larger G: more
- *                       L2 locality, less even FP64 load); 0 keeps them in order
+ *                       L2 locality, less even FP64 load), the chunks of both ends of the cell order last;
+ *                       small launches go from the middle of the cell order outwards; 0 keeps them in order
  *   area_table:         split = 0, Q = 2, j_tile = 0 (with j_tile = 1 refused), FP32_MIXED (FP64 contexts
  *                       keep it and ignore it, like the other push shapes): 1 takes the face AREAs of Eq. 18
  *                       for far-field warps from per-cell polynomial fits of the integrand instead of
