@@ -389,9 +389,11 @@ typedef struct grpic_batch grpic_batch;
  * is captured once in a CUDA graph on a stream the batch owns (`stream` is unused).  The
  * contexts stay owned by the caller and must outlive every grpic_batch_step and
  * grpic_batch_info of the batch; grpic_batch_destroy touches none of them (the batch keeps its own
- * copy of the first context's allocator).  The batch is built for the particle counts loaded at
- * creation (re-create it after loading more).  Every batched step sorts.  Returns
- * GRPIC_ERR_INVALID for mismatched contexts. */
+ * copy of the first context's allocator).  The batch is built for the species and particle counts
+ * loaded at creation (re-create it after loading more: grpic_batch_step then returns
+ * GRPIC_ERR_INVALID); within them a context may be reloaded with other particles, charges and masses,
+ * retuned or stepped on its own between batched steps, each of which takes it as it stands.  Every
+ * batched step sorts.  Returns GRPIC_ERR_INVALID for mismatched contexts. */
 grpic_status grpic_batch_create(grpic_ctx* const* ctxs, int n, void* stream, grpic_batch** out);
 
 /* Advance every instance nsteps timesteps (graph replays), ordered after each context's pending

@@ -1324,6 +1324,44 @@ grpic_status grpic_get_profile(grpic_ctx* c, double times_ms[6], int64_t counts[
 }  // extern "C"
 
 // ---- batched engine ----------------------------------------------------------------------------
+namespace {
+
+// What a batch's tables and graphs hold of one context.
+struct BatchHeld {
+  struct Store {
+    bool loaded;
+    void* buf[2];
+    long long cap;
+    double qm, qmacro;
+    bool operator==(const Store& o) const {
+      return loaded == o.loaded && buf[0] == o.buf[0] && buf[1] == o.buf[1] && cap == o.cap && qm == o.qm &&
+             qmacro == o.qmacro;
+    }
+  } sp[kMaxSpecies];
+  int bcur, far_min_blocks, spread;
+  const void* atab;
+  bool operator==(const BatchHeld& o) const {
+    for (int s = 0; s < kMaxSpecies; ++s)
+      if (!(sp[s] == o.sp[s])) return false;
+    return bcur == o.bcur && far_min_blocks == o.far_min_blocks && spread == o.spread && atab == o.atab;
+  }
+};
+
+BatchHeld batch_held(const grpic_ctx* c) {
+  BatchHeld h{};
+  for (int s = 0; s < kMaxSpecies; ++s) {
+    const SpeciesStore& S = c->sp[s];
+    h.sp[s] = BatchHeld::Store{S.loaded, {S.buf[0], S.buf[1]}, S.cap, S.qm, S.qmacro};
+  }
+  h.bcur = c->bcur;
+  h.far_min_blocks = c->tune.far_min_blocks;
+  h.spread = c->tune.spread;
+  h.atab = area_table_of(c);
+  return h;
+}
+
+}  // namespace
+
 struct grpic_batch {
   std::vector<grpic_ctx*> ctxs;
   // the batch's own copy of the device allocator (its tables must be freed with it even after
@@ -1345,7 +1383,14 @@ struct grpic_batch {
   int npairs = 0;
   int persist_blocks = 0;
   int sms = 1;
-  std::vector<long long> pair_n;  // work upper bound of each pair when the batch was built
+  std::vector<TileGrid> tiles_of;  // field patches of each instance
+  // pair of each (instance, species), -1 where nothing was loaded when the batch was built, and the pairs' work upper bound
+  std::vector<int> pair_of;
+  std::vector<long long> pair_n;
+  // what the tables and graphs hold of the contexts (a context may be reloaded, retuned or stepped on its own between
+  // batched steps), and the particle bounds of the captured push launches, 4 an instance
+  std::vector<BatchHeld> held;
+  std::vector<long long> captured_n;
   // One captured step per step parity k: every step flips each particle store (the sort) and each d
   // buffer (the E step), so replaying graph[k] when each context's (store, d) parity equals its
   // parity at capture XOR k lets the FP32 push run as the single-context kernel per (instance,
@@ -1408,34 +1453,22 @@ void append_blocks(std::vector<BlockEntry>& v, int inst, long long items, int bs
   for (long long q = 0; q < nb; ++q) v.push_back(BlockEntry{inst, (int)q});
 }
 
+// The descriptors of the instances as their contexts stand.
 template <typename T>
-grpic_status batch_build(grpic_batch* b) {
+std::vector<InstDesc<T>> batch_descs(grpic_batch* b) {
   const int n = (int)b->ctxs.size();
   std::vector<InstDesc<T>> desc(n);
-  std::vector<BlockEntry> tile, all, part;
-  std::vector<int> pairs, cur_init, dcur_init(n, 0);
-  std::vector<long long> bin_base;
-  long long nbins = 0;
-  // device ping-pong indices: one int per (instance, species)
-  b->cur = static_cast<int*>(batch_alloc(b, sizeof(int) * 4 * n));
-  if (!b->cur) return GRPIC_ERR_OOM;
-  b->dcur = static_cast<int*>(batch_alloc(b, sizeof(int) * n));
-  if (!b->dcur) return GRPIC_ERR_OOM;
-  cur_init.assign(4 * n, 0);
-  std::vector<const Grid*> grids(n);
-  std::vector<TileGrid> tiles(n);
-  for (int i = 0; i < n; ++i) grids[i] = &b->ctxs[i]->g;
-  batch_field_tiles(grids.data(), n, sizeof(T), b->sms, tiles.data());
+  long long bin_base = 0;
   for (int i = 0; i < n; ++i) {
     grpic_ctx* c = b->ctxs[i];
     InstDesc<T>& D = desc[i];
     D.g = c->g;
     D.K32 = field_consts<float>(c->g);
     D.K64 = field_consts<double>(c->g);
-    // b[0]: the context's current b (b^{n-1/2} at a step boundary), b[1]: the other buffer
+    // a step reads d from the device-selected parity and writes the other; it writes b^n to the
+    // other b buffer and returns to the current one (so b needs no parity)
     for (int q = 0; q < 3; ++q) {
-      D.FS.d[0][q] = field_plane<T>(c, false, 0, q);
-      D.FS.d[1][q] = field_plane<T>(c, false, 1, q);
+      for (int w = 0; w < 2; ++w) D.FS.d[w][q] = field_plane<T>(c, false, w, q);
       D.FS.b[0][q] = field_plane<T>(c, true, c->bcur, q);
       D.FS.b[1][q] = field_plane<T>(c, true, 1 - c->bcur, q);
       D.FS.J[q] = c->J + (size_t)q * c->g.ncell;
@@ -1444,34 +1477,67 @@ grpic_status batch_build(grpic_batch* b) {
     D.FS.kin = static_cast<const T*>(c->kin);
     D.FS.loc = c->loc;
     D.FS.met = c->met;
-    c->met_held = true;
     D.dcur = b->dcur + i;
-    dcur_init[i] = c->dcur;
     D.st = c->st;
-    const Grid& g = c->g;
-    D.tiles = tiles[i];
-    for (long long q = 0; q < D.tiles.count(); ++q) tile.push_back(BlockEntry{i, (int)q});
-    append_blocks(all, i, g.ncell, 256);
+    D.tiles = b->tiles_of[i];
     for (int s = 0; s < kMaxSpecies; ++s) {
       SpeciesStore& S = c->sp[s];
       SpeciesDesc<T>& SD = D.sp[s];
-      SD.active = S.loaded ? 1 : 0;
+      SD.active = b->pair_of[4 * i + s] >= 0 ? 1 : 0;
       SD.qm = S.qm;
       SD.qmacro = S.qmacro;
-      SD.C = make_consts<T>(g, Species{S.qm, S.qmacro});
+      SD.C = make_consts<T>(c->g, Species{S.qm, S.qmacro});
       SD.cur = b->cur + 4 * i + s;
       SD.bin_base = 0;
-      if (!S.loaded) continue;
+      if (!SD.active) continue;
       SD.buf[0] = particles_view<T>(c, s, 0);
       SD.buf[1] = particles_view<T>(c, s, 1);
-      SD.bin_base = nbins;
-      nbins += g.ncell + 1;
+      // (the bound of the tables: the live count on the device decides)
+      SD.buf[0].n = SD.buf[1].n = S.loaded ? b->pair_n[b->pair_of[4 * i + s]] : 0;
+      SD.bin_base = bin_base;
+      bin_base += c->g.ncell + 1;
+    }
+  }
+  b->held.resize(n);
+  for (int i = 0; i < n; ++i) b->held[i] = batch_held(b->ctxs[i]);
+  return desc;
+}
+
+template <typename T>
+grpic_status batch_build(grpic_batch* b) {
+  const int n = (int)b->ctxs.size();
+  std::vector<BlockEntry> tile, all, part;
+  std::vector<int> pairs, cur_init, dcur_init(n, 0);
+  long long nbins = 0;
+  // device ping-pong indices: one int per (instance, species)
+  b->cur = static_cast<int*>(batch_alloc(b, sizeof(int) * 4 * n));
+  if (!b->cur) return GRPIC_ERR_OOM;
+  b->dcur = static_cast<int*>(batch_alloc(b, sizeof(int) * n));
+  if (!b->dcur) return GRPIC_ERR_OOM;
+  cur_init.assign(4 * n, 0);
+  std::vector<const Grid*> grids(n);
+  b->tiles_of.resize(n);
+  for (int i = 0; i < n; ++i) grids[i] = &b->ctxs[i]->g;
+  batch_field_tiles(grids.data(), n, sizeof(T), b->sms, b->tiles_of.data());
+  b->pair_of.assign(4 * n, -1);
+  for (int i = 0; i < n; ++i) {
+    grpic_ctx* c = b->ctxs[i];
+    c->met_held = true;
+    dcur_init[i] = c->dcur;
+    for (long long q = 0; q < b->tiles_of[i].count(); ++q) tile.push_back(BlockEntry{i, (int)q});
+    append_blocks(all, i, c->g.ncell, 256);
+    for (int s = 0; s < kMaxSpecies; ++s) {
+      const SpeciesStore& S = c->sp[s];
+      if (!S.loaded) continue;
+      nbins += c->g.ncell + 1;
       cur_init[4 * i + s] = S.cur;
+      b->pair_of[4 * i + s] = (int)pairs.size();
       pairs.push_back(4 * i + s);
       b->pair_n.push_back(S.n);
       append_blocks(part, 4 * i + s, S.n, 128);
     }
   }
+  const std::vector<InstDesc<T>> desc = batch_descs<T>(b);
   b->npairs = (int)pairs.size();
   b->nbins = std::max<long long>(nbins, 1);
   b->ntile = (int)tile.size();
@@ -1503,6 +1569,34 @@ grpic_status batch_build(grpic_batch* b) {
   cudaMemcpyAsync(b->pair_base + b->npairs, pair_of_inst.data(), sizeof(int) * 4 * n, cudaMemcpyHostToDevice, st);
   cudaMemcpyAsync(b->cur, cur_init.data(), sizeof(int) * 4 * n, cudaMemcpyHostToDevice, st);
   return cudaStreamSynchronize(st) == cudaSuccess ? GRPIC_OK : GRPIC_ERR_CUDA;
+}
+
+void batch_drop_graphs(grpic_batch* b) {
+  for (int kk = 0; kk < 2; ++kk)
+    if (b->graph[kk]) {
+      cudaGraphExecDestroy(b->graph[kk]);
+      b->graph[kk] = nullptr;
+    }
+}
+
+// Bring the descriptors in line with contexts that were reloaded or retuned since, and drop graphs whose push launches
+// hold other values or smaller bounds than the contexts now have.
+template <typename T>
+grpic_status batch_refresh(grpic_batch* b) {
+  bool same = true, fits = true;
+  for (size_t i = 0; i < b->ctxs.size(); ++i) {
+    same = same && batch_held(b->ctxs[i]) == b->held[i];
+    for (int s = 0; s < kMaxSpecies && !b->captured_n.empty(); ++s)
+      fits = fits && b->ctxs[i]->sp[s].n <= b->captured_n[4 * i + s];
+  }
+  if (!same || !fits) {
+    if (cudaStreamSynchronize(b->stream) != cudaSuccess) return GRPIC_ERR_CUDA;
+    batch_drop_graphs(b);
+  }
+  if (same) return GRPIC_OK;
+  const std::vector<InstDesc<T>> desc = batch_descs<T>(b);
+  cudaMemcpyAsync(b->desc, desc.data(), sizeof(InstDesc<T>) * desc.size(), cudaMemcpyHostToDevice, b->stream);
+  return cudaStreamSynchronize(b->stream) == cudaSuccess ? GRPIC_OK : GRPIC_ERR_CUDA;
 }
 
 // The FP32-mixed push of a batched step at step parity k (see grpic_batch): per (instance,
@@ -1617,11 +1711,15 @@ grpic_status grpic_batch_create(grpic_ctx* const* ctxs, int n, void* stream, grp
 
 grpic_status grpic_batch_step(grpic_batch* b, int nsteps) {
   if (!b || nsteps < 0) return GRPIC_ERR_INVALID;
-  // the batch was built for the particle counts of its creation
-  size_t p = 0;
-  for (grpic_ctx* c : b->ctxs)
-    for (int s = 0; s < kMaxSpecies; ++s)
-      if (c->sp[s].loaded && (p >= b->pair_n.size() || c->sp[s].n > b->pair_n[p++])) return GRPIC_ERR_INVALID;
+  // the batch was built for the species and particle counts of its creation
+  for (size_t i = 0; i < b->ctxs.size(); ++i)
+    for (int s = 0; s < kMaxSpecies; ++s) {
+      const int p = b->pair_of[4 * i + s];
+      const SpeciesStore& S = b->ctxs[i]->sp[s];
+      if (S.loaded && (p < 0 || S.n > b->pair_n[p])) return GRPIC_ERR_INVALID;
+    }
+  const grpic_status fresh = b->mixed ? batch_refresh<float>(b) : batch_refresh<double>(b);
+  if (fresh != GRPIC_OK) return fresh;
   // order after each context's pending work; refresh the device ping-pong indices
   std::vector<int> cur(4 * b->ctxs.size(), 0);
   for (size_t i = 0; i < b->ctxs.size(); ++i) {
@@ -1649,13 +1747,11 @@ grpic_status grpic_batch_step(grpic_batch* b, int nsteps) {
     }
   }
   if (k < 0) {
-    for (int kk = 0; kk < 2; ++kk)
-      if (b->graph[kk]) {
-        cudaGraphExecDestroy(b->graph[kk]);
-        b->graph[kk] = nullptr;
-      }
+    batch_drop_graphs(b);
     b->cur0 = cur;
     b->dcur0 = dpar;
+    b->captured_n.resize(cur.size());
+    for (size_t q = 0; q < cur.size(); ++q) b->captured_n[q] = b->ctxs[q / 4]->sp[q % 4].n;
     for (int kk = 0; kk < 2; ++kk) {
       cudaGraph_t graph = nullptr;
       if (cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return GRPIC_ERR_CUDA;
@@ -1705,11 +1801,7 @@ grpic_status grpic_batch_set_blocks_per_sm(grpic_batch* b, int blocks_per_sm) {
   if (b->persist_blocks == b->sms * blocks_per_sm) return GRPIC_OK;
   if (b->stream) cudaStreamSynchronize(b->stream);
   b->persist_blocks = b->sms * blocks_per_sm;
-  for (int kk = 0; kk < 2; ++kk)
-    if (b->graph[kk]) {
-      cudaGraphExecDestroy(b->graph[kk]);
-      b->graph[kk] = nullptr;  // re-captured with the new grid by the next grpic_batch_step
-    }
+  batch_drop_graphs(b);  // captured with the new grid by the next grpic_batch_step
   return GRPIC_OK;
 }
 
@@ -1723,8 +1815,7 @@ grpic_status grpic_batch_info(grpic_batch* b, int64_t* kernels_per_step, int64_t
 grpic_status grpic_batch_destroy(grpic_batch* b) {
   if (!b) return GRPIC_ERR_INVALID;
   if (b->stream) cudaStreamSynchronize(b->stream);
-  for (int kk = 0; kk < 2; ++kk)
-    if (b->graph[kk]) cudaGraphExecDestroy(b->graph[kk]);
+  batch_drop_graphs(b);
   for (void* p : b->allocs) batch_free(b, p);
   if (b->ev) cudaEventDestroy(b->ev);
   if (b->ev_fork) cudaEventDestroy(b->ev_fork);
