@@ -538,20 +538,32 @@ grpic_status read_status(grpic_ctx* c) {
   return GRPIC_OK;
 }
 
+// Room for n particles.  Where the stores have to grow, what was loaded goes with them: the species counts as not loaded
+// until the load that asked for them has filled the new ones, so that nothing runs on them should that load fail.
 grpic_status ensure_capacity(grpic_ctx* c, int s, long long n) {
   SpeciesStore& S = c->sp[s];
   long long want = std::max<long long>(n, c->cfg.max_particles);
   if (c->cfg.max_particles > 0 && n > c->cfg.max_particles)
     return fail(c, GRPIC_ERR_CAPACITY, "more particles than max_particles");
   if (S.cap >= want && S.buf[0]) return GRPIC_OK;
-  for (int b = 0; b < 2; ++b) {
-    dev_free(c, S.buf[b]);
-    S.buf[b] = nullptr;
-  }
+  auto drop = [c, &S] {
+    for (int b = 0; b < 2; ++b) {
+      dev_free(c, S.buf[b]);
+      S.buf[b] = nullptr;
+    }
+    S.cap = 0;
+  };
+  S.loaded = false;
+  S.n = 0;
+  S.shadow_pending = false;
+  drop();
   const size_t bytes = (size_t)std::max<long long>(want, 1) * particle_bytes(c);
   for (int b = 0; b < 2; ++b) {
     S.buf[b] = dev_alloc(c, bytes);
-    if (!S.buf[b]) return fail(c, GRPIC_ERR_OOM, "particle store allocation failed");
+    if (!S.buf[b]) {
+      drop();
+      return fail(c, GRPIC_ERR_OOM, "particle store allocation failed");
+    }
   }
   S.cap = std::max<long long>(want, 1);
   return GRPIC_OK;
