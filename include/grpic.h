@@ -153,6 +153,12 @@ typedef struct grpic_ctx grpic_ctx;
 /* Create a context on the current CUDA device.  Validates the configuration (Courant:
  * c dt < 1/sqrt(3), Sec. 5), computes r_+ = m + sqrt(m^2 - a^2), and flags every field location
  * as advanced or excised (decided in FP64).  `stream` is a cudaStream_t (NULL = default stream).
+ * An FP64 context with m > 0 also takes a table of the metric at the field locations, 192 bytes per
+ * cell, where that is at most an eighth of the device's free memory.  It only saves time: the field
+ * updates give the same bits without it.  Where an allocation of the library fails, tables that came
+ * from the same allocator on the same device are freed, whichever context they belong to, and the
+ * allocation is tried again; so free_fn may be called for a context from a thread that uses another
+ * context with the same alloc and alloc_user.
  * Returns GRPIC_ERR_INVALID / GRPIC_ERR_CFL on bad input, GRPIC_ERR_OOM if allocation fails. */
 grpic_status grpic_create(const grpic_config* cfg, void* stream, grpic_ctx** out);
 

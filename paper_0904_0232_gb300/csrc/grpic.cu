@@ -4,6 +4,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -28,6 +29,15 @@ struct SpeciesStore {
   bool bins_zero = false;
   bool shadow_pending = false;
   bool loaded = false;
+};
+
+// FP64 contexts: the metric table of the field kernels.  It only saves time, and any allocation of the library may take
+// its memory from any thread (give_up_metric_table): the mutex is held while a launch that reads p is enqueued, and a
+// batched step counts among the users while it runs.
+struct MetricTable {
+  std::mutex mu;
+  double2* p = nullptr;
+  int users = 0;
 };
 
 // What the host reads back: the status word and the species' live counts (both buffers).
@@ -55,8 +65,7 @@ struct grpic_ctx {
   void* tgt = nullptr;     // absorbing layers: 6 planes of T, the target d and b (null without layers)
   void* kin = nullptr;     // inner absorbing layer: relaxation table over g.kbox0 / g.kboxn (T)
   double* J = nullptr;     // 3 planes
-  double2* met = nullptr;  // FP64: metric table of the field kernels (may be given up for memory, see dev_alloc)
-  bool met_held = false;   // a batch's tables refer to it
+  MetricTable met;
   float4* atab = nullptr;  // per-cell area fits of the far-field deposit (built when tune.area_table is set)
   uint16_t* loc = nullptr;  // per-cell location flags
   // field ping-pong state: buffer of the current d and b; bprev: buffer holding b^{n-1/2} after the
@@ -94,7 +103,7 @@ struct grpic_ctx {
 
 namespace {
 
-void* raw_alloc(grpic_ctx* c, size_t bytes) {
+void* raw_alloc(const grpic_ctx* c, size_t bytes) {
   if (c->cfg.alloc) return c->cfg.alloc(bytes, c->cfg.alloc_user);
   void* p = nullptr;
   if (cudaMalloc(&p, bytes) != cudaSuccess) {
@@ -113,16 +122,71 @@ void dev_free(grpic_ctx* c, void* p) {
   cudaFree(p);
 }
 
-// Device memory of the context.  The metric table only saves time, so it makes room for anything else: where an
-// allocation fails it is freed (unless a batch refers to it) and the allocation tried again.
+// The contexts that hold a metric table.
+struct TableOwners {
+  std::mutex mu;
+  std::vector<grpic_ctx*> list;
+};
+TableOwners& table_owners() {
+  static TableOwners o;
+  return o;
+}
+
+bool same_allocator(const grpic_ctx* c, grpic_alloc_fn alloc, void* user) {
+  return c->cfg.alloc == alloc && (!alloc || c->cfg.alloc_user == user);
+}
+
+// Device memory of the context.  Where an allocation fails, metric tables from the same allocator make room.
 void* dev_alloc(grpic_ctx* c, size_t bytes) {
   if (bytes == 0) bytes = 256;
   void* p = raw_alloc(c, bytes);
-  if (p || !c->met || c->met_held) return p;
-  cudaStreamSynchronize(c->stream);
-  dev_free(c, c->met);
-  c->met = nullptr;
-  return raw_alloc(c, bytes);
+  while (!p && give_up_metric_table(c->cfg.alloc, c->cfg.alloc_user)) p = raw_alloc(c, bytes);
+  return p;
+}
+
+// Is a graph being captured from the stream?  A launch in it may be replayed after the table has gone.
+bool capturing(cudaStream_t st) {
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) {
+    cudaGetLastError();
+    return true;
+  }
+  return cs != cudaStreamCaptureStatusNone;
+}
+
+// The table for launches that are enqueued while `use` lives, or null (the kernels then evaluate the metric: the same bits).
+const double2* metric_table(grpic_ctx* c, std::unique_lock<std::mutex>& use) {
+  if (c->mixed) return nullptr;
+  use = std::unique_lock<std::mutex>(c->met.mu);
+  return c->met.p && !capturing(c->stream) ? c->met.p : nullptr;
+}
+
+// The table costs 192 B a cell, more than the fields, J and flags of an FP64 context together (122 B): it is taken where
+// that is at most an eighth of the free memory, so that little is lost to programs beside the library, which cannot have it
+// given up.
+constexpr size_t kTableShare = 8;
+void create_metric_table(grpic_ctx* c) {
+  const size_t bytes = sizeof(double2) * kMetricPlanes * (size_t)c->g.ncell;
+  size_t free_bytes = 0, total = 0;
+  if (cudaMemGetInfo(&free_bytes, &total) != cudaSuccess || bytes > free_bytes / kTableShare) {
+    cudaGetLastError();
+    return;
+  }
+  c->met.p = static_cast<double2*>(raw_alloc(c, bytes));
+  if (!c->met.p) return;
+  launch_metric_table(c->g, c->loc, c->met.p, c->stream);
+  std::lock_guard<std::mutex> lk(table_owners().mu);
+  table_owners().list.push_back(c);
+}
+
+void destroy_metric_table(grpic_ctx* c) {
+  {
+    std::lock_guard<std::mutex> lk(table_owners().mu);
+    std::vector<grpic_ctx*>& l = table_owners().list;
+    l.erase(std::remove(l.begin(), l.end(), c), l.end());
+  }
+  dev_free(c, c->met.p);
+  c->met.p = nullptr;
 }
 
 grpic_status fail(grpic_ctx* c, grpic_status s, const std::string& msg) {
@@ -357,7 +421,8 @@ void enqueue_stage(grpic_ctx* c, int stage) {
       }
       A.kin = static_cast<const T*>(c->kin);
       A.loc = c->loc;
-      A.met = c->met;
+      std::unique_lock<std::mutex> table_use;
+      A.met = metric_table(c, table_use);
       A.K = field_consts<T>(c->g);
       const T dx4 = grid_dx4<T>(c->g);
       A.coef = centred ? dx4 : dx4 * T(0.5);
@@ -412,7 +477,8 @@ void enqueue_stage(grpic_ctx* c, int stage) {
       }
       A.kin = static_cast<const T*>(c->kin);
       A.loc = c->loc;
-      A.met = c->met;
+      std::unique_lock<std::mutex> table_use;
+      A.met = metric_table(c, table_use);
       A.K = field_consts<T>(c->g);
       const T dx4 = grid_dx4<T>(c->g);
       A.coef = dx4 * T(0.5);
@@ -597,6 +663,24 @@ grpic_status grpic_create(const grpic_config* cfg, void* stream, grpic_ctx** out
 
 }  // extern "C"
 
+bool grpic::give_up_metric_table(grpic_alloc_fn alloc, void* user) {
+  int device = 0;
+  cudaGetDevice(&device);
+  std::lock_guard<std::mutex> lk(table_owners().mu);
+  std::vector<grpic_ctx*>& owners = table_owners().list;
+  for (size_t i = 0; i < owners.size(); ++i) {
+    grpic_ctx* c = owners[i];
+    if (c->device != device || !same_allocator(c, alloc, user)) continue;
+    std::lock_guard<std::mutex> use(c->met.mu);
+    if (c->met.users > 0 || capturing(c->stream) || cudaStreamSynchronize(c->stream) != cudaSuccess) continue;
+    dev_free(c, c->met.p);
+    c->met.p = nullptr;
+    owners.erase(owners.begin() + i);
+    return true;
+  }
+  return false;
+}
+
 grpic_status grpic::create_context(const grpic_config* cfg, void* stream, bool metric_table, grpic_ctx** out) {
   if (!cfg || !out) return GRPIC_ERR_INVALID;
   *out = nullptr;
@@ -718,8 +802,7 @@ grpic_status grpic::create_context(const grpic_config* cfg, void* stream, bool m
       launch_inner_kappa_table<double>(g, static_cast<double*>(c->kin), c->stream);
   }
   if (!c->mixed && metric_table && g.m > 0.0) {
-    c->met = static_cast<double2*>(raw_alloc(c, sizeof(double2) * kMetricPlanes * (size_t)ncell));
-    if (c->met) launch_metric_table(g, c->loc, c->met, c->stream);
+    create_metric_table(c);
   }
   grpic_status s = cuda_check(c, cudaGetLastError(), "create");
   if (s == GRPIC_OK) s = cuda_check(c, cudaStreamSynchronize(c->stream), "create sync");
@@ -740,7 +823,7 @@ grpic_status grpic_destroy(grpic_ctx* c) {
   dev_free(c, c->tgt);
   dev_free(c, c->kin);
   dev_free(c, c->atab);
-  dev_free(c, c->met);
+  destroy_metric_table(c);
   dev_free(c, c->dstar);
   dev_free(c, c->J);
   dev_free(c, c->loc);
@@ -1351,15 +1434,21 @@ struct BatchHeld {
     }
   } sp[kMaxSpecies];
   int bcur, far_min_blocks, spread;
-  const void* atab;
+  const void *atab, *met;
   bool operator==(const BatchHeld& o) const {
     for (int s = 0; s < kMaxSpecies; ++s)
       if (!(sp[s] == o.sp[s])) return false;
-    return bcur == o.bcur && far_min_blocks == o.far_min_blocks && spread == o.spread && atab == o.atab;
+    return bcur == o.bcur && far_min_blocks == o.far_min_blocks && spread == o.spread && atab == o.atab &&
+           met == o.met;
   }
 };
 
-BatchHeld batch_held(const grpic_ctx* c) {
+const double2* batch_table(grpic_ctx* c) {
+  std::lock_guard<std::mutex> lk(c->met.mu);
+  return c->met.p;
+}
+
+BatchHeld batch_held(grpic_ctx* c) {
   BatchHeld h{};
   for (int s = 0; s < kMaxSpecies; ++s) {
     const SpeciesStore& S = c->sp[s];
@@ -1369,8 +1458,25 @@ BatchHeld batch_held(const grpic_ctx* c) {
   h.far_min_blocks = c->tune.far_min_blocks;
   h.spread = c->tune.spread;
   h.atab = area_table_of(c);
+  h.met = batch_table(c);
   return h;
 }
+
+// A batched step keeps the tables that its descriptors refer to for as long as it runs; between steps they can be given up.
+struct TableUse {
+  const std::vector<grpic_ctx*>& ctxs;
+  explicit TableUse(const std::vector<grpic_ctx*>& v) : ctxs(v) { add(1); }
+  ~TableUse() { add(-1); }
+  TableUse(const TableUse&) = delete;
+
+ private:
+  void add(int d) {
+    for (grpic_ctx* c : ctxs) {
+      std::lock_guard<std::mutex> lk(c->met.mu);
+      c->met.users += d;
+    }
+  }
+};
 
 }  // namespace
 
@@ -1421,12 +1527,14 @@ namespace {
 
 void* batch_alloc(grpic_batch* b, size_t bytes) {
   void* p = nullptr;
-  if (b->alloc) {
-    p = b->alloc(bytes, b->alloc_user);
-  } else if (cudaMalloc(&p, bytes) != cudaSuccess) {
-    cudaGetLastError();
-    p = nullptr;
-  }
+  do {
+    if (b->alloc) {
+      p = b->alloc(bytes, b->alloc_user);
+    } else if (cudaMalloc(&p, bytes) != cudaSuccess) {
+      cudaGetLastError();
+      p = nullptr;
+    }
+  } while (!p && give_up_metric_table(b->alloc, b->alloc_user));
   if (p) b->allocs.push_back(p);
   return p;
 }
@@ -1488,7 +1596,7 @@ std::vector<InstDesc<T>> batch_descs(grpic_batch* b) {
     for (int q = 0; q < 6; ++q) D.FS.tgt[q] = target_plane<T>(c, q);
     D.FS.kin = static_cast<const T*>(c->kin);
     D.FS.loc = c->loc;
-    D.FS.met = c->met;
+    D.FS.met = batch_table(c);
     D.dcur = b->dcur + i;
     D.st = c->st;
     D.tiles = b->tiles_of[i];
@@ -1534,7 +1642,6 @@ grpic_status batch_build(grpic_batch* b) {
   b->pair_of.assign(4 * n, -1);
   for (int i = 0; i < n; ++i) {
     grpic_ctx* c = b->ctxs[i];
-    c->met_held = true;
     dcur_init[i] = c->dcur;
     for (long long q = 0; q < b->tiles_of[i].count(); ++q) tile.push_back(BlockEntry{i, (int)q});
     append_blocks(all, i, c->g.ncell, 256);
@@ -1730,6 +1837,7 @@ grpic_status grpic_batch_step(grpic_batch* b, int nsteps) {
       const SpeciesStore& S = b->ctxs[i]->sp[s];
       if (S.loaded && (p < 0 || S.n > b->pair_n[p])) return GRPIC_ERR_INVALID;
     }
+  const TableUse tables(b->ctxs);
   const grpic_status fresh = b->mixed ? batch_refresh<float>(b) : batch_refresh<double>(b);
   if (fresh != GRPIC_OK) return fresh;
   // order after each context's pending work; refresh the device ping-pong indices

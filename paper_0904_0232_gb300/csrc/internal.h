@@ -9,4 +9,8 @@ namespace grpic {
 // server's runs, whose admission charges the memory that grpic_request_bytes states).
 grpic_status create_context(const grpic_config* cfg, void* stream, bool metric_table, grpic_ctx** out);
 
+// Free one metric table that came from this allocator (null: cudaMalloc) on the current device and is not in use by a
+// running batched step.  Returns whether there was one.
+bool give_up_metric_table(grpic_alloc_fn alloc, void* user);
+
 }  // namespace grpic

@@ -145,12 +145,15 @@ struct grpic_server {
 namespace {
 
 void* s_alloc(grpic_server* s, size_t bytes) {
-  if (s->alloc) return s->alloc(bytes, s->user);
   void* p = nullptr;
-  if (cudaMalloc(&p, bytes) != cudaSuccess) {
-    cudaGetLastError();
-    return nullptr;
-  }
+  do {
+    if (s->alloc) {
+      p = s->alloc(bytes, s->user);
+    } else if (cudaMalloc(&p, bytes) != cudaSuccess) {
+      cudaGetLastError();
+      p = nullptr;
+    }
+  } while (!p && grpic::give_up_metric_table(s->alloc, s->user));
   return p;
 }
 
