@@ -229,9 +229,10 @@ grpic_status grpic_request_bytes(const grpic_request* r, size_t* bytes) {
   const double tsz = r->cfg.precision == GRPIC_FP32_MIXED ? 4.0 : 8.0;
   const double n = (double)interior_slots(*r);
   // 12 field planes (two d and two b buffers; 6 more for the absorbing layers' target), FP64 J,
-  // location flags, sort counts and offsets
+  // location flags, and the sort bins, an int a cell and species: those of species 0 and 1 always, 2 and 3 together
   const bool layers = r->cfg.absorb_inner > 0.0 || r->cfg.absorb_outer > 0.0;
-  const double fields = cells * ((layers ? 18.0 : 12.0) * tsz + 3.0 * 8.0 + 2.0 + 8.0);
+  const double bins = r->nspecies > 2 ? 16.0 : 8.0;
+  const double fields = cells * ((layers ? 18.0 : 12.0) * tsz + 3.0 * 8.0 + 2.0 + bins);
   const double particles = n * r->nspecies * 2.0 * (8.0 * tsz + 8.0);
   const double staging = n * (4.0 * 8.0 * (1 + r->nspecies) + 4.0);
   *bytes = (size_t)(fields + particles + staging) + (size_t)(1 << 20);
