@@ -61,12 +61,17 @@ __host__ __device__ constexpr int nb_hi(int t, int s, int ax) {
   return half(s, ax) == half(t, ax) ? 0 : (half(t, ax) == 1 ? 1 : 0);
 }
 
-// Reciprocal square root and reciprocal: the hardware approximations in FP32 (relative error
+// Square root with its reciprocal, reciprocal and quotient: the hardware approximations in FP32 (relative error
 // ~1e-7, below the FP32 rounding of the stencil sums), FastOps64 in FP64.
-__device__ __forceinline__ float rsqrt_t(float v) { return rsqrtf(v); }
-__device__ __forceinline__ double rsqrt_t(double v) { return FastOps64::rsqrt(v); }
+__device__ __forceinline__ float root_t(float v, float& inv) {
+  inv = rsqrtf(v);
+  return v * inv;
+}
+__device__ __forceinline__ double root_t(double v, double& inv) { return FastOps64::root_and_rsqrt(v, &inv); }
 __device__ __forceinline__ float rcp_t(float v) { return __fdividef(1.f, v); }
 __device__ __forceinline__ double rcp_t(double v) { return FastOps64::rcp(v); }
+__device__ __forceinline__ float div_t(float a, float b) { return a * __fdividef(1.f, b); }
+__device__ __forceinline__ double div_t(double a, double b) { return FastOps64::div(a, b); }
 // A product that stays one (in FP64, where the metric table has to hold what the kernels would evaluate, no product is
 // left for the compiler to fuse with a sum, which it does differently from place to place).
 __device__ __forceinline__ float mul_t(float a, float b) { return a * b; }
@@ -110,18 +115,17 @@ __device__ __forceinline__ Pt<T> metric_pt(const FieldConsts<T>& K, int l, T xr,
   const T q = K.a2 * Z * Z;
   const T p = fma(X, X, fma(Y, Y, fma(Z, Z, -K.a2)));
   const T disc = fma(p, p, T(4) * q);
-  const T rD = rsqrt_t(disc);  // 1 / D
-  const T D = mul_t(disc, rD);
-  const T r2 = p >= T(0) ? T(0.5) * (p + D) : mul_t(T(2) * q, rcp_t(D - p));
+  T rD, ir;  // 1 / D, 1 / r
+  const T D = root_t(disc, rD);
+  const T r2 = p >= T(0) ? T(0.5) * (p + D) : div_t(T(2) * q, D - p);
   if (!(r2 > T(0))) return P;
-  const T ir = rsqrt_t(r2);
-  const T r = r2 * ir;
+  const T r = root_t(r2, ir);
   const T irho2 = rcp_t(r2 + K.a2);
   if constexpr (sizeof(T) == sizeof(float)) {
     P.f = K.two_m * r * rD;
   } else {
     const T F = mul_t(K.two_m, r);
-    P.f = F * rcp_t(D + F);
+    P.f = div_t(F, D + F);
   }
   P.k0 = (r * X - mul_t(K.a, Y)) * irho2;
   P.k1 = (r * Y + mul_t(K.a, X)) * irho2;

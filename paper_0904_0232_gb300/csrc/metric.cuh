@@ -99,84 +99,153 @@ struct SeededOps64 {
   }
 };
 
-// FP64 reciprocal, square root and reciprocal square root to FP64 accuracy with 1, 2 and 2 FP64 operations.  This GPU issues
+// FP64 reciprocal, square root and reciprocal square root, rounded as well as the IEEE operations' to a hundredth of a unit
+// in the last place, with 1, 2 and 3 FP64 operations (3 for a root and its reciprocal together).  This GPU issues
 // one FP64 warp instruction per 16 cycles and SM, 64 times slower than FP32 and integer ones, and its FP64 kernels are
 // bound by their count (IEEE 1/x, sqrt x and 1/sqrt x take about 9, 10 and 20), so everything else is done beside the FP64
 // pipe:
 //   1. the argument's mantissa as two floats xh + xl (46 bits), y0 ~ xh^-1/2 (or xh^-1) from the FP32 approximation,
 //      r = 1 - x y0^2 (1 - x y0) in FP32 with fused multiply-adds, whose rounding (2^-24 of r ~ 2^-21) leaves
 //      y = y0 (1 + r/2 + 3 r^2/8) (y0 (1 + r + r^2)) within about 2^-44; the sum is an integer addition to y0's bits;
-//   2. in FP64 the residual e = 1 - x y^2 (with s = x y for the root) or 1 - x y;
-//   3. the first-order step y (1 + e/2), s (1 + e/2) or y (1 + e), whose correction is below 2^12 units in the last place:
-//      formed in FP32, rounded to an integer and added to the bits (where that crosses a power of two, which changes the
-//      unit, in FP64).  The truncation is of order e^2.
-// The result is within one unit in the last place (measured: 0.75).  Arguments are positive normal numbers (rcp:
-// of either sign); root gives 0 for 0 and subnormals.  Others give no useful value, and callers screen them.
+//   2. in FP64 the residuals: 1 - x y; with s = x y, x - s^2 and 1 - s y.  s is rounded, s = x y (1 + n), which the first of
+//      these holds twice and the second once: e = 2 (1 - s y) - (x - s^2) / x = 1 - x y^2 to order n^2;
+//   3. the first-order step y (1 + e), s (1 + (x - s^2) / 2x) or y (1 + e/2), whose correction is below 2^12 units in the last
+//      place: formed in FP32, rounded to an integer and added to the bits (in FP64 where either side of that is not in the
+//      result's binade, whose unit it is in).  The truncation is of order e^2.
+// So the result is the exact one rounded, but for the FP32 correction's own error of below 2^-7 units (measured over 5e7
+// arguments: 0.500 units off at most, rms 4.7e-17 relative as IEEE; 1/sqrt x in two IEEE operations 1.49 and 6.7e-17).  Arguments lie in
+// 2^-890 .. 2^890, and root gives 0 for 0 and subnormals.  Others give no useful value, and callers screen them (or use
+// CheckedOps64).
+// Few instructions count as well: the push's two copies of them lie at the limit of the instruction cache.
 struct FastOps64 {
  private:
-  // mantissa of x in [1, 2), or [1, 4) where odd, as xh + xl
-  __device__ static __forceinline__ void split(int hi, int lo, int odd, float* xh, float* xl) {
-    const unsigned m = ((unsigned)(hi & 0xfffff) << 3) | ((unsigned)lo >> 29);
-    *xh = __uint_as_float(((127u + odd) << 23) | m);
-    const float low = __uint_as_float(0x4B000000u | (((unsigned)lo & 0x1fffffffu) >> 6)) - 8388608.f;
-    *xl = low * (odd ? 0x1p-45f : 0x1p-46f);
+  // the upper 23 of a double's mantissa bits under the exponent field `field` of a float, and the 23 after them as a float of
+  // that scale
+  __device__ static __forceinline__ void split(int hi, int lo, unsigned field, float* xh, float* xl) {
+    *xh = __uint_as_float((__funnelshift_l((unsigned)lo, (unsigned)hi, 3) & 0x7fffffu) | field);
+    const unsigned base = field - (23u << 23);
+    *xl = __uint_as_float(base | (((unsigned)lo & 0x1fffffffu) >> 6)) - __uint_as_float(base);
   }
-  // y0 + c (y0 in [0.5, 1]) times 2^-shift, as a double
-  __device__ static __forceinline__ double assemble(float y0, float c, int shift) {
-    const long long bits = ((long long)__float_as_uint(y0) << 29) + ((long long)(896 - shift) << 52);
+  // y0 + c (y0 in [0.5, 1]) as a double, its exponent field raised by field (a high word)
+  __device__ static __forceinline__ double assemble(float y0, float c, int field) {
+    const long long bits = ((long long)__float_as_uint(y0) << 29) + ((long long)field << 32);
     return __longlong_as_double(bits + __float2int_rn(c * 0x1p53f));
   }
-  // y (1 + e scale), |e| < 2^-40
-  __device__ static __forceinline__ double correct(double y, double e, float scale) {
-    const int eh = __double2hiint(e);
-    const unsigned ee = ((unsigned)eh >> 20) & 0x7ffu;
-    const float ef = ee < 923u ? 0.f
-                               : __uint_as_float(((unsigned)eh & 0x80000000u) | ((ee - 896u) << 23) |
-                                                 (((unsigned)eh & 0xfffffu) << 3) | ((unsigned)__double2loint(e) >> 29));
-    const float m = __uint_as_float(0x3f800000u | (((unsigned)__double2hiint(y) & 0xfffffu) << 3) |
-                                    ((unsigned)__double2loint(y) >> 29));
-    const long long b0 = __double_as_longlong(y), b1 = b0 + __float2int_rn(ef * (m * scale));
-    if (((b0 ^ b1) >> 52) != 0) return crossing(y, e, scale);
-    return __longlong_as_double(b1);
+  // v as a float, its exponent field lowered by field (a high word) and 0 where that is too small
+  __device__ static __forceinline__ float small_float(double v, int field) {
+    const int hi = __double2hiint(v);
+    const unsigned m = (unsigned)max((hi & 0x7fffffff) - field, 0);
+    return __uint_as_float(__funnelshift_l((unsigned)__double2loint(v), m, 3) | ((unsigned)hi & 0x80000000u));
   }
-  __device__ static __noinline__ double crossing(double y, double e, float scale) {
-    return fma(y * e, scale == 0x1p52f ? 1.0 : 0.5, y);
+  static constexpr int kNoField = 896 << 20;  // between the fields of a double and a float of one value
+  // v moved by n units, where v and the result both have the exponent field (a high word) that n's unit belongs to
+  __device__ static __forceinline__ bool add_units(double v, float n, int field, double* out) {
+    *out = __longlong_as_double(__double_as_longlong(v) + __float2int_rn(n));
+    return (((__double2hiint(v) ^ field) | (__double2hiint(*out) ^ field)) >> 20) == 0;
   }
-  __device__ static __forceinline__ double rsqrt_start(double x) {
+  struct Start {
+    double y;   // x^-1/2 within 2^-43
+    float yf;   // y 2^h to FP32, in [0.5, 1], where x 4^-h is in [1, 4)
+    int x, r;   // exponent fields of 4^h and 2^h (high words)
+  };
+  __device__ static __forceinline__ Start rsqrt_start(double x) {
     const int hi = __double2hiint(x), lo = __double2loint(x);
-    const int E = (hi >> 20) - 1023, odd = E & 1;
+    Start b;
+    b.x = ((hi - 0x00100000) | 0x00100000) & 0x7ff00000;
+    b.r = (int)((unsigned)b.x >> 1) + (1023 << 19);
     float xh, xl;
-    split(hi, lo, odd, &xh, &xl);
+    split(hi, lo, (127u << 23) + ((~(unsigned)hi & 0x00100000u) << 3), &xh, &xl);
     const float y0 = fminf(fmaxf(rsqrtf(xh), 0.5f), 1.f);
     const float t = __fmul_rn(xh, y0);
     float r = __fmaf_rn(-t, y0, 1.f);
     r = __fmaf_rn(-__fmaf_rn(xh, y0, -t), y0, r);
     r = __fmaf_rn(-__fmul_rn(xl, y0), y0, r);
-    return assemble(y0, y0 * (r * __fmaf_rn(0.375f, r, 0.5f)), (E - odd) >> 1);
+    const float c = y0 * (r * __fmaf_rn(0.375f, r, 0.5f));
+    b.y = assemble(y0, c, kNoField + (1023 << 20) - b.r);
+    b.yf = __fadd_rn(y0, c);
+    return b;
+  }
+  // d 4^-h to FP32
+  __device__ static __forceinline__ float scaled(const Start& b, double d) {
+    return small_float(d, b.x + (kNoField - (1023 << 20)));
+  }
+  // root of x from s = x y, d = x - s^2 (s (d / x) / 2 in units of 2^(h - 52): (d 4^-h) (y 2^h) / 2 2^52)
+  __device__ static __forceinline__ double root_of(double x, const Start& b, double s, double d, float df) {
+    double v;
+    if (!add_units(s, df * (b.yf * 0x1p51f), b.r, &v)) v = root_apart(s, d, b.y);
+    return (__double2hiint(x) & 0x7fffffff) < 0x00100000 ? 0.0 : v;
+  }
+  // and its reciprocal from also e1 = 1 - s y
+  __device__ static __forceinline__ double rsqrt_of(const Start& b, double d, float df, double e1) {
+    const float e = __fmaf_rn(2.f, small_float(e1, kNoField), -(df * __fmul_rn(b.yf, b.yf)));
+    double v;
+    if (!add_units(b.y, e * (b.yf * 0x1p52f), (2045 << 20) - b.r, &v)) v = rsqrt_apart(b.y, d, e1);
+    return v;
+  }
+  // across a power of two (out of line with their operations, which would be issued, predicated off, for every argument)
+  __device__ static __noinline__ double rcp_apart(double y, double e) { return fma(y, e, y); }
+  __device__ static __noinline__ double root_apart(double s, double d, double y) { return fma(0.5 * y, d, s); }
+  __device__ static __noinline__ double rsqrt_apart(double y, double d, double e1) {
+    return fma(0.5 * y, fma(2.0, e1, -d * y * y), y);
   }
 
  public:
   __device__ static __forceinline__ double rcp(double x) {
-    const int hi = __double2hiint(x), lo = __double2loint(x);
+    const int hi = __double2hiint(x), lo = __double2loint(x), field = hi & 0x7ff00000;
     float xh, xl, y0;
-    split(hi, lo, 0, &xh, &xl);
+    split(hi, lo, 127u << 23, &xh, &xl);
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y0) : "f"(xh));
     y0 = fminf(fmaxf(y0, 0.5f), 1.f);
     float r = __fmaf_rn(-xh, y0, 1.f);
     r = __fmaf_rn(-xl, y0, r);
-    const double y = assemble(y0, y0 * __fmaf_rn(r, r, r), ((hi & 0x7fffffff) >> 20) - 1023);
-    const double ys = __hiloint2double(__double2hiint(y) | (hi & 0x80000000), __double2loint(y));
-    return correct(ys, fma(-x, ys, 1.0), 0x1p52f);
-  }
-  __device__ static __forceinline__ double rsqrt(double x) {
-    const double y = rsqrt_start(x);
-    return correct(y, fma(-x * y, y, 1.0), 0x1p51f);
+    const float c = y0 * __fmaf_rn(r, r, r);
+    const double y = assemble(y0, c, kNoField + (1023 << 20) - field);
+    const double e = fma(-x, y, 1.0);
+    double v;
+    if (!add_units(y, small_float(e, kNoField) * (__fadd_rn(y0, c) * 0x1p53f), (2045 << 20) - field, &v))
+      v = rcp_apart(y, e);
+    return v;
   }
   __device__ static __forceinline__ double root(double x) {
-    const double y = rsqrt_start(x), s = x * y;
-    const double v = correct(s, fma(-s, y, 1.0), 0x1p51f);
-    return (__double2hiint(x) & 0x7fffffff) < 0x00100000 ? 0.0 : v;
+    const Start b = rsqrt_start(x);
+    const double s = x * b.y, d = fma(-s, s, x);
+    return root_of(x, b, s, d, scaled(b, d));
   }
+  __device__ static __forceinline__ double rsqrt(double x) {
+    const Start b = rsqrt_start(x);
+    const double s = x * b.y, d = fma(-s, s, x);
+    return rsqrt_of(b, d, scaled(b, d), fma(-s, b.y, 1.0));
+  }
+  // root(x) and its reciprocal rsqrt(x)
+  __device__ static __forceinline__ double root_and_rsqrt(double x, double* ri) {
+    const Start b = rsqrt_start(x);
+    const double s = x * b.y, d = fma(-s, s, x);
+    const float df = scaled(b, d);
+    *ri = rsqrt_of(b, d, df, fma(-s, b.y, 1.0));
+    return root_of(x, b, s, d, df);
+  }
+  // a / b, its residual taken once: 4 operations, as well rounded as the others (b as for rcp)
+  __device__ static __forceinline__ double div(double a, double b) {
+    const double y = rcp(b), q = a * y;
+    return fma(fma(-b, q, a), y, q);
+  }
+};
+
+// The same for any argument: those out of FastOps64's range take the IEEE operations, out of line.
+struct CheckedOps64 {
+  __device__ static __forceinline__ double div(double a, double b) {
+    const bool finite = (__double2hiint(a) & 0x7ff00000) != 0x7ff00000;
+    return finite && in_range(__double2hiint(b)) ? FastOps64::div(a, b) : ieee_div(a, b);
+  }
+  __device__ static __forceinline__ double root(double x) {
+    return in_range(__double2hiint(x)) ? FastOps64::root(x) : ieee_root(x);
+  }
+
+ private:
+  // high word of a positive number from 2^-890, below 2^890
+  __device__ static __forceinline__ bool in_range(int hi) { return (unsigned)hi - (133u << 20) < 1780u << 20; }
+  __device__ static __noinline__ double ieee_div(double a, double b) { return a / b; }
+  __device__ static __noinline__ double ieee_root(double x) { return sqrt(x); }
 };
 
 // x / 2 for a positive normal x, without an FP64 operation.
@@ -241,7 +310,7 @@ __device__ __forceinline__ Kerr<S> kerr_eval(S x, S y, S z, S m, S a) {
 // kerr_eval in FP64 with FastOps64; since the root satisfies Sigma = r^4 + a^2 z^2 = r^2 D, 1 / Sigma and f = 2 m r / D
 // need no division.  The root for p = R^2 - a^2 < 0 is out of line (its operations would be issued for every point).
 static __device__ __noinline__ double kerr_root_inside(double p, double q4, double D) {
-  return halve(q4 * FastOps64::rcp(D - p));
+  return halve(FastOps64::div(q4, D - p));
 }
 __device__ __forceinline__ Kerr<double> kerr_eval_fast(double x, double y, double z, double two_m, double a, double a2,
                                                        double a2_4) {
@@ -249,8 +318,7 @@ __device__ __forceinline__ Kerr<double> kerr_eval_fast(double x, double y, doubl
   const double q4 = a2_4 * (z * z);
   const double p = fma(x, x, fma(y, y, fma(z, z, -a2)));
   const double D2 = fma(p, p, q4);
-  K.inv_D = FastOps64::rsqrt(D2);
-  K.D = D2 * K.inv_D;
+  K.D = FastOps64::root_and_rsqrt(D2, &K.inv_D);
   double r2 = halve(p + K.D);
   if (__double2hiint(p) < 0) r2 = kerr_root_inside(p, q4, K.D);
   if (__double2hiint(D2) < 0x00100000 || __double2hiint(r2) < 0x00100000) {  // r = 0
@@ -260,8 +328,7 @@ __device__ __forceinline__ Kerr<double> kerr_eval_fast(double x, double y, doubl
     return K;
   }
   K.flat = false;
-  K.inv_r = FastOps64::rsqrt(r2);
-  K.r = r2 * K.inv_r;
+  K.r = FastOps64::root_and_rsqrt(r2, &K.inv_r);
   K.inv_rho2 = FastOps64::rcp(r2 + a2);
   K.inv_sig = K.inv_D * (K.inv_r * K.inv_r);
   K.f = two_m * K.r * K.inv_D;

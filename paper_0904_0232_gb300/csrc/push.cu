@@ -175,7 +175,7 @@ __global__ void k_load(const Grid g, const Particles<T> P, long long n, const do
         bad |= ST_LOAD_INVALID;
       } else {
         // raise: u^i = u_i - f k_i (k.u - u_4)
-        const double fkul = f * (ku - (fk - S) * FastOps64::rcp(A));
+        const double fkul = f * (ku - FastOps64::div(fk - S, A));
 #pragma unroll
         for (int q = 0; q < 3; ++q) u[q] = fma(-kk[q], fkul, u[q]);
         u[3] = S;
@@ -188,7 +188,7 @@ __global__ void k_load(const Grid g, const Particles<T> P, long long n, const do
       } else if (!(S2 >= 0.0)) {
         bad |= ST_LOAD_INVALID;
       } else {
-        u[3] = (fk + FastOps64::root(S2)) * FastOps64::rcp(A);
+        u[3] = FastOps64::div(fk + FastOps64::root(S2), A);
         if (!(u[3] > 0.0)) bad |= ST_LOAD_INVALID;
       }
     }

@@ -163,6 +163,13 @@ __device__ __forceinline__ bool finite_t(double v) { return (__double2hiint(v) &
 __device__ __forceinline__ bool below_one(float v) { return fabsf(v) < 1.f; }
 __device__ __forceinline__ bool below_one(double v) { return (__double2hiint(v) & 0x7fffffff) < 0x3ff00000; }
 
+// a / b, in FP64 from 1 / b to FP64 accuracy and the residual (3 operations)
+__device__ __forceinline__ float quotient(float a, float b, float) { return a / b; }
+__device__ __forceinline__ double quotient(double a, double b, double inv) {
+  const double q = a * inv;
+  return fma(fma(-b, q, a), inv, q);
+}
+
 template <typename T>
 __device__ __forceinline__ T lerp(T a, T b, T w) {
   return fma(w, b - a, a);
@@ -381,14 +388,16 @@ __device__ __forceinline__ void accel(const Grid& g, const Fields<T>& F, const C
 // corner at (oI, oJ) relative to the centre along (I, J) = (K+1, K+2) mod 3, split at the fractions (u, v).  The Q x Q
 // Gauss nodes of the four rectangles make a 2Q x 2Q lattice, on which p = R^2 - a^2, 4 q = 4 a^2 z^2 and the spin
 // term of k_K's numerator are sums of a row and a column term.  With D = sqrt(p^2 + 4 q), r^2 = (p + D) / 2 and
-// f = 2 m r / D the integrand 1 + f (1 - k_K^2) (k being null, Eq. 6) is N / M,
-//   M = D rho^4, N = M + 2 m r (rho^4 - num^2), k_K = num / rho^2    (K = 0: num = r x - a y, 1: r y + a x)
-//   M = D r,     N = M + 2 m (r^2 - z^2)                             (K = 2),
-// so that a node takes two roots and one reciprocal root, sqrt(N / M) = N / sqrt(N M).
+// f = 2 m r / D the integrand 1 + f (1 - k_K^2) (k being null, Eq. 6) is 1 + F / M,
+//   M = D rho^4, F = 2 m r (rho^4 - num^2), k_K = num / rho^2    (K = 0: num = r x - a y, 1: r y + a x)
+//   M = D r,     F = 2 m (r^2 - z^2)                             (K = 2),
+// so that a node takes three roots and one reciprocal.
 // FP64 operations bound the push in FP64 (one FP64 warp instruction per 16 cycles and SM): 19 a node (15 for K = 2) and 96
 // nodes a particle-step at Q = 2, where one IEEE evaluation of the integrand per node took about 78.
-// Measured: push of 1.82 M particles at 64^3, Q = 2: 25.8 -> 10.7 ms (4600 issued FP64 operations a particle-step with
-// 5-operation roots 15.5 ms, 3180 with FastOps64's: 83 % of the pipe's cycles).
+// Measured: push of 1.82 M particles at 64^3, Q = 2: 25.8 -> 10.6 ms (4600 issued FP64 operations a particle-step with
+// 5-operation roots 15.5 ms, 3190 with FastOps64's: 88 % of the pipe's cycles).  Error of a node, rms over 4e5 positions
+// from R = 3.5 to 52 with m = 2, a = 1.8: 6.8e-17 relative, as for one IEEE evaluation (N / sqrt(N M) with N = M + F, of as many
+// operations, 8.7e-17).
 // r = 0 takes the flat limit 1.
 // A00 = [u,1] x [v,1], A10 = [0,u] x [v,1], A01 = [u,1] x [0,v], A11 = [0,u] x [0,v].
 template <int Q, int K>
@@ -432,18 +441,18 @@ __device__ __forceinline__ void lattice_areas(const Consts<double>& C, double XK
         double r2 = halve(p + D);
         if (__double2hiint(p) < 0) r2 = kerr_root_inside(p, q4, D);
         const double r = FastOps64::root(r2);
-        double M, N;
+        double M, F;
         if (K == 2) {
           M = D * r;
-          N = fma(C.two_m, r2 - zz, M);
+          F = C.two_m * (r2 - zz);
         } else {
           const double num = fma(r, XK, K == 0 ? tR : tJ[j]);
           const double rho2 = r2 + C.a2;
           const double rho4 = rho2 * rho2;
           M = D * rho4;
-          N = fma(C.two_m * r, fma(-num, num, rho4), M);
+          F = C.two_m * r * fma(-num, num, rho4);
         }
-        double val = N * FastOps64::rsqrt(N * M);
+        double val = FastOps64::root(fma(F, FastOps64::rcp(M), 1.0));
         if (__double2hiint(r2) < 0x00100000) val = 1.0;  // r = 0: the flat limit
         if (Q == 2)
           S[si][j / Q] += val;  // unit Gauss weights
@@ -952,7 +961,7 @@ __device__ __forceinline__ Move<T> push_move(const Grid& g, const Fields<T>& F, 
     accel<T, MIXED, WIDE>(g, F, C, xs, us, a, flags, n64);
     if (stage == 0) {
       if constexpr (sizeof(T) == sizeof(double))
-        h = C.dt * FastOps64::rcp(gamma_step<T, FastOps64>(us[3], a[3], C.inv_c, C.dt, &fb));
+        h = CheckedOps64::div(C.dt, gamma_step<T, CheckedOps64>(us[3], a[3], C.inv_c, C.dt, &fb));
       else
         h = C.dt / gamma_step<T>(us[3], a[3], C.inv_c, C.dt, &fb);
     }
@@ -967,7 +976,7 @@ __device__ __forceinline__ Move<T> push_move(const Grid& g, const Fields<T>& F, 
     }
   }
   T x0[3], x1[4], u1[4], dx[3];
-  const T h6 = sizeof(T) == sizeof(double) ? h * T(1.0 / 6.0) : h / T(6);
+  const T h6 = quotient(h, T(6), T(1.0 / 6.0));
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     const T xq = reload(P.x[q] + i), d = h6 * sx[q];
@@ -980,10 +989,7 @@ __device__ __forceinline__ Move<T> push_move(const Grid& g, const Fields<T>& F, 
   }
   x1[3] -= C.cdt;  // x^4 is stored relative to c t
   T gbar = T(1);
-  if (C.gamma_in_j) {
-    const T u4s = reload(P.u[3] + i) + u1[3];
-    gbar = sizeof(T) == sizeof(double) ? u4s * (T(0.5) * C.inv_c) : u4s / (T(2) * C.c);
-  }
+  if (C.gamma_in_j) gbar = quotient(reload(P.u[3] + i) + u1[3], T(2) * C.c, T(0.5) * C.inv_c);
   bool finite = true;
 #pragma unroll
   for (int q = 0; q < 4; ++q) finite = finite && finite_t(x1[q]) && finite_t(u1[q]);
