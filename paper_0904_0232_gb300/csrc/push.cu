@@ -108,18 +108,13 @@ __global__ void __launch_bounds__(128, 4) k_push_deposit_batch(const InstDesc<do
 __device__ __forceinline__ float from_f64(double v, float) { return narrow(v); }
 __device__ __forceinline__ double from_f64(double v, double) { return v; }
 
-// Is the point inside r <= r_+?  Screened in FP32 (far from the hole nothing else is evaluated), decided from the FP64
-// radius r (negative: not evaluated yet) and, where that is within rounding of r_+, from the IEEE evaluation.
+// Is the point inside r <= r_+?  Screened in FP32 (far from the hole nothing else is evaluated), decided by the IEEE
+// evaluation.
 __device__ __forceinline__ bool inside_horizon(const Grid& g, double X, double Y, double Z) {
   const float xf = narrow(X), yf = narrow(Y), zf = narrow(Z), rp = (float)g.r_plus + fabsf((float)g.a);
   if (xf * xf + yf * yf + zf * zf > 1.01f * rp * rp + 1e-3f) return false;  // r >= R - |a| > r_+
   const Kerr<double> K = kerr_eval<double>(X, Y, Z, g.m, g.a);
   return K.flat || K.r <= g.r_plus;
-}
-
-// v > 0, normal and finite (from the bits)
-__device__ __forceinline__ bool normal_positive(double v) {
-  return (unsigned)__double2hiint(v) - 0x00100000u < 0x7fe00000u;
 }
 
 // Completion of u^a from its spatial part.  Covariant u_i (umode 1): g^mn u_m u_n = -c^2 with g^mn = eta^mn - f k^m k^n,
@@ -170,12 +165,13 @@ __global__ void k_load(const Grid g, const Particles<T> P, long long n, const do
     if (umode == 1) {
       const double A = 1.0 + f;
       const double S2 = fma(fk, fk, A * fma(-fk, ku, uu));
-      const double S = FastOps64::root(S2);
-      if (!normal_positive(S2)) {
+      // (S^2 beyond FP64: loaded with an infinite u^4, which the first step reports, where the metric is not flat)
+      if (!(S2 > 0.0) || (f == 0.0 && !finite_t(S2))) {
         bad |= ST_LOAD_INVALID;
       } else {
         // raise: u^i = u_i - f k_i (k.u - u_4)
-        const double fkul = f * (ku - FastOps64::div(fk - S, A));
+        const double S = CheckedOps64::root(S2);
+        const double fkul = f * (ku - CheckedOps64::div(fk - S, A));
 #pragma unroll
         for (int q = 0; q < 3; ++q) u[q] = fma(-kk[q], fkul, u[q]);
         u[3] = S;
@@ -188,7 +184,7 @@ __global__ void k_load(const Grid g, const Particles<T> P, long long n, const do
       } else if (!(S2 >= 0.0)) {
         bad |= ST_LOAD_INVALID;
       } else {
-        u[3] = FastOps64::div(fk + FastOps64::root(S2), A);
+        u[3] = CheckedOps64::div(fk + CheckedOps64::root(S2), A);
         if (!(u[3] > 0.0)) bad |= ST_LOAD_INVALID;
       }
     }
