@@ -634,6 +634,12 @@ __device__ __forceinline__ void e_step_tile(const Grid& g, const EStepArgs<T>& A
 // Resident blocks per SM: 64 registers a thread for the FP32 patches, 128 for the FP64 ones.
 constexpr int patch_blocks(size_t word, int rows) { return (word == 4 ? 32 : 16) / rows; }
 
+// Chunks of at most z planes, as many as nzi planes take, made as equal as they can be.
+inline int even_chunk(int nzi, int z) {
+  const int nc = (nzi + z - 1) / z;
+  return (nzi + nc - 1) / nc;
+}
+
 // Patches over the advanced cells [2, n-3] per axis (31 x (rows - 1) cells each), and the split of z that minimises the
 // estimated time: a chunk marches `halo` planes beyond its own and the busiest of the `slots` runs
 // ceil(patches / slots) of them.
@@ -645,8 +651,8 @@ TileGrid tile_grid(const Grid& g, int rows, int slots, double* cost_out = nullpt
   t.ntx = (g.nx - 4 + ox - 1) / ox;
   t.nty = (g.ny - 4 + oy - 1) / oy;
   double best = 1e300;
-  for (int nc = (nzi + 63) / 64; nc <= nzi; ++nc) {
-    const int zc = (nzi + nc - 1) / nc;
+  for (int z = std::min(nzi, 64); z >= 1; --z) {  // (by the length: by the number of chunks, a long grid has too many)
+    const int zc = even_chunk(nzi, z);
     const long long nt = (long long)t.ntx * t.nty * ((nzi + zc - 1) / zc);
     const double per_slot = std::ceil((double)nt / slots);
     const double cost = per_slot * (zc + halo);  // time ~ blocks of the busiest slot x planes marched
@@ -1036,14 +1042,13 @@ void launch_e_step(const Grid& g, const EStepArgs<T>& A, int sms, cudaStream_t s
 constexpr int kBatchRows = 16;
 void batch_field_tiles(const Grid* const* grids, int n, size_t word, int sms, TileGrid* tiles) {
   const int slots = sms * patch_blocks(word, kBatchRows);
+  for (int i = 0; i < n; ++i) tiles[i] = tile_grid(*grids[i], kBatchRows, 1);
   double best = 1e300;
   int zbest = 64;
   for (int zc = 64; zc >= 1; zc -= zc > 16 ? 4 : 1) {
     long long nt = 0;
-    for (int i = 0; i < n; ++i) {
-      TileGrid t = tile_grid(*grids[i], kBatchRows, 1);
-      nt += (long long)t.ntx * t.nty * ((grids[i]->nz - 4 + zc - 1) / zc);
-    }
+    for (int i = 0; i < n; ++i)
+      nt += (long long)tiles[i].ntx * tiles[i].nty * ((grids[i]->nz - 4 + zc - 1) / zc);
     const double cost = std::ceil((double)nt / slots) * (zc + 2);
     if (cost < best * 0.999) {
       best = cost;
@@ -1051,7 +1056,6 @@ void batch_field_tiles(const Grid* const* grids, int n, size_t word, int sms, Ti
     }
   }
   for (int i = 0; i < n; ++i) {
-    tiles[i] = tile_grid(*grids[i], kBatchRows, 1);
     tiles[i].zchunk = zbest;
     tiles[i].ntz = (grids[i]->nz - 4 + zbest - 1) / zbest;
   }
