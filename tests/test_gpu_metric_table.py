@@ -64,7 +64,8 @@ def _started(mem):
 
 @pytest.fixture(scope="module")
 def expected():
-    ctx = _started(Memory())
+    mem = Memory()  # (its callbacks have to outlive the context)
+    ctx = _started(mem)
     out = {}
     for n in range(1, 41):
         G.grpic_step(ctx, 1)
