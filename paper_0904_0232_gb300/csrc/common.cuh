@@ -396,11 +396,9 @@ struct BlockEntry {
 template <typename T>
 struct SpeciesDesc {
   Consts<T> C;          // launch constants of this (instance, species)
-  double qm, qmacro;
   Particles<T> buf[2];  // the two ping-pong buffers (n = work upper bound, n_dev = live count)
   int* cur;             // device int: index of the current buffer
   long long bin_base;   // first sort bin of this (instance, species) in the batch's bin array
-  int active;
 };
 
 template <typename T>

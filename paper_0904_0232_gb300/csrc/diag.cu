@@ -55,8 +55,7 @@ __device__ __forceinline__ void cloud64(const Particles<T>& P, long long i, doub
     }
 }
 
-template <typename T>
-__global__ void k_charge_density(const Particles<T> P, double q, int nx, int ny, int nz, double inv_c,
+__global__ void k_charge_density(const Particles<double> P, double q, int nx, int ny, int nz, double inv_c,
                                  bool with_gamma, double* __restrict__ rho) {
   const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (i >= P.n || i >= (long long)(*P.n_dev) || P.key[i] == kDead) return;
@@ -320,16 +319,15 @@ template <typename T>
 void launch_charge_density(const Particles<T>& P, double q, const Grid& g, bool with_gamma, double* rho,
                            cudaStream_t stream) {
   if (P.n <= 0) return;
+  const unsigned nb = (unsigned)((P.n + 255) / 256);
   if constexpr (sizeof(T) == sizeof(float)) {
-    const unsigned nb = (unsigned)((P.n + 255) / 256);
     if (with_gamma)
       k_charge_density_runs<true><<<nb, 256, 0, stream>>>(P, q, g.nx, g.ny, g.nz, 1.0 / g.c, rho);
     else
       k_charge_density_runs<false><<<nb, 256, 0, stream>>>(P, q, g.nx, g.ny, g.nz, 1.0 / g.c, rho);
-    return;
+  } else {
+    k_charge_density<<<nb, 256, 0, stream>>>(P, q, g.nx, g.ny, g.nz, 1.0 / g.c, with_gamma, rho);
   }
-  k_charge_density<T><<<(unsigned)((P.n + 255) / 256), 256, 0, stream>>>(P, q, g.nx, g.ny, g.nz, 1.0 / g.c,
-                                                                         with_gamma, rho);
 }
 
 template <typename T>

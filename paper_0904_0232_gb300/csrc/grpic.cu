@@ -1603,17 +1603,15 @@ std::vector<InstDesc<T>> batch_descs(grpic_batch* b) {
     for (int s = 0; s < kMaxSpecies; ++s) {
       SpeciesStore& S = c->sp[s];
       SpeciesDesc<T>& SD = D.sp[s];
-      SD.active = b->pair_of[4 * i + s] >= 0 ? 1 : 0;
-      SD.qm = S.qm;
-      SD.qmacro = S.qmacro;
       SD.C = make_consts<T>(c->g, Species{S.qm, S.qmacro});
       SD.cur = b->cur + 4 * i + s;
       SD.bin_base = 0;
-      if (!SD.active) continue;
+      const int pair = b->pair_of[4 * i + s];
+      if (pair < 0) continue;
       SD.buf[0] = particles_view<T>(c, s, 0);
       SD.buf[1] = particles_view<T>(c, s, 1);
       // (the bound of the tables: the live count on the device decides)
-      SD.buf[0].n = SD.buf[1].n = S.loaded ? b->pair_n[b->pair_of[4 * i + s]] : 0;
+      SD.buf[0].n = SD.buf[1].n = S.loaded ? b->pair_n[pair] : 0;
       SD.bin_base = bin_base;
       bin_base += c->g.ncell + 1;
     }

@@ -211,12 +211,7 @@ struct FastOps64 {
     const double s = x * b.y, d = fma(-s, s, x);
     return root_of(x, b, s, d, scaled(b, d));
   }
-  __device__ static __forceinline__ double rsqrt(double x) {
-    const Start b = rsqrt_start(x);
-    const double s = x * b.y, d = fma(-s, s, x);
-    return rsqrt_of(b, d, scaled(b, d), fma(-s, b.y, 1.0));
-  }
-  // root(x) and its reciprocal rsqrt(x)
+  // root(x), and its reciprocal to *ri
   __device__ static __forceinline__ double root_and_rsqrt(double x, double* ri) {
     const Start b = rsqrt_start(x);
     const double s = x * b.y, d = fma(-s, s, x);
@@ -342,7 +337,12 @@ __device__ __forceinline__ Kerr<double> kerr_eval_fast(double x, double y, doubl
   return kerr_eval_fast(x, y, z, 2.0 * m, a, a2, 4.0 * a2);
 }
 
-// christoffel_uu (below) in FP64 without forming d_i k_j.  With u.r = u^i d_i r, k_x = (r x - a y) / rho^2 and so on,
+// Gamma^a_mn u^m u^n = g^ab (u^m d_m g_bn u^n - 1/2 d_b g_mn u^m u^n) for g = eta + f k k.
+// With s = k.u, D_b = u^m d_m k_b, E_b = u^n d_b k_n and d_4 = 0:
+//   w_b = (u.df) s k_b + f s D_b + f (u.D) k_b - 1/2 s^2 d_b f - f s E_b
+//   Gamma u u = eta^ab w_b - f k^a (k^b w_b)
+// with grad r from the implicit quartic, r_x = x r / D, r_y = y r / D, r_z = z (r^2 + a^2) / (r D), and without forming
+// d_i k_j: with u.r = u^i d_i r, k_x = (r x - a y) / rho^2 and so on,
 //   D_x = [x u.r + r u^x - a u^y - 2 r (u.r) k_x] / rho^2,  D_y alike,  D_z = (u^z - k_z u.r) / r,
 //   E_j = A d_j r + ((r u^x + a u^y) / rho^2, (r u^y - a u^x) / rho^2, u^z / r)_j,
 //   A = [u^x x + u^y y - 2 r (u^x k_x + u^y k_y)] / rho^2 - u^z k_z / r,
@@ -382,67 +382,6 @@ __device__ __forceinline__ void christoffel_uu_fast(const Kerr<double>& K, doubl
   out[1] = fma(-fk, k1, w1);
   out[2] = fma(-fk, k2, w2);
   out[3] = fk - c1;
-}
-
-// Gamma^a_mn u^m u^n = g^ab (u^m d_m g_bn u^n - 1/2 d_b g_mn u^m u^n) for g = eta + f k k.
-// With s = k.u, D_b = u^m d_m k_b, E_b = u^n d_b k_n and d_4 = 0:
-//   w_b = (u.df) s k_b + f s D_b + f (u.D) k_b - 1/2 s^2 d_b f - f s E_b
-//   Gamma u u = eta^ab w_b - f k^a (k^b w_b)
-template <typename S, typename Ops = IeeeOps>
-__device__ __forceinline__ void christoffel_uu(const Kerr<S>& K, S x, S y, S z, S a, const S u[4], S out[4]) {
-  if (K.flat) {
-    out[0] = out[1] = out[2] = out[3] = S(0);
-    return;
-  }
-  const S r = K.r, f = K.f;
-  const S k0 = K.k0, k1 = K.k1, k2 = K.k2;
-  const S r2 = r * r, a2 = a * a;
-  const S inv_rho2 = K.inv_rho2;
-  const S inv_D = K.inv_D;
-  const S inv_r = K.inv_r;
-  // grad r from the implicit quartic: r_x = x r / D, r_y = y r / D, r_z = z (r^2 + a^2) / (r D)
-  const S rx = x * r * inv_D;
-  const S ry = y * r * inv_D;
-  const S rz = z * (r2 + a2) * inv_D * inv_r;
-  // grad f: df/dr = f (3/r - 4 r^3/Sigma), df/dz|_r = -2 a^2 z f / Sigma, Sigma = r^4 + a^2 z^2
-  const S inv_sig = K.inv_sig;
-  const S fr = f * (S(3) * inv_r - S(4) * r2 * r * inv_sig);
-  const S fx = fr * rx;
-  const S fy = fr * ry;
-  const S fz = fr * rz - S(2) * a2 * z * f * inv_sig;
-  // Jacobian J[i][j] = d_i k_j
-  const S ri[3] = {rx, ry, rz};
-  S Jk[3][3];
-#pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    const S tr = S(2) * r * ri[i];
-    Jk[i][0] = (x * ri[i] + (i == 0 ? r : S(0)) - (i == 1 ? a : S(0)) - tr * k0) * inv_rho2;
-    Jk[i][1] = (y * ri[i] + (i == 1 ? r : S(0)) + (i == 0 ? a : S(0)) - tr * k1) * inv_rho2;
-    Jk[i][2] = ((i == 2 ? S(1) : S(0)) - k2 * ri[i]) * inv_r;
-  }
-  const S s = k0 * u[0] + k1 * u[1] + k2 * u[2] + u[3];
-  const S uf = u[0] * fx + u[1] * fy + u[2] * fz;
-  S Dv[3], Ev[3];
-#pragma unroll
-  for (int j = 0; j < 3; ++j) {
-    Dv[j] = u[0] * Jk[0][j] + u[1] * Jk[1][j] + u[2] * Jk[2][j];
-    Ev[j] = u[0] * Jk[j][0] + u[1] * Jk[j][1] + u[2] * Jk[j][2];
-  }
-  const S uD = u[0] * Dv[0] + u[1] * Dv[1] + u[2] * Dv[2];
-  const S fg[3] = {fx, fy, fz};
-  const S kv[3] = {k0, k1, k2};
-  const S c1 = uf * s + f * uD;  // coefficient of k_b in w_b (and w_4 itself)
-  const S fs = f * s;
-  const S hs2 = S(0.5) * s * s;
-  S w[3];
-#pragma unroll
-  for (int j = 0; j < 3; ++j) w[j] = c1 * kv[j] + fs * (Dv[j] - Ev[j]) - hs2 * fg[j];
-  const S w3 = c1;
-  const S kw = k0 * w[0] + k1 * w[1] + k2 * w[2] - w3;
-  out[0] = w[0] - f * k0 * kw;
-  out[1] = w[1] - f * k1 * kw;
-  out[2] = w[2] - f * k2 * kw;
-  out[3] = -w3 + f * kw;
 }
 
 // Field tensor at a point from the prognostic pair: covariant b = (F_yz, F_zx, F_xy) and

@@ -104,7 +104,7 @@ __device__ __forceinline__ Kerr<float> kerr_far(float x, float y, float z, float
   return K;
 }
 
-// Gamma^a_mn u^m u^n of christoffel_uu (metric.cuh) in FP32, the x and y components of its
+// Gamma^a_mn u^m u^n (as christoffel_uu_fast, metric.cuh) in FP32, the x and y components of its
 // 3-vectors, and of each row of the Jacobian d_i k_j, as packed pairs.
 __device__ __forceinline__ void christoffel_uu_x2(const Kerr<float>& K, float x, float y, float z, float a,
                                                   const float u[4], float out[4]) {
@@ -116,7 +116,7 @@ __device__ __forceinline__ void christoffel_uu_x2(const Kerr<float>& K, float x,
   const float2 kxy = make_float2(K.k0, K.k1), xy = make_float2(x, y);
   const float r2 = r * r, a2 = a * a;
   const float inv_rho2 = K.inv_rho2, inv_D = K.inv_D, inv_r = K.inv_r, inv_sig = K.inv_sig;
-  // grad r (r_x, r_y) = (x, y) r / D, r_z = z (r^2 + a^2) / (r D); grad f as in christoffel_uu
+  // grad r (r_x, r_y) = (x, y) r / D, r_z = z (r^2 + a^2) / (r D); grad f by d_r f and d_z f
   const float2 rxy = mul2(xy, f2(r * inv_D));
   const float rz = z * (r2 + a2) * inv_D * inv_r;
   const float fr = f * (3.f * inv_r - 4.f * r2 * r * inv_sig);
