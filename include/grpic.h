@@ -300,7 +300,8 @@ grpic_status grpic_gauss_residual(grpic_ctx* ctx, double* res, int mem, double* 
  *              kernel pushes the rest
  *   far_min_blocks:     4, 5 or 6 resident 128-thread blocks per SM for the far-field (split = 1)
  *                       or per-warp (split = 0: 4 or 5) kernel at Q = 2 (register budget 128,
- *                       96, 80 per thread); other Q use fixed choices
+ *                       96, 80 per thread); other Q use fixed choices, and so do launches of at most 311296
+ *                       particles without j_tile (split = 0), which run as one-warp blocks at 128 registers
  *   near_blocks_per_sm: persistent blocks per SM of the near-hole kernel (>= 1)
  *   sort_interval:      counting sort every k timesteps (>= 1)
  *   overlap:            split = 1 only, as above
@@ -310,7 +311,8 @@ grpic_status grpic_gauss_residual(grpic_ctx* ctx, double* res, int mem, double* 
  *                       groups of G consecutive chunks, spreading the near-hole (FP64-heavy) chunks over
  *                       the launch while each group keeps neighbouring cells together (larger G: more
  *                       L2 locality, less even FP64 load), the chunks of both ends of the cell order last;
- *                       small launches go from the middle of the cell order outwards; 0 keeps them in order
+ *                       launches of at most 311296 particles go from the middle of the cell order outwards
+ *                       whatever G; 0 keeps them in order
  *   area_table:         split = 0, Q = 2, j_tile = 0 (with j_tile = 1 refused), FP32_MIXED (FP64 contexts
  *                       keep it and ignore it, like the other push shapes): 1 takes the face AREAs of Eq. 18
  *                       for far-field warps from per-cell polynomial fits of the integrand instead of
@@ -381,17 +383,18 @@ grpic_status grpic_sort_particles_static(int nx, int ny, int nz, int64_t n, cons
                                          int64_t* n_out, void* stream);
 
 /* ---------------------------------------------------------------------------------------
- * Batched engine: many independent contexts advanced together.  Each stage of the timestep
- * is one persistent launch over all (instance, work item) pairs read from a device table;
- * the per-step stage sequence is captured once in a CUDA graph and replayed.
+ * Batched engine: many independent contexts advanced together.  The stages of the timestep but the
+ * FP32-mixed push are launches over all (instance, work item) pairs read from a device table; that push
+ * is the single-context kernel per instance and species, on parallel branches.  The per-step stage
+ * sequence is captured once in a CUDA graph and replayed.
  * Not in the paper: it runs the paper's cycle for several simulations at once.
  * ------------------------------------------------------------------------------------- */
 typedef struct grpic_batch grpic_batch;
 
 /* Group n contexts with the same precision, quadrature order and field-update form.  The
  * batch builds one device descriptor per instance and tables of (instance, work block) items
- * for every stage; each batched stage is one launch over such a table (persistent grid-stride
- * for the field and sort stages, one block per item for the push), and one step's stage sequence
+ * for every stage (one block per item for the fields and the FP64 push, persistent grid-stride for
+ * zeroing J and the sort), and one step's stage sequence
  * is captured once in a CUDA graph on a stream the batch owns (`stream` is unused).  The
  * contexts stay owned by the caller and must outlive every grpic_batch_step and
  * grpic_batch_info of the batch; grpic_batch_destroy touches none of them (the batch keeps its own
@@ -409,7 +412,7 @@ grpic_status grpic_batch_step(grpic_batch* b, int nsteps);
 /* Kernels launched per batched step, and the total number of work blocks in the stage tables. */
 grpic_status grpic_batch_info(grpic_batch* b, int64_t* kernels_per_step, int64_t* work_blocks);
 
-/* Persistent blocks per SM of the batch's launches (1..32, default 8; what the autotuner
+/* Persistent blocks per SM of the batch's grid-stride launches (1..32, default 8; what the autotuner
  * chooses).  Takes effect at the next grpic_batch_step, which captures the graph again. */
 grpic_status grpic_batch_set_blocks_per_sm(grpic_batch* b, int blocks_per_sm);
 

@@ -133,8 +133,8 @@ struct BStepArgs {
 };
 
 // E step: d_out = d + coef (4 pi/c J - div h(b, x)) at advanced edge locations, d copied elsewhere.  Time-centred: a
-// launch with x = d, coef = dx4 / 2 gives the midpoint predictor d*, a second with x = d*, coef = dx4 the new d (relaxed
-// toward tgt in the absorbing layers when tgt is set); literal: one launch with x = d, coef = dx4.
+// launch with x = d, coef = dx4 / 2 gives the midpoint predictor d*, a second with x = d*, coef = dx4 the new d
+// (relaxed toward tgt in the absorbing layers when tgt is set); literal: one launch with x = d, coef = dx4.
 template <typename T>
 struct EStepArgs {
   const T* b[3];
@@ -285,8 +285,8 @@ void launch_area_table(const Grid& g, float4* tab, cudaStream_t st);
 
 // Split FP32-mixed push.  near_radius: particles with R(x_n) below it are classified near
 // (marked kNear, listed; count[0] = list length, count[1] = work cursor) and pushed by
-// launch_push_near (nblocks persistent blocks; new sort keys to keys[slot]); the rest by launch_push_far (FP32 only; minb selects
-// the register budget), concurrently.  launch_near_keys then copies keys[slot] to P.key.
+// launch_push_near (nblocks persistent blocks; new sort keys to keys[slot]); the rest by launch_push_far (FP32 only;
+// minb selects the register budget), concurrently.  launch_near_keys then copies keys[slot] to P.key.
 void launch_classify_near(const Grid& g, const Particles<float>& P, uint32_t* list, int* count,
                           cudaStream_t stream);
 void launch_push_far(const Grid& g, const Fields<float>& F, const Particles<float>& P, const Species& sp,
@@ -302,17 +302,21 @@ unsigned coprime_multiplier(unsigned n);
 // Block -> work-chunk map of the push launches: groups of 2^lg consecutive chunks are permuted,
 // group g -> g * perm mod (number of full groups), perm coprime to that number (1 keeps the order;
 // a partial last group stays in place).  With `tail` groups at either end set apart, the others are permuted among
-// themselves and go first, the lower end's and the upper end's after them.  perm = 0: from the middle outwards.  Cell-sorted particles put the FP64-heavy chunks near the
-// hole in one contiguous run; the permutation spreads them over the whole launch, so the FP64
-// pipes of all SMs share that work alongside FP32 work, while the blocks of a group, which run at
-// about the same time, keep neighbouring cells together (their field stencils and J nodes stay in
+// themselves and go first, the lower end's and the upper end's after them.  perm = 0: from the middle outwards.
+// Cell-sorted particles put the FP64-heavy chunks near the hole in one contiguous run; the permutation spreads them
+// over the whole launch, so the FP64 pipes of all SMs share that work alongside FP32 work, while the blocks of a
+// group, which run at about the same time, keep neighbouring cells together (their field stencils and J nodes stay in
 // L2).  Larger groups favour that locality, smaller ones the spreading of FP64 work.
 __device__ __forceinline__ unsigned spread_chunk(unsigned b, unsigned n, unsigned perm, int lg, unsigned tail = 0) {
   if (perm == 0u) return b & 1u ? (n - 1) / 2 + (b + 1) / 2 : (n - 1) / 2 - b / 2;
   const unsigned nfull = n >> lg;
   if (perm == 1u || b >= (nfull << lg)) return b;
   const unsigned mask = (1u << lg) - 1u, main = nfull - 2 * tail, i = b >> lg;
-  const unsigned group = i < main ? tail + (unsigned)(((unsigned long long)i * perm) % main) : i - main < tail ? i - main : i;
+  unsigned group = i;
+  if (i < main)
+    group = tail + (unsigned)(((unsigned long long)i * perm) % main);
+  else if (i - main < tail)
+    group = i - main;
   return (group << lg) | (b & mask);
 }
 inline unsigned spread_multiplier(unsigned n, int lg, unsigned tail = 0) {
@@ -328,12 +332,13 @@ inline int spread_log2(int group) {
 }
 // A push launch of few blocks: warps near the hole take several times as long as the others (FP64 pipe), so where an SM
 // gets only a handful of warps, blocks of one warp (a register file holds as many warps of them) spread the near ones
-// over the SMs, and another species' launch runs beside it (grpic.cu).  Larger launches keep blocks of four warps, whose
-// common cells stay in L1.
+// over the SMs, and another species' launch runs beside it (grpic.cu).  Larger launches keep blocks of four warps,
+// whose common cells stay in L1.
 // Measured, us per push stage, 128-thread blocks one after another / small launches as here: 2 x 46 K particles at 32^3
 // 228 / 105 (FP64 695 / 603), 2 x 400 K + 2 x 85 K at 64 x 64 x 128 380 / 238; blocks of one warp for 2 x 0.9 M
 // particles at 64^3 cost 1142 instead of 941.
-constexpr long long kSmallPush = 311296;  // 4 waves of 128-thread blocks at 4 an SM
+constexpr unsigned kSms = 152;  // of the GB300, on which this line and kTailWaves (push_far.cu) were measured
+constexpr long long kSmallPush = 4ll * kSms * 4 * 128;  // 4 waves of 128-thread blocks at 4 an SM: 311296
 inline bool small_push(long long n) { return n <= kSmallPush; }
 // Unsplit alternative: one launch, far-field or FP32-mixed code chosen per warp by the same
 // near_radius criterion.  atab (non-null, Q = 2, no tile): far-field warps deposit with the
@@ -366,8 +371,8 @@ void launch_max_id(const Particles<T>& P, unsigned long long* max_id, cudaStream
 size_t invariant_acc_bytes();
 constexpr int kInvariantStride = 64;  // tracked subsample: ids divisible by this
 
-// Counting sort by cell of the species of a context; removed particles (key == kDead) are dropped.  bins: ncell + 1 ints,
-// zero on entry; tiles: scan_tiles(ncell + 1) ints; n_out: the live count (device).
+// Counting sort by cell of the species of a context; removed particles (key == kDead) are dropped.  bins: ncell + 1
+// ints, zero on entry; tiles: scan_tiles(ncell + 1) ints; n_out: the live count (device).
 template <typename T>
 struct SortJob {
   Particles<T> src, dst;

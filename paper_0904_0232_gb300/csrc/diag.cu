@@ -62,8 +62,8 @@ __global__ void k_charge_density(const Particles<double> P, double q, int nx, in
   cloud64(P, i, q, nx, ny, nz, inv_c, with_gamma, rho);
 }
 
-// v = (hi 2^64 + lo) 2^-s in FP64, v > 0 and below 2^(32 W), rounded once (halves upwards): the integers become the bits of
-// the result, since conversions would run on the FP64 pipe.
+// v = (hi 2^64 + lo) 2^-s in FP64, v > 0 and below 2^(32 W), rounded once (halves upwards): the integers become the
+// bits of the result, since conversions would run on the FP64 pipe.
 template <int W>
 __device__ __forceinline__ double scaled_double(unsigned long long hi, unsigned long long lo, int s) {
   unsigned w[4] = {(unsigned)lo, (unsigned)(lo >> 32), (unsigned)hi, (unsigned)(hi >> 32)};
@@ -77,22 +77,24 @@ __device__ __forceinline__ double scaled_double(unsigned long long hi, unsigned 
       top -= 32;
     }
   const int lz = __clz(w[W - 1]);
-  const unsigned m1 = __funnelshift_l(w[W - 2], w[W - 1], lz), m0 = __funnelshift_l(W > 2 ? w[W - 3] : 0u, w[W - 2], lz);
+  const unsigned m1 = __funnelshift_l(w[W - 2], w[W - 1], lz);
+  const unsigned m0 = __funnelshift_l(W > 2 ? w[W - 3] : 0u, w[W - 2], lz);
   // the leading one of m1 >> 11 adds 1 to the exponent field
   const unsigned long long m = ((unsigned long long)m1 << 21 | m0 >> 11) + ((m0 >> 10) & 1u);
   return __longlong_as_double((long long)m + ((long long)((1022 + top - lz - s) << 20) << 32));
 }
 
-// FP32 positions.  One FP64 warp instruction takes 16 cycles of an SM, and the eight weights of a particle, its floors and
-// conversions took about 36 of them besides eight atomics.  But a weight of an FP32 coordinate x >= 1 is an integer multiple
-// of 2^-23, so the sum of a node's weights over the particles of a cell is an exact integer (69 bits, with gamma 32 more),
-// rounded once when it is complete.  A warp finds the runs of equal cells among its particles (after a sort nearly all
-// particles of a cell) and cuts them to kRun; a few lanes take a run from shared memory: one FP64 multiplication and one
-// atomic a node for up to kRun particles.  Without gamma four lanes a run, each an x pair of its nodes (the lower node's sum
-// is that of w_y w_z less the upper's); with gamma eight, for the wider products make the pair slower (136 us for 123 below).
-// kRun = 8: the sums stay in 64-bit parts, and with 8 particles a cell the 4 or 5 runs of a warp fill its lanes.
-// gamma: u^4 as a 32-bit integer times a power of two common to the warp, exact while the exponents of its particles lie
-// within 8.  A warp with a wider range, or a coordinate below 1 or beyond the last cell, takes cloud64.
+// FP32 positions.  One FP64 warp instruction takes 16 cycles of an SM, and the eight weights of a particle, its
+// floors and conversions took about 36 of them besides eight atomics.  But a weight of an FP32 coordinate x >= 1 is
+// an integer multiple of 2^-23, so the sum of a node's weights over the particles of a cell is an exact integer (69
+// bits, with gamma 32 more), rounded once when it is complete.  A warp finds the runs of equal cells among its
+// particles (after a sort nearly all particles of a cell) and cuts them to kRun; a few lanes take a run from shared
+// memory: one FP64 multiplication and one atomic a node for up to kRun particles.  Without gamma four lanes a run,
+// each an x pair of its nodes (the lower node's sum is that of w_y w_z less the upper's); with gamma eight, for the
+// wider products make the pair slower (136 us for 123 below).  kRun = 8: the sums stay in 64-bit parts, and with 8
+// particles a cell the 4 or 5 runs of a warp fill its lanes.
+// gamma: u^4 as a 32-bit integer times a power of two common to the warp, exact while the exponents of its particles
+// lie within 8.  A warp with a wider range, or a coordinate below 1 or beyond the last cell, takes cloud64.
 // Bound by instruction issue (73 % of the slots).  Measured (6.4 M particles a species, 8 a cell, 96^3): 487 -> 82 us a
 // species, with gamma 123.
 constexpr int kRun = 8;
@@ -163,7 +165,8 @@ __global__ void __launch_bounds__(256)
     unsigned long long hi = 0, lo = 0, sum = 0, sum_hi = 0;
     for (int p = first; p < first + len; ++p) {
       const uint4 w = s_w[warp][p];
-      const unsigned long long a = (unsigned long long)(unsigned)((int)w.y * sgy + ofy) * (unsigned)((int)w.z * sgz + ofz);
+      const unsigned wy = (unsigned)((int)w.y * sgy + ofy), wz = (unsigned)((int)w.z * sgz + ofz);
+      const unsigned long long a = (unsigned long long)wy * wz;
       if (GAMMA) {
         const unsigned long long b = (unsigned long long)(unsigned)((int)w.x * sgx + ofx) * w.w, l = a * b;
         lo += l;

@@ -10,27 +10,25 @@
 // (Eqs. 4-6), |k| = 1 and G = f / (1 + f), lowering the tensor of Eq. 8 and eliminating gives
 //   e = -d + G [k x b + d - k (k.d)],      h = b - G [b + d x k - k (k.b)]
 // (from h = [b - f d x k + f k (k.b)] / (1 + f) and e = f k x h + (f - 1) d - f k (k.d): the k (k.b) and
-// k (k.(d x k)) terms vanish in k x h).  e_L needs neither b_L nor its eight-point mean, and h splits into a
-// part of b alone and G d x k, so the E step forms the b part and G k once for its two conversions.
+// k (k.(d x k)) terms vanish in k x h).  e_L needs neither b_L nor its eight-point mean.
 //
-// One launch per update.  A block owns a 32 x BY patch of (x, y) columns and marches up z through
-// a chunk of planes: it evaluates the conversion for the whole patch of the next plane into
-// shared memory and updates the cells whose stencil lies inside the patch.  Neighbouring patches
-// overlap by the stencil's reach (1 cell for the B step; 3 for the time-centred E step, whose
-// midpoint predictor d* = d + (dx4/2) rhs(b, d) is converted again before the update), so each
-// cell is written exactly once by one block, from inputs that no block of the launch modifies.
-// The output is the other buffer of a ping-pong pair (every cell written; a copy where the
-// location is not advanced), except the time-centred second B half-step, which overwrites the
-// b^{n-1/2} buffer it reads only at the cell it writes.  Per cell the launch moves the
-// prognostic words once: the conversions and the predictor live in registers and shared memory,
+// A B half-step is one launch, and so is the literal E step; the time-centred E step is two, the midpoint predictor
+// d* = d + (dx4/2) rhs(b, d) into memory that is free by then (the idle b buffer) and the update from h(b, d*).
+// A block owns a 32 x BY patch of (x, y) columns and marches up z through a chunk of planes: it evaluates the
+// conversion for the whole patch of the next plane into shared memory and updates the cells whose stencil lies inside
+// the patch.  Neighbouring patches overlap by the stencil's reach, one cell, so each cell is written exactly once by
+// one block, from inputs that no block of the launch modifies.  The output is another buffer than the inputs
+// (every cell written; a copy where the location is not advanced), except the time-centred second B half-step, which
+// overwrites the b^{n-1/2} buffer it reads only at the cell it writes.  Per cell a launch moves the words that it reads
+// and writes once: the conversions live in registers and shared memory,
 // and in FP32 the metric is evaluated where it is needed instead of being read from memory (48 B per cell and step, as
 // much as the fields themselves).  In FP64 it is read from a table (launch_metric_table): its 40 operations at each
 // of three locations are two thirds of the kernel's, and the FP64 pipe takes longer for them than HBM for 96 B
 // (B step at 96^3: 420 us evaluated, 138 us read).
 //
 // What bounds them: FP32 the issue of instructions, FP64 the FP64 pipe.  Hence sums over pairs of planes are
-// carried from one plane of the march to the next instead of being formed again, a patch synchronises once
-// (B) or twice (E) a plane, and FP64 reciprocals and roots are FastOps64's.
+// carried from one plane of the march to the next instead of being formed again, a patch synchronises once a plane,
+// and FP64 reciprocals and roots are FastOps64's.
 // Measured (GB300, microseconds a launch, no layers; before: the E step as one march with a halo of 3, IEEE FP64
 // divides and roots, the metric evaluated in FP64, patches over all cells and chunks of at least 4 planes):
 //            FP32 64^3   128^3      192^3       64x64x128   FP64 32^3    64^3         96^3
@@ -161,8 +159,8 @@ __device__ __forceinline__ T edge_e(const Pt<T>& P, T dL, T sdM, T sdN, T sbM, T
   return fma(G, t, -dL);
 }
 
-// h_Q at a face: bQ is b_Q there, sbM, sbN the sums of the four nearest points of the other two b components (M = Q + 1,
-// N = Q + 2 mod 3), sdM, sdN the sums of the two nearest points of d_M and d_N; (d x k)_Q = d_M k_N - d_N k_M.
+// h_Q at a face: bQ is b_Q there, sbM, sbN the sums of the four nearest points of the other two b components (M = Q +
+// 1, N = Q + 2 mod 3), sdM, sdN the sums of the two nearest points of d_M and d_N; (d x k)_Q = d_M k_N - d_N k_M.
 // FP64: b_Q - G [b_Q - k_Q (k.b) + (d x k)_Q].
 // FP32: [b_Q - f (d x k)_Q + f k_Q (k.b)] / (1 + f) as it stands.  Where b is large beside d (a strong
 // uniform field), d is what the differences of these h leave of their rounding to FP32, so another form of equal
@@ -286,9 +284,10 @@ __device__ __forceinline__ void cp_async_wait() {
 
 // The staged halo patch of a block: (BY + 2) x kSX elements, at most two per thread (threads
 // 32 x BY); element e of the patch is column e % kSX, row e / kSX, at grid (x0 - 1 + column,
-// y0 - 1 + row) where (x0, y0) is the grid position of thread (0, 0).  Columns and rows beyond the grid are left out, and
-// planes beyond it take the nearest one: only cells of the outer index layer reach them, and those are not converted.
-// (Copies that clamp the columns too, many lanes reading one address, made a patch at a grid's edge twice as slow.)
+// y0 - 1 + row) where (x0, y0) is the grid position of thread (0, 0).  Columns and rows beyond the grid are left out,
+// and planes beyond it take the nearest one: only cells of the outer index layer reach them, and those are not
+// converted.  (Copies that clamp the columns too, many lanes reading one address, made a patch at a grid's edge twice
+// as slow.)
 template <int BY>
 struct Stager {
   int s0, s1;       // element in a staged component; negative: none
@@ -317,8 +316,8 @@ struct Stager {
   }
 };
 
-// The outer two index layers are never advanced: a step into another buffer copies them, each block its share (blocks of
-// their own beside the patches filled both slots of an SM with patches while other SMs had none: FP64 at 64^3 80 us
+// The outer two index layers are never advanced: a step into another buffer copies them, each block its share (blocks
+// of their own beside the patches filled both slots of an SM with patches while other SMs had none: FP64 at 64^3 80 us
 // instead of 46).  Cells by index: the z layers, then the y layers of the planes between them, then the x layers of the
 // rows between those.
 __device__ __forceinline__ int outer_layer(int q, int n) { return q < 2 ? q : n - 4 + q; }  // q = 0..3
@@ -504,9 +503,9 @@ __device__ __forceinline__ void b_step_tile(const Grid& g, const BStepArgs<T>& A
 // (One launch for both, with h of d and of d* in one march, overlaps patches by 3 cells instead of 1 and needs
 // two barriers a plane and 80 registers: slower at every size, see the figures above.)
 // Patch: threads (tx, ty) at x = x0 + tx, y = y0 + ty, h at the patch of each plane of the chunk and of the plane
-// below it; cells with tx >= 1 and ty >= 1 are updated (the divergence reaches -1).  Iteration q reads the staged planes
-// q and q + 1 (q + 2 in flight) for h of plane q and updates plane q - 1 from the h that the last iteration left in
-// the other half of H: one barrier a plane.
+// below it; cells with tx >= 1 and ty >= 1 are updated (the divergence reaches -1).  Iteration q reads the staged
+// planes q and q + 1 (q + 2 in flight) for h of plane q and updates plane q - 1 from the h that the last iteration
+// left in the other half of H: one barrier a plane.
 template <typename T, int BY>
 struct EStepSmem {
   Plane3<T, BY> Sb[4], Sx[4];
@@ -667,14 +666,16 @@ TileGrid tile_grid(const Grid& g, int rows, int slots, double* cost_out = nullpt
 }
 
 template <typename T, int BY>
-__global__ void __launch_bounds__(kTX * BY, patch_blocks(sizeof(T), BY)) k_b_step(const Grid g, const BStepArgs<T> A, const TileGrid t) {
+__global__ void __launch_bounds__(kTX * BY, patch_blocks(sizeof(T), BY))
+    k_b_step(const Grid g, const BStepArgs<T> A, const TileGrid t) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   auto& sm = *reinterpret_cast<BStepSmem<T, BY>*>(smem_raw);
   b_step_tile<T, BY>(g, A, t, blockIdx.x, sm);
 }
 
 template <typename T, int BY>
-__global__ void __launch_bounds__(kTX * BY, patch_blocks(sizeof(T), BY)) k_e_step(const Grid g, const EStepArgs<T> A, const TileGrid t) {
+__global__ void __launch_bounds__(kTX * BY, patch_blocks(sizeof(T), BY))
+    k_e_step(const Grid g, const EStepArgs<T> A, const TileGrid t) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   auto& sm = *reinterpret_cast<EStepSmem<T, BY>*>(smem_raw);
   e_step_tile<T, BY>(g, A, t, blockIdx.x, sm);

@@ -80,8 +80,8 @@ struct grpic_ctx {
   int* bins2 = nullptr;          // sort bins of species 2 and 3 (those of 0 and 1 follow J)
   SpeciesStore sp[kMaxSpecies];
   long long steps = 0;
-  long long pushes = 0;
-  grpic_status step_status = GRPIC_OK;  // status of this context after the last batched step  // push stages run: particle x^4 is stored relative to c dt * pushes
+  long long pushes = 0;  // push stages run: particle x^4 is stored relative to c dt * pushes
+  grpic_status step_status = GRPIC_OK;  // status of this context after the last batched step
   int since_sort = 0;
   grpic_stats totals{};
   // invariant baselines: per species E and L of the tracked particles, by id / stride
@@ -154,16 +154,17 @@ bool capturing(cudaStream_t st) {
   return cs != cudaStreamCaptureStatusNone;
 }
 
-// The table for launches that are enqueued while `use` lives, or null (the kernels then evaluate the metric: the same bits).
+// The table for launches that are enqueued while `use` lives, or null (the kernels then evaluate the metric: the same
+// bits).
 const double2* metric_table(grpic_ctx* c, std::unique_lock<std::mutex>& use) {
   if (c->mixed) return nullptr;
   use = std::unique_lock<std::mutex>(c->met.mu);
   return c->met.p && !capturing(c->stream) ? c->met.p : nullptr;
 }
 
-// The table costs 192 B a cell, more than the fields, J and flags of an FP64 context together (122 B): it is taken where
-// that is at most an eighth of the free memory, so that little is lost to programs beside the library, which cannot have it
-// given up.
+// The table costs 192 B a cell, more than the fields, J and flags of an FP64 context together (122 B): it is taken
+// where that is at most an eighth of the free memory, so that little is lost to programs beside the library, which
+// cannot have it given up.
 constexpr size_t kTableShare = 8;
 void create_metric_table(grpic_ctx* c) {
   const size_t bytes = sizeof(double2) * kMetricPlanes * (size_t)c->g.ncell;
@@ -298,12 +299,12 @@ void enqueue_rho(grpic_ctx* c, bool with_gamma, double* rho) {
 // The area fits the per-warp select push uses, or null.
 const float4* area_table_of(const grpic_ctx* c) { return c->tune.area_table ? c->atab : nullptr; }
 
-// One push launch per species, launch(species, stream).  The smaller half of them go to the side stream, ahead of and beside
-// the others (all add into J atomically), and the context stream waits for them: small launches (small_push) do not fill the
-// GPU, and the blocks of one take the SMs that the last blocks of another leave idle.  The buffers belong to the context
-// stream, which is joined before anything else uses them.
-// Large ones beside each other, us per push stage: 2 x 2.1 M particles at 64^3 840 -> 831, 2 x 1.6 M at 75 x 50 x 91, Q = 3,
-// 927 -> 914, 2 x 16.8 M at 128^3 5715 -> 5705.
+// One push launch per species, launch(species, stream).  The smaller half of them go to the side stream, ahead of and
+// beside the others (all add into J atomically), and the context stream waits for them: small launches (small_push)
+// do not fill the GPU, and the blocks of one take the SMs that the last blocks of another leave idle.  The buffers
+// belong to the context stream, which is joined before anything else uses them.
+// Large ones beside each other, us per push stage: 2 x 2.1 M particles at 64^3 840 -> 831, 2 x 1.6 M at 75 x 50 x 91,
+// Q = 3, 927 -> 914, 2 x 16.8 M at 128^3 5715 -> 5705.
 template <typename Launch>
 void enqueue_species_pushes(grpic_ctx* c, Launch launch) {
   int order[kMaxSpecies], n = 0;
@@ -462,8 +463,8 @@ void enqueue_stage(grpic_ctx* c, int stage) {
       c->pushes += 1;
       break;
     case GRPIC_STAGE_E: {
-      // the predictor goes to the idle b buffer (b^n: the next first half-step writes all of it), or to planes of its own
-      // where that buffer is still to be read (grpic_stage)
+      // the predictor goes to the idle b buffer (b^n: the next first half-step writes all of it), or to planes of its
+      // own where that buffer is still to be read (grpic_stage)
       const bool literal = literal_fields(c);
       EStepArgs<T> A;
       for (int q = 0; q < 3; ++q) {
@@ -604,8 +605,9 @@ grpic_status read_status(grpic_ctx* c) {
   return GRPIC_OK;
 }
 
-// Room for n particles.  Where the stores have to grow, what was loaded goes with them: the species counts as not loaded
-// until the load that asked for them has filled the new ones, so that nothing runs on them should that load fail.
+// Room for n particles.  Where the stores have to grow, what was loaded goes with them: the species counts as not
+// loaded until the load that asked for them has filled the new ones, so that nothing runs on them should that load
+// fail.
 grpic_status ensure_capacity(grpic_ctx* c, int s, long long n) {
   SpeciesStore& S = c->sp[s];
   long long want = std::max<long long>(n, c->cfg.max_particles);
@@ -1163,7 +1165,8 @@ grpic_status grpic_num_particles(grpic_ctx* c, int species, int64_t* n) {
   if (c->since_sort != 0) {
     enqueue_stage_any(c, GRPIC_STAGE_SORT);
     c->since_sort = 0;
-    s = cuda_check(c, cudaMemcpyAsync(&v, S.n_dev + S.cur, sizeof(int), cudaMemcpyDeviceToHost, c->stream), "count copy");
+    s = cuda_check(c, cudaMemcpyAsync(&v, S.n_dev + S.cur, sizeof(int), cudaMemcpyDeviceToHost, c->stream),
+                   "count copy");
     if (s == GRPIC_OK) s = cuda_check(c, cudaStreamSynchronize(c->stream), "count sync");
     if (s != GRPIC_OK) return s;
   }
@@ -1462,7 +1465,8 @@ BatchHeld batch_held(grpic_ctx* c) {
   return h;
 }
 
-// A batched step keeps the tables that its descriptors refer to for as long as it runs; between steps they can be given up.
+// A batched step keeps the tables that its descriptors refer to for as long as it runs; between steps they can be
+// given up.
 struct TableUse {
   const std::vector<grpic_ctx*>& ctxs;
   explicit TableUse(const std::vector<grpic_ctx*>& v) : ctxs(v) { add(1); }
@@ -1502,7 +1506,8 @@ struct grpic_batch {
   int persist_blocks = 0;
   int sms = 1;
   std::vector<TileGrid> tiles_of;  // field patches of each instance
-  // pair of each (instance, species), -1 where nothing was loaded when the batch was built, and the pairs' work upper bound
+  // pair of each (instance, species), -1 where nothing was loaded when the batch was built, and the pairs' work upper
+  // bound
   std::vector<int> pair_of;
   std::vector<long long> pair_n;
   // what the tables and graphs hold of the contexts (a context may be reloaded, retuned or stepped on its own between
@@ -1821,7 +1826,8 @@ grpic_status grpic_batch_create(grpic_ctx* const* ctxs, int n, void* stream, grp
   // kernels per step: B halves 2, zero J 1, push (FP32-mixed: one per pair; FP64: 1), E 2 (literal 1), d parity 1,
   // sort 5 (+2 with particles; and 1 memset)
   const int push_launches = b->npart > 0 ? (b->mixed ? b->npairs : 1) : 0;
-  b->kernels_per_step = 2 + 1 + push_launches + (b->literal ? 1 : 2) + 1 + (b->npairs ? 5 + 2 * (b->npart > 0 ? 1 : 0) : 0);
+  const int sort_launches = b->npairs ? 5 + 2 * (b->npart > 0 ? 1 : 0) : 0;
+  b->kernels_per_step = 2 + 1 + push_launches + (b->literal ? 1 : 2) + 1 + sort_launches;
   *out = b;
   return GRPIC_OK;
 }

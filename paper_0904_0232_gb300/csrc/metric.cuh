@@ -99,28 +99,28 @@ struct SeededOps64 {
   }
 };
 
-// FP64 reciprocal, square root and reciprocal square root, rounded as well as the IEEE operations' to a hundredth of a unit
-// in the last place, with 1, 2 and 3 FP64 operations (3 for a root and its reciprocal together).  This GPU issues
-// one FP64 warp instruction per 16 cycles and SM, 64 times slower than FP32 and integer ones, and its FP64 kernels are
-// bound by their count (IEEE 1/x, sqrt x and 1/sqrt x take about 9, 10 and 20), so everything else is done beside the FP64
-// pipe:
+// FP64 reciprocal, square root and reciprocal square root, rounded as well as the IEEE operations' to a hundredth of
+// a unit in the last place, with 1, 2 and 3 FP64 operations (3 for a root and its reciprocal together).  This GPU
+// issues one FP64 warp instruction per 16 cycles and SM, 64 times slower than FP32 and integer ones, and its FP64
+// kernels are bound by their count (IEEE 1/x, sqrt x and 1/sqrt x take about 9, 10 and 20), so everything else is
+// done beside the FP64 pipe:
 //   1. the argument's mantissa as two floats xh + xl (46 bits), y0 ~ xh^-1/2 (or xh^-1) from the FP32 approximation,
 //      r = 1 - x y0^2 (1 - x y0) in FP32 with fused multiply-adds, whose rounding (2^-24 of r ~ 2^-21) leaves
 //      y = y0 (1 + r/2 + 3 r^2/8) (y0 (1 + r + r^2)) within about 2^-44; the sum is an integer addition to y0's bits;
-//   2. in FP64 the residuals: 1 - x y; with s = x y, x - s^2 and 1 - s y.  s is rounded, s = x y (1 + n), which the first of
-//      these holds twice and the second once: e = 2 (1 - s y) - (x - s^2) / x = 1 - x y^2 to order n^2;
-//   3. the first-order step y (1 + e), s (1 + (x - s^2) / 2x) or y (1 + e/2), whose correction is below 2^12 units in the last
-//      place: formed in FP32, rounded to an integer and added to the bits (in FP64 where either side of that is not in the
-//      result's binade, whose unit it is in).  The truncation is of order e^2.
-// So the result is the exact one rounded, but for the FP32 correction's own error of below 2^-7 units (measured over 5e7
-// arguments: 0.500 units off at most, rms 4.7e-17 relative as IEEE; 1/sqrt x in two IEEE operations 1.49 and 6.7e-17).  Arguments lie in
-// 2^-890 .. 2^890, and root gives 0 for 0 and subnormals.  Others give no useful value, and callers screen them (or use
-// CheckedOps64).
+//   2. in FP64 the residuals: 1 - x y; with s = x y, x - s^2 and 1 - s y.  s is rounded, s = x y (1 + n), which the
+//      first of these holds twice and the second once: e = 2 (1 - s y) - (x - s^2) / x = 1 - x y^2 to order n^2;
+//   3. the first-order step y (1 + e), s (1 + (x - s^2) / 2x) or y (1 + e/2), whose correction is below 2^12 units in
+//      the last place: formed in FP32, rounded to an integer and added to the bits (in FP64 where either side of that
+//      is not in the result's binade, whose unit it is in).  The truncation is of order e^2.
+// So the result is the exact one rounded, but for the FP32 correction's own error of below 2^-7 units (measured over
+// 5e7 arguments: 0.500 units off at most, rms 4.7e-17 relative as IEEE; 1/sqrt x in two IEEE operations 1.49 and
+// 6.7e-17).  Arguments lie in 2^-890 .. 2^890, and root gives 0 for 0 and subnormals.  Others give no useful value,
+// and callers screen them (or use CheckedOps64).
 // Few instructions count as well: the push's two copies of them lie at the limit of the instruction cache.
 struct FastOps64 {
  private:
-  // the upper 23 of a double's mantissa bits under the exponent field `field` of a float, and the 23 after them as a float of
-  // that scale
+  // the upper 23 of a double's mantissa bits under the exponent field `field` of a float, and the 23 after them as a
+  // float of that scale
   __device__ static __forceinline__ void split(int hi, int lo, unsigned field, float* xh, float* xl) {
     *xh = __uint_as_float((__funnelshift_l((unsigned)lo, (unsigned)hi, 3) & 0x7fffffu) | field);
     const unsigned base = field - (23u << 23);
@@ -182,7 +182,8 @@ struct FastOps64 {
     if (!add_units(b.y, e * (b.yf * 0x1p52f), (2045 << 20) - b.r, &v)) v = rsqrt_apart(b.y, d, e1);
     return v;
   }
-  // across a power of two (out of line with their operations, which would be issued, predicated off, for every argument)
+  // across a power of two (out of line with their operations, which would be issued, predicated off, for every
+  // argument)
   __device__ static __noinline__ double rcp_apart(double y, double e) { return fma(y, e, y); }
   __device__ static __noinline__ double root_apart(double s, double d, double y) { return fma(0.5 * y, d, s); }
   __device__ static __noinline__ double rsqrt_apart(double y, double d, double e1) {
@@ -244,7 +245,9 @@ struct CheckedOps64 {
 };
 
 // x / 2 for a positive normal x, without an FP64 operation.
-__device__ __forceinline__ double halve(double x) { return __hiloint2double(__double2hiint(x) - 0x00100000, __double2loint(x)); }
+__device__ __forceinline__ double halve(double x) {
+  return __hiloint2double(__double2hiint(x) - 0x00100000, __double2loint(x));
+}
 
 template <typename S>
 struct Kerr {

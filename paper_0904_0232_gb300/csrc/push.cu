@@ -11,8 +11,8 @@ namespace grpic {
 namespace {
 
 template <typename T, int Q, bool MIXED, int THREADS>
-__global__ void __launch_bounds__(THREADS, 4 * (128 / THREADS)) k_push_deposit(const Grid g, const Fields<T> F, const Particles<T> P,
-                                                           const Consts<T> C, DevStatus* st) {
+__global__ void __launch_bounds__(THREADS, 4 * (128 / THREADS))
+    k_push_deposit(const Grid g, const Fields<T> F, const Particles<T> P, const Consts<T> C, DevStatus* st) {
   const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   unsigned flags = 0, n64 = 0;
   bool active = i < P.n && i < (long long)(*P.n_dev);
@@ -117,14 +117,14 @@ __device__ __forceinline__ bool inside_horizon(const Grid& g, double X, double Y
   return K.flat || K.r <= g.r_plus;
 }
 
-// Completion of u^a from its spatial part.  Covariant u_i (umode 1): g^mn u_m u_n = -c^2 with g^mn = eta^mn - f k^m k^n,
-// k^m = (k_i, -1), is (1 + f) u_4^2 - 2 f (k.u) u_4 - C = 0, C = |u|^2 - f (k.u)^2 + c^2; for its roots
+// Completion of u^a from its spatial part.  Covariant u_i (umode 1): g^mn u_m u_n = -c^2 with g^mn = eta^mn - f k^m
+// k^n, k^m = (k_i, -1), is (1 + f) u_4^2 - 2 f (k.u) u_4 - C = 0, C = |u|^2 - f (k.u)^2 + c^2; for its roots
 // u_4 = [f (k.u) -+ S] / (1 + f), S^2 = f^2 (k.u)^2 + (1 + f) C, u^4 = -u_4 + f (k.u - u_4) is +-S, so the
 // future-directed one has u^4 = S.  Contravariant u^i (umode 2): (1 - f) u4^2 - 2 f (k.u) u4 - C = 0 with
 // C = |u|^2 + f (k.u)^2 + c^2, u^4 = [f (k.u) + S] / (1 - f), S^2 = f^2 (k.u)^2 + (1 - f) C.
-// The load is bound by the FP64 pipe: one FP64 evaluation of the metric by FastOps64 and 20 operations a particle (two IEEE
-// evaluations and the two roots of each quadratic before: 5.1 ms for 15.6 M particles of an FP32-mixed context; 2.2 ms with
-// the constants formed and the signs compared in FP64 as well; now 2.0 ms).
+// The load is bound by the FP64 pipe: one FP64 evaluation of the metric by FastOps64 and 20 operations a particle
+// (two IEEE evaluations and the two roots of each quadratic before: 5.1 ms for 15.6 M particles of an FP32-mixed
+// context; 2.2 ms with the constants formed and the signs compared in FP64 as well; now 2.0 ms).
 // FP64 products of the grid's constants, formed once on the host.
 struct LoadConsts {
   double two_m, a2, a2_4, c2;

@@ -259,9 +259,9 @@ __device__ __noinline__ void metric_christoffel_fp64(const Consts<float>& C, flo
   out[7] = narrow(gd[3]);
 }
 
-// Node indices of the gathers and deposits (ncell < 2^31).  32 bits save address arithmetic: the push of 2 x 2.1 M particles at
-// 64^3 936 -> 917 us, at 75 x 50 x 91, Q = 3, 1108 -> 1085.  The kernels with area fits keep 64 (WIDE): with 32 their 96-register
-// build went from 5764 to 5966 us (2 x 16.8 M particles, 128^3).
+// Node indices of the gathers and deposits (ncell < 2^31).  32 bits save address arithmetic: the push of 2 x 2.1 M
+// particles at 64^3 936 -> 917 us, at 75 x 50 x 91, Q = 3, 1108 -> 1085.  The kernels with area fits keep 64 (WIDE):
+// with 32 their 96-register build went from 5764 to 5966 us (2 x 16.8 M particles, 128^3).
 template <bool WIDE>
 using NodeIndex = std::conditional_t<WIDE, long long, int>;
 
@@ -392,12 +392,12 @@ __device__ __forceinline__ void accel(const Grid& g, const Fields<T>& F, const C
 //   M = D rho^4, F = 2 m r (rho^4 - num^2), k_K = num / rho^2    (K = 0: num = r x - a y, 1: r y + a x)
 //   M = D r,     F = 2 m (r^2 - z^2)                             (K = 2),
 // so that a node takes three roots and one reciprocal.
-// FP64 operations bound the push in FP64 (one FP64 warp instruction per 16 cycles and SM): 19 a node (15 for K = 2) and 96
-// nodes a particle-step at Q = 2, where one IEEE evaluation of the integrand per node took about 78.
+// FP64 operations bound the push in FP64 (one FP64 warp instruction per 16 cycles and SM): 19 a node (15 for K = 2)
+// and 96 nodes a particle-step at Q = 2, where one IEEE evaluation of the integrand per node took about 78.
 // Measured: push of 1.82 M particles at 64^3, Q = 2: 25.8 -> 10.6 ms (4600 issued FP64 operations a particle-step with
-// 5-operation roots 15.5 ms, 3190 with FastOps64's: 88 % of the pipe's cycles).  Error of a node, rms over 4e5 positions
-// from R = 3.5 to 52 with m = 2, a = 1.8: 6.8e-17 relative, as for one IEEE evaluation (N / sqrt(N M) with N = M + F, of as many
-// operations, 8.7e-17).
+// 5-operation roots 15.5 ms, 3190 with FastOps64's: 88 % of the pipe's cycles).  Error of a node, rms over 4e5
+// positions from R = 3.5 to 52 with m = 2, a = 1.8: 6.8e-17 relative, as for one IEEE evaluation (N / sqrt(N M) with
+// N = M + F, of as many operations, 8.7e-17).
 // r = 0 takes the flat limit 1.
 // A00 = [u,1] x [v,1], A10 = [0,u] x [v,1], A01 = [u,1] x [0,v], A11 = [0,u] x [0,v].
 template <int Q, int K>
@@ -572,8 +572,8 @@ __device__ __forceinline__ float col_coord(const FaceLattice& L, int jb) {
   return fmaf(0.5f * (hi_j - lo_j), gx, 0.5f * (lo_j + hi_j));
 }
 // FP32-mixed: r^2 of one node of a hot cell, and 2 / D with it.  h = p / 2, q, D2 = h^2 + q, their FP32 root r2 (of the
-// p > 0 form) and 2 / D come in; the cancellation-free root where p <= 0, then one FP64 Newton step on the FP64 p64, q64
-// where the policy asks for it, and 2 / D = 2 r^2 / Sigma from the corrected root (near the ring the FP32 D has
+// p > 0 form) and 2 / D come in; the cancellation-free root where p <= 0, then one FP64 Newton step on the FP64 p64,
+// q64 where the policy asks for it, and 2 / D = 2 r^2 / Sigma from the corrected root (near the ring the FP32 D has
 // lost its digits).  Straight-line but for the rare closed form, so that a row's nodes overlap.
 __device__ __forceinline__ void hot_node(const Consts<float>& C, float h, float q, double p64, double q64, float& r2,
                                          float& rD2, unsigned& n64) {
@@ -687,13 +687,14 @@ __device__ __forceinline__ void table_areas(const float4* __restrict__ t, float 
 // FP32 r below r_fp64) go through hot_node before the integrand; r = 0 gives the flat limit.  FP64 p and q are sums of
 // FP64 face, row and column terms, like their FP32 counterparts.
 // (Marked nodes evaluated one at a time after the lattice, each a serial chain of FP64 and integer operations with a
-// warp's lanes out of step: 136 us instead of 114 for 46 K particles at 32^3, a quarter of them near; 128^3 2.95 -> 2.89 ms.)
-// ROWS: rows of the lattice in flight (1 or 2).  FP32-mixed code takes 1: its rows carry the corrections, and with two of them
-// unrolled the far and the FP32-mixed copies of a kernel no longer fit the instruction cache together (no_instruction 2.1
-// cycles per issue, with one row 0.9 before the corrections moved into the rows).  Push stage 2 -> 1: 2 x 2.1 M particles at
-// 64^3 834 -> 791 us, 2 x 1.6 M at 75 x 50 x 91, Q = 3, 918 -> 870, 2 x 15.6 M at 128^3 with fits over steps 4-203 6.75 ->
-// 6.59 ms.  A far-field lattice with 1 loses its overlap (822 and 937 us), and so do the near warps of small launches (2 x 46 K
-// particles at 32^3: 104 -> 107).
+// warp's lanes out of step: 136 us instead of 114 for 46 K particles at 32^3, a quarter of them near; 128^3 2.95 ->
+// 2.89 ms.)
+// ROWS: rows of the lattice in flight (1 or 2).  FP32-mixed code takes 1: its rows carry the corrections, and with
+// two of them unrolled the far and the FP32-mixed copies of a kernel no longer fit the instruction cache together
+// (no_instruction 2.1 cycles per issue, with one row 0.9 before the corrections moved into the rows).  Push stage 2
+// -> 1: 2 x 2.1 M particles at 64^3 834 -> 791 us, 2 x 1.6 M at 75 x 50 x 91, Q = 3, 918 -> 870, 2 x 15.6 M at 128^3
+// with fits over steps 4-203 6.75 -> 6.59 ms.  A far-field lattice with 1 loses its overlap (822 and 937 us), and so
+// do the near warps of small launches (2 x 46 K particles at 32^3: 104 -> 107).
 template <int Q, bool MIXED, bool TAB, bool WIDE, int ROWS>
 __device__ __forceinline__ void deposit_lattice(const Grid& g, const Fields<float>& F, const Consts<float>& C,
                                                 const float x0[3], const float dx[3], float qg, float inv_dt,

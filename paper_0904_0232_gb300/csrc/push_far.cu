@@ -216,15 +216,15 @@ unsigned coprime_multiplier(unsigned n) {
   return m % n;
 }
 
-// A block near the hole takes several times as long as another, so one that starts late leaves the GPU idle but for its SM.
-// The last kTailWaves waves of a spread launch (152 SMs, as many blocks an SM as the kernel is compiled for), at most half of
-// it, take the chunks from both ends of the cell order, the farthest from the hole; the others go before them, permuted.
-// Push stage without / with, us: 2 x 2.1 M particles at 64^3 916 / 840, 2 x 1.6 M at 75 x 50 x 91, Q = 3, 1087 / 927,
-// 2 x 400 K + 2 x 85 K at 64 x 64 x 128 249 / 238, 2 x 16.8 M at 128^3 with fits 5765 / 5715.  4 waves give 860 and 1004 for the
-// first and second, 13 give 854 and 935.
-// Launches in blocks of one warp (small_push) are mostly resident at once: they go from the middle of the cell order outwards, so
-// that the blocks near the hole come first and are dealt to the SMs in turn (2 x 46 K particles at 32^3 111 -> 105 us; a batch
-// of eight runs of 32^3 to 64^3 cells 7.06 -> 6.98 ms for four steps).
+// A block near the hole takes several times as long as another, so one that starts late leaves the GPU idle but for
+// its SM.  The last kTailWaves waves of a spread launch (kSms SMs, as many blocks an SM as the kernel is compiled for),
+// at most half of it, take the chunks from both ends of the cell order, the farthest from the hole; the others go
+// before them, permuted.  Push stage without / with, us: 2 x 2.1 M particles at 64^3 916 / 840, 2 x 1.6 M at
+// 75 x 50 x 91, Q = 3, 1087 / 927, 2 x 400 K + 2 x 85 K at 64 x 64 x 128 249 / 238, 2 x 16.8 M at 128^3 with fits
+// 5765 / 5715.  4 waves give 860 and 1004 for the first and second, 13 give 854 and 935.
+// Launches in blocks of one warp (small_push) are mostly resident at once: they go from the middle of the cell order
+// outwards, so that the blocks near the hole come first and are dealt to the SMs in turn (2 x 46 K particles at 32^3
+// 111 -> 105 us; a batch of eight runs of 32^3 to 64^3 cells 7.06 -> 6.98 ms for four steps).
 constexpr unsigned kTailWaves = 8;
 
 template <int Q, int MINB, bool TILE, bool TAB, int THREADS>
@@ -234,10 +234,12 @@ void launch_select(const Grid& g, const Fields<float>& F, const Particles<float>
   const unsigned nb = blocks_for(P.n, THREADS);
   // groups of `spread` chunks of 128 particles
   const int lg = spread > 0 ? spread_log2(spread * (128 / THREADS)) : 0;
-  const unsigned tail = spread > 0 ? std::min(kTailWaves * (152u * MINB * (128 / THREADS)) / 2 >> lg, (nb >> lg) / 4) : 0u;
+  constexpr unsigned kWave = kSms * MINB * (128 / THREADS);
+  const unsigned tail = spread > 0 ? std::min(kTailWaves * kWave / 2 >> lg, (nb >> lg) / 4) : 0u;
   const unsigned perm = spread == 0 ? 1u : THREADS == 32 ? 0u : spread_multiplier(nb, lg, tail);
-  k_push_select<Q, MINB, TILE, TAB, THREADS><<<nb, THREADS, 0, stream>>>(g, F, P, C, (float)(rn * rn), perm, lg, tail, st,
-                                                                         atab);
+  const float r_near2 = (float)(rn * rn);
+  k_push_select<Q, MINB, TILE, TAB, THREADS>
+      <<<nb, THREADS, 0, stream>>>(g, F, P, C, r_near2, perm, lg, tail, st, atab);
 }
 
 void launch_push_select(const Grid& g, const Fields<float>& F, const Particles<float>& P, const Species& sp,

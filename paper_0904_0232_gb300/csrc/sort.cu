@@ -11,8 +11,9 @@
 // cell the order is not stable.  The bins have to be zero before a sort; the step's zeroing of J takes them along.
 // (Tile sums counted by the histogram, one atomic a warp: sorted particles meet on one tile's address, 4.4 ms for
 // 31 M particles instead of 0.1.)
-// Measured, us per sort of all species (a launch each of seven kernels per species before): 2 x 46 K particles at 32^3 69 -> 27,
-// 4 species with 0.97 M at 64 x 64 x 128 157 -> 62, 2 x 1.8 M at 64^3 150 -> 102, 2 x 15.6 M at 128^3 971 -> 915.
+// Measured, us per sort of all species (a launch each of seven kernels per species before): 2 x 46 K particles at
+// 32^3 69 -> 27, 4 species with 0.97 M at 64 x 64 x 128 157 -> 62, 2 x 1.8 M at 64^3 150 -> 102, 2 x 15.6 M at 128^3
+// 971 -> 915.
 #include <algorithm>
 
 #include "common.cuh"
@@ -327,8 +328,8 @@ void launch_sort(const Grid& g, const SortJobs<T>& jobs, cudaStream_t stream) {
   for (int q = 0; q < jobs.n; ++q) n = std::max(n, jobs.job[q].src.n);
   if (n > 0) k_hist<T><<<dim3(blocks_for(n, 256), jobs.n), 256, 0, stream>>>(jobs, g.ncell);
   k_job_tile_sums<T><<<dim3(ntiles, jobs.n), kScanThreads, 0, stream>>>(jobs, nbins);
-  // beyond 16384 tiles (320^3 cells) the blocks' own sums over the tiles before them, of order ntiles^2, would cost more
-  // than a launch
+  // beyond 16384 tiles (320^3 cells) the blocks' own sums over the tiles before them, of order ntiles^2, would cost
+  // more than a launch
   const bool scanned = ntiles > 16384;
   for (int q = 0; scanned && q < jobs.n; ++q)
     k_scan_tile_sums<<<1, kScanThreads, 0, stream>>>(jobs.job[q].tiles, ntiles);

@@ -1,6 +1,6 @@
-"""A batch over contexts that change between its steps: reloaded with fewer and then more particles (up to the counts of
-its creation), other charges, other stores (a load beyond the capacity moves them) or another launch shape, it steps them
-as they stand.  Each is compared with the same contexts stepped on their own."""
+"""A batch over contexts that change between its steps: reloaded with fewer and then more particles (up to the
+counts of its creation), other charges, other stores (a load beyond the capacity moves them) or another launch
+shape, it steps them as they stand. Each is compared with the same contexts stepped on their own."""
 import numpy as np
 import pytest
 

@@ -1,7 +1,7 @@
-"""FP64 reciprocal, quotient, root and reciprocal root of the FP64 kernels (FastOps64): each within 0.51 units in the last
-place of the exact value (0.5 for a correctly rounded one, and below 2^-7 for the FP32 correction), for arguments over the
-whole range, beside powers of two and perfect squares.  The root of 0 and of subnormals is 0, and CheckedOps64 gives special
-arguments what IEEE gives them."""
+"""FP64 reciprocal, quotient, root and reciprocal root of the FP64 kernels (FastOps64): each within 0.51 units
+in the last place of the exact value (0.5 for a correctly rounded one, and below 2^-7 for the FP32
+correction), for arguments over the whole range, beside powers of two and perfect squares. The root of 0 and
+of subnormals is 0, and CheckedOps64 gives special arguments what IEEE gives them."""
 import ctypes
 import os
 import subprocess

@@ -1,6 +1,6 @@
-"""Steps of a grid with very many planes are enqueued as fast as others: the choice of the field launches' chunks does not
-grow with the number of planes (4 ms a launch at a million planes where each number of chunks is tried, 5 us where each
-length up to 64 is; bound: 2.5 ms a launch)."""
+"""Steps of a grid with very many planes are enqueued as fast as others: the choice of the field launches'
+chunks does not grow with the number of planes (4 ms a launch at a million planes where each number of chunks
+is tried, 5 us where each length up to 64 is; bound: 2.5 ms a launch)."""
 import time
 
 import pytest

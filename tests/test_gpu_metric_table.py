@@ -1,6 +1,6 @@
-"""The metric table of an FP64 context makes room for any other allocation of the library from the same allocator: another
-context's, a batch's own tables, its own after it has been in a batch; also while another thread steps the context.  The
-field takes the same bits with and without it."""
+"""The metric table of an FP64 context makes room for any other allocation of the library from the same
+allocator: another context's, a batch's own tables, its own after it has been in a batch; also while another
+thread steps the context. The field takes the same bits with and without it."""
 import ctypes
 import threading
 

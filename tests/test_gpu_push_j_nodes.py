@@ -62,7 +62,8 @@ def test_nodes_against_the_oracle(references, count, quad, shape):
     J = sim.get_fields()[2]
     r = np.arange(N) - 0.5 * (N - 1)
     R = np.sqrt(r[:, None, None] ** 2 + r[None, :, None] ** 2 + r[None, None, :] ** 2)
-    for lo, hi in ((0.0, 7.0), (7.0, 12.0), (12.0, 60.0)):  # nodes below r_fp64 = 4 m among them, the other near ones, far
+    # nodes below r_fp64 = 4 m among them, the other near ones, far
+    for lo, hi in ((0.0, 7.0), (7.0, 12.0), (12.0, 60.0)):
         skip = mask | (R < lo) | (R >= hi)
         assert np.abs(Jr[:, ~skip]).max() > 0.0
         assert rel_l2_masked(J, Jr, skip) <= TOL["fp32_mixed"]["J"], (lo, rel_l2_masked(J, Jr, skip))

@@ -1,5 +1,6 @@
-"""What the server allocates to admit a run stays within the estimate that it charges, for one to four species, with and
-without particles, in both precisions.  The grids are large enough that a word a cell is more than the estimate's slack."""
+"""What the server allocates to admit a run stays within the estimate that it charges, for one to four
+species, with and without particles, in both precisions. The grids are large enough that a word a cell is more
+than the estimate's slack."""
 import ctypes
 
 import pytest
