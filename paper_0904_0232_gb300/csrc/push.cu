@@ -108,6 +108,11 @@ __global__ void __launch_bounds__(128, 4) k_push_deposit_batch(const InstDesc<do
 __device__ __forceinline__ float from_f64(double v, float) { return narrow(v); }
 __device__ __forceinline__ double from_f64(double v, double) { return v; }
 
+// v > 0, infinity included (from the bits; NaN fails)
+__device__ __forceinline__ bool positive(double v) {
+  return (unsigned long long)__double_as_longlong(v) - 1 < 0x7ff0000000000000ull;
+}
+
 // Is the point inside r <= r_+?  Screened in FP32 (far from the hole nothing else is evaluated), decided by the IEEE
 // evaluation.
 __device__ __forceinline__ bool inside_horizon(const Grid& g, double X, double Y, double Z) {
@@ -166,12 +171,12 @@ __global__ void k_load(const Grid g, const Particles<T> P, long long n, const do
       const double A = 1.0 + f;
       const double S2 = fma(fk, fk, A * fma(-fk, ku, uu));
       // (S^2 beyond FP64: loaded with an infinite u^4, which the first step reports, where the metric is not flat)
-      if (!(S2 > 0.0) || (f == 0.0 && !finite_t(S2))) {
+      if (!positive(S2) || (!finite_t(S2) && !positive(f))) {
         bad |= ST_LOAD_INVALID;
       } else {
-        // raise: u^i = u_i - f k_i (k.u - u_4)
+        // raise: u^i = u_i - f k_i (k.u - u_4), k.u - u_4 = (k.u + S) / (1 + f)
         const double S = CheckedOps64::root(S2);
-        const double fkul = f * (ku - CheckedOps64::div(fk - S, A));
+        const double fkul = f * ((ku + S) * FastOps64::rcp(A));
 #pragma unroll
         for (int q = 0; q < 3; ++q) u[q] = fma(-kk[q], fkul, u[q]);
         u[3] = S;

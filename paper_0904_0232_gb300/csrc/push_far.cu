@@ -218,8 +218,9 @@ unsigned coprime_multiplier(unsigned n) {
 
 // A block near the hole takes several times as long as another, so one that starts late leaves the GPU idle but for
 // its SM.  The last kTailWaves waves of a spread launch (kSms SMs, as many blocks an SM as the kernel is compiled for),
-// at most half of it, take the chunks from both ends of the cell order, the farthest from the hole; the others go
-// before them, permuted.  Push stage without / with, us: 2 x 2.1 M particles at 64^3 916 / 840, 2 x 1.6 M at
+// at most half of it, take the chunks from both ends of the cell order, the farthest from a hole in the middle of the
+// grid (near one end of a z-slab: no worse than one permutation of all, 642 -> 522 us a push of 2 x 1 M particles in
+// half of 64^3 with the other changes of the time); the others go before them, permuted.  Push stage without / with, us: 2 x 2.1 M particles at 64^3 916 / 840, 2 x 1.6 M at
 // 75 x 50 x 91, Q = 3, 1087 / 927, 2 x 400 K + 2 x 85 K at 64 x 64 x 128 249 / 238, 2 x 16.8 M at 128^3 with fits
 // 5765 / 5715.  4 waves give 860 and 1004 for the first and second, 13 give 854 and 935.
 // Launches in blocks of one warp (small_push) are mostly resident at once: they go from the middle of the cell order

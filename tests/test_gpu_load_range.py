@@ -1,5 +1,6 @@
-"""Loads of velocities whose square is beyond FP64.  The completed u^4 is infinite, which the load takes (the first step
-reports it) except for covariant u_i where the metric is flat, whose completion is not a number."""
+"""Velocities at the edge of FP64.  Where the square is beyond it the completed u^4 is infinite, which the load takes (the
+first step reports it) except for covariant u_i where the metric is flat, whose completion is not a number; a u^4 of 0 makes
+the step infinite."""
 import numpy as np
 import pytest
 
@@ -50,3 +51,15 @@ def test_large_velocities_are_completed(umode):
     _, uo, io = sim.get_particles(0)
     want = np.hypot(np.hypot(u[0], u[2]), 1.0)
     assert np.all(np.abs(uo[3, np.argsort(io)] - want) <= 4e-16 * want)
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32_mixed"])
+def test_a_step_without_a_clock_rate_is_reported_as_such(prec):
+    """u^4 = 0, given in full: the proper-time step dt / gamma is infinite and the state after it not finite."""
+    sim = Simulation(N, N, N, 0.0, 0.0, 1.0, 0.4, precision=prec)
+    x = np.full((4, 1), 5.25)
+    x[3] = 0.0
+    sim.load_particles(0, 0.0, 0.0, x, np.array([[0.1], [0.0], [0.0], [0.0]]), np.zeros(1, dtype=np.uint32))
+    with pytest.raises(GrpicError) as err:
+        sim.step(1)
+    assert err.value.code == 5  # GRPIC_ERR_NONFINITE
