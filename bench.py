@@ -49,10 +49,11 @@ FP32_PEAK_NOMINAL = 152 * 128 * 2 * 2.070e9
 # dram__bytes_write of one launch over its particles), from ncu captures at the bench size, per
 # variant (far-field area fits on or off, resident blocks per SM), valid for the push sources whose
 # hash is recorded with them.
-PUSH_TRAFFIC = {"sha": "ec9ca8bbcc078ad0",
-                "bytes_per_particle": {"area_table0_minb4": 1522.5e6 / 15.61e6,
-                                       "area_table0_minb5": 1699.0e6 / 15.61e6,
-                                       "area_table1_minb5": 2594.4e6 / 15.61e6}}
+PUSH_TRAFFIC = {"sha": "4e08eafbf2acecc7",
+                "bytes_per_particle": {"area_table0_minb4": 1523.1e6 / 15.61e6,
+                                       "area_table0_minb5": 1698.9e6 / 15.61e6,
+                                       "area_table1_minb4": 2477.9e6 / 15.61e6,
+                                       "area_table1_minb5": 2595.1e6 / 15.61e6}}
 
 
 def push_variant(tuning):

@@ -26,7 +26,8 @@ namespace {
 __device__ __forceinline__ double to_f64(float v) { return widen(v); }
 __device__ __forceinline__ double to_f64(double v) { return v; }
 
-// The cloud of one particle in FP64: eight atomics.
+// The cloud of one particle in FP64: eight atomics.  The weights are formed without the charge, so that their rounding is
+// the same for particles of opposite charge at one place (a pair plasma's start) and cancels with it.
 template <typename T>
 __device__ __forceinline__ void cloud64(const Particles<T>& P, long long i, double q, int nx, int ny, int nz,
                                         double inv_c, bool with_gamma, double* __restrict__ rho) {
@@ -43,15 +44,15 @@ __device__ __forceinline__ void cloud64(const Particles<T>& P, long long i, doub
     c[ax] = k;
   }
   const double qq = with_gamma ? q * to_f64(P.u[3][i]) * inv_c : q;
-  const double qx[2] = {qq * (1.0 - w[0]), qq * w[0]}, wy[2] = {1.0 - w[1], w[1]}, wz[2] = {1.0 - w[2], w[2]};
+  const double wx[2] = {1.0 - w[0], w[0]}, wy[2] = {1.0 - w[1], w[1]}, wz[2] = {1.0 - w[2], w[2]};
   double* r = rho + ((long long)c[2] * ny + c[1]) * nx + c[0];
 #pragma unroll
   for (int dj = 0; dj < 2; ++dj)
 #pragma unroll
     for (int di = 0; di < 2; ++di) {
-      const double qxy = qx[di] * wy[dj];
+      const double wxy = wx[di] * wy[dj];
 #pragma unroll
-      for (int dk = 0; dk < 2; ++dk) atomicAdd(r + (long long)dk * nx * ny + dj * nx + di, qxy * wz[dk]);
+      for (int dk = 0; dk < 2; ++dk) atomicAdd(r + (long long)dk * nx * ny + dj * nx + di, qq * (wxy * wz[dk]));
     }
 }
 
