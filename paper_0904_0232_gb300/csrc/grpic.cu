@@ -128,8 +128,8 @@ struct TableOwners {
   std::vector<grpic_ctx*> list;
 };
 TableOwners& table_owners() {
-  static TableOwners o;
-  return o;
+  static TableOwners* const o = new TableOwners();  // (never destroyed: contexts may be, after static objects)
+  return *o;
 }
 
 bool same_allocator(const grpic_ctx* c, grpic_alloc_fn alloc, void* user) {
